@@ -485,7 +485,7 @@ def run_ours(args):
     achieved = (flops / args.steps) / (force_ms / force_launches / 1e3) / 1e12 if force_ms > 0 else None
     f32 = prm["precision"] == 1
     peak = fp32_peak_tflops(SM_MAX_MHZ) if f32 else peak64_measured
-    roofline = {"kernel": "k_force32" if f32 else "k_force64", "bound": "alu" if f32 else "fp64",
+    roofline = {"kernel": "k_force32" if f32 else "k_sum64", "bound": "alu" if f32 else "fp64",
                 "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak if achieved else None,
                 "traffic": recorded_traffic("k_force32", args.workload, n, prm.get("key_frame", 0),
                                             ctx.bh_get_tuning()) if prm["precision"] == 1 else None,
@@ -550,7 +550,7 @@ def run_ours(args):
         # brings the ill-conditioned particles to the gate)
         refine_ms = stages.get("refine", {}).get("ms_per_step", 0.0)
         rate32r = (pp + pc) / args.steps / ((force_ms / force_launches + refine_ms) / 1e3)
-        fp64 = {"kernel": "k_force64", "kernel_ms": ms64, "interactions_per_s": rate64,
+        fp64 = {"kernel": "k_sum64", "kernel_ms": ms64, "interactions_per_s": rate64,
                 "fp32_kernel_interactions_per_s": rate32, "fp32_with_refinement_interactions_per_s": rate32r,
                 "fp32_over_fp64": rate32r / rate64}
         for x in (ctxe, ctx32):

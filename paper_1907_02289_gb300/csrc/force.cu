@@ -7,12 +7,12 @@
 //   list cells:     centre-of-mass monopole (Sec. 5.1) and, for order 2, the
 //                   traceless quadrupole about the centre of mass.
 //
-// This file: the plain FP64 kernel (absolute coordinates, one warp per group,
-// list entries staged 32 at a time in shared memory and broadcast to the
-// lanes), the per-evaluation FP32 hi/lo split used by the FP32 kernel
-// (force32.cu), and the dispatcher.  Pairs that may be in contact
-// (r^2 <= r_coll^2 up to rounding) are re-evaluated in the oracle's exact
-// operation order, so the r <= r_coll decision is the oracle's.
+// This file: the plain FP64 kernels (absolute coordinates) of the force and
+// of the self-gravity potential, the per-evaluation FP32 hi/lo split used by
+// the FP32 kernel (force32.cu), and the dispatcher.  Pairs that may be in
+// contact (r^2 <= r_coll^2 up to rounding) are re-evaluated in the oracle's
+// exact operation order, so the r <= r_coll decision is the oracle's.
+#include <algorithm>
 #include <cmath>
 
 #include "force_common.cuh"
@@ -23,220 +23,290 @@ namespace {
 
 constexpr int kWarps = 4;
 
-struct __align__(32) D4 {
+struct __align__(16) D4 {
     double x, y, z, w;
 };
 
 struct Smem64 {
-    D4 pj[32];
-    uint32_t jid[32];
-    double cl[32][10];  // M, c3, Q6
+    union {
+        struct {
+            D4 pj[32];
+            uint32_t jid[32];
+        } p;
+        double cl[32][10];  // M, c3, Q6
+    };
 };
 
-__global__ void __launch_bounds__(32 * kWarps) k_force64(
-    int64_t ng, const unsigned long long* __restrict__ dng, const unsigned long long* __restrict__ abort,
-    const int32_t* __restrict__ groups, const uint32_t* __restrict__ begin,
-    const uint32_t* __restrict__ end, const int64_t* __restrict__ jj_off, const uint32_t* __restrict__ JJ,
-    const int64_t* __restrict__ pc_off, const int32_t* __restrict__ C, const double* __restrict__ x,
-    const double* __restrict__ y, const double* __restrict__ z, const double* __restrict__ vx,
-    const double* __restrict__ vy, const double* __restrict__ vz, const double* __restrict__ m,
-    const double* __restrict__ M, const double* __restrict__ cx, const double* __restrict__ cy,
-    const double* __restrict__ cz, const double* __restrict__ Q, ForceParams fp, bool add_central,
-    double* __restrict__ ax, double* __restrict__ ay, double* __restrict__ az, uint32_t n, int64_t nn,
-    int* status) {
-    __shared__ Smem64 sm[kWarps];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int64_t k = (int64_t)blockIdx.x * kWarps + w;
-    if (dng) ng = min(ng, (int64_t)*dng);  // device-sized list build
-    if (k >= ng || (abort && *abort)) return;  // (abort: that build outgrew its buffers)
-    Smem64& S = sm[w];
-    const int32_t g = groups[k];
-    const uint32_t b = begin[g], e = end[g];
-    const int64_t j0 = jj_off[k], j1 = jj_off[k + 1], c0 = pc_off[k], c1 = pc_off[k + 1];
-    for (uint32_t i0 = b; i0 < e; i0 += 32) {
-        const uint32_t i = i0 + lane;
-        const bool valid = i < e;
-        const uint32_t ii = valid ? i : b;
-        const double xi = x[ii], yi = y[ii], zi = z[ii];
-        double ag[3] = {0.0, 0.0, 0.0}, an[3] = {0.0, 0.0, 0.0};
-        // the group's own particles first (segment 0), then the other list particles
-        for (int seg = 0; seg < 2; ++seg) {
-            const int64_t s0 = seg == 0 ? (int64_t)b : j0, s1 = seg == 0 ? (int64_t)e : j1;
-            for (int64_t t0 = s0; t0 < s1; t0 += 32) {
-                const int nt = (int)min((int64_t)32, s1 - t0);
-                if (lane < nt) {
-                    uint32_t j = seg == 0 ? (uint32_t)(t0 + lane) : JJ[t0 + lane];
-                    if (j >= n) {
-                        atomicOr(status, kStatBounds);
-                        j = b;
-                    }
-                    S.pj[lane] = D4{x[j], y[j], z[j], m[j]};
-                    S.jid[lane] = j;
-                }
-                __syncwarp();
-                for (int q = 0; q < nt; ++q) {
-                    const D4 pj = S.pj[q];
-                    const double dx = pj.x - xi, dy = pj.y - yi, dz = pj.z - zi;
-                    const double r2 = dx * dx + dy * dy + dz * dz;
-                    if (r2 > fp.rc2_hi) {
-                        const double s2 = r2 + fp.eps2;
-                        const double ri = rsqrt(s2);
-                        const double f = pj.w * ri * ri * ri;
-                        ag[0] += f * dx;
-                        ag[1] += f * dy;
-                        ag[2] += f * dz;
-                    } else {
-                        const uint32_t j = S.jid[q];
-                        if (valid && j != i)
-                            exact_pair64(fp, xi, yi, zi, vx[ii], vy[ii], vz[ii], m[ii], pj.x, pj.y, pj.z, vx[j],
-                                         vy[j], vz[j], pj.w, an);
-                    }
-                }
-                __syncwarp();
-            }
-        }
-        for (int64_t t0 = c0; t0 < c1; t0 += 32) {
-            const int nt = (int)min((int64_t)32, c1 - t0);
-            if (lane < nt) {
-                int32_t cc = C[t0 + lane];
-                if (cc < 0 || cc >= nn) {
-                    atomicOr(status, kStatBounds);
-                    cc = 0;
-                }
-                S.cl[lane][0] = M[cc];
-                S.cl[lane][1] = cx[cc];
-                S.cl[lane][2] = cy[cc];
-                S.cl[lane][3] = cz[cc];
-                if (fp.order >= 2)
-#pragma unroll
-                    for (int a = 0; a < 6; ++a) S.cl[lane][4 + a] = Q[6 * (int64_t)cc + a];
-            }
-            __syncwarp();
-            for (int q = 0; q < nt; ++q) {
-                const double* cl = S.cl[q];
-                const double dx = cl[1] - xi, dy = cl[2] - yi, dz = cl[3] - zi;  // d = c - x_i = -R
-                const double R2 = dx * dx + dy * dy + dz * dz + fp.eps2;
-                const double ri = rsqrt(R2);
-                const double ri2 = ri * ri;
-                const double ri3 = ri * ri2;
-                const double mono = cl[0] * ri3;
-                ag[0] += mono * dx;
-                ag[1] += mono * dy;
-                ag[2] += mono * dz;
-                if (fp.order >= 2) {
-                    const double qx = cl[4] * dx + cl[7] * dy + cl[8] * dz;
-                    const double qy = cl[7] * dx + cl[5] * dy + cl[9] * dz;
-                    const double qz = cl[8] * dx + cl[9] * dy + cl[6] * dz;
-                    const double dqd = dx * qx + dy * qy + dz * qz;
-                    const double ri5 = ri3 * ri2;
-                    const double s = 2.5 * dqd * ri2;
-                    ag[0] += ri5 * (s * dx - qx);
-                    ag[1] += ri5 * (s * dy - qy);
-                    ag[2] += ri5 * (s * dz - qz);
-                }
-            }
-            __syncwarp();
-        }
-        if (valid) {
-            double a[3] = {fp.G * ag[0] + an[0], fp.G * ag[1] + an[1], fp.G * ag[2] + an[2]};
-            if (add_central) central64(fp.GMc, xi, yi, zi, a);
-            ax[i] = a[0];
-            ay[i] = a[1];
-            az[i] = a[2];
-        }
-    }
+struct Args64 {
+    int64_t ng;
+    const unsigned long long* dng;    // device group count (device-sized list builds; NULL: ng)
+    const unsigned long long* abort;  // nonzero: that build outgrew its buffers, nothing is done
+    const int32_t* groups;
+    const uint32_t *begin, *end;
+    const int64_t* jj_off;
+    const uint32_t* JJ;
+    const int64_t* pc_off;
+    const int32_t* C;
+    const double *x, *y, *z, *vx, *vy, *vz, *m;
+    const double *M, *cx, *cy, *cz, *Q;
+    ForceParams fp;
+    bool add_central;
+    double *ax, *ay, *az;  // force
+    double* phi;           // potential
+    uint32_t n;
+    int64_t nn;
+    int* status;
+    int lcap, full;  // items: log2 of the largest, and how many of those a group of n_g has
+};
+
+// ---- 1 / sqrt(s) -----------------------------------------------------------
+// The FP64 pipe (2 lanes per clock and SM: one warp instruction takes it 16
+// cycles) bounds these kernels; the integer and FP32 pipes idle beside it.
+// So the inverse square root and its powers are taken from a hardware
+// estimate y0 (21 significant bits) by the binomial series of
+// s^(-k/2) = y0^k (1 - e)^(-k/2), e = 1 - s y0^2 (|e| <= 2^-18 or so):
+//   (1 - e)^(-1/2) = 1 + e/2 + 3/8 e^2 + O(e^3),
+//   (1 - e)^(-3/2) = 1 + 3/2 e + 15/8 e^2 + O(e^3)
+// with y0^2 exact (42 bits, squared as an integer), e exact to one rounding
+// (FMA), and the e^2 term, below 2^-36, in FP32: what is left out is below
+// 2^-53 of the result.  One FP64 comparison, conversion or product saved is
+// worth 30 integer instructions here.
+struct RSeed {
+    double y0, a, e;  // estimate, its square, 1 - s y0^2
+    double q;         // kq e^2
+};
+
+// Whether s is far enough from overflow and underflow for the series (its
+// powers included); else the callers take the library functions.
+__device__ __forceinline__ bool rseed_ok(double s) {
+    return (uint32_t)((__double2hiint(s) >> 20) - 423) < 1200u;  // 2^-600 <= s < 2^600
 }
 
+__device__ __forceinline__ RSeed rseed(double s, float kq) {
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(s));
+    const uint32_t h = (uint32_t)__double2hiint(y);
+    RSeed r;
+    r.y0 = __hiloint2double((int)h, 0);
+    const uint32_t m = (h & 0xfffffu) | 0x100000u;
+    const uint64_t sq = (uint64_t)m * m;  // in [2^40, 2^42)
+    const uint32_t p = (uint32_t)(sq >> 41);
+    r.a = __longlong_as_double((long long)(((uint64_t)(2u * (h >> 20) - 1024u + p) << 52) + (sq << (12 - p))));
+    r.e = fma(-s, r.a, 1.0);
+    // kq e^2 in FP32, by integer conversions (the FP64 ones take the FP64 pipe);
+    // an e below 2^-126 counts as that
+    const uint32_t eh = max((uint32_t)__double2hiint(r.e) & 0x7fffffffu, 897u << 20);
+    const float ef = __uint_as_float((eh - (896u << 20)) << 3);
+    const uint32_t qb = __float_as_uint(__fmul_rn(__fmul_rn(kq, ef), ef));
+    r.q = __hiloint2double((int)((qb >> 3) + (896u << 20)), (int)(qb << 29));
+    return r;
+}
 
-// Self-gravity potential of every particle over its group's lists, FP64:
-// the potential of the gravity Eq. (1) applies (held at its r_coll value
-// inside r_coll) for the group's own particles (j != i) and the list
-// particles, then the monopole + quadrupole potential of the list cells.
-// Same staging as k_force64.
-__global__ void __launch_bounds__(32 * kWarps) k_potential64(
-    int64_t ng, const int32_t* __restrict__ groups, const uint32_t* __restrict__ begin,
-    const uint32_t* __restrict__ end, const int64_t* __restrict__ jj_off, const uint32_t* __restrict__ JJ,
-    const int64_t* __restrict__ pc_off, const int32_t* __restrict__ C, const double* __restrict__ x,
-    const double* __restrict__ y, const double* __restrict__ z, const double* __restrict__ m,
-    const double* __restrict__ M, const double* __restrict__ cx, const double* __restrict__ cy,
-    const double* __restrict__ cz, const double* __restrict__ Q, ForceParams fp, double* __restrict__ phi,
-    uint32_t n, int64_t nn, int* status) {
-    __shared__ Smem64 sm[kWarps];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int64_t k = (int64_t)blockIdx.x * kWarps + w;
-    if (k >= ng) return;
-    Smem64& S = sm[w];
-    const int32_t g = groups[k];
-    const uint32_t b = begin[g], e = end[g];
-    const int64_t j0 = jj_off[k], j1 = jj_off[k + 1], c0 = pc_off[k], c1 = pc_off[k + 1];
-    const double s2c = fp.rc2 + fp.eps2, sc = sqrt(s2c);
-    for (uint32_t i0 = b; i0 < e; i0 += 32) {
-        const uint32_t i = i0 + lane;
-        const bool valid = i < e;
-        const uint32_t ii = valid ? i : b;
-        const double xi = x[ii], yi = y[ii], zi = z[ii];
-        double acc = 0.0;
-        for (int seg = 0; seg < 2; ++seg) {
-            const int64_t s0 = seg == 0 ? (int64_t)b : j0, s1 = seg == 0 ? (int64_t)e : j1;
-            for (int64_t t0 = s0; t0 < s1; t0 += 32) {
-                const int nt = (int)min((int64_t)32, s1 - t0);
-                if (lane < nt) {
-                    uint32_t j = seg == 0 ? (uint32_t)(t0 + lane) : JJ[t0 + lane];
-                    if (j >= n) {
-                        atomicOr(status, kStatBounds);
-                        j = b;
+// m s^(-3/2)
+__device__ __forceinline__ double inv_cube(double m, double s) {
+    if (!rseed_ok(s)) {
+        const double ri = rsqrt(s);
+        return m * ri * ri * ri;
+    }
+    const RSeed r = rseed(s, 1.875f);
+    const double f0 = (m * r.y0) * r.a;
+    return fma(f0, fma(1.5, r.e, r.q), f0);
+}
+
+// s^(-1/2)
+__device__ __forceinline__ double inv_sqrt(double s) {
+    if (!rseed_ok(s)) return rsqrt(s);
+    const RSeed r = rseed(s, 0.375f);
+    return fma(r.y0, fma(0.5, r.e, r.q), r.y0);
+}
+
+// ---- the kernels -----------------------------------------------------------
+// Sum over the group's own particles and its list particles, then its list
+// cells, for one item of a group: 2^k of its particles whose list is split
+// over 32 / 2^k lanes each.  A group of n_i particles is cut along the binary
+// digits of n_i (62 = 32 + 16 + 8 + 4 + 2), so every lane has a particle and
+// the FP64 pipe does no work for padding (32-lane chunks left 26% of it idle
+// for the 2^20 ring's groups, more than half for groups of 8 to 20); with few
+// particles the largest item is cut down too, so that all SMs have work.  A
+// warp per item; list entries staged 32 at a time in shared memory, the next
+// 32 loaded while these are evaluated.  Measured against one warp per group
+// in 32-lane chunks with rsqrt(), sqrt() and divisions: force evaluation of a
+// 2^17 ring 6.07 -> 2.78 ms (62.8e6 -> 38.8e6 FP64 warp instructions, pipe 53
+// -> 71% busy), of the 2^20 ring 39.9 -> 24.4 ms, potential of a 2^18 ring
+// 13.5 -> 4.2 ms, a 4096-particle cube's evaluation 3.30 -> 1.28 ms in all.
+template <bool POT, int ORDER, bool EPS>
+__device__ __forceinline__ void item64(const Args64& A, Smem64& S, int64_t k, uint32_t b, uint32_t e, uint32_t i0,
+                                       int lsz, int lane) {
+    const ForceParams& fp = A.fp;
+    const int nsp = 32 >> lsz;
+    const int s = lane >> lsz;
+    const uint32_t i = i0 + (uint32_t)(lane & ((1 << lsz) - 1));
+    const double xi = A.x[i], yi = A.y[i], zi = A.z[i];
+    double g0 = 0.0, g1 = 0.0, g2 = 0.0;     // G-free sums (potential: g0)
+    double an[3] = {0.0, 0.0, 0.0};          // pairs evaluated exactly, G included
+    const long long rc2_hi = __double_as_longlong(fp.rc2_hi), rc2 = __double_as_longlong(fp.rc2);
+    const double inv_sc = POT && fp.rc2 + fp.eps2 > 0.0 ? 1.0 / sqrt(fp.rc2 + fp.eps2) : 0.0;
+    const double half_sc3 = 0.5 * inv_sc * inv_sc * inv_sc;
+    {
+        const int64_t j0 = A.jj_off[k], own = (int64_t)(e - b), tot = own + (A.jj_off[k + 1] - j0);
+        auto index = [&](int64_t t) -> uint32_t {
+            if (t < own) return b + (uint32_t)t;
+            if (t >= tot) return b;
+            const uint32_t j = A.JJ[j0 + t - own];
+            if (j < A.n) return j;
+            atomicOr(A.status, kStatBounds);
+            return b;
+        };
+        auto load = [&](uint32_t j) { return D4{A.x[j], A.y[j], A.z[j], A.m[j]}; };
+        uint32_t j = index(lane), jn = index(lane + 32);
+        D4 d = load(j);
+        for (int64_t t0 = 0; t0 < tot; t0 += 32) {
+            S.p.pj[lane] = d;
+            S.p.jid[lane] = j;
+            __syncwarp();
+            j = jn;
+            d = load(j);
+            jn = index(t0 + 64 + lane);
+            const int nt = (int)min((int64_t)32, tot - t0);
+            for (int q = s; q < nt; q += nsp) {
+                const D4 pj = S.p.pj[q];
+                const double dx = pj.x - xi, dy = pj.y - yi, dz = pj.z - zi;
+                const double r2 = dx * dx + dy * dy + dz * dz;
+                const long long rb = __double_as_longlong(r2);  // r2 >= 0: orders as its bits
+                if (POT) {
+                    if (rb > rc2) {
+                        g0 = fma(-pj.w, inv_sqrt(EPS ? r2 + fp.eps2 : r2), g0);
+                    } else if (rb != 0 && S.p.jid[q] != i) {
+                        g0 -= pj.w * inv_sc + pj.w * (fp.rc2 - r2) * half_sc3;
                     }
-                    S.pj[lane] = D4{x[j], y[j], z[j], m[j]};
-                    S.jid[lane] = j;
+                } else {
+                    if (rb > rc2_hi) {
+                        const double f = inv_cube(pj.w, EPS ? r2 + fp.eps2 : r2);
+                        g0 = fma(f, dx, g0);
+                        g1 = fma(f, dy, g1);
+                        g2 = fma(f, dz, g2);
+                    } else {
+                        const uint32_t jq = S.p.jid[q];
+                        if (jq != i)
+                            exact_pair64(fp, xi, yi, zi, A.vx[i], A.vy[i], A.vz[i], A.m[i], pj.x, pj.y, pj.z, A.vx[jq],
+                                         A.vy[jq], A.vz[jq], pj.w, an);
+                    }
                 }
-                __syncwarp();
-                for (int q = 0; q < nt; ++q) {
-                    const D4 pj = S.pj[q];
-                    if (S.jid[q] == i) continue;
-                    const double dx = pj.x - xi, dy = pj.y - yi, dz = pj.z - zi;
-                    const double r2 = dx * dx + dy * dy + dz * dz;
-                    if (r2 == 0.0) continue;
-                    if (r2 > fp.rc2)
-                        acc -= pj.w / sqrt(r2 + fp.eps2);
-                    else
-                        acc -= pj.w / sc + pj.w * (fp.rc2 - r2) / (2.0 * s2c * sc);
-                }
-                __syncwarp();
             }
+            __syncwarp();
         }
-        for (int64_t t0 = c0; t0 < c1; t0 += 32) {
-            const int nt = (int)min((int64_t)32, c1 - t0);
-            if (lane < nt) {
-                int32_t cc = C[t0 + lane];
-                if (cc < 0 || cc >= nn) {
-                    atomicOr(status, kStatBounds);
-                    cc = 0;
-                }
-                S.cl[lane][0] = M[cc];
-                S.cl[lane][1] = cx[cc];
-                S.cl[lane][2] = cy[cc];
-                S.cl[lane][3] = cz[cc];
-                if (fp.order >= 2)
+    }
+    {
+        const int64_t c0 = A.pc_off[k], c1 = A.pc_off[k + 1];
+        constexpr int NC = ORDER >= 2 ? 10 : 4;
+        auto index = [&](int64_t t) -> int32_t {
+            if (t >= c1) return 0;
+            const int32_t cc = A.C[t];
+            if (cc >= 0 && cc < A.nn) return cc;
+            atomicOr(A.status, kStatBounds);
+            return 0;
+        };
+        double v[NC];
+        auto load = [&](int32_t cc) {
+            v[0] = A.M[cc];
+            v[1] = A.cx[cc];
+            v[2] = A.cy[cc];
+            v[3] = A.cz[cc];
+            if (ORDER >= 2) {
+                const double2* Q = reinterpret_cast<const double2*>(A.Q) + 3 * (int64_t)cc;
 #pragma unroll
-                    for (int a = 0; a < 6; ++a) S.cl[lane][4 + a] = Q[6 * (int64_t)cc + a];
+                for (int a = 0; a < 3; ++a) {
+                    const double2 u = Q[a];
+                    v[NC - 6 + 2 * a] = u.x;
+                    v[NC - 5 + 2 * a] = u.y;
+                }
             }
+        };
+        int32_t cn = index(c0 + lane);
+        load(cn);
+        cn = index(c0 + 32 + lane);
+        for (int64_t t0 = c0; t0 < c1; t0 += 32) {
+#pragma unroll
+            for (int a = 0; a < NC; ++a) S.cl[lane][a] = v[a];
             __syncwarp();
-            for (int q = 0; q < nt; ++q) {
+            load(cn);
+            cn = index(t0 + 64 + lane);
+            const int nt = (int)min((int64_t)32, c1 - t0);
+            for (int q = s; q < nt; q += nsp) {
                 const double* cl = S.cl[q];
-                const double Rx = xi - cl[1], Ry = yi - cl[2], Rz = zi - cl[3];
-                const double R2 = Rx * Rx + Ry * Ry + Rz * Rz + fp.eps2;
-                const double R = sqrt(R2);
-                acc -= cl[0] / R;
-                if (fp.order >= 2) {
-                    const double qx = cl[4] * Rx + cl[7] * Ry + cl[8] * Rz;
-                    const double qy = cl[7] * Rx + cl[5] * Ry + cl[9] * Rz;
-                    const double qz = cl[8] * Rx + cl[9] * Ry + cl[6] * Rz;
-                    acc -= 0.5 * (Rx * qx + Ry * qy + Rz * qz) / (R2 * R2 * R);
+                const double dx = cl[1] - xi, dy = cl[2] - yi, dz = cl[3] - zi;  // d = c - x_i = -R
+                const double R2 = EPS ? fma(dx, dx, fma(dy, dy, fma(dz, dz, fp.eps2))) : dx * dx + dy * dy + dz * dz;
+                if (ORDER < 2) {
+                    if (POT) {
+                        g0 = fma(-cl[0], inv_sqrt(R2), g0);
+                    } else {
+                        const double f = inv_cube(cl[0], R2);
+                        g0 = fma(f, dx, g0);
+                        g1 = fma(f, dy, g1);
+                        g2 = fma(f, dz, g2);
+                    }
+                    continue;
+                }
+                const double ri = inv_sqrt(R2), ri2 = ri * ri;
+                const double qx = cl[NC - 6] * dx + cl[NC - 3] * dy + cl[NC - 2] * dz;
+                const double qy = cl[NC - 3] * dx + cl[NC - 5] * dy + cl[NC - 1] * dz;
+                const double qz = cl[NC - 2] * dx + cl[NC - 1] * dy + cl[NC - 4] * dz;
+                const double dqd = dx * qx + dy * qy + dz * qz;
+                if (POT) {  // -(M + (d.Qd) / (2 R^4)) / R
+                    g0 = fma(-ri, fma(0.5 * dqd, ri2 * ri2, cl[0]), g0);
+                } else {    // ((M R^2 + 5/2 (d.Qd) / R^2) d - Q d) / R^5
+                    const double ri5 = ri2 * ri2 * ri;
+                    const double w = fma(2.5, dqd * ri2, cl[0] * R2);
+                    g0 = fma(ri5, fma(w, dx, -qx), g0);
+                    g1 = fma(ri5, fma(w, dy, -qy), g1);
+                    g2 = fma(ri5, fma(w, dz, -qz), g2);
                 }
             }
             __syncwarp();
         }
-        if (valid) phi[i] = fp.G * acc;
+    }
+    if (POT) {
+        for (int o = 1 << lsz; o < 32; o <<= 1) g0 += __shfl_xor_sync(0xffffffffu, g0, o);
+        if (s == 0) A.phi[i] = fp.G * g0;
+        return;
+    }
+    double a[3] = {fma(fp.G, g0, an[0]), fma(fp.G, g1, an[1]), fma(fp.G, g2, an[2])};
+    for (int o = 1 << lsz; o < 32; o <<= 1)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) a[c] += __shfl_xor_sync(0xffffffffu, a[c], o);
+    if (s != 0) return;
+    if (A.add_central) central64(fp.GMc, xi, yi, zi, a);
+    A.ax[i] = a[0];
+    A.ay[i] = a[1];
+    A.az[i] = a[2];
+}
+
+template <bool POT, int ORDER, bool EPS>
+__global__ void __launch_bounds__(32 * kWarps) k_sum64(const Args64 A) {
+    __shared__ Smem64 sm[kWarps];
+    if (A.abort && *A.abort) return;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int64_t ng = A.dng ? min(A.ng, (int64_t)*A.dng) : A.ng;
+    const int slots = A.full + A.lcap;
+    // item u = (group, slot): slots below `full` take the group's whole items
+    // of 2^lcap particles (every full-th one), the others the one item of
+    // each smaller power of two that the size's binary digits ask for
+    for (int64_t u = (int64_t)blockIdx.x * kWarps + w; u < ng * slots; u += (int64_t)gridDim.x * kWarps) {
+        const int64_t k = u / slots;
+        const int slot = (int)(u - k * slots);
+        const int32_t g = A.groups[k];
+        const uint32_t b = A.begin[g], e = A.end[g], ni = e - b;
+        if (slot < A.full) {
+            for (uint32_t c = slot; c < ni >> A.lcap; c += A.full) {
+                item64<POT, ORDER, EPS>(A, sm[w], k, b, e, b + (c << A.lcap), A.lcap, lane);
+                __syncwarp();
+            }
+        } else {
+            const int bit = slot - A.full;
+            if ((ni >> bit) & 1u)
+                item64<POT, ORDER, EPS>(A, sm[w], k, b, e, b + ((ni >> (bit + 1)) << (bit + 1)), bit, lane);
+            __syncwarp();
+        }
     }
 }
 
@@ -323,21 +393,72 @@ int stage_split(Ctx* c, const bh_particles* p) {
     return BH_OK;
 }
 
+namespace {
+
+Args64 args64(const Ctx* c, const bh_particles* p, const ForceParams& fp) {
+    Args64 A = {};
+    A.ng = c->n_groups;
+    A.groups = c->groups.p;
+    A.begin = c->begin.p;
+    A.end = c->end.p;
+    A.jj_off = c->cnt_j.p;
+    A.JJ = c->JJ.p;
+    A.pc_off = c->cnt_c.p;
+    A.C = c->C.p;
+    A.x = p->x;
+    A.y = p->y;
+    A.z = p->z;
+    A.vx = p->vx;
+    A.vy = p->vy;
+    A.vz = p->vz;
+    A.m = p->m;
+    A.M = c->M.p;
+    A.cx = c->cx.p;
+    A.cy = c->cy.p;
+    A.cz = c->cz.p;
+    A.Q = c->Q.p;
+    A.fp = fp;
+    A.n = (uint32_t)c->n;
+    A.nn = c->n_nodes;
+    A.status = c->d_status;
+    return A;
+}
+
+template <bool POT>
+int launch_sum64(Ctx* c, Args64& A) {
+    // largest item: 32 particles, or fewer when that gives less than 8 items
+    // per SM (each item then splits its lists over more lanes)
+    A.lcap = 5;
+    while (A.lcap > 0 && (c->n >> A.lcap) < 8 * (int64_t)c->num_sms) --A.lcap;
+    A.full = std::max(1, c->prm.n_g >> A.lcap);
+    // (device-sized build: the expected groups; the kernel strides over more)
+    const int64_t ng = A.dng ? std::min(A.ng, std::max<int64_t>(c->dev_slots, 1)) : A.ng;
+    const int64_t nb = (ng * (A.full + A.lcap) + kWarps - 1) / kWarps;
+    const unsigned grid = (unsigned)std::min<int64_t>(nb, (int64_t)1 << 30);
+    const bool eps = A.fp.eps2 != 0.0;
+    auto kern = A.fp.order >= 2 ? (eps ? k_sum64<POT, 2, true> : k_sum64<POT, 2, false>)
+                                : (eps ? k_sum64<POT, 1, true> : k_sum64<POT, 1, false>);
+    kern<<<grid, 32 * kWarps, 0, c->stream>>>(A);
+    BH_LAUNCH(c);
+    return BH_OK;
+}
+
+}  // namespace
+
 int stage_force(Ctx* c, bh_particles* p, bool add_central) {
-    const int64_t ng = c->n_groups;
     const ForceParams fp = force_params(c);
     add_central = add_central && c->prm.M_central != 0.0;
     if (c->prm.precision == BH_PREC_FP64) {
-        const unsigned nb = blocks_for(ng, kWarps);
+        Args64 A = args64(c, p, fp);
+        A.dng = c->dev_build ? c->d_sz + kSzNg : nullptr;
+        A.abort = c->abort;
+        A.add_central = add_central;
+        A.ax = p->ax;
+        A.ay = p->ay;
+        A.az = p->az;
         BH_TRY(timing_begin(c));
         BH_TRY(stage_begin(c, BH_STAGE_FORCE));
-        const unsigned long long* dng = c->dev_build ? c->d_sz + kSzNg : nullptr;
-        k_force64<<<nb, 32 * kWarps, 0, c->stream>>>(ng, dng, c->abort, c->groups.p, c->begin.p, c->end.p, c->cnt_j.p, c->JJ.p,
-                                                     c->cnt_c.p, c->C.p, p->x, p->y, p->z, p->vx, p->vy, p->vz,
-                                                     p->m, c->M.p, c->cx.p, c->cy.p, c->cz.p, c->Q.p, fp,
-                                                     add_central, p->ax, p->ay, p->az, (uint32_t)c->n,
-                                                     c->n_nodes, c->d_status);
-        BH_LAUNCH(c);
+        BH_TRY(launch_sum64<false>(c, A));
         BH_TRY(stage_end(c));
         return timing_end(c);
     }
@@ -352,10 +473,9 @@ int stage_potential(Ctx* c, const bh_particles* p, double* phi, double* W) {
         phi = c->pot.p;
     }
     const ForceParams fp = force_params(c);
-    k_potential64<<<blocks_for(c->n_groups, kWarps), 32 * kWarps, 0, c->stream>>>(
-        c->n_groups, c->groups.p, c->begin.p, c->end.p, c->cnt_j.p, c->JJ.p, c->cnt_c.p, c->C.p, p->x, p->y, p->z,
-        p->m, c->M.p, c->cx.p, c->cy.p, c->cz.p, c->Q.p, fp, phi, (uint32_t)c->n, c->n_nodes, c->d_status);
-    BH_LAUNCH(c);
+    Args64 A = args64(c, p, fp);
+    A.phi = phi;
+    BH_TRY(launch_sum64<true>(c, A));
     if (W) {
         BH_TRY(grow(c, c->diag, (size_t)kWBlocks + 1, "potential energy sums"));
         k_wsum_partial<<<kWBlocks, kWThreads, 0, c->stream>>>(c->n, p->m, phi, c->diag.p);
