@@ -56,8 +56,21 @@ struct Args64 {
     uint32_t n;
     int64_t nn;
     int* status;
-    int lcap, full;  // items: log2 of the largest, and how many of those a group of n_g has
+    const int64_t* off;    // patches: particle offsets (np + 1)
+    int np, n_g, slots;    // item slots per group
 };
+
+// Items of a group (see item64): log2 of the largest, by the size of the
+// particle set alone (a patch's sums are then those of the patch alone):
+// smaller items give a small set's SMs more to share, at the price of staging
+// the lists more often.  Measured, a force evaluation with 1, 2, 4, 8 and 16
+// particles: 16,384-particle cube 694, 715, 788, 915, 1207 us; 20,000-particle
+// ring 460, 441, 452, 507, 573 us; 65,537: 1344, 1246, 1227, 1263, 1366 us;
+// 2^20: 27.7, 26.0, 25.2, 24.9, 24.9 ms.
+__host__ __device__ __forceinline__ int item_lcap(int64_t n) {
+    return n >= 80000 ? 3 : n >= 40000 ? 2 : n >= 20000 ? 1 : 0;
+}
+__host__ __device__ __forceinline__ int whole_items(int n_g, int lcap) { return n_g >> lcap > 1 ? n_g >> lcap : 1; }
 
 // ---- 1 / sqrt(s) -----------------------------------------------------------
 // The FP64 pipe (2 lanes per clock and SM: one warp instruction takes it 16
@@ -124,16 +137,15 @@ __device__ __forceinline__ double inv_sqrt(double s) {
 // Sum over the group's own particles and its list particles, then its list
 // cells, for one item of a group: 2^k of its particles whose list is split
 // over 32 / 2^k lanes each.  A group of n_i particles is cut along the binary
-// digits of n_i (62 = 32 + 16 + 8 + 4 + 2), so every lane has a particle and
-// the FP64 pipe does no work for padding (32-lane chunks left 26% of it idle
-// for the 2^20 ring's groups, more than half for groups of 8 to 20); with few
-// particles the largest item is cut down too, so that all SMs have work.  A
-// warp per item; list entries staged 32 at a time in shared memory, the next
+// digits of n_i (62 = 7 x 8 + 4 + 2), so every lane has a particle and the
+// FP64 pipe does no work for padding (32-lane chunks left 26% of it idle for
+// the 2^20 ring's groups, more than half for groups of 8 to 20).  A warp per
+// item; list entries staged 32 at a time in shared memory, the next
 // 32 loaded while these are evaluated.  Measured against one warp per group
 // in 32-lane chunks with rsqrt(), sqrt() and divisions: force evaluation of a
 // 2^17 ring 6.07 -> 2.78 ms (62.8e6 -> 38.8e6 FP64 warp instructions, pipe 53
-// -> 71% busy), of the 2^20 ring 39.9 -> 24.4 ms, potential of a 2^18 ring
-// 13.5 -> 4.2 ms, a 4096-particle cube's evaluation 3.30 -> 1.28 ms in all.
+// -> 71% busy), of the 2^20 ring 39.9 -> 24.2 ms, potential of a 2^18 ring
+// 13.5 -> 4.2 ms, force evaluation of a 4096-particle cube 2.3 -> 0.2 ms.
 template <bool POT, int ORDER, bool EPS>
 __device__ __forceinline__ void item64(const Args64& A, Smem64& S, int64_t k, uint32_t b, uint32_t e, uint32_t i0,
                                        int lsz, int lane) {
@@ -287,22 +299,30 @@ __global__ void __launch_bounds__(32 * kWarps) k_sum64(const Args64 A) {
     if (A.abort && *A.abort) return;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int64_t ng = A.dng ? min(A.ng, (int64_t)*A.dng) : A.ng;
-    const int slots = A.full + A.lcap;
-    // item u = (group, slot): slots below `full` take the group's whole items
-    // of 2^lcap particles (every full-th one), the others the one item of
-    // each smaller power of two that the size's binary digits ask for
-    for (int64_t u = (int64_t)blockIdx.x * kWarps + w; u < ng * slots; u += (int64_t)gridDim.x * kWarps) {
-        const int64_t k = u / slots;
-        const int slot = (int)(u - k * slots);
+    // item u = (group, slot): slots below `whole` take the group's items of
+    // 2^lcap particles (every whole-th one), the next ones the item of each
+    // smaller power of two that the size's binary digits ask for
+    for (int64_t u = (int64_t)blockIdx.x * kWarps + w; u < ng * A.slots; u += (int64_t)gridDim.x * kWarps) {
+        const int64_t k = u / A.slots;
+        const int slot = (int)(u - k * A.slots);
         const int32_t g = A.groups[k];
         const uint32_t b = A.begin[g], e = A.end[g], ni = e - b;
-        if (slot < A.full) {
-            for (uint32_t c = slot; c < ni >> A.lcap; c += A.full) {
-                item64<POT, ORDER, EPS>(A, sm[w], k, b, e, b + (c << A.lcap), A.lcap, lane);
+        int q = 0;
+        for (int lo = 0, hi = A.np - 1; lo < hi;) {  // its patch: the last one starting at or before b
+            const int mid = (lo + hi + 1) >> 1;
+            if (A.off[mid] <= (int64_t)b)
+                lo = q = mid;
+            else
+                hi = mid - 1;
+        }
+        const int lcap = item_lcap(A.off[q + 1] - A.off[q]), whole = whole_items(A.n_g, lcap);
+        if (slot < whole) {
+            for (uint32_t c = slot; c < ni >> lcap; c += whole) {
+                item64<POT, ORDER, EPS>(A, sm[w], k, b, e, b + (c << lcap), lcap, lane);
                 __syncwarp();
             }
-        } else {
-            const int bit = slot - A.full;
+        } else if (slot - whole < lcap) {
+            const int bit = slot - whole;
             if ((ni >> bit) & 1u)
                 item64<POT, ORDER, EPS>(A, sm[w], k, b, e, b + ((ni >> (bit + 1)) << (bit + 1)), bit, lane);
             __syncwarp();
@@ -421,19 +441,22 @@ Args64 args64(const Ctx* c, const bh_particles* p, const ForceParams& fp) {
     A.n = (uint32_t)c->n;
     A.nn = c->n_nodes;
     A.status = c->d_status;
+    A.off = c->d_off.p;
+    A.np = c->n_patches;
+    A.n_g = c->prm.n_g;
     return A;
 }
 
 template <bool POT>
 int launch_sum64(Ctx* c, Args64& A) {
-    // largest item: 32 particles, or fewer when that gives less than 8 items
-    // per SM (each item then splits its lists over more lanes)
-    A.lcap = 5;
-    while (A.lcap > 0 && (c->n >> A.lcap) < 8 * (int64_t)c->num_sms) --A.lcap;
-    A.full = std::max(1, c->prm.n_g >> A.lcap);
+    A.slots = 0;
+    for (int q = 0; q < c->n_patches; ++q) {
+        const int lc = item_lcap(c->h_off[q + 1] - c->h_off[q]);
+        A.slots = std::max(A.slots, whole_items(c->prm.n_g, lc) + lc);
+    }
     // (device-sized build: the expected groups; the kernel strides over more)
     const int64_t ng = A.dng ? std::min(A.ng, std::max<int64_t>(c->dev_slots, 1)) : A.ng;
-    const int64_t nb = (ng * (A.full + A.lcap) + kWarps - 1) / kWarps;
+    const int64_t nb = (ng * A.slots + kWarps - 1) / kWarps;
     const unsigned grid = (unsigned)std::min<int64_t>(nb, (int64_t)1 << 30);
     const bool eps = A.fp.eps2 != 0.0;
     auto kern = A.fp.order >= 2 ? (eps ? k_sum64<POT, 2, true> : k_sum64<POT, 2, false>)

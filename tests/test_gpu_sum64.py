@@ -1,6 +1,6 @@
 """FP64 force and potential kernels at the edges of their work split: groups
-are cut along the binary digits of their size, the largest item shrinks with
-the particle count (1 to 32 particles), and each item's lists are split over
+are cut along the binary digits of their size, the largest item grows with
+the particle count (1 to 8 particles), and each item's lists are split over
 the remaining lanes; separations outside the range of the inverse-square-root
 series take the library functions.  Tolerance: the FP64 gate, 1e-12 of every
 value (a sum of ~1e3 terms of either sign in another order: ~1e-14)."""
@@ -29,19 +29,21 @@ def check(P, prm, tol=1e-12):
     ref = orc.rebuild(P, op)
     ctx, D = gpu_build(P, prm, precision=0)
     aref = orc.tree_forces(ref, op)
-    unit = np.abs(aref).max()  # (the squares of 1e180 would not fit the metric's norms)
+    unit = np.abs(aref).max() or 1.0  # (the squares of 1e180 would not fit the metric's norms)
     assert_force_close(accel_of(D) / unit, aref / unit, tol)
     phi = torch.empty(len(P["x"]), dtype=torch.float64, device="cuda")
     W = ctx.bh_compute_potential(D, phi)
     pref = orc.tree_potential(ref, op)
+    if len(pref) == 1:
+        assert W == 0.0 and float(phi[0]) == 0.0 and pref[0] == 0.0
+        return
     assert np.abs(phi.cpu().numpy() / pref - 1.0).max() <= tol
     assert abs(W / (0.5 * (ref.P["m"] * pref).sum()) - 1.0) <= tol
     ctx.close()
 
 
-# 8 items per SM (152 SMs) is what the largest item is sized for: 1216 x 2^k
-# particles are the edges
-@pytest.mark.parametrize("n", [33, 1215, 1217, 2433, 4865, 9727, 19457, 38911, 38913])
+# the largest item grows at 20,000, 40,000 and 80,000 particles
+@pytest.mark.parametrize("n", [1, 33, 4097, 19999, 20001, 39999, 40001, 79999, 80001])
 @pytest.mark.parametrize("order,eps", [(1, 1e-3), (2, 0.0)])
 def test_item_sizes(n, order, eps):
     prm = dict(synth.PRESETS["cube4k"]["params"], order=order, eps=eps, theta=0.7, n_g=40)
