@@ -262,7 +262,7 @@ int build_tree(Ctx* c, bh_particles* p) {
     BH_TRY(stage_boxes(c));
     BH_TRY(stage_end(c));
     BH_TRY(stage_moments(c, p));
-    BH_STAGE(c, BH_STAGE_GROUPS, stage_groups(c));
+    BH_STAGE(c, BH_STAGE_GROUPS, BH_OK);  // (found with the octree: the stage takes no time of its own)
     c->have_tree = true;
     return BH_OK;
 }
@@ -512,9 +512,8 @@ int size_dev_build(Ctx* c, const int64_t cap[5]) {
     BH_TRY(grow(c, c->qlo, 3 * (size_t)nodes, "node qlo"));
     BH_TRY(grow(c, c->qhi, 3 * (size_t)nodes, "node qhi"));
     BH_TRY(grow(c, c->wnode, (size_t)nodes, "walk records"));
-    BH_TRY(grow(c, c->split_cnt, (size_t)nodes, "split counts"));
-    BH_TRY(grow(c, c->split_bnd, 9 * (size_t)nodes, "split bounds"));
-    BH_TRY(grow(c, c->split_off, (size_t)nodes / 256 + 2, "split tile sums"));
+    BH_TRY(grow(c, c->tree_cnt, (size_t)tree_count_words(n), "node counts"));
+    BH_TRY(grow(c, c->tree_range, (size_t)n, "node ranges"));
     if (f32) {
         BH_TRY(grow(c, c->cell32, 3 * (size_t)nodes, "FP32 cell records"));
         BH_TRY(grow(c, c->cell32lo, (size_t)nodes, "FP32 cell mass corrections"));
@@ -584,7 +583,6 @@ int capture_rebuild(Ctx* c, bh_particles* p) {
         rc = capture_if(c, kOvfNodes, c->body_stream[0], [&]() -> int {
             BH_TRY(stage_boxes(c));
             BH_TRY(stage_moments(c, p));
-            BH_TRY(stage_groups(c));
             BH_TRY(stage_lists_dev_walk(c));
             return capture_if(c, kOvfLists, c->body_stream[1], [&]() -> int { return stage_lists_dev_fill(c); });
         });
@@ -998,10 +996,10 @@ int bh_destroy(bh_ctx* ctx) {
     }
     release(c->sort_hist); release(c->digit_hist); release(c->pscratch); release(c->scan_tmp);
     release(c->level); release(c->nchild); release(c->begin); release(c->end); release(c->parent);
-    release(c->first_child); release(c->qlo); release(c->qhi); release(c->wnode); release(c->split_cnt);
-    release(c->split_off); release(c->split_bnd); release(c->M); release(c->cx); release(c->cy);
-    release(c->cz); release(c->Q); release(c->cell32); release(c->cell32lo); release(c->refine); release(c->cbnd); release(c->cslot); release(c->cflag); release(c->phi); release(c->plo); release(c->contacts); release(c->gmark);
-    release(c->gflag); release(c->gpos); release(c->groups); release(c->order); release(c->cnt_p);
+    release(c->first_child); release(c->qlo); release(c->qhi); release(c->wnode); release(c->tree_range); release(c->tree_cnt);
+    release(c->M); release(c->cx); release(c->cy);
+    release(c->cz); release(c->Q); release(c->cell32); release(c->cell32lo); release(c->refine); release(c->cbnd); release(c->cslot); release(c->cflag); release(c->phi); release(c->plo); release(c->contacts);
+    release(c->groups); release(c->order); release(c->cnt_p);
     release(c->cnt_c); release(c->cnt_j); release(c->cnt_jm); release(c->stash_p); release(c->stash_c); release(c->P); release(c->C); release(c->JJ); release(c->ipp);
     release(c->hbuf); release(c->hid);
     for (auto& pr : c->ev_force) {

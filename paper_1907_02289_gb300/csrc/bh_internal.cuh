@@ -147,9 +147,8 @@ struct Ctx {
     DBuf<int32_t> parent, first_child;
     DBuf<uint32_t> qlo, qhi;         // 3 per node
     DBuf<WalkNode> wnode;
-    DBuf<uint32_t> split_cnt;        // per node of a level
-    DBuf<uint32_t> split_off;
-    DBuf<uint32_t> split_bnd;        // 9 per node of a level
+    DBuf<uint16_t> tree_range;       // per particle: levels of the nodes that begin there
+    DBuf<uint32_t> tree_cnt;         // per (level, particle tile): nodes that begin there, then first ids
 
     // moments
     DBuf<double> M, cx, cy, cz, Q;   // Q: 6 per node
@@ -171,8 +170,6 @@ struct Ctx {
 
     // groups
     int64_t n_groups = 0;
-    DBuf<int32_t> gmark;             // per particle: group node starting here, or -1
-    DBuf<uint32_t> gflag, gpos;
     DBuf<int32_t> groups;            // node ids ordered by begin
     DBuf<int32_t> order;             // force-kernel processing order of groups
     DBuf<unsigned long long> order_cnt;  // order buckets: counts/starts and cursors
@@ -300,12 +297,11 @@ cudaError_t sort_pairs_with(cudaStream_t s, uint64_t* keys, uint32_t* idx, uint6
                             int64_t n, uint32_t* scratch);
 
 // tree.cu
-int stage_octree(Ctx* c);                          // level-by-level split; sets n_nodes
-int stage_octree_dev(Ctx* c);                      // the same, device-sized (c->dev_build)
+int stage_octree(Ctx* c);                          // nodes and groups; sets n_nodes, n_groups
+int64_t tree_count_words(int64_t n);               // words of tree_cnt for n particles
 int stage_boxes(Ctx* c);                           // integer boxes + walk records
 int stage_moments(Ctx* c, const bh_particles* p);  // M, c, Q (+ FP32 cell records)
 int stage_moments64(Ctx* c, const bh_particles* p);  // FP64 M, c, Q whatever the precision
-int stage_groups(Ctx* c);                          // groups ordered by begin
 
 // walk.cu
 int stage_lists(Ctx* c);                           // walk (count, fill) + particle expansion

@@ -1,7 +1,7 @@
 // tree.cu -- Sec. 4.2 step 3a, second half, and the node refresh of the
-// list-reusing step: level-by-level octree over sorted keys, integer node
-// boxes on the key grid, node moments (mass, centre of mass, traceless
-// quadrupole) and the groups (maximal nodes with at most n_g particles).
+// list-reusing step: octree over sorted keys and its groups (maximal nodes
+// with at most n_g particles), integer node boxes on the key grid, and node
+// moments (mass, centre of mass, traceless quadrupole).
 //
 // Numbering: breadth first, key order within a level (a node's children are
 // contiguous and in octant order).  A node at level l splits on the digit of
@@ -37,221 +37,280 @@ __device__ __forceinline__ void level_range(int64_t& ls, int64_t& cnt, const uns
     }
 }
 
-// Roots: node q is the root of patch q (particles [off[q], off[q+1])).
-__global__ void k_roots(uint8_t* level, uint32_t* begin, uint32_t* end, int32_t* parent,
-                        const int64_t* __restrict__ off, int np) {
-    const int q = blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= np) return;
-    level[q] = 0;
-    begin[q] = (uint32_t)off[q];
-    end[q] = (uint32_t)off[q + 1];
-    parent[q] = -1;
+// ---- octree ----------------------------------------------------------------
+// The sorted keys fix the whole tree at once; no level waits for the one
+// above it.  With common(a, b) the levels two keys share (the deepest level
+// at which they lie in one cell), c = common(i - 1, i) and the patch's end
+// past every cell:
+//   particle i is the first of its cell at every level above c;
+//   the level-l cell that starts at i holds more than m particles iff
+//     common(i, i + m) >= l;
+//   so the nodes that begin at i are, if the level-c cell around i splits
+//     (more than n_leaf particles), those of levels c + 1 to
+//     max(c, min(common(i, i + n_leaf), 20)) + 1, a chain of first children;
+//   and the group that begins at i, if there is one, is the highest of them
+//     with at most n_g particles (or the leaf).
+// One pass counts the nodes per level (and the groups) of each tile of
+// particles, a scan over (level, tile) turns the counts into node ids (breadth
+// first, key order within a level), a second pass writes the nodes and the
+// group list, and a pass over the nodes links each to its children.  Against
+// one counting, scanning and writing round per level, with binary searches
+// for the children (each of a top level's a serial chain through memory), and
+// a host wait per level for the eager build: a list-constructing evaluation
+// of a 65,537-particle ring 1.49 -> 1.00 ms, 4 graph steps of 64 patches 23.2
+// -> 22.7 ms, of the 2^26 ring 543.8 -> 542.8 ms.
+constexpr int kTreeThreads = 256, kTreeItems = 4, kTreeTile = kTreeThreads * kTreeItems;
+constexpr int kTreeRows = kLevels + 2;  // levels 0..21, then the groups
+static_assert(kTreeItems * (kTreeThreads / 32) == 32, "one lane per (round, warp) when ranks are scanned");
+
+// Levels at which two keys lie in the same cell: the deepest (0..21).
+__device__ __forceinline__ int common(uint64_t a, uint64_t b) {
+    const uint64_t x = a ^ b;
+    return x ? (__clzll((long long)x) - 1) / 3 : kLevels;
 }
 
-// Child boundaries of a node [b, e) of level lev: bnd[o] = first particle
-// with octant digit >= o (o = 0..8), found by binary search; returns the
-// number of non-empty children (0 when the node does not split).
-__device__ __forceinline__ uint32_t split_bounds(const uint64_t* __restrict__ key, uint32_t b, uint32_t e, int lev,
-                                                 int n_leaf, uint32_t (&bnd)[9]) {
-    uint32_t nch = 0;
-    if (e - b > (uint32_t)n_leaf && lev < kLevels) {
-        const int shift = 3 * (kLevels - 1 - lev);
-        uint32_t lo = b, prev = b;
-        bnd[0] = b;
-        for (int o = 1; o < 8; ++o) {
-            uint32_t hi = e;
-            while (lo < hi) {
-                uint32_t mid = lo + ((hi - lo) >> 1);
-                if ((int)((key[mid] >> shift) & 7u) < o)
-                    lo = mid + 1;
-                else
-                    hi = mid;
-            }
-            bnd[o] = lo;
-            nch += (lo > prev);
-            prev = lo;
-        }
-        bnd[8] = e;
-        nch += (e > prev);
-    }
-    return nch;
-}
-
-// Child boundaries of each node of one level (9 per node, see split_bounds).
-__global__ void k_split_count(const uint64_t* __restrict__ key, const uint32_t* __restrict__ begin,
-                              const uint32_t* __restrict__ end, int64_t ls, int64_t cnt, int lev,
-                              int n_leaf, uint32_t* __restrict__ nch_out, uint32_t* __restrict__ bnd) {
-    int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= cnt) return;
-    uint32_t bb[9];
-    const uint32_t nch = split_bounds(key, begin[ls + t], end[ls + t], lev, n_leaf, bb);
-    if (nch > 0)
-#pragma unroll
-        for (int o = 0; o < 9; ++o) bnd[9 * t + o] = bb[o];
-    nch_out[t] = nch;
-}
-
-__global__ void k_split_write(const uint32_t* __restrict__ nch_in, const uint32_t* __restrict__ off,
-                              const uint32_t* __restrict__ bnd, int64_t ls, int64_t cnt, int64_t le,
-                              int lev, uint8_t* level, uint32_t* begin, uint32_t* end,
-                              int32_t* parent, int32_t* first_child, uint8_t* nchild) {
-    int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= cnt) return;
-    const int64_t node = ls + t;
-    const uint32_t nch = nch_in[t];
-    if (nch == 0) {
-        first_child[node] = -1;
-        nchild[node] = 0;
-        return;
-    }
-    const int64_t fc = le + off[t];
-    first_child[node] = (int32_t)fc;
-    nchild[node] = (uint8_t)nch;
-    int k = 0;
-    for (int o = 0; o < 8; ++o) {
-        uint32_t b0 = bnd[9 * t + o], b1 = bnd[9 * t + o + 1];
-        if (b1 > b0) {
-            int64_t ch = fc + k++;
-            level[ch] = (uint8_t)(lev + 1);
-            begin[ch] = b0;
-            end[ch] = b1;
-            parent[ch] = (int32_t)node;
+// Whether the level-c cell that holds particle i has more than m particles
+// (patch [ps, pe)).  Most answers come from three keys: yes if i + m is in the
+// cell; no if neither i + m/2 nor i - m/2 is (m + 1 particles in a row that
+// hold i reach m/2 past it on one side); else from the cell's first particle.
+__device__ __forceinline__ bool cell_above(const uint64_t* __restrict__ key, int64_t i, uint64_t ki, int64_t ps,
+                                           int64_t pe, int c, int64_t m) {
+    if (i + m < pe && common(ki, key[i + m]) >= c) return true;
+    const int64_t h = m >> 1;
+    if (!(i + h < pe && common(ki, key[i + h]) >= c) && !(i - h >= ps && common(key[i - h], ki) >= c)) return false;
+    int64_t lo = max(ps, i - m), b = i;
+    if (common(key[lo], ki) >= c) {
+        if (lo == i - m) return true;
+        b = lo;
+    } else {
+        while (lo + 1 < b) {
+            const int64_t mid = (lo + b) >> 1;
+            if (common(key[mid], ki) >= c)
+                b = mid;
+            else
+                lo = mid;
         }
     }
+    return b + m < pe && common(key[b], key[b + m]) >= c;
 }
 
-// ---- device-sized octree ---------------------------------------------------
-// For a list-constructing step captured as one graph nothing is read back:
-// the level bounds live on the device (sz[kSzLvl + l] = first node of level
-// l), every level runs the same three launches (one node per thread, the
-// threads striding over tiles of kLvTile nodes): counts and child bounds
-// with per-tile sums; one block scanning the tile sums, which writes the next
-// level's end, cut at the node capacity with the overflow flagged; the child
-// writes.  The numbering is the one of the level loop above.
-constexpr int kLvTile = 256;  // nodes per tile = threads per block
-
-__global__ void k_lvl_init(unsigned long long* sz, int np) {
-    if (threadIdx.x != 0) return;
-    sz[kSzLvl] = 0;
-    sz[kSzLvl + 1] = (unsigned long long)np;
-    sz[kSzOvf] = 0;
-    sz[kSzNeedNodes] = 0;
+// Patch that holds particle i: the last one starting at or before it.
+__device__ __forceinline__ int patch_at(const int64_t* __restrict__ off, int np, int64_t i) {
+    int q = 0;
+    for (int lo = 0, hi = np - 1; lo < hi;) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (off[mid] <= i)
+            lo = q = mid;
+        else
+            hi = mid - 1;
+    }
+    return q;
 }
 
-// Exclusive scan over the block (kLvTile threads); *total = block sum.
-__device__ __forceinline__ uint32_t lv_exclusive(uint32_t v, uint32_t* wt, uint32_t* total) {
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    uint32_t x = v;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
-        if (lane >= o) x += y;
+// Levels l0..l1 of the nodes that begin at a particle (l0 > kLevels: none) and
+// the level lg of the group that does (kNoGroup: none), in 16 bits.
+constexpr int kNoGroup = 31;
+struct NodeRange {
+    int l0 = kLevels + 1, l1 = -1, lg = kNoGroup;
+    __device__ __forceinline__ uint16_t code() const { return (uint16_t)(l0 | (l1 & 31) << 5 | lg << 10); }
+    __device__ __forceinline__ static NodeRange of(uint16_t v) {
+        NodeRange r;
+        r.l0 = v & 31;
+        r.l1 = r.l0 > kLevels ? -1 : (v >> 5) & 31;
+        r.lg = v >> 10;
+        return r;
     }
-    if (lane == 31) wt[w] = x;
-    __syncthreads();
-    if (w == 0) {
-        const uint32_t t = lane < kLvTile / 32 ? wt[lane] : 0u;
-        uint32_t q = t;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t y = __shfl_up_sync(0xffffffffu, q, o);
-            if (lane >= o) q += y;
-        }
-        if (lane < kLvTile / 32) wt[lane] = q - t;
-        if (lane == kLvTile / 32 - 1) *total = q;
-    }
-    __syncthreads();
-    const uint32_t r = wt[w] + x - v;
-    __syncthreads();
+};
+
+__device__ __forceinline__ NodeRange node_range(const uint64_t* __restrict__ key, int64_t i,
+                                                const int64_t* __restrict__ off, int np, int n_leaf, int n_g) {
+    NodeRange r;
+    const int q = patch_at(off, np, i);
+    const int64_t ps = off[q], pe = off[q + 1];
+    const uint64_t ki = key[i];
+    const int c = i > ps ? common(key[i - 1], ki) : -1;
+    if (c >= kLevels || (c >= 0 && !cell_above(key, i, ki, ps, pe, c, n_leaf))) return r;
+    const int d = i + n_leaf < pe ? common(ki, key[i + n_leaf]) : -1;
+    r.l0 = c + 1;
+    r.l1 = max(c, min(d, kLevels - 1)) + 1;
+    const int dg = i + n_g < pe ? common(ki, key[i + n_g]) : -1;
+    if (dg >= r.l0)
+        r.lg = min(dg + 1, r.l1);
+    else if (c < 0 || cell_above(key, i, ki, ps, pe, c, n_g))
+        r.lg = r.l0;
     return r;
 }
 
-__global__ void __launch_bounds__(kLvTile) k_split_count_d(const uint64_t* __restrict__ key,
-                                                           const uint32_t* __restrict__ begin,
-                                                           const uint32_t* __restrict__ end,
-                                                           const unsigned long long* __restrict__ sz, int lev,
-                                                           int n_leaf, uint32_t* __restrict__ nch_out,
-                                                           uint32_t* __restrict__ bnd, uint32_t* __restrict__ tsum) {
-    __shared__ uint32_t wt[kLvTile / 32];
-    __shared__ uint32_t tot;
-    const int64_t ls = (int64_t)sz[kSzLvl + lev], cnt = (int64_t)sz[kSzLvl + lev + 1] - ls;
-    const int64_t nt = (cnt + kLvTile - 1) / kLvTile;
-    for (int64_t tile = blockIdx.x; tile < nt; tile += gridDim.x) {
-        const int64_t t = tile * kLvTile + threadIdx.x;
-        uint32_t nch = 0;
-        if (t < cnt) {
-            uint32_t bb[9];
-            nch = split_bounds(key, begin[ls + t], end[ls + t], lev, n_leaf, bb);
-            if (nch > 0)
+// Each particle's node range, and the nodes per level, and groups, of each
+// tile: cnt[row * ntiles + tile].
+__global__ void __launch_bounds__(kTreeThreads) k_tree_count(const uint64_t* __restrict__ key, int64_t n,
+                                                             const int64_t* __restrict__ off, int np, int n_leaf,
+                                                             int n_g, int64_t ntiles, uint16_t* __restrict__ range,
+                                                             uint32_t* __restrict__ cnt) {
+    __shared__ uint32_t h[kTreeRows];
+    if (threadIdx.x < kTreeRows) h[threadIdx.x] = 0;
+    __syncthreads();
+    const int lane = threadIdx.x & 31;
+#pragma unroll 1
+    for (int r = 0; r < kTreeItems; ++r) {
+        const int64_t i = (int64_t)blockIdx.x * kTreeTile + r * kTreeThreads + threadIdx.x;
+        NodeRange q;
+        if (i < n) {
+            q = node_range(key, i, off, np, n_leaf, n_g);
+            range[i] = q.code();
+        }
+        const int l0 = __reduce_min_sync(0xffffffffu, q.l0), l1 = __reduce_max_sync(0xffffffffu, q.l1);
+        for (int l = l0; l <= l1; ++l) {
+            const unsigned m = __ballot_sync(0xffffffffu, l >= q.l0 && l <= q.l1);
+            if (lane == 0 && m) atomicAdd(&h[l], (uint32_t)__popc(m));
+        }
+        const unsigned mg = __ballot_sync(0xffffffffu, q.lg != kNoGroup);
+        if (lane == 0 && mg) atomicAdd(&h[kLevels + 1], (uint32_t)__popc(mg));
+    }
+    __syncthreads();
+    if (threadIdx.x < kTreeRows) cnt[(int64_t)threadIdx.x * ntiles + blockIdx.x] = h[threadIdx.x];
+}
+
+// The level bounds, the node and group counts from the scanned counts: sz
+// words kSzLvl.. and kSzNg, cut at the node capacity (overflow flagged).
+__global__ void k_tree_sizes(const uint32_t* __restrict__ scan, int64_t ntiles,
+                             const unsigned long long* __restrict__ total, unsigned long long cap,
+                             unsigned long long* sz) {
+    const int l = threadIdx.x;
+    const unsigned long long nodes = scan[(int64_t)(kLevels + 1) * ntiles];
+    if (l < kLevels + 3) {
+        const unsigned long long v = l <= kLevels ? (unsigned long long)scan[(int64_t)l * ntiles] : nodes;
+        sz[kSzLvl + l] = v < cap ? v : cap;
+    }
+    if (l == 0) {
+        sz[kSzNg] = *total - nodes;
+        sz[kSzOvf] = nodes > cap ? kOvfNodes : 0ull;
+        sz[kSzNeedNodes] = nodes > cap ? nodes : 0ull;
+    }
+}
+
+// Nodes (level, begin, first child; end and parent of the roots) and groups.
+__global__ void __launch_bounds__(kTreeThreads) k_tree_write(
+    const uint16_t* __restrict__ range, int64_t n, const int64_t* __restrict__ off, int np, int64_t ntiles,
+    const uint32_t* __restrict__ scan, int64_t cap, uint8_t* __restrict__ level,
+    uint32_t* __restrict__ begin, uint32_t* __restrict__ end, int32_t* __restrict__ parent,
+    int32_t* __restrict__ first_child, uint8_t* __restrict__ nchild, int32_t* __restrict__ groups) {
+    __shared__ uint32_t base[kTreeRows][32];  // per (round, warp): nodes of the row before it in the tile, then ids
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const unsigned lt = (1u << lane) - 1u;
+    for (int t = threadIdx.x; t < kTreeRows * 32; t += kTreeThreads) (&base[0][0])[t] = 0;
+    __syncthreads();
+    NodeRange q[kTreeItems];
 #pragma unroll
-                for (int o = 0; o < 9; ++o) bnd[9 * t + o] = bb[o];
-            nch_out[t] = nch;
+    for (int r = 0; r < kTreeItems; ++r) {
+        const int64_t i = (int64_t)blockIdx.x * kTreeTile + r * kTreeThreads + threadIdx.x;
+        if (i < n) q[r] = NodeRange::of(range[i]);
+        const int l0 = __reduce_min_sync(0xffffffffu, q[r].l0), l1 = __reduce_max_sync(0xffffffffu, q[r].l1);
+        for (int l = l0; l <= l1; ++l) {
+            const unsigned m = __ballot_sync(0xffffffffu, l >= q[r].l0 && l <= q[r].l1);
+            if (lane == 0) base[l][r * (kTreeThreads / 32) + w] = __popc(m);
         }
-        lv_exclusive(nch, wt, &tot);
-        if (threadIdx.x == 0) tsum[tile] = tot;
+        const unsigned mg = __ballot_sync(0xffffffffu, q[r].lg != kNoGroup);
+        if (lane == 0) base[kLevels + 1][r * (kTreeThreads / 32) + w] = __popc(mg);
+    }
+    __syncthreads();
+    for (int row = w; row < kTreeRows; row += kTreeThreads / 32) {  // counts -> ids
+        const uint32_t v = base[row][lane];
+        uint32_t x = v;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += y;
+        }
+        base[row][lane] = scan[(int64_t)row * ntiles + blockIdx.x] + x - v;
+    }
+    __syncthreads();
+    const uint32_t nodes = scan[(int64_t)(kLevels + 1) * ntiles];
+#pragma unroll
+    for (int r = 0; r < kTreeItems; ++r) {
+        const int64_t i = (int64_t)blockIdx.x * kTreeTile + r * kTreeThreads + threadIdx.x;
+        const int slot = r * (kTreeThreads / 32) + w;
+        const int l0 = __reduce_min_sync(0xffffffffu, q[r].l0), l1 = __reduce_max_sync(0xffffffffu, q[r].l1);
+        int64_t prev = -1, gnode = -1;
+        for (int l = l0; l <= l1; ++l) {
+            const bool has = l >= q[r].l0 && l <= q[r].l1;
+            const unsigned m = __ballot_sync(0xffffffffu, has);
+            if (!has) continue;
+            const int64_t id = (int64_t)base[l][slot] + __popc(m & lt);
+            if (l == q[r].lg) gnode = id;
+            if (prev >= 0 && prev < cap) first_child[prev] = (int32_t)id;
+            if (id < cap) {
+                level[id] = (uint8_t)l;
+                begin[id] = (uint32_t)i;
+                if (l == 0) {
+                    parent[id] = -1;
+                    end[id] = (uint32_t)off[patch_at(off, np, i) + 1];
+                }
+                if (l == q[r].l1) {
+                    first_child[id] = -1;
+                    nchild[id] = 0;
+                }
+            }
+            prev = id;
+        }
+        const unsigned mg = __ballot_sync(0xffffffffu, q[r].lg != kNoGroup);
+        if (q[r].lg != kNoGroup) groups[(int64_t)base[kLevels + 1][slot] + __popc(mg & lt) - nodes] = (int32_t)gnode;
     }
 }
 
-// One block: tile sums -> tile offsets; the next level ends at
-// min(le + total, cap).
-__global__ void __launch_bounds__(kLvTile) k_split_scan_d(unsigned long long* sz, int lev,
-                                                          uint32_t* __restrict__ tsum, int64_t cap) {
-    __shared__ uint32_t wt[kLvTile / 32];
-    __shared__ uint32_t tot;
-    const int64_t ls = (int64_t)sz[kSzLvl + lev], le = (int64_t)sz[kSzLvl + lev + 1], cnt = le - ls;
-    const int64_t nt = (cnt + kLvTile - 1) / kLvTile;
-    unsigned long long carry = 0;
-    for (int64_t b0 = 0; b0 < nt; b0 += kLvTile) {
-        const int64_t i = b0 + threadIdx.x;
-        const uint32_t v = i < nt ? tsum[i] : 0u;
-        const uint32_t e = lv_exclusive(v, wt, &tot);
-        if (i < nt) tsum[i] = (uint32_t)(carry + e);
-        carry += tot;
-    }
-    if (threadIdx.x == 0) {
-        const unsigned long long want = (unsigned long long)le + carry;
-        sz[kSzLvl + lev + 2] = want < (unsigned long long)cap ? want : (unsigned long long)cap;
-        if (want > (unsigned long long)cap) {
-            sz[kSzOvf] |= kOvfNodes;
-            if (want > sz[kSzNeedNodes]) sz[kSzNeedNodes] = want;
-        }
-    }
-}
-
-__global__ void __launch_bounds__(kLvTile) k_split_write_d(
-    const unsigned long long* __restrict__ sz, int lev, const uint32_t* __restrict__ nch_in,
-    const uint32_t* __restrict__ bnd, const uint32_t* __restrict__ tsum, int64_t cap, uint8_t* level,
-    uint32_t* begin, uint32_t* end, int32_t* parent, int32_t* first_child, uint8_t* nchild) {
-    __shared__ uint32_t wt[kLvTile / 32];
-    __shared__ uint32_t tot;
-    const int64_t ls = (int64_t)sz[kSzLvl + lev], le = (int64_t)sz[kSzLvl + lev + 1], cnt = le - ls;
-    const int64_t nt = (cnt + kLvTile - 1) / kLvTile;
-    for (int64_t tile = blockIdx.x; tile < nt; tile += gridDim.x) {
-        const int64_t t = tile * kLvTile + threadIdx.x;
-        const uint32_t nch = t < cnt ? nch_in[t] : 0u;
-        const uint32_t off = tsum[tile] + lv_exclusive(nch, wt, &tot);
-        if (t >= cnt) continue;
-        const int64_t node = ls + t;
-        if (nch == 0) {
-            first_child[node] = -1;
-            nchild[node] = 0;
-            continue;
-        }
-        const int64_t fc = le + off;
-        first_child[node] = (int32_t)fc;
-        nchild[node] = (uint8_t)nch;
-        int k = 0;
-        for (int o = 0; o < 8; ++o) {
-            const uint32_t b0 = bnd[9 * t + o], b1 = bnd[9 * t + o + 1];
-            if (b1 > b0) {
-                const int64_t ch = fc + k++;
-                if (ch >= cap) continue;  // past the capacity (flagged by the scan)
-                level[ch] = (uint8_t)(lev + 1);
-                begin[ch] = b0;
-                end[ch] = b1;
-                parent[ch] = (int32_t)node;
+// Children of every node that splits: parent links, child count, and each
+// child's end (the next one's begin; the last one's by a search forward).
+__global__ void __launch_bounds__(128) k_tree_link(const uint64_t* __restrict__ key, const int64_t* __restrict__ off,
+                                                   int np, const unsigned long long* __restrict__ sz,
+                                                   const uint8_t* __restrict__ level,
+                                                   const uint32_t* __restrict__ begin, uint32_t* __restrict__ end,
+                                                   int32_t* __restrict__ parent,
+                                                   const int32_t* __restrict__ first_child,
+                                                   uint8_t* __restrict__ nchild) {
+    if (sz[kSzOvf]) return;  // (a device-sized build that outgrew its nodes)
+    const int64_t nn = (int64_t)sz[kSzLvl + kLevels + 2];
+    for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < nn; k += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t f = first_child[k];
+        if (f < 0) continue;
+        const int l = level[k];
+        const int64_t lim = min((int64_t)8, (int64_t)sz[kSzLvl + l + 2] - f);  // nodes of level l + 1 from f on
+        const uint32_t b = begin[k];
+        const int64_t pe = off[patch_at(off, np, b) + 1];
+        uint32_t cb[8];
+        uint64_t ck[8];
+#pragma unroll
+        for (int t = 0; t < 8; ++t) cb[t] = t < lim ? begin[f + t] : 0xffffffffu;
+#pragma unroll
+        for (int t = 0; t < 8; ++t) ck[t] = (int64_t)cb[t] < pe ? key[cb[t]] : 0ull;
+        int nch = 0;
+        bool in = true;
+        uint32_t last = b;
+#pragma unroll
+        for (int t = 0; t < 8; ++t) {
+            in = in && (int64_t)cb[t] < pe && common(ck[0], ck[t]) >= l;
+            if (in) {
+                ++nch;
+                parent[f + t] = (int32_t)k;
+                if (t > 0) end[f + t - 1] = cb[t];
+                last = cb[t];
             }
         }
+        nchild[k] = (uint8_t)nch;
+        // end of the last child = end of node k
+        int64_t lo = last, step = 1;
+        while (lo + step < pe && common(ck[0], key[lo + step]) >= l) {
+            lo += step;
+            step <<= 1;
+        }
+        int64_t hi = min(lo + step, pe);  // key[lo] is in the node, key[hi] (or the patch's end) is not
+        while (lo + 1 < hi) {
+            const int64_t mid = (lo + hi) >> 1;
+            if (common(ck[0], key[mid]) >= l)
+                lo = mid;
+            else
+                hi = mid;
+        }
+        end[f + nch - 1] = (uint32_t)hi;
     }
 }
 
@@ -515,32 +574,6 @@ __global__ void k_moments32(int64_t ls, int64_t cnt, const unsigned long long* _
     }
 }
 
-__global__ void k_group_mark(int64_t nn, const unsigned long long* __restrict__ dnn,
-                             const uint32_t* __restrict__ begin, const uint32_t* __restrict__ end,
-                             const int32_t* __restrict__ parent, const uint8_t* __restrict__ nchild,
-                             int n_g, int32_t* __restrict__ gmark) {
-    if (dnn) nn = min(nn, (int64_t)*dnn);
-    for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < nn; k += (int64_t)gridDim.x * blockDim.x) {
-        const uint32_t cnt = end[k] - begin[k];
-        const bool small = cnt <= (uint32_t)n_g || nchild[k] == 0;
-        // a root (of any patch: parent -1) or the child of a node above n_g
-        const int32_t p = parent[k];
-        const bool top = p < 0 || (end[p] - begin[p]) > (uint32_t)n_g;
-        if (small && top) gmark[begin[k]] = (int32_t)k;
-    }
-}
-
-__global__ void k_group_flag(const int32_t* __restrict__ gmark, int64_t n, uint32_t* __restrict__ flag) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) flag[i] = gmark[i] >= 0 ? 1u : 0u;
-}
-
-__global__ void k_group_compact(const int32_t* __restrict__ gmark, const uint32_t* __restrict__ pos,
-                                int64_t n, int32_t* __restrict__ groups) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n && gmark[i] >= 0) groups[pos[i]] = gmark[i];
-}
-
 // Grid of a device-sized level launch: enough blocks for the previous
 // build's nodes on that level with the build's room to grow (the kernels
 // stride, so any count is covered; this only sets the parallelism).
@@ -553,77 +586,61 @@ unsigned dev_level_grid(const Ctx* c, int lev, int threads) {
 int grow_nodes(Ctx* c, size_t need) {
     if (need <= c->level.cap) return BH_OK;
     size_t cap = need + need / 2 + 1024;
-    BH_TRY(grow(c, c->level, cap, "node level", true));
-    BH_TRY(grow(c, c->nchild, cap, "node nchild", true));
-    BH_TRY(grow(c, c->begin, cap, "node begin", true));
-    BH_TRY(grow(c, c->end, cap, "node end", true));
-    BH_TRY(grow(c, c->parent, cap, "node parent", true));
-    BH_TRY(grow(c, c->first_child, cap, "node first_child", true));
+    BH_TRY(grow(c, c->level, cap, "node level"));
+    BH_TRY(grow(c, c->nchild, cap, "node nchild"));
+    BH_TRY(grow(c, c->begin, cap, "node begin"));
+    BH_TRY(grow(c, c->end, cap, "node end"));
+    BH_TRY(grow(c, c->parent, cap, "node parent"));
+    BH_TRY(grow(c, c->first_child, cap, "node first_child"));
     return BH_OK;
 }
 
 }  // namespace
 
-// Device-sized octree: node arrays hold c->cap_nodes nodes (grown by the
-// caller); c->n_nodes is that capacity until the sizes are read back.
-int stage_octree_dev(Ctx* c) {
-    const int np = c->n_patches;
-    const int64_t cap = c->cap_nodes;
-    const uint64_t* key = c->key[c->key_cur].p;
-    const int64_t tiles = (cap + kLvTile - 1) / kLvTile;
-    BH_TRY(grow(c, c->split_cnt, (size_t)cap, "split counts"));
-    BH_TRY(grow(c, c->split_bnd, 9 * (size_t)cap, "split bounds"));
-    BH_TRY(grow(c, c->split_off, (size_t)tiles + 1, "split tile sums"));
-    k_roots<<<blocks_for(np, 64), 64, 0, c->stream>>>(c->level.p, c->begin.p, c->end.p, c->parent.p, c->d_off.p, np);
-    BH_LAUNCH(c);
-    k_lvl_init<<<1, 32, 0, c->stream>>>(c->d_sz, np);
-    BH_LAUNCH(c);
-    for (int lev = 0; lev <= kLevels; ++lev) {
-        const unsigned grid = dev_level_grid(c, lev, kLvTile);
-        k_split_count_d<<<grid, kLvTile, 0, c->stream>>>(key, c->begin.p, c->end.p, c->d_sz, lev, c->prm.n_leaf,
-                                                         c->split_cnt.p, c->split_bnd.p, c->split_off.p);
-        BH_LAUNCH(c);
-        k_split_scan_d<<<1, kLvTile, 0, c->stream>>>(c->d_sz, lev, c->split_off.p, cap);
-        BH_LAUNCH(c);
-        k_split_write_d<<<grid, kLvTile, 0, c->stream>>>(c->d_sz, lev, c->split_cnt.p, c->split_bnd.p,
-                                                         c->split_off.p, cap, c->level.p, c->begin.p, c->end.p,
-                                                         c->parent.p, c->first_child.p, c->nchild.p);
-        BH_LAUNCH(c);
-    }
-    c->n_nodes = cap;
-    return BH_OK;
-}
+int64_t tree_count_words(int64_t n) { return kTreeRows * ((n + kTreeTile - 1) / kTreeTile); }
 
+// Nodes and groups.  Eager: the counts are read back once, to size the
+// arrays.  Device-sized (c->dev_build): the arrays hold c->cap_nodes nodes and
+// one group per particle; c->n_nodes and c->n_groups are those bounds until
+// the sizes are read back.
 int stage_octree(Ctx* c) {
-    if (c->dev_build) return stage_octree_dev(c);
-    const int64_t n = c->n;
+    const int64_t n = c->n, ntiles = (n + kTreeTile - 1) / kTreeTile;
+    const int np = c->n_patches, n_leaf = c->prm.n_leaf, n_g = c->prm.n_g;
+    const bool dev = c->dev_build;
     const uint64_t* key = c->key[c->key_cur].p;
-    const int np = c->n_patches;
-    BH_TRY(grow_nodes(c, (size_t)(n / 2 + 64 + np)));
-    k_roots<<<blocks_for(np, 64), 64, 0, c->stream>>>(c->level.p, c->begin.p, c->end.p, c->parent.p, c->d_off.p, np);
+    BH_TRY(grow(c, c->tree_cnt, (size_t)tree_count_words(n), "node counts"));
+    BH_TRY(grow(c, c->tree_range, (size_t)n, "node ranges"));
+    uint32_t* cnt = c->tree_cnt.p;
+    k_tree_count<<<(unsigned)ntiles, kTreeThreads, 0, c->stream>>>(key, n, c->d_off.p, np, n_leaf, n_g, ntiles,
+                                                                 c->tree_range.p, cnt);
     BH_LAUNCH(c);
-    c->lvl_start.assign({0, (int64_t)np});
-    for (int lev = 0;; ++lev) {
-        const int64_t ls = c->lvl_start[lev], le = c->lvl_start[lev + 1], cnt = le - ls;
-        BH_TRY(grow(c, c->split_cnt, (size_t)cnt, "split counts"));
-        BH_TRY(grow(c, c->split_off, (size_t)cnt, "split offsets"));
-        BH_TRY(grow(c, c->split_bnd, (size_t)cnt * 9, "split bounds"));
-        k_split_count<<<blocks_for(cnt, 128), 128, 0, c->stream>>>(key, c->begin.p, c->end.p, ls, cnt, lev,
-                                                                   c->prm.n_leaf, c->split_cnt.p, c->split_bnd.p);
-        BH_LAUNCH(c);
-        BH_TRY(scan_u32(c, c->split_cnt.p, c->split_off.p, cnt, c->d_small));
-        unsigned long long total = 0;
-        BH_CUDA(c, cudaMemcpyAsync(&total, c->d_small, sizeof(total), cudaMemcpyDeviceToHost, c->stream));
+    BH_TRY(scan_u32(c, cnt, cnt, tree_count_words(n), c->d_small));
+    k_tree_sizes<<<1, 32, 0, c->stream>>>(cnt, ntiles, c->d_small, dev ? (unsigned long long)c->cap_nodes : ~0ull,
+                                          c->d_sz);
+    BH_LAUNCH(c);
+    if (dev) {
+        c->n_nodes = c->cap_nodes;
+        c->n_groups = n;
+    } else {
+        unsigned long long sz[kSzWords];
+        BH_CUDA(c, cudaMemcpyAsync(sz, c->d_sz, sizeof(sz), cudaMemcpyDeviceToHost, c->stream));
         BH_CUDA(c, cudaStreamSynchronize(c->stream));
-        BH_TRY(grow_nodes(c, (size_t)(le + total)));
-        k_split_write<<<blocks_for(cnt, 128), 128, 0, c->stream>>>(
-            c->split_cnt.p, c->split_off.p, c->split_bnd.p, ls, cnt, le, lev, c->level.p, c->begin.p,
-            c->end.p, c->parent.p, c->first_child.p, c->nchild.p);
-        BH_LAUNCH(c);
-        if (total == 0) break;
-        c->lvl_start.push_back(le + (int64_t)total);
+        c->n_nodes = (int64_t)sz[kSzLvl + kLevels + 2];
+        c->n_groups = (int64_t)sz[kSzNg];
+        c->lvl_start.assign(1, 0);
+        for (int l = 0; l <= kLevels && sz[kSzLvl + l + 1] > sz[kSzLvl + l]; ++l)
+            c->lvl_start.push_back((int64_t)sz[kSzLvl + l + 1]);
+        BH_TRY(grow_nodes(c, (size_t)c->n_nodes));
+        BH_TRY(grow(c, c->groups, (size_t)c->n_groups + 1, "groups"));
     }
-    c->n_nodes = c->lvl_start.back();
+    k_tree_write<<<(unsigned)ntiles, kTreeThreads, 0, c->stream>>>(
+        c->tree_range.p, n, c->d_off.p, np, ntiles, cnt, c->n_nodes, c->level.p, c->begin.p, c->end.p, c->parent.p,
+        c->first_child.p, c->nchild.p, c->groups.p);
+    BH_LAUNCH(c);
+    k_tree_link<<<blocks_for(c->n_nodes, 128), 128, 0, c->stream>>>(key, c->d_off.p, np, c->d_sz, c->level.p,
+                                                                    c->begin.p, c->end.p, c->parent.p,
+                                                                    c->first_child.p, c->nchild.p);
+    BH_LAUNCH(c);
     return BH_OK;
 }
 
@@ -703,33 +720,5 @@ int stage_moments64(Ctx* c, const bh_particles* p) {
     }
     return stage_end(c);
 }
-
-int stage_groups(Ctx* c) {
-    const int64_t n = c->n, nn = c->n_nodes;
-    const bool dev = c->dev_build;
-    BH_TRY(grow(c, c->gmark, (size_t)n, "group marks"));
-    BH_TRY(grow(c, c->gflag, (size_t)n, "group flags"));
-    BH_TRY(grow(c, c->gpos, (size_t)n, "group positions"));
-    BH_CUDA(c, cudaMemsetAsync(c->gmark.p, 0xff, n * sizeof(int32_t), c->stream));
-    k_group_mark<<<blocks_for(nn, 256), 256, 0, c->stream>>>(
-        nn, dev ? c->d_sz + kSzLvl + kLevels + 2 : nullptr, c->begin.p, c->end.p, c->parent.p, c->nchild.p,
-        c->prm.n_g, c->gmark.p);
-    BH_LAUNCH(c);
-    k_group_flag<<<blocks_for(n, 256), 256, 0, c->stream>>>(c->gmark.p, n, c->gflag.p);
-    BH_LAUNCH(c);
-    unsigned long long* total = dev ? c->d_sz + kSzNg : c->d_small;
-    BH_TRY(scan_u32(c, c->gflag.p, c->gpos.p, n, total));
-    unsigned long long ng = (unsigned long long)n;  // device-sized: at most one group per particle
-    if (!dev) {
-        BH_CUDA(c, cudaMemcpyAsync(&ng, c->d_small, sizeof(ng), cudaMemcpyDeviceToHost, c->stream));
-        BH_CUDA(c, cudaStreamSynchronize(c->stream));
-    }
-    BH_TRY(grow(c, c->groups, (size_t)ng + 1, "groups"));
-    k_group_compact<<<blocks_for(n, 256), 256, 0, c->stream>>>(c->gmark.p, c->gpos.p, n, c->groups.p);
-    BH_LAUNCH(c);
-    c->n_groups = (int64_t)ng;
-    return BH_OK;
-}
-
 
 }  // namespace bh
