@@ -54,9 +54,10 @@ int grow(Ctx* c, DBuf<T>& b, size_t n, const char* what, bool keep = false) {
 }
 
 // Per-node packed record read by the walk (one 32-byte load per visit):
-// a = (qlo.x | level << 21 | leaf flag, qlo.y | leaf count << 21, qlo.z,
+// a = (qlo.x | level << 21 | leaf flag, qlo.y | count << 21, qlo.z,
 // successor of the subtree or -1), b = (qhi.xyz, first child, or for a leaf
-// its first particle).  A leaf count of kWalkCntMax means "that many or
+// its first particle); the count is a leaf's particles or an inner node's
+// children.  A leaf count of kWalkCntMax means "that many or
 // more": the walk then reads the node's end.
 struct WalkNode {
     uint4 a, b;

@@ -372,10 +372,10 @@ __global__ void k_boxes(const uint64_t* __restrict__ key, int64_t ls, int64_t cn
         }
         WalkNode w;
         // a leaf carries its first particle and (up to kWalkCntMax - 1) its
-        // particle count instead of a first child
-        const uint32_t leafcnt = nc == 0 ? min(end[k] - begin[k], kWalkCntMax) : 0u;
+        // particle count instead of a first child and the child count
+        const uint32_t cnt = nc == 0 ? min(end[k] - begin[k], kWalkCntMax) : (uint32_t)nc;
         w.a = make_uint4(lo[0] | ((uint32_t)level[k] << kLevels) | (nc == 0 ? kWalkLeaf : 0u),
-                         lo[1] | (leafcnt << kLevels), lo[2],
+                         lo[1] | (cnt << kLevels), lo[2],
                          (uint32_t)skip_of(k, parent, first_child, nchild, status));
         w.b = make_uint4(hi[0], hi[1], hi[2], nc == 0 ? begin[k] : (uint32_t)first_child[k]);
         wnode[k] = w;
