@@ -48,9 +48,10 @@ extern "C" {
 #define BH_E_CUDA 3          /* a CUDA call failed                           */
 #define BH_E_LIST_OVERFLOW 4 /* list or node buffer too small (needed size   */
                              /* is reported by bh_get_sizes)                 */
-#define BH_E_TIMEOUT 5       /* reserved: no kernel of this library waits on */
-                             /* the device (no spin on a flag, a barrier or  */
-                             /* another kernel), so it is never returned     */
+#define BH_E_TIMEOUT 5       /* a tile of the key sort gave up waiting for the */
+                             /* counts of an earlier one (a bounded wait on a */
+                             /* running block: never in a correct run; no     */
+                             /* other kernel of this library waits)           */
 #define BH_E_STATE 6         /* call out of order (e.g. forces before lists) */
 
 #define BH_PREC_FP64 0 /* plain FP64 force kernel                              */
@@ -448,7 +449,7 @@ int bh_measure_peak(int kind, double* tflops);
  * All eight 8-bit passes run, so all 64 key bits are sorted.
  * The first call on each device does set-up with that device current: it
  * looks up the scratch array's address (cudaGetSymbolAddress) and sets the
- * sort kernel's shared-memory limit; make that first call before capturing
+ * sort kernels' shared-memory limit; make that first call before capturing
  * any stream on that device.  The looked-up address belongs to the device's
  * primary context: after cudaDeviceReset (or anything else that destroys
  * that context) this entry point must not be called again in the process.

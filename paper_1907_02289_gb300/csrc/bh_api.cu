@@ -164,7 +164,7 @@ int setup_patches(Ctx* c, int n_patches, const int64_t* off) {
     std::vector<uint2> map;
     std::vector<int> poff;
     if (n_patches > 1) {
-        c->n_tiles = sort_tiles_for(c->h_off, &meta);
+        c->n_tiles = sort_tiles_for(c->h_off, &meta, &c->n_sort_slots);
         BH_TRY(grow(c, c->tile_meta, meta.size(), "sort tile table"));
         BH_CUDA(c, cudaMemcpyAsync(c->tile_meta.p, meta.data(), meta.size() * sizeof(uint32_t),
                                    cudaMemcpyHostToDevice, c->stream));
@@ -994,7 +994,7 @@ int bh_destroy(bh_ctx* ctx) {
         release(c->key[b]);
         release(c->idx[b]);
     }
-    release(c->sort_hist); release(c->digit_hist); release(c->pscratch); release(c->scan_tmp);
+    release(c->sort_scratch); release(c->pscratch); release(c->scan_tmp);
     release(c->level); release(c->nchild); release(c->begin); release(c->end); release(c->parent);
     release(c->first_child); release(c->qlo); release(c->qhi); release(c->wnode); release(c->tree_range); release(c->tree_cnt);
     release(c->M); release(c->cx); release(c->cy);

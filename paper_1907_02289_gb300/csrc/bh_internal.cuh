@@ -117,6 +117,7 @@ struct Ctx {
     DBuf<int64_t> d_off;                // the same on the device
     DBuf<uint32_t> tile_meta;           // sort tiles per patch (4 words per tile), n_patches > 1
     int64_t n_tiles = 0;
+    int n_sort_slots = 0;               // patches of more than one sort tile
     DBuf<uint2> box_map;                // root-box blocks of the patches: (patch, block within it)
     DBuf<int> box_poff;                 // first root-box block of each patch (n_patches + 1)
     int n_box_blocks = 0;
@@ -133,8 +134,7 @@ struct Ctx {
     DBuf<uint64_t> key[2];
     DBuf<uint32_t> idx[2];
     int key_cur = 0;           // buffer holding the sorted keys / perm
-    DBuf<uint32_t> sort_hist;
-    DBuf<uint32_t> digit_hist; // 8 x 256 global digit counts
+    DBuf<uint32_t> sort_scratch;  // look-back words, digit counts, tickets
     DBuf<double> pscratch;     // permutation scratch (8 arrays x 8 bytes per particle)
     DBuf<double> cyl;          // cylindrical frame: phi[n], r[n]
     DBuf<unsigned long long> box_part;  // root-box partials (6 per block, as ordered integers)
@@ -282,20 +282,19 @@ int scan_u32(Ctx* c, const uint32_t* in, uint32_t* out, int64_t n, unsigned long
              const unsigned long long* dn = nullptr);
 int scan_i64(Ctx* c, const int64_t* in, int64_t* out, int64_t n, unsigned long long* d_total,
              const unsigned long long* dn = nullptr);
-int64_t scan_sums_count(int64_t n);
-cudaError_t scan_u32_with(cudaStream_t s, const uint32_t* in, uint32_t* out, int64_t n, uint32_t* sums);
 
 // sort.cu
 int stage_keys(Ctx* c, const bh_particles* p);     // root box + keys (+ status on NaN)
 int stage_sort(Ctx* c);                            // stable LSD radix sort of (key, idx)
 int stage_permute(Ctx* c, bh_particles* p);        // gather particle arrays into key order
 int setup_patches(Ctx* c, int n_patches, const int64_t* off);  // bh_api.cu
-int64_t sort_tiles_for(const std::vector<int64_t>& off, std::vector<uint32_t>* meta);  // sort.cu
+int64_t sort_tiles_for(const std::vector<int64_t>& off, std::vector<uint32_t>* meta, int* nslots);  // sort.cu
 // context-free sort over caller buffers (sort.cu); scratch >= sort_scratch_words(n) words
 int64_t sort_scratch_words(int64_t n);
 cudaError_t sort_setup_device();
 cudaError_t sort_pairs_with(cudaStream_t s, uint64_t* keys, uint32_t* idx, uint64_t* ktmp, uint32_t* itmp,
-                            int64_t n, uint32_t* scratch);
+                            int64_t n, int num_sms, uint32_t* scratch, int* status);
+int sort_launches();                               // kernels of one such sort of more than one tile
 
 // tree.cu
 int stage_octree(Ctx* c);                          // nodes and groups; sets n_nodes, n_groups

@@ -1282,8 +1282,8 @@ int build_order32(Ctx* c) {
             c->sort_attr_device = c->device;
         }
         BH_CUDA(c, sort_pairs_with(c->stream, c->ord_key[0].p, c->ord_idx[0].p, c->ord_key[1].p, c->ord_idx[1].p, ng,
-                                   c->ord_scratch.p));
-        c->n_launches += 1 + 8 * 5;
+                                   c->num_sms, c->ord_scratch.p, c->d_status));
+        c->n_launches += sort_launches();
         BH_CUDA(c, cudaMemcpyAsync(c->order.p, c->ord_idx[0].p, ng * sizeof(int32_t), cudaMemcpyDeviceToDevice,
                                    c->stream));
         return BH_OK;

@@ -1,6 +1,6 @@
 // noalloc.cu -- bh_sort_keys_static: the stable radix sort of sort.cu over
-// caller buffers, with its scratch (per-tile digit histograms and scan block
-// sums) in one fixed array in device global memory instead of memory from
+// caller buffers, with its scratch (look-back words per tile, digit counts
+// and tickets) in one fixed array in device global memory instead of memory from
 // cudaMalloc.  Nothing in this file allocates.
 #include <cstdarg>
 #include <cstdio>
@@ -12,9 +12,10 @@ namespace bh {
 namespace {
 
 // Largest n this entry point accepts, and the scratch that n needs:
-// 256 digit counts per 4096-key tile plus the scan's block sums (1 MiB).
+// 256 look-back words per tile plus the digit counts and tickets (1 MiB holds
+// them, since a tile is more than 4096 keys).
 constexpr int64_t kStaticSortMaxN = BH_SORT_STATIC_MAX_N;
-constexpr int64_t kStaticWords = 256 * (kStaticSortMaxN / 4096) + (256 * (kStaticSortMaxN / 4096) + 2047) / 2048;
+constexpr int64_t kStaticWords = 256 * (kStaticSortMaxN / 4096) + 128;
 
 static __device__ __align__(256) uint32_t g_sort_scratch[kStaticWords];
 
@@ -22,6 +23,7 @@ constexpr int kMaxDevices = 64;
 
 struct DeviceSlot {
     bool ready = false;
+    int num_sms = 0;
     uint32_t* scratch = nullptr;
 };
 
@@ -44,7 +46,7 @@ int report(char* err, size_t err_len, int code, const char* fmt, ...) {
 // The cached address belongs to the device's primary context: it is not valid
 // after that context is destroyed (cudaDeviceReset), after which this entry
 // point must not be called again in the process.
-int device_scratch(uint32_t** out, char* err, size_t err_len) {
+int device_scratch(uint32_t** out, int* num_sms, char* err, size_t err_len) {
     int dev = -1;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return report(err, err_len, BH_E_CUDA, "cudaGetDevice: %s", cudaGetErrorString(e));
@@ -63,10 +65,14 @@ int device_scratch(uint32_t** out, char* err, size_t err_len) {
         if (e != cudaSuccess)
             return report(err, err_len, BH_E_CUDA, "setting the sort kernel's shared-memory limit on device %d: %s",
                           dev, cudaGetErrorString(e));
+        e = cudaDeviceGetAttribute(&s.num_sms, cudaDevAttrMultiProcessorCount, dev);
+        if (e != cudaSuccess)
+            return report(err, err_len, BH_E_CUDA, "cudaDeviceGetAttribute: %s", cudaGetErrorString(e));
         s.scratch = static_cast<uint32_t*>(p);
         s.ready = true;
     }
     *out = s.scratch;
+    *num_sms = s.num_sms;
     return BH_OK;
 }
 
@@ -98,12 +104,12 @@ extern "C" int bh_sort_keys_static(uint64_t* keys, uint32_t* idx, uint64_t* keys
         return report(err, err_len, BH_E_INVAL, "sort of n = %lld needs %lld scratch words, %lld available",
                       (long long)n, (long long)sort_scratch_words(n), (long long)kStaticWords);
     uint32_t* scratch = nullptr;
-    int rc = device_scratch(&scratch, err, err_len);
+    int num_sms = 0;
+    int rc = device_scratch(&scratch, &num_sms, err, err_len);
     if (rc != BH_OK) return rc;
-    // The histograms are fully written by every upsweep and the block sums by
-    // every reduce before they are read, so no part of the scratch has to
-    // start at zero.
-    cudaError_t e = sort_pairs_with((cudaStream_t)stream, keys, idx, keys_tmp, idx_tmp, n, scratch);
+    // (the sort clears the part of the scratch it uses first; no status word:
+    // a look-back that gave up, which cannot happen, would leave keys unsorted)
+    cudaError_t e = sort_pairs_with((cudaStream_t)stream, keys, idx, keys_tmp, idx_tmp, n, num_sms, scratch, nullptr);
     if (e != cudaSuccess) return report(err, err_len, BH_E_CUDA, "sort launch: %s", cudaGetErrorString(e));
     return BH_OK;
 }

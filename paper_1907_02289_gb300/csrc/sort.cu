@@ -191,10 +191,10 @@ __device__ __forceinline__ uint32_t quantise(double v, double lo, double S) {
 }
 
 // Keys of every particle on its patch's grid (patch by binary search of the
-// offsets); idx = the particle's index.
+// offsets).
 __global__ void k_keys(const double* __restrict__ x, const double* __restrict__ y,
                        const double* __restrict__ z, int64_t n, const int64_t* __restrict__ off, int np,
-                       const double* __restrict__ boxes, uint64_t* __restrict__ key, uint32_t* __restrict__ idx) {
+                       const double* __restrict__ boxes, uint64_t* __restrict__ key) {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     int q = 0;
@@ -210,182 +210,316 @@ __global__ void k_keys(const double* __restrict__ x, const double* __restrict__ 
     uint32_t qx = quantise(x[i], box[0], S), qy = quantise(y[i], box[1], S),
              qz = quantise(z[i], box[2], S);
     key[i] = (spread3(qx) << 2) | (spread3(qy) << 1) | spread3(qz);
-    idx[i] = (uint32_t)i;
 }
 
 // ---------------------------------------------------------------------------
-// Radix sort: 8-bit digits, passes over bits [8p, 8p+8).  Per pass:
-//   upsweep   per-tile digit histogram, stored digit-major hist[d * ntiles + t]
-//   scan      exclusive scan of hist -> global start of (digit, tile)
-//   downsweep stable in-tile ranking (warp match + per-warp counters), local
-//             reorder through shared memory, coalesced scatter.
+// Radix sort: 8-bit digits, stable, one launch per digit (passes over bits
+// [8p, 8p+8)) after one that counts all eight digits of every key.  A block
+// takes the next tile (an atomic ticket, so every earlier tile has been taken
+// by a running block), ranks its keys (ballots within a warp, per-warp digit
+// counters), publishes its digit counts, reorders the keys by digit in shared
+// memory, and finds the counts of all earlier tiles by looking back over the
+// published words (a tile's own count, or the running total up to it) before
+// the coalesced scatter: each pass reads and writes every key once, where
+// counting, scanning and scattering launches read them twice.
 // Stability: ranks follow (tile, warp, round, lane) = input order.
 //
 // Several patches (independent particle sets, each sorted on its own): tiles
-// never straddle a patch, and the histogram of patch p is stored as its own
-// digit-major block after those of patches 0..p-1, so the one scan orders
-// the output by (patch, digit, tile).  tmeta holds per tile {first key, key
-// count, first tile of its patch, tile count of its patch}; NULL means one
-// patch cut into uniform tiles.
+// never straddle a patch, and the look-back of a tile ends at its patch's
+// first.  tmeta holds per tile {first key, key count | digit-count slot << 13,
+// first tile of its patch, tile count of its patch}; NULL means one patch cut
+// into uniform tiles.  A patch of one tile needs no counts over the patch.
+//
+// Look-back words: digit pass + 1 in the top 4 bits (the words are cleared
+// once per sort, so those of an earlier pass never match), a flag for a
+// running total, and the count; 32 bits below 2^27 keys, else 64.
+// Measured against counting, scanning and scattering launches (42 launches,
+// and a host wait for the digit counts): 3,000,001 keys 469 -> 360 us, the
+// evaluation of a 65,537-particle ring 860 -> 675 us.
 // ---------------------------------------------------------------------------
-constexpr int kSortThreads = 256;
+constexpr int kSortThreads = 384;
 constexpr int kSortWarps = kSortThreads / 32;
-constexpr int kSortItems = 16;                       // per lane
-constexpr int kSortTile = kSortThreads * kSortItems; // 4096
+constexpr int kSortItems = 12;                       // per lane
+constexpr int kSortTile = kSortThreads * kSortItems; // 4608
 constexpr int kRadix = 256;
+constexpr int kSlotShift = 13;                       // kSortTile < 2^13
+constexpr int64_t kSort32 = (int64_t)1 << 27;        // keys that 32-bit look-back words count
+constexpr int kSortHist = 8 * kRadix;                // digit counts per slot
+constexpr int kSortPolls = 1 << 22;                  // look-back polls before a tile gives up
 
 struct TileInfo {
     int64_t start;  // first key of the tile
     int cnt;        // keys in the tile
-    int64_t hbase;  // histogram slot of (digit 0, this tile)
-    int nt;         // tile count of the tile's patch (histogram stride)
+    int slot;       // digit counts of its patch
+    int first, nt;  // first tile and tile count of its patch
 };
 
-__device__ __forceinline__ TileInfo tile_info(const uint32_t* __restrict__ tmeta, int64_t n, int ntiles) {
-    const int t = blockIdx.x;
+__device__ __forceinline__ TileInfo tile_info(const uint32_t* __restrict__ tmeta, int64_t n, int ntiles, int t) {
     TileInfo ti;
     if (tmeta) {
         const uint4 m = reinterpret_cast<const uint4*>(tmeta)[t];
         ti.start = m.x;
-        ti.cnt = (int)m.y;
-        ti.hbase = (int64_t)kRadix * m.z + (t - (int)m.z);
+        ti.cnt = (int)(m.y & ((1u << kSlotShift) - 1u));
+        ti.slot = (int)(m.y >> kSlotShift);
+        ti.first = (int)m.z;
         ti.nt = (int)m.w;
     } else {
         ti.start = (int64_t)t * kSortTile;
         const int64_t r = n - ti.start;
         ti.cnt = (int)(r < kSortTile ? r : kSortTile);
-        ti.hbase = t;
+        ti.slot = 0;
+        ti.first = 0;
         ti.nt = ntiles;
     }
     return ti;
 }
 
-__global__ void k_digit_hist(const uint64_t* __restrict__ key, int64_t n, uint32_t* __restrict__ hist) {
+// Digit counts of every pass, per patch of more than one tile: hist[slot][pass][digit].
+__global__ void __launch_bounds__(256) k_digit_hist(const uint64_t* __restrict__ key, int64_t n, int ntiles,
+                                                    const uint32_t* __restrict__ tmeta, uint32_t* __restrict__ hist) {
     __shared__ uint32_t h[8][kRadix];
-    for (int i = threadIdx.x; i < 8 * kRadix; i += blockDim.x) (&h[0][0])[i] = 0;
-    __syncthreads();
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        uint64_t k = key[i];
+    const int per = (ntiles + gridDim.x - 1) / gridDim.x;
+    const int t0 = blockIdx.x * per, t1 = min(t0 + per, ntiles);
+    int slot = -1;
+    auto flush = [&]() {
+        __syncthreads();
+        if (slot >= 0)
+            for (int i = threadIdx.x; i < kSortHist; i += blockDim.x)
+                if ((&h[0][0])[i]) atomicAdd(&hist[(int64_t)slot * kSortHist + i], (&h[0][0])[i]);
+        __syncthreads();
+        for (int i = threadIdx.x; i < kSortHist; i += blockDim.x) (&h[0][0])[i] = 0;
+        __syncthreads();
+    };
+    for (int t = t0; t < t1; ++t) {
+        const TileInfo ti = tile_info(tmeta, n, ntiles, t);
+        if (ti.nt == 1) continue;
+        if (ti.slot != slot) {
+            flush();
+            slot = ti.slot;
+        }
+#pragma unroll 6
+        for (int i = threadIdx.x; i < ti.cnt; i += 256) {
+            const uint64_t k = key[ti.start + i];
 #pragma unroll
-        for (int p = 0; p < 8; ++p) atomicAdd(&h[p][(k >> (8 * p)) & 0xff], 1u);
+            for (int p = 0; p < 8; ++p) atomicAdd(&h[p][(k >> (8 * p)) & 0xff], 1u);
+        }
     }
-    __syncthreads();
-    for (int i = threadIdx.x; i < 8 * kRadix; i += blockDim.x)
-        if ((&h[0][0])[i]) atomicAdd(&hist[i], (&h[0][0])[i]);
+    if (slot >= 0) flush();
 }
 
-__global__ void __launch_bounds__(kSortThreads) k_upsweep(const uint64_t* __restrict__ key, int64_t n,
-                                                         int shift, uint32_t* __restrict__ hist,
-                                                         int ntiles, const uint32_t* __restrict__ tmeta) {
-    __shared__ uint32_t h[kRadix];
-    h[threadIdx.x] = 0;
-    __syncthreads();
-    const TileInfo ti = tile_info(tmeta, n, ntiles);
-#pragma unroll 4
-    for (int k = 0; k < kSortItems; ++k) {
-        const int r = k * kSortThreads + threadIdx.x;
-        if (r < ti.cnt) atomicAdd(&h[(key[ti.start + r] >> shift) & 0xff], 1u);
+template <class W>
+struct Look {
+    static constexpr int kTag = 8 * sizeof(W) - 4;
+    static constexpr W kTotal = (W)1 << (kTag - 1), kCount = kTotal - 1;
+    __device__ __forceinline__ static W load(const W* p) {
+        W v;
+        if constexpr (sizeof(W) == 4)
+            asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+        else
+            asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+        return v;
     }
-    __syncthreads();
-    hist[ti.hbase + (int64_t)threadIdx.x * ti.nt] = h[threadIdx.x];
-}
+    __device__ __forceinline__ static void store(W* p, W v) {
+        if constexpr (sizeof(W) == 4)
+            asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+        else
+            asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+    }
+};
 
-struct DownSmem {
+struct SweepSmem {
     uint32_t whist[kSortWarps][kRadix];
     uint32_t tstart[kRadix];
     uint32_t goff[kRadix];
-    uint32_t wtot[kSortWarps];
-    uint64_t skey[kSortTile];
-    uint32_t sidx[kSortTile];
+    unsigned long long wtot[kRadix / 32];
+    int tile;
+    union {
+        uint64_t skey[kSortTile];
+        uint32_t sidx[kSortTile];
+    };
 };
 
-__global__ void __launch_bounds__(kSortThreads) k_downsweep(
-    const uint64_t* __restrict__ kin, const uint32_t* __restrict__ iin, int64_t n, int shift,
-    const uint32_t* __restrict__ offs, int ntiles, uint64_t* __restrict__ kout,
-    uint32_t* __restrict__ iout, const uint32_t* __restrict__ tmeta) {
+// FIRST: the index of a key is its position (iin is not read).
+template <class W, bool FIRST>
+__global__ void __launch_bounds__(kSortThreads, 3) k_sweep(
+    const uint64_t* __restrict__ kin, const uint32_t* __restrict__ iin, int64_t n, int pass, int ntiles,
+    const uint32_t* __restrict__ tmeta, const uint32_t* __restrict__ hist, W* words, uint32_t* ticket,
+    uint64_t* __restrict__ kout, uint32_t* __restrict__ iout, int* status) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    DownSmem& S = *reinterpret_cast<DownSmem*>(smem_raw);
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    for (int i = threadIdx.x; i < kSortWarps * kRadix; i += kSortThreads) (&S.whist[0][0])[i] = 0;
-    const TileInfo ti = tile_info(tmeta, n, ntiles);
-    S.goff[threadIdx.x] = offs[ti.hbase + (int64_t)threadIdx.x * ti.nt];
+    SweepSmem& S = *reinterpret_cast<SweepSmem*>(smem_raw);
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, shift = 8 * pass;
+    if (tid == 0) S.tile = (int)atomicAdd(ticket, 1u);
+    for (int i = tid; i < kSortWarps * kRadix; i += kSortThreads) (&S.whist[0][0])[i] = 0;
     __syncthreads();
-
-    const int64_t tbase = ti.start, tend = ti.start + ti.cnt;
-    const int64_t wbase = tbase + (int64_t)w * (32 * kSortItems);
+    const int tile = S.tile;
+    const TileInfo ti = tile_info(tmeta, n, ntiles, tile);
+    const int wbase = w * (32 * kSortItems);
     const unsigned lt = (1u << lane) - 1u;
     uint64_t kr[kSortItems];
-    uint32_t ir[kSortItems], lr[kSortItems];
+    uint32_t pr[kSortItems];
 #pragma unroll
     for (int r = 0; r < kSortItems; ++r) {
-        int64_t pos = wbase + r * 32 + lane;
-        bool valid = pos < tend;
-        uint64_t k = valid ? kin[pos] : 0;
-        uint32_t d = valid ? (uint32_t)((k >> shift) & 0xff) : 0x100u;
-        unsigned peers = __match_any_sync(0xffffffffu, d);
-        int leader = __ffs(peers) - 1;
-        uint32_t old = 0;
-        if (lane == leader && valid) {
-            old = S.whist[w][d];
-            S.whist[w][d] = old + __popc(peers);
+        const int pos = wbase + r * 32 + lane;
+        kr[r] = pos < ti.cnt ? kin[ti.start + pos] : ~0ull;
+    }
+#pragma unroll
+    for (int r = 0; r < kSortItems; ++r) {
+        const bool valid = wbase + r * 32 + lane < ti.cnt;
+        const uint32_t d = (uint32_t)(kr[r] >> shift) & 0xffu;
+        unsigned peers = __ballot_sync(0xffffffffu, valid);
+#pragma unroll
+        for (int b = 0; b < 8; ++b) {
+            const bool bit = (d >> b) & 1u;
+            const unsigned m = __ballot_sync(0xffffffffu, bit);
+            peers &= bit ? m : ~m;
         }
-        old = __shfl_sync(0xffffffffu, old, leader);
-        kr[r] = k;
-        ir[r] = valid ? iin[pos] : 0u;
-        lr[r] = old + __popc(peers & lt);
+        const uint32_t old = S.whist[w][d];
         __syncwarp();
+        if (valid && (peers & lt) == 0) S.whist[w][d] = old + __popc(peers);
+        __syncwarp();
+        pr[r] = old + __popc(peers & lt);
     }
     __syncthreads();
-    // per digit: exclusive over warps; tile total; exclusive over digits
-    {
-        const int d = threadIdx.x;  // kSortThreads == kRadix
-        uint32_t run = 0;
+    // per digit: exclusive over warps; tile count; exclusive over digits (of
+    // the tile, and of the patch)
+    W* mine = words + (int64_t)tile * kRadix;
+    const W tag = (W)(pass + 1) << Look<W>::kTag;
+    uint32_t total = 0, base = 0;
+    unsigned long long x = 0, own = 0;
+    if (tid < kRadix) {
 #pragma unroll
         for (int ww = 0; ww < kSortWarps; ++ww) {
-            uint32_t t = S.whist[ww][d];
-            S.whist[ww][d] = run;
-            run += t;
+            const uint32_t t = S.whist[ww][tid];
+            S.whist[ww][tid] = total;
+            total += t;
         }
-        uint32_t x = run;
+        if (ti.nt > 1)
+            Look<W>::store(&mine[tid], tag | (tile == ti.first ? Look<W>::kTotal : (W)0) | (W)total);
+        const uint32_t hc = ti.nt > 1 ? hist[(int64_t)ti.slot * kSortHist + pass * kRadix + tid] : total;
+        own = (unsigned long long)hc << 32 | total;
+        x = own;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
-            uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+            const unsigned long long y = __shfl_up_sync(0xffffffffu, x, o);
             if (lane >= o) x += y;
         }
         if (lane == 31) S.wtot[w] = x;
-        __syncthreads();
-        uint32_t add = 0;
-        for (int ww = 0; ww < w; ++ww) add += S.wtot[ww];
-        S.tstart[d] = add + x - run;
+    }
+    __syncthreads();
+    if (tid < kRadix) {
+        x -= own;
+        for (int ww = 0; ww < w; ++ww) x += S.wtot[ww];
+        S.tstart[tid] = (uint32_t)x;
+        base = (uint32_t)(x >> 32);
     }
     __syncthreads();
 #pragma unroll
-    for (int r = 0; r < kSortItems; ++r) {
-        int64_t pos = wbase + r * 32 + lane;
-        if (pos < tend) {
-            uint32_t d = (uint32_t)((kr[r] >> shift) & 0xff);
-            uint32_t p = S.tstart[d] + S.whist[w][d] + lr[r];
-            S.skey[p] = kr[r];
-            S.sidx[p] = ir[r];
+    for (int r = 0; r < kSortItems; ++r)
+        if (wbase + r * 32 + lane < ti.cnt) {
+            const uint32_t d = (uint32_t)(kr[r] >> shift) & 0xffu;
+            pr[r] += S.tstart[d] + S.whist[w][d];
+            S.skey[pr[r]] = kr[r];
         }
+    if (tid < kRadix) {
+        W excl = 0;
+        if (tile > ti.first) {
+            int polls = 0;
+            for (int t = tile - 1; t >= ti.first;) {
+                const W v = Look<W>::load(&words[(int64_t)t * kRadix + tid]);
+                if (v >> Look<W>::kTag == (W)(pass + 1)) {
+                    excl += v & Look<W>::kCount;
+                    if (v & Look<W>::kTotal) break;
+                    --t;
+                } else if (++polls > kSortPolls) {  // (the earlier tile is running: never)
+                    if (status) atomicOr(status, kStatTimeout);
+                    break;
+                }
+            }
+            Look<W>::store(&mine[tid], tag | Look<W>::kTotal | (excl + (W)total));
+        }
+        // the patch's first output is its first key's position
+        const int64_t p0 = tmeta ? ti.start - (int64_t)(tile - ti.first) * kSortTile : 0;
+        S.goff[tid] = (uint32_t)p0 + base + (uint32_t)excl - S.tstart[tid];
     }
     __syncthreads();
-    const int tn = ti.cnt;
-    for (int q = threadIdx.x; q < tn; q += kSortThreads) {
-        uint64_t k = S.skey[q];
-        uint32_t d = (uint32_t)((k >> shift) & 0xff);
-        uint64_t g = (uint64_t)S.goff[d] + (uint64_t)(q - S.tstart[d]);
-        kout[g] = k;
-        iout[g] = S.sidx[q];
+    uint32_t g[kSortItems];
+#pragma unroll
+    for (int r = 0; r < kSortItems; ++r) {
+        const int q = r * kSortThreads + tid;
+        g[r] = 0xffffffffu;
+        if (q < ti.cnt) {
+            const uint64_t k = S.skey[q];
+            g[r] = S.goff[(uint32_t)(k >> shift) & 0xffu] + (uint32_t)q;
+            if ((int64_t)g[r] < n) kout[g[r]] = k;  // (past it only after a look-back that gave up)
+        }
     }
+    uint32_t ir[kSortItems];
+#pragma unroll
+    for (int r = 0; r < kSortItems; ++r) {
+        const int pos = wbase + r * 32 + lane;
+        ir[r] = FIRST ? (uint32_t)(ti.start + pos) : pos < ti.cnt ? iin[ti.start + pos] : 0u;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < kSortItems; ++r)
+        if (wbase + r * 32 + lane < ti.cnt) S.sidx[pr[r]] = ir[r];
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < kSortItems; ++r)
+        if ((int64_t)g[r] < n) iout[g[r]] = S.sidx[r * kSortThreads + tid];
 }
+
+// Scratch of a sort: look-back words, digit counts and tickets, cleared
+// together at its start.
+struct SortScratch {
+    int64_t words, total;  // 32-bit words of the look-back part and in all
+};
+
+SortScratch sort_scratch(int64_t n, int64_t ntiles, int64_t nslots) {
+    SortScratch z;
+    z.words = ntiles * kRadix * (n < kSort32 ? 1 : 2);
+    z.total = z.words + nslots * kSortHist + 8;
+    return z;
+}
+
+// Sort (key[0]) into (key[0], idx[0]): eight passes, the first one numbering
+// the keys by position.
+template <class W>
+cudaError_t sort_passes(cudaStream_t s, uint64_t* const (&kb)[2], uint32_t* const (&ib)[2], int64_t n,
+                        const uint32_t* tmeta, int ntiles, int nslots, int num_sms, uint32_t* scratch, int* status) {
+    const SortScratch z = sort_scratch(n, ntiles, nslots);
+    W* words = reinterpret_cast<W*>(scratch);
+    uint32_t* hist = scratch + z.words;
+    uint32_t* ticket = hist + (int64_t)nslots * kSortHist;
+    cudaError_t e = cudaMemsetAsync(scratch, 0, (size_t)z.total * sizeof(uint32_t), s);
+    if (e != cudaSuccess) return e;
+    if (nslots > 0) {
+        const int nb = std::min(ntiles, 4 * num_sms);
+        k_digit_hist<<<nb, 256, 0, s>>>(kb[0], n, ntiles, tmeta, hist);
+    }
+    const int smem = (int)sizeof(SweepSmem);
+    for (int pass = 0; pass < 8; ++pass) {
+        const int a = pass & 1, b = 1 - a;
+        auto kern = pass == 0 ? k_sweep<W, true> : k_sweep<W, false>;
+        kern<<<ntiles, kSortThreads, smem, s>>>(kb[a], ib[a], n, pass, ntiles, tmeta, hist, words, ticket + pass, kb[b],
+                                                ib[b], status);
+    }
+    return cudaGetLastError();
+}
+
+cudaError_t sort_any(cudaStream_t s, uint64_t* const (&kb)[2], uint32_t* const (&ib)[2], int64_t n,
+                     const uint32_t* tmeta, int ntiles, int nslots, int num_sms, uint32_t* scratch, int* status) {
+    return n < kSort32 ? sort_passes<uint32_t>(s, kb, ib, n, tmeta, ntiles, nslots, num_sms, scratch, status)
+                       : sort_passes<unsigned long long>(s, kb, ib, n, tmeta, ntiles, nslots, num_sms, scratch, status);
+}
+constexpr int kSortLaunches = 9;  // kernels of one sort
 
 // All particle arrays (8-byte elements) gathered into key order in one pass:
 // the permutation is read once and every array's load is in flight at once;
-// dst[a] = scratch + a n (copied back by the caller).
+// into scratch + a n, then copied back to dst[a] (the same arrays).
 struct Gather8 {
     const unsigned long long* src[8];
+    unsigned long long* dst[8];
     int na;
 };
 
@@ -405,6 +539,20 @@ __global__ void k_gather_all(Gather8 G, unsigned long long* __restrict__ scratch
 #pragma unroll
     for (int a = 0; a < 8; ++a)
         if (a < G.na) scratch[(int64_t)a * n + i] = v[a];
+}
+
+// The gathered arrays back into place (one launch; eight copies of a small
+// set's arrays cost their launches).
+__global__ void k_copy_back(Gather8 G, const unsigned long long* __restrict__ scratch, int64_t n) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    unsigned long long v[8];
+#pragma unroll
+    for (int a = 0; a < 8; ++a)
+        if (a < G.na) v[a] = scratch[(int64_t)a * n + i];
+#pragma unroll
+    for (int a = 0; a < 8; ++a)
+        if (a < G.na) G.dst[a][i] = v[a];
 }
 
 }  // namespace
@@ -449,8 +597,7 @@ int stage_keys(Ctx* c, const bh_particles* p) {
                                              c->d_status);
         BH_LAUNCH(c);
     }
-    k_keys<<<blocks_for(n, 256), 256, 0, c->stream>>>(cx, cy, p->z, n, c->d_off.p, np, c->d_box, c->key[0].p,
-                                                      c->idx[0].p);
+    k_keys<<<blocks_for(n, 256), 256, 0, c->stream>>>(cx, cy, p->z, n, c->d_off.p, np, c->d_box, c->key[0].p);
     BH_LAUNCH(c);
     c->key_cur = 0;
     return BH_OK;
@@ -458,41 +605,20 @@ int stage_keys(Ctx* c, const bh_particles* p) {
 
 int stage_sort(Ctx* c) {
     const int64_t n = c->n;
-    const uint32_t* tmeta = c->n_patches > 1 ? c->tile_meta.p : nullptr;
-    const int ntiles = c->n_patches > 1 ? (int)c->n_tiles : (int)((n + kSortTile - 1) / kSortTile);
-    BH_TRY(grow(c, c->digit_hist, 8 * kRadix, "digit histogram"));
-    BH_TRY(grow(c, c->sort_hist, (size_t)kRadix * ntiles, "sort histogram"));
-    BH_CUDA(c, cudaMemsetAsync(c->digit_hist.p, 0, 8 * kRadix * sizeof(uint32_t), c->stream));
-    // passes whose digit is the same for every key leave the order as it is
-    // and are skipped (a device-sized build runs all eight: nothing is read
-    // back; the sort is stable, so the result is the same)
-    uint32_t h[8 * kRadix] = {};
-    if (!c->dev_build) {
-        k_digit_hist<<<c->num_sms * 2, 256, 0, c->stream>>>(c->key[c->key_cur].p, n, c->digit_hist.p);
-        BH_LAUNCH(c);
-        BH_CUDA(c, cudaMemcpyAsync(h, c->digit_hist.p, sizeof(h), cudaMemcpyDeviceToHost, c->stream));
-        BH_CUDA(c, cudaStreamSynchronize(c->stream));
-    }
-    const int smem = (int)sizeof(DownSmem);
+    const bool batch = c->n_patches > 1;
+    const uint32_t* tmeta = batch ? c->tile_meta.p : nullptr;
+    const int ntiles = batch ? (int)c->n_tiles : (int)((n + kSortTile - 1) / kSortTile);
+    const int nslots = batch ? c->n_sort_slots : ntiles > 1 ? 1 : 0;
+    BH_TRY(grow(c, c->sort_scratch, (size_t)sort_scratch(n, ntiles, nslots).total, "sort scratch"));
     if (c->sort_attr_device != c->device) {  // once per device
-        BH_CUDA(c, cudaFuncSetAttribute(k_downsweep, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+        BH_CUDA(c, sort_setup_device());
         c->sort_attr_device = c->device;
     }
-    for (int pass = 0; pass < 8; ++pass) {
-        bool trivial = false;
-        for (int d = 0; d < kRadix; ++d)
-            if ((int64_t)h[pass * kRadix + d] == n) trivial = true;
-        if (trivial) continue;  // every key has the same digit: order unchanged
-        const int shift = 8 * pass, a = c->key_cur, b = 1 - a;
-        k_upsweep<<<ntiles, kSortThreads, 0, c->stream>>>(c->key[a].p, n, shift, c->sort_hist.p, ntiles, tmeta);
-        BH_LAUNCH(c);
-        BH_TRY(scan_u32(c, c->sort_hist.p, c->sort_hist.p, (int64_t)kRadix * ntiles, nullptr));
-        k_downsweep<<<ntiles, kSortThreads, smem, c->stream>>>(c->key[a].p, c->idx[a].p, n, shift,
-                                                               c->sort_hist.p, ntiles, c->key[b].p,
-                                                               c->idx[b].p, tmeta);
-        BH_LAUNCH(c);
-        c->key_cur = b;
-    }
+    uint64_t* const kb[2] = {c->key[0].p, c->key[1].p};
+    uint32_t* const ib[2] = {c->idx[0].p, c->idx[1].p};
+    BH_CUDA(c, sort_any(c->stream, kb, ib, n, tmeta, ntiles, nslots, c->num_sms, c->sort_scratch.p, c->d_status));
+    c->n_launches += kSortLaunches - (nslots > 0 ? 0 : 1);
+    c->key_cur = 0;
     return BH_OK;
 }
 
@@ -504,78 +630,66 @@ int stage_permute(Ctx* c, bh_particles* p) {
                                    (unsigned long long*)p->vy, (unsigned long long*)p->vz,
                                    (unsigned long long*)p->m,  (unsigned long long*)p->id};
     const uint32_t* perm = c->idx[c->key_cur].p;
-    Gather8 G;
-    unsigned long long* dst[8];
-    G.na = 0;
+    Gather8 G = {};
     for (int a = 0; a < 8; ++a)
         if (arrs[a]) {
-            dst[G.na] = arrs[a];
+            G.dst[G.na] = arrs[a];
             G.src[G.na++] = arrs[a];
         }
     unsigned long long* scratch = (unsigned long long*)c->pscratch.p;
     k_gather_all<<<blocks_for(n, 256), 256, 0, c->stream>>>(G, scratch, perm, n, c->d_status);
     BH_LAUNCH(c);
-    for (int a = 0; a < G.na; ++a)
-        BH_CUDA(c, cudaMemcpyAsync(dst[a], scratch + (int64_t)a * n, n * sizeof(double), cudaMemcpyDeviceToDevice,
-                                   c->stream));
+    k_copy_back<<<blocks_for(n, 256), 256, 0, c->stream>>>(G, scratch, n);
+    BH_LAUNCH(c);
     return BH_OK;
 }
 
-// Sort tiles of the patches: 4 words per tile (see TileInfo).
-int64_t sort_tiles_for(const std::vector<int64_t>& off, std::vector<uint32_t>* meta) {
+// Sort tiles of the patches: 4 words per tile (see k_sweep); *nslots = patches
+// of more than one tile.
+int64_t sort_tiles_for(const std::vector<int64_t>& off, std::vector<uint32_t>* meta, int* nslots) {
     int64_t t = 0;
+    *nslots = 0;
     for (size_t q = 0; q + 1 < off.size(); ++q) {
         const int64_t np = off[q + 1] - off[q], nt = (np + kSortTile - 1) / kSortTile, t0 = t;
+        const uint32_t slot = nt > 1 ? (uint32_t)(*nslots)++ : 0u;
         for (int64_t u = 0; u < nt; ++u, ++t) {
-            if (meta) {
-                const int64_t st = off[q] + u * kSortTile, r = off[q + 1] - st;
-                meta->push_back((uint32_t)st);
-                meta->push_back((uint32_t)(r < kSortTile ? r : kSortTile));
-                meta->push_back((uint32_t)t0);
-                meta->push_back((uint32_t)nt);
-            }
+            const int64_t st = off[q] + u * kSortTile, r = off[q + 1] - st;
+            meta->push_back((uint32_t)st);
+            meta->push_back((uint32_t)(r < kSortTile ? r : kSortTile) | slot << kSlotShift);
+            meta->push_back((uint32_t)t0);
+            meta->push_back((uint32_t)nt);
         }
     }
     return t;
 }
 
-// Context-free form of stage_sort for callers that supply every buffer: all
-// eight passes run (no host read-back of the digit histogram, so nothing here
-// synchronises), ending in (keys, idx) again.  idx is set to 0..n-1 first.
+// Context-free form of stage_sort for callers that supply every buffer,
+// ending in (keys, idx) again; nothing here synchronises.
 int64_t sort_scratch_words(int64_t n) {
     const int64_t ntiles = (n + kSortTile - 1) / kSortTile;
-    return kRadix * ntiles + scan_sums_count(kRadix * ntiles);
+    return sort_scratch(n, ntiles, 1).total;
 }
 
 cudaError_t sort_setup_device() {
-    return cudaFuncSetAttribute(k_downsweep, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(DownSmem));
+    const int smem = (int)sizeof(SweepSmem);
+    const void* kerns[4] = {(const void*)k_sweep<uint32_t, true>, (const void*)k_sweep<uint32_t, false>,
+                            (const void*)k_sweep<unsigned long long, true>,
+                            (const void*)k_sweep<unsigned long long, false>};
+    for (const void* k : kerns) {
+        const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
-
-namespace {
-__global__ void k_iota(uint32_t* __restrict__ idx, int64_t n) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) idx[i] = (uint32_t)i;
-}
-}  // namespace
 
 cudaError_t sort_pairs_with(cudaStream_t s, uint64_t* keys, uint32_t* idx, uint64_t* ktmp, uint32_t* itmp,
-                            int64_t n, uint32_t* scratch) {
+                            int64_t n, int num_sms, uint32_t* scratch, int* status) {
     if (n <= 0) return cudaSuccess;
     const int ntiles = (int)((n + kSortTile - 1) / kSortTile);
-    uint32_t* hist = scratch;
-    uint32_t* sums = scratch + (int64_t)kRadix * ntiles;
-    k_iota<<<blocks_for(n, 256), 256, 0, s>>>(idx, n);
-    uint64_t* kb[2] = {keys, ktmp};
-    uint32_t* ib[2] = {idx, itmp};
-    for (int pass = 0; pass < 8; ++pass) {
-        const int a = pass & 1, b = 1 - a;
-        k_upsweep<<<ntiles, kSortThreads, 0, s>>>(kb[a], n, 8 * pass, hist, ntiles, nullptr);
-        cudaError_t e = scan_u32_with(s, hist, hist, (int64_t)kRadix * ntiles, sums);
-        if (e != cudaSuccess) return e;
-        k_downsweep<<<ntiles, kSortThreads, sizeof(DownSmem), s>>>(kb[a], ib[a], n, 8 * pass, hist, ntiles,
-                                                                   kb[b], ib[b], nullptr);
-    }
-    return cudaGetLastError();
+    uint64_t* const kb[2] = {keys, ktmp};
+    uint32_t* const ib[2] = {idx, itmp};
+    return sort_any(s, kb, ib, n, nullptr, ntiles, ntiles > 1 ? 1 : 0, num_sms, scratch, status);
 }
+int sort_launches() { return kSortLaunches; }
 
 }  // namespace bh
