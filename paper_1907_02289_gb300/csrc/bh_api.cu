@@ -227,10 +227,14 @@ int check_particles(Ctx* c, const bh_particles* p, bool need_v) {
     return BH_OK;
 }
 
+}  // namespace
+
+// (the last of h_pin's words; the callers' own read-backs use the first ones)
 int read_status(Ctx* c) {
-    int st = 0;
-    BH_CUDA(c, cudaMemcpyAsync(&st, c->d_status, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+    BH_CUDA(c, cudaMemcpyAsync(c->h_pin + 63, c->d_status, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
     BH_CUDA(c, cudaStreamSynchronize(c->stream));
+    int st;
+    memcpy(&st, c->h_pin + 63, sizeof(int));
     if (st) BH_CUDA(c, cudaMemsetAsync(c->d_status, 0, sizeof(int), c->stream));
     if (st & kStatNonFinite) return fail(c, BH_E_INVAL, "non-finite particle coordinate");
     if (st & kStatAxis) return fail(c, BH_E_INVAL, "the cylindrical key frame needs every particle off the axis (r > 0)");
@@ -241,6 +245,8 @@ int read_status(Ctx* c) {
         return fail(c, BH_E_INVAL, "a contact acceleration term reached 1024 or was not finite (kappa, eta too large?)");
     return BH_OK;
 }
+
+namespace {
 
 int build_tree(Ctx* c, bh_particles* p) {
     BH_TRY(check_particles(c, p, true));
@@ -254,7 +260,6 @@ int build_tree(Ctx* c, bh_particles* p) {
         BH_TRY(setup_patches(c, 1, off));
     }
     BH_STAGE(c, BH_STAGE_KEYS, stage_keys(c, p));
-    BH_TRY(read_status(c));  // non-finite coordinates; a particle on the axis of the cylindrical frame
     BH_STAGE(c, BH_STAGE_SORT, stage_sort(c));
     BH_STAGE(c, BH_STAGE_PERMUTE, stage_permute(c, p));
     BH_TRY(stage_begin(c, BH_STAGE_TREE));
@@ -525,8 +530,8 @@ int size_dev_build(Ctx* c, const int64_t cap[5]) {
     for (auto* b : {&c->cnt_p, &c->cnt_c, &c->cnt_j, &c->cnt_jm})
         BH_TRY(grow(c, *b, (size_t)n + 1, "list offsets"));
     BH_TRY(grow(c, c->order, (size_t)n + 1, "group order"));
-    // scans over up to n group counts (8-byte words, 2048 per tile)
-    BH_TRY(grow(c, c->scan_tmp, ((size_t)n / 2048 + 2) * sizeof(int64_t), "scan block sums"));
+    // three scans over up to n group counts (8-byte words, 2048 per tile)
+    BH_TRY(grow(c, c->scan_tmp, 3 * ((size_t)n / 2048 + 2) * sizeof(int64_t), "scan block sums"));
     BH_TRY(grow(c, c->stash_p, (size_t)std::max<int64_t>(1, cap[1] * c->walk_cap_p), "stashed particle lists"));
     BH_TRY(grow(c, c->stash_c, (size_t)std::max<int64_t>(1, cap[1] * c->walk_cap_c), "stashed cell lists"));
     BH_TRY(grow(c, c->P, (size_t)cap[2] + 1, "particle lists"));
@@ -651,10 +656,9 @@ int graph_rebuild_step(Ctx* c, bh_particles* p) {
     if (!rebuild_graph_fits(c, p)) BH_TRY(capture_rebuild(c, p));
     BH_TRY(launch_graph(c, c->rgraph_exec, c->gt_rebuild));
     c->n_launches += c->rgraph_launches;
-    unsigned long long sz[kSzWords], sm[24];
-    BH_CUDA(c, cudaMemcpyAsync(sz, c->d_sz, sizeof(sz), cudaMemcpyDeviceToHost, c->stream));
-    BH_CUDA(c, cudaMemcpyAsync(sm, c->d_small, sizeof(sm), cudaMemcpyDeviceToHost, c->stream));
-    BH_CUDA(c, cudaStreamSynchronize(c->stream));
+    const unsigned long long *sz = c->h_pin, *sm = c->h_pin + kSzWords;  // (24 words)
+    BH_CUDA(c, cudaMemcpyAsync(c->h_pin, c->d_sz, kSzWords * sizeof(*sz), cudaMemcpyDeviceToHost, c->stream));
+    BH_CUDA(c, cudaMemcpyAsync(c->h_pin + kSzWords, c->d_small, 24 * sizeof(*sm), cudaMemcpyDeviceToHost, c->stream));
     BH_TRY(read_status(c));
     ++c->n_graph_builds;
     if (sz[kSzOvf] != 0) {
@@ -678,6 +682,7 @@ int graph_rebuild_step(Ctx* c, bh_particles* p) {
     c->n_int_pp = (int64_t)sm[8];
     c->n_int_pc = (int64_t)sm[9];
     c->n_int_pp_far = c->prm.precision == BH_PREC_FP32 ? (int64_t)sm[10] : 0;
+    c->far_pending = false;
     if (sm[11] == 0) ++c->n_one_walk_builds;
     c->walk_cap_p = (int64_t)(((sm[12] + sm[12] / 4 + 4) + 3) & ~3ull);
     c->walk_cap_c = (int64_t)(((sm[13] + sm[13] / 4 + 4) + 3) & ~3ull);
@@ -932,6 +937,8 @@ static int create_ctx(const char* who, const bh_params* p, int n_patches, const 
     if (e == cudaSuccess) e = cudaMalloc(&c->d_box, 8 * sizeof(double) * (size_t)n_patches);
     if (e == cudaSuccess) e = cudaMalloc(&c->d_small, 64 * sizeof(unsigned long long));
     if (e == cudaSuccess) e = cudaMalloc(&c->d_sz, bh::kSzWords * sizeof(unsigned long long));
+    if (e == cudaSuccess) e = cudaHostAlloc(&c->h_pin, 64 * sizeof(unsigned long long), cudaHostAllocDefault);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->count_event, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->d_sz, 0, bh::kSzWords * sizeof(unsigned long long), c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->d_status, 0, sizeof(int), c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
@@ -983,6 +990,8 @@ int bh_destroy(bh_ctx* ctx) {
     cudaFree(c->d_box);
     cudaFree(c->d_small);
     cudaFree(c->d_sz);
+    if (c->h_pin) cudaFreeHost(c->h_pin);
+    if (c->count_event) cudaEventDestroy(c->count_event);
     using bh::release;
     release(c->d_off); release(c->tile_meta); release(c->box_map); release(c->box_poff); release(c->d_rcq); release(c->d_rfar); release(c->d_period); release(c->cyl); release(c->box_part); release(c->order_cnt); release(c->warp_time); release(c->contact_acc); release(c->diag); release(c->pot);
     for (int b = 0; b < 2; ++b) {
@@ -1359,6 +1368,13 @@ int bh_get_counters(bh_ctx* ctx, bh_counters* out) {
     out->n_rebuilds = c->n_rebuilds;
     out->n_launches = c->n_launches;
     out->n_contacts = c->n_contacts;
+    if (c->far_pending) {  // an eager list build since: read its count now
+        unsigned long long hf = 0;
+        BH_CUDA(c, cudaMemcpyAsync(&hf, c->d_small + 10, sizeof(hf), cudaMemcpyDeviceToHost, c->stream));
+        BH_CUDA(c, cudaStreamSynchronize(c->stream));
+        c->n_int_pp_far = (int64_t)hf;
+        c->far_pending = false;
+    }
     out->n_pp_far = c->n_int_pp_far;
     out->n_one_walk_builds = c->n_one_walk_builds;
     out->n_h2d_bytes = c->h2d_bytes;

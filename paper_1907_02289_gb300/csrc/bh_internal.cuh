@@ -129,6 +129,8 @@ struct Ctx {
     int* d_status = nullptr;
     double* d_box = nullptr;   // per patch: lo[3], L, S, spare x3 (8 doubles)
     unsigned long long* d_small = nullptr;  // scan totals etc. (64 words)
+    unsigned long long* h_pin = nullptr;    // page-locked words for size read-backs (64)
+    cudaEvent_t count_event = nullptr;      // the contact count has been copied to h_pin
 
     // keys and sort
     DBuf<uint64_t> key[2];
@@ -234,6 +236,7 @@ struct Ctx {
     int64_t n_pp = 0, n_pc = 0, n_jj = 0;
     int64_t n_int_pp = 0, n_int_pc = 0;
     int64_t n_int_pp_far = 0;            // FP32 path: pp interactions with far list particles
+    bool far_pending = false;            // a list build ran since n_int_pp_far was read (word 10 of d_small)
     DBuf<int64_t> cnt_p, cnt_c, cnt_j;   // per group counts, then offsets (ng + 1)
     DBuf<int64_t> cnt_jm;                // FP32 path: per group index of the first far list particle
     DBuf<int32_t> stash_p, stash_c;      // per group list slots of the one-walk build
@@ -276,12 +279,12 @@ inline unsigned blocks_for(int64_t n, int threads) {
 }
 
 // ---- stage entry points (one translation unit each) ------------------------
-// scan.cu: exclusive prefix sums; *total written to d_total (device) if given.
-// With dn, the element count is read on the device (*dn, at most n).
-int scan_u32(Ctx* c, const uint32_t* in, uint32_t* out, int64_t n, unsigned long long* d_total,
-             const unsigned long long* dn = nullptr);
-int scan_i64(Ctx* c, const int64_t* in, int64_t* out, int64_t n, unsigned long long* d_total,
-             const unsigned long long* dn = nullptr);
+// scan.cu: exclusive prefix sums in place, n >= 1; the total goes to *d_total
+// (device).  scan3_i64: three arrays of n (+ 1) elements, totals to
+// d_total[0..2] and to each array's element n; with dn, the element count is
+// read on the device (*dn, at most n).
+int scan_u32(Ctx* c, uint32_t* v, int64_t n, unsigned long long* d_total);
+int scan3_i64(Ctx* c, int64_t* const (&v)[3], int64_t n, unsigned long long* d_total, const unsigned long long* dn);
 
 // sort.cu
 int stage_keys(Ctx* c, const bh_particles* p);     // root box + keys (+ status on NaN)
@@ -313,6 +316,9 @@ int stage_split(Ctx* c, const bh_particles* p);    // FP32 hi/lo split of partic
 int build_order32(Ctx* c);                         // FP32 kernel's group order (per list build)
 int stage_force(Ctx* c, bh_particles* p, bool add_central);
 int stage_potential(Ctx* c, const bh_particles* p, double* phi, double* W);  // self-gravity potential (FP64)
+
+// bh_api.cu: wait for the stream and report the device status word
+int read_status(Ctx* c);
 
 // bh_api.cu: force-kernel and stage timing (no-ops unless enabled, or while
 // capturing a graph); stage_end closes the innermost stage begun

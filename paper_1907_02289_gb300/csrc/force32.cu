@@ -745,11 +745,11 @@ __device__ __forceinline__ void group_chunk(const Args& A, Smem32& S, int64_t k,
             // an ill-conditioned sum (terms far larger than the total) goes to
             // the refinement pass, which rewrites a_i
             const double kg = A.kref * A.fp.G;
-            if (A.refine && hc) {  // judged with its contact term, after the contact pass
+            if (hc) {  // judged with its contact term, after the contact pass
                 A.cbnd[i] = bnd;
                 A.cslot[i] = (uint32_t)k;
                 A.cflag[i] = 1u;
-            } else if (A.refine && a[0] * a[0] + a[1] * a[1] + a[2] * a[2] < kg * kg * (double)bnd) {
+            } else if (a[0] * a[0] + a[1] * a[1] + a[2] * a[2] < kg * kg * (double)bnd) {
                 const unsigned long long q = atomicAdd(A.nrefine, 1ull);
                 A.refine[q] = make_uint2(i, (uint32_t)k);
             }
@@ -896,30 +896,33 @@ __global__ void k_order_keys(int64_t ng, const int32_t* __restrict__ groups, con
     keys[k] = ((uint64_t)(k / window) << 8) | (uint64_t)order_bucket(k, groups, begin, end, jj_off, pc_off, chunk, by_cost);
 }
 
-// exclusive prefix of the bucket counts (one block of kOrderBuckets threads)
-__global__ void k_order_prefix(unsigned long long* cnt) {
-    __shared__ unsigned long long v[kOrderBuckets];
-    v[threadIdx.x] = cnt[threadIdx.x];
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        unsigned long long run = 0;
-        for (int b = 0; b < kOrderBuckets; ++b) {
-            const unsigned long long t = v[b];
-            v[b] = run;
-            run += t;
-        }
-    }
-    __syncthreads();
-    cnt[threadIdx.x] = v[threadIdx.x];
-}
-
 __global__ void k_order_scatter(int64_t ng, const unsigned long long* __restrict__ dng,
                                 const int32_t* __restrict__ groups, const uint32_t* __restrict__ begin,
                                 const uint32_t* __restrict__ end, const int64_t* __restrict__ jj_off,
                                 const int64_t* __restrict__ pc_off, uint32_t chunk, bool by_cost,
-                                const unsigned long long* __restrict__ start, unsigned long long* cursor,
+                                const unsigned long long* __restrict__ cnt, unsigned long long* cursor,
                                 int32_t* __restrict__ order) {
     if (dng) ng = min(ng, (int64_t)*dng);
+    // exclusive prefix of the bucket counts, by the block's first warp
+    __shared__ unsigned long long start[kOrderBuckets];
+    constexpr int PL = kOrderBuckets / 32;
+    if (threadIdx.x < 32) {
+        unsigned long long v[PL], sum = 0;
+#pragma unroll
+        for (int b = 0; b < PL; ++b) {
+            v[b] = sum;
+            sum += cnt[threadIdx.x * PL + b];
+        }
+        unsigned long long x = sum;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned long long y = __shfl_up_sync(0xffffffffu, x, o);
+            if (threadIdx.x >= o) x += y;
+        }
+#pragma unroll
+        for (int b = 0; b < PL; ++b) start[threadIdx.x * PL + b] = x - sum + v[b];
+    }
+    __syncthreads();
     for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < ng; k += (int64_t)gridDim.x * blockDim.x) {
         const int b = order_bucket(k, groups, begin, end, jj_off, pc_off, chunk, by_cost);
         order[start[b] + atomicAdd(&cursor[b], 1ull)] = (int32_t)k;
@@ -933,10 +936,11 @@ __global__ void k_order_scatter(int64_t ng, const unsigned long long* __restrict
 // The candidates arrive in no fixed order (warps append them as they go), so
 // the terms are summed per particle in 64-bit fixed point (units of 2^-50,
 // terms below 2^10 in magnitude): integer addition does not depend on the
-// order, which keeps every run bit-reproducible.  Three passes: clear the
-// accumulators of the particles involved, add the terms, then move each
-// particle's sum into its acceleration (the first pass to take it adds the
-// whole sum, every later one adds zero).
+// order, which keeps every run bit-reproducible.  Two passes: add the terms;
+// then the first thread to claim a particle's flag moves its sum into the
+// acceleration, leaves the accumulator at zero for the next evaluation, and
+// judges whether the particle is refined.  Both take the number of pairs from
+// the device, so the host issues them without waiting for it.
 constexpr double kFix = 1125899906842624.0;  // 2^50
 constexpr double kFixMax = 1024.0;
 
@@ -950,22 +954,14 @@ __device__ __forceinline__ int64_t contact_count(const unsigned long long* count
     return np;
 }
 
-__global__ void k_contacts_clear(const uint2* __restrict__ pairs, const unsigned long long* __restrict__ count,
-                                 int64_t cap, unsigned long long* __restrict__ acc, int* status) {
-    const int64_t np = contact_count(count, cap, status, true);
-    for (int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; u < np; u += (int64_t)gridDim.x * blockDim.x) {
-        const uint32_t i = pairs[u].x;
-        acc[3 * (int64_t)i] = acc[3 * (int64_t)i + 1] = acc[3 * (int64_t)i + 2] = 0ull;
-    }
-}
-
 __global__ void k_contacts64(const uint2* __restrict__ pairs, const unsigned long long* __restrict__ count,
                              int64_t cap, ForceParams fp, const double* __restrict__ x,
                              const double* __restrict__ y, const double* __restrict__ z,
                              const double* __restrict__ vx, const double* __restrict__ vy,
                              const double* __restrict__ vz, const double* __restrict__ m,
-                             unsigned long long* __restrict__ acc, unsigned long long* n_touch, int* status) {
-    const int64_t np = contact_count(count, cap, status, false);
+                             unsigned long long* __restrict__ acc, unsigned long long* n_touch, int* status,
+                             bool flag) {
+    const int64_t np = contact_count(count, cap, status, flag);
     unsigned long long touching = 0;
     for (int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; u < np; u += (int64_t)gridDim.x * blockDim.x) {
         const uint2 pr = pairs[u];
@@ -986,21 +982,6 @@ __global__ void k_contacts64(const uint2* __restrict__ pairs, const unsigned lon
     if (touching) atomicAdd(n_touch, touching);
 }
 
-__global__ void k_contacts_apply(const uint2* __restrict__ pairs, const unsigned long long* __restrict__ count,
-                                 int64_t cap, unsigned long long* __restrict__ acc, double* ax, double* ay,
-                                 double* az, int* status) {
-    const int64_t np = contact_count(count, cap, status, false);
-    for (int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; u < np; u += (int64_t)gridDim.x * blockDim.x) {
-        const uint32_t i = pairs[u].x;
-        double* out[3] = {ax, ay, az};
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            const long long v = (long long)atomicExch(&acc[3 * (int64_t)i + c], 0ull);
-            if (v != 0) atomicAdd(&out[c][i], (double)v / kFix);
-        }
-    }
-}
-
 // ---- refinement of ill-conditioned particles ------------------------------
 // A particle whose FP32 sum is ill-conditioned (|a_i| small against the sum
 // of |tile partial sums|, e.g. where the pull of its neighbours nearly
@@ -1013,7 +994,7 @@ __global__ void k_contacts_apply(const uint2* __restrict__ pairs, const unsigned
 // queued particle; the lanes split the entries and the partial sums are
 // reduced in df.  The result replaces a_i; the pass runs after the contact
 // pass, whose terms it includes.  A particle with a contact candidate is
-// judged only after that pass (k_flag_contacts): the spring term can cancel
+// judged only after that pass (k_contacts_apply): the spring term can cancel
 // the pull of the neighbour it touches.
 struct RefineConsts {
     df rc2, eps2, rc2eps2;  // r_coll^2, eps^2, r_coll^2 + eps^2
@@ -1083,11 +1064,11 @@ __device__ __forceinline__ void ref_pc(const Args& A, const RefineConsts& K, flo
     for (int c = 0; c < 3; ++c) acc[c] = df_add(acc[c], t[c]);
 }
 
-// After the contact pass: each particle with a contact candidate (claimed
-// once through its flag) is queued when its tree part, gravity and contact,
-// is small against its FP32 bound.
-__global__ void k_flag_contacts(const Args A, const uint2* __restrict__ pairs, const unsigned long long* count,
-                                int64_t cap) {
+// After the contact terms: each particle with a contact candidate (claimed
+// once through its flag) gets their sum, and is queued when its tree part,
+// gravity and contact, is small against its FP32 bound.
+__global__ void k_contacts_apply(const Args A, const uint2* __restrict__ pairs, const unsigned long long* count,
+                                 int64_t cap, unsigned long long* __restrict__ acc) {
     int64_t np = (int64_t)*count;
     if (np > cap) np = cap;
     const double kg = A.kref * A.fp.G;
@@ -1095,6 +1076,15 @@ __global__ void k_flag_contacts(const Args A, const uint2* __restrict__ pairs, c
         const uint32_t i = pairs[u].x;
         if (i >= A.n || atomicExch(&A.cflag[i], 0u) == 0u) continue;
         double a[3] = {A.ax[i], A.ay[i], A.az[i]};
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            const long long v = (long long)acc[3 * (int64_t)i + q];
+            acc[3 * (int64_t)i + q] = 0ull;
+            a[q] += (double)v / kFix;
+        }
+        A.ax[i] = a[0];
+        A.ay[i] = a[1];
+        A.az[i] = a[2];
         if (A.add_central) {  // the tree part: the central term taken off again
             double c[3] = {0.0, 0.0, 0.0};
             central_newton(A.fp.GMc, A.x[i], A.y[i], A.z[i], c);
@@ -1295,8 +1285,6 @@ int build_order32(Ctx* c) {
     k_order_hist<<<nb, 256, 0, c->stream>>>(ng, dng, c->groups.p, c->begin.p, c->end.p, c->cnt_j.p, c->cnt_c.p, chunk,
                                             by_cost, cnt);
     BH_LAUNCH(c);
-    k_order_prefix<<<1, kOrderBuckets, 0, c->stream>>>(cnt);
-    BH_LAUNCH(c);
     k_order_scatter<<<nb, 256, 0, c->stream>>>(ng, dng, c->groups.p, c->begin.p, c->end.p, c->cnt_j.p, c->cnt_c.p,
                                                chunk, by_cost, cnt, cnt + kOrderBuckets, c->order.p);
     BH_LAUNCH(c);
@@ -1315,7 +1303,6 @@ RefineConsts refine_consts(const ForceParams& fp) {
 // The refinement pass over the particles the force kernel queued (count
 // read on the device, so it can run inside a captured graph).
 int refine_pass(Ctx* c, const Args& A, const ForceParams& fp) {
-    if (!A.refine) return BH_OK;
     BH_TRY(stage_begin(c, BH_STAGE_REFINE));
     k_refine32<<<(unsigned)(c->num_sms * 4), 256, 0, c->stream>>>(A, refine_consts(fp), c->cell32lo.p,
                                                                    (int64_t)c->refine.cap);
@@ -1323,25 +1310,15 @@ int refine_pass(Ctx* c, const Args& A, const ForceParams& fp) {
     return stage_end(c);
 }
 
-// The particles with contact candidates, judged after the contact pass.
-int flag_pass(Ctx* c, const Args& A, unsigned nb) {
-    if (!A.refine) return BH_OK;
-    BH_TRY(stage_begin(c, BH_STAGE_REFINE));
-    k_flag_contacts<<<nb, 128, 0, c->stream>>>(A, A.contacts, A.ncontact, A.contact_cap);
-    BH_LAUNCH(c);
-    return stage_end(c);
-}
-
-int contact_pass(Ctx* c, const Args& A, const ForceParams& fp, bh_particles* p, unsigned nb) {
-    BH_TRY(stage_begin(c, BH_STAGE_CONTACTS));
+int contact_pass(Ctx* c, const Args& A, const ForceParams& fp, bh_particles* p) {
+    const unsigned nb = (unsigned)(c->num_sms * 4);
     unsigned long long* acc = c->contact_acc.p;
-    k_contacts_clear<<<nb, 128, 0, c->stream>>>(A.contacts, A.ncontact, A.contact_cap, acc, c->d_status);
-    BH_LAUNCH(c);
+    BH_TRY(stage_begin(c, BH_STAGE_CONTACTS));
+    // (an overflow is flagged in a captured step; eagerly the host sees the count)
     k_contacts64<<<nb, 128, 0, c->stream>>>(A.contacts, A.ncontact, A.contact_cap, fp, p->x, p->y, p->z, p->vx, p->vy,
-                                            p->vz, p->m, acc, c->d_small + 18, c->d_status);
+                                            p->vz, p->m, acc, c->d_small + 18, c->d_status, c->capturing);
     BH_LAUNCH(c);
-    k_contacts_apply<<<nb, 128, 0, c->stream>>>(A.contacts, A.ncontact, A.contact_cap, acc, p->ax, p->ay, p->az,
-                                                c->d_status);
+    k_contacts_apply<<<nb, 128, 0, c->stream>>>(A, A.contacts, A.ncontact, A.contact_cap, acc);
     BH_LAUNCH(c);
     return stage_end(c);
 }
@@ -1373,15 +1350,16 @@ int launch_force32(Ctx* c, bh_particles* p, const ForceParams& fp, bool add_cent
     const bool contact = c->prm.r_coll > 0.0;
     const int64_t cap = c->n > 65536 ? c->n : 65536;
     if (contact && c->contacts.cap < (size_t)cap) BH_TRY(grow(c, c->contacts, (size_t)cap, "contact pairs"));
-    if (contact) BH_TRY(grow(c, c->contact_acc, 3 * (size_t)c->n, "contact sums"));
+    if (contact && c->contact_acc.cap < 3 * (size_t)c->n) {  // zero between evaluations
+        BH_TRY(grow(c, c->contact_acc, 3 * (size_t)c->n, "contact sums"));
+        BH_CUDA(c, cudaMemsetAsync(c->contact_acc.p, 0, c->contact_acc.cap * sizeof(unsigned long long), c->stream));
+    }
     A.contacts = reinterpret_cast<uint2*>(c->contacts.p);
     A.contact_cap = (int64_t)c->contacts.cap;
     if (c->capturing && c->tune.graph_contact_room > 0)  // the room a graph step may use
         A.contact_cap = std::min(A.contact_cap, (int64_t)c->tune.graph_contact_room);
     A.ncontact = c->d_small + 16;
     c->contact_stats = contact;
-    BH_CUDA(c, cudaMemsetAsync(A.ncontact, 0, sizeof(unsigned long long), c->stream));
-    BH_CUDA(c, cudaMemsetAsync(c->d_small + 18, 0, sizeof(unsigned long long), c->stream));  // pairs in contact
     A.n = (uint32_t)c->n;
     A.nn = c->n_nodes;
     A.status = c->d_status;
@@ -1406,7 +1384,6 @@ int launch_force32(Ctx* c, bh_particles* p, const ForceParams& fp, bool add_cent
     A.warp_time = nullptr;
     A.kref = BH_REFINE_K;
     A.nrefine = c->d_small + 20;
-    A.refine = nullptr;
     A.cbnd = nullptr;
     A.cslot = nullptr;
     A.cflag = nullptr;
@@ -1414,19 +1391,17 @@ int launch_force32(Ctx* c, bh_particles* p, const ForceParams& fp, bool add_cent
     A.vy = p->vy;
     A.vz = p->vz;
     A.m = p->m;
-    if (A.kref > 0.0) {
-        BH_TRY(grow(c, c->refine, (size_t)c->n, "refinement queue"));
-        A.refine = c->refine.p;
-        if (contact) {
-            const bool fresh = c->cflag.cap < (size_t)c->n;
-            BH_TRY(grow(c, c->cbnd, (size_t)c->n, "contact-particle bounds"));
-            BH_TRY(grow(c, c->cslot, (size_t)c->n, "contact-particle list slots"));
-            BH_TRY(grow(c, c->cflag, (size_t)c->n, "contact-particle flags"));
-            if (fresh) BH_CUDA(c, cudaMemsetAsync(c->cflag.p, 0, c->cflag.cap * sizeof(unsigned), c->stream));
-            A.cbnd = c->cbnd.p;
-            A.cslot = c->cslot.p;
-            A.cflag = c->cflag.p;
-        }
+    BH_TRY(grow(c, c->refine, (size_t)c->n, "refinement queue"));
+    A.refine = c->refine.p;
+    if (contact) {
+        const bool fresh = c->cflag.cap < (size_t)c->n;
+        BH_TRY(grow(c, c->cbnd, (size_t)c->n, "contact-particle bounds"));
+        BH_TRY(grow(c, c->cslot, (size_t)c->n, "contact-particle list slots"));
+        BH_TRY(grow(c, c->cflag, (size_t)c->n, "contact-particle flags"));
+        if (fresh) BH_CUDA(c, cudaMemsetAsync(c->cflag.p, 0, c->cflag.cap * sizeof(unsigned), c->stream));
+        A.cbnd = c->cbnd.p;
+        A.cslot = c->cslot.p;
+        A.cflag = c->cflag.p;
     }
     unsigned nb;
     if (c->tune.sched == BH_SCHED_GRID && !A.dng) {
@@ -1437,7 +1412,6 @@ int launch_force32(Ctx* c, bh_particles* p, const ForceParams& fp, bool add_cent
         if ((int64_t)nb > need) nb = (unsigned)(need > 0 ? need : 1);
         if (c->tune.sched == BH_SCHED_DYNAMIC) {
             A.ticket = c->d_small + 17;
-            BH_CUDA(c, cudaMemsetAsync(A.ticket, 0, sizeof(unsigned long long), c->stream));
         }
         if (c->timing && !c->capturing) {
             BH_TRY(grow(c, c->warp_time, 2 * (size_t)nb * W, "warp times"));
@@ -1446,48 +1420,36 @@ int launch_force32(Ctx* c, bh_particles* p, const ForceParams& fp, bool add_cent
         }
     }
     c->f32_blocks = nb;
-    c->refine_pending = A.refine != nullptr;  // its count is read when asked for
+    c->refine_pending = true;  // its count is read when asked for
     for (int attempt = 0; attempt < 2; ++attempt) {
-        BH_CUDA(c, cudaMemsetAsync(A.nrefine, 0, sizeof(unsigned long long), c->stream));
+        // words 16..20: contact candidates, ticket, pairs in contact, (unused), refinement queue
+        BH_CUDA(c, cudaMemsetAsync(c->d_small + 16, 0, 5 * sizeof(unsigned long long), c->stream));
         BH_TRY(timing_begin(c));
         BH_TRY(stage_begin(c, BH_STAGE_FORCE));
         kern<<<nb, 32 * W, smem, c->stream>>>(A);
         BH_LAUNCH(c);
         BH_TRY(stage_end(c));
         BH_TRY(timing_end(c));
-        if (!contact) {
-            BH_TRY(refine_pass(c, A, fp));
-            break;
+        // the passes that follow take their counts from the device
+        const bool read = contact && !c->capturing;
+        if (read) {
+            BH_CUDA(c, cudaMemcpyAsync(c->h_pin, A.ncontact, sizeof(unsigned long long), cudaMemcpyDeviceToHost,
+                                       c->stream));
+            BH_CUDA(c, cudaEventRecord(c->count_event, c->stream));
         }
-        if (c->capturing) {
-            // inside a captured graph: no read-back; the passes take the count
-            // from the device and an overflow is flagged in the status word
-            const unsigned nbc = (unsigned)(c->num_sms * 4);
-            BH_TRY(contact_pass(c, A, fp, p, nbc));
-            BH_TRY(flag_pass(c, A, nbc));
-            BH_TRY(refine_pass(c, A, fp));
-            break;
-        }
-        // size the FP64 contact pass (one read-back per evaluation); on
-        // overflow grow the list and evaluate again
-        unsigned long long np = 0;
-        BH_CUDA(c, cudaMemcpyAsync(&np, A.ncontact, sizeof(np), cudaMemcpyDeviceToHost, c->stream));
-        BH_CUDA(c, cudaStreamSynchronize(c->stream));
-        c->n_contacts = (int64_t)np;
-        if ((int64_t)np > A.contact_cap) {
-            BH_TRY(grow(c, c->contacts, (size_t)(np + np / 4 + 1024), "contact pairs"));
-            A.contacts = reinterpret_cast<uint2*>(c->contacts.p);
-            A.contact_cap = (int64_t)c->contacts.cap;
-            BH_CUDA(c, cudaMemsetAsync(A.ncontact, 0, sizeof(unsigned long long), c->stream));
-            if (A.ticket) BH_CUDA(c, cudaMemsetAsync(A.ticket, 0, sizeof(unsigned long long), c->stream));
-            continue;
-        }
-        if (np > 0) {
-            BH_TRY(contact_pass(c, A, fp, p, blocks_for((int64_t)np, 128)));
-            BH_TRY(flag_pass(c, A, blocks_for((int64_t)np, 128)));
-        }
+        if (contact) BH_TRY(contact_pass(c, A, fp, p));
         BH_TRY(refine_pass(c, A, fp));
-        break;
+        if (!read) break;
+        // the host waits for the count alone (the passes run on); on overflow
+        // it grows the list and evaluates again.  Inside a captured graph
+        // nothing is read back: an overflow is flagged in the status word.
+        BH_CUDA(c, cudaEventSynchronize(c->count_event));
+        const int64_t np = (int64_t)c->h_pin[0];
+        c->n_contacts = np;
+        if (np <= A.contact_cap) break;
+        BH_TRY(grow(c, c->contacts, (size_t)(np + np / 4 + 1024), "contact pairs"));
+        A.contacts = reinterpret_cast<uint2*>(c->contacts.p);
+        A.contact_cap = (int64_t)c->contacts.cap;
     }
     return BH_OK;
 }

@@ -1,6 +1,5 @@
 // scan.cu -- device-wide exclusive prefix sums (reduce, scan block sums,
-// scan tiles with offsets).  Used for radix-sort digit offsets, octree child
-// offsets, group compaction and list offsets.
+// scan tiles with offsets).  Used for octree node ids and list offsets.
 #include <algorithm>
 
 #include "bh_internal.cuh"
@@ -48,10 +47,21 @@ __device__ __forceinline__ int64_t count_of(int64_t n, const unsigned long long*
     return v < (unsigned long long)n ? (int64_t)v : n;
 }
 
+// Up to three arrays of one length in one launch: blockIdx.y is the array, its
+// block sums start at blockIdx.y * stride.
 template <typename T>
-__global__ void k_reduce(const T* __restrict__ in, int64_t n, const unsigned long long* dn, T* __restrict__ sums) {
+struct ScanArrays {
+    const T* in[3];
+    T* out[3];
+};
+
+template <typename T>
+__global__ void k_reduce(ScanArrays<T> a, int64_t n, const unsigned long long* dn, T* __restrict__ sums,
+                         int64_t stride) {
     __shared__ T wt[kThreads / 32];
     __shared__ T tot;
+    const T* __restrict__ in = a.in[blockIdx.y];
+    sums += blockIdx.y * stride;
     n = count_of(n, dn);
     const int64_t nt = (n + kTile - 1) / kTile;
     for (int64_t tile = blockIdx.x; tile < nt; tile += gridDim.x) {
@@ -67,11 +77,14 @@ __global__ void k_reduce(const T* __restrict__ in, int64_t n, const unsigned lon
     }
 }
 
-// One block: exclusive scan of the block sums in place; total to *d_total.
+// One block per array: exclusive scan of the block sums in place; total to
+// d_total[array] and, with close, to element n of the output.
 template <typename T>
-__global__ void k_scan_sums(T* sums, int64_t n, const unsigned long long* dn, unsigned long long* d_total) {
+__global__ void k_scan_sums(ScanArrays<T> a, T* sums, int64_t stride, int64_t n, const unsigned long long* dn,
+                            unsigned long long* d_total, bool close) {
     __shared__ T wt[kThreads / 32];
     __shared__ T tot;
+    sums += blockIdx.y * stride;
     n = count_of(n, dn);
     const int64_t nb = (n + kTile - 1) / kTile;
     T carry = 0;
@@ -83,16 +96,20 @@ __global__ void k_scan_sums(T* sums, int64_t n, const unsigned long long* dn, un
         carry += tot;
         __syncthreads();
     }
-    if (threadIdx.x == 0 && d_total) *d_total = (unsigned long long)carry;
+    if (threadIdx.x == 0 && d_total) d_total[blockIdx.y] = (unsigned long long)carry;
+    if (threadIdx.x == 0 && close) a.out[blockIdx.y][n] = carry;
 }
 
 // Blocked arrangement: thread t owns items [t*kItems, (t+1)*kItems) of the tile.
 template <typename T>
-__global__ void k_scan_apply(const T* __restrict__ in, T* __restrict__ out, int64_t n, const unsigned long long* dn,
-                             const T* __restrict__ sums) {
+__global__ void k_scan_apply(ScanArrays<T> a, int64_t n, const unsigned long long* dn, const T* __restrict__ sums,
+                             int64_t stride) {
     __shared__ T wt[kThreads / 32];
     __shared__ T tot;
     __shared__ T stage[kTile];
+    const T* in = a.in[blockIdx.y];  // (may be the output)
+    T* out = a.out[blockIdx.y];
+    sums += blockIdx.y * stride;
     n = count_of(n, dn);
     const int64_t nt = (n + kTile - 1) / kTile;
     for (int64_t tile = blockIdx.x; tile < nt; tile += gridDim.x) {
@@ -126,33 +143,29 @@ __global__ void k_scan_apply(const T* __restrict__ in, T* __restrict__ out, int6
 // dn == nullptr: n elements, one tile per block.  Otherwise *dn elements
 // (read on the device, at most n) over a grid fixed here.
 template <typename T>
-int scan_impl(Ctx* c, const T* in, T* out, int64_t n, unsigned long long* d_total, const unsigned long long* dn) {
-    if (n <= 0) {
-        if (d_total) BH_CUDA(c, cudaMemsetAsync(d_total, 0, sizeof(unsigned long long), c->stream));
-        return BH_OK;
-    }
+int scan_impl(Ctx* c, const ScanArrays<T>& a, int na, int64_t n, unsigned long long* d_total,
+              const unsigned long long* dn, bool close) {
     const int64_t nb = (n + kTile - 1) / kTile;
-    BH_TRY(grow(c, c->scan_tmp, (size_t)nb * sizeof(T), "scan block sums"));
+    BH_TRY(grow(c, c->scan_tmp, (size_t)(na * nb) * sizeof(T), "scan block sums"));
     T* sums = (T*)c->scan_tmp.p;
-    const unsigned grid = dn ? (unsigned)std::min<int64_t>(nb, 4 * (int64_t)c->num_sms) : (unsigned)nb;
-    k_reduce<T><<<grid, kThreads, 0, c->stream>>>(in, n, dn, sums);
+    const dim3 grid(dn ? (unsigned)std::min<int64_t>(nb, 4 * (int64_t)c->num_sms) : (unsigned)nb, na);
+    k_reduce<T><<<grid, kThreads, 0, c->stream>>>(a, n, dn, sums, nb);
     BH_LAUNCH(c);
-    k_scan_sums<T><<<1, kThreads, 0, c->stream>>>(sums, n, dn, d_total);
+    k_scan_sums<T><<<dim3(1, na), kThreads, 0, c->stream>>>(a, sums, nb, n, dn, d_total, close);
     BH_LAUNCH(c);
-    k_scan_apply<T><<<grid, kThreads, 0, c->stream>>>(in, out, n, dn, sums);
+    k_scan_apply<T><<<grid, kThreads, 0, c->stream>>>(a, n, dn, sums, nb);
     BH_LAUNCH(c);
     return BH_OK;
 }
 
 }  // namespace
 
-int scan_u32(Ctx* c, const uint32_t* in, uint32_t* out, int64_t n, unsigned long long* d_total,
-             const unsigned long long* dn) {
-    return scan_impl<uint32_t>(c, in, out, n, d_total, dn);
+int scan_u32(Ctx* c, uint32_t* v, int64_t n, unsigned long long* d_total) {
+    return scan_impl<uint32_t>(c, {{v}, {v}}, 1, n, d_total, nullptr, false);
 }
-int scan_i64(Ctx* c, const int64_t* in, int64_t* out, int64_t n, unsigned long long* d_total,
-             const unsigned long long* dn) {
-    return scan_impl<int64_t>(c, in, out, n, d_total, dn);
+
+int scan3_i64(Ctx* c, int64_t* const (&v)[3], int64_t n, unsigned long long* d_total, const unsigned long long* dn) {
+    return scan_impl<int64_t>(c, {{v[0], v[1], v[2]}, {v[0], v[1], v[2]}}, 3, n, d_total, dn, true);
 }
 
 }  // namespace bh

@@ -521,12 +521,13 @@ struct Gather8 {
     const unsigned long long* src[8];
     unsigned long long* dst[8];
     int na;
+    const int* stop;  // status word: with an error in it the particles stay as they are (NULL: not asked)
 };
 
 __global__ void k_gather_all(Gather8 G, unsigned long long* __restrict__ scratch, const uint32_t* __restrict__ perm,
                              int64_t n, int* status) {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
+    if (i >= n || (G.stop && *G.stop)) return;
     const uint32_t j = perm[i];
     if (j >= n) {
         atomicOr(status, kStatBounds);
@@ -545,7 +546,7 @@ __global__ void k_gather_all(Gather8 G, unsigned long long* __restrict__ scratch
 // set's arrays cost their launches).
 __global__ void k_copy_back(Gather8 G, const unsigned long long* __restrict__ scratch, int64_t n) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
+    if (i >= n || (G.stop && *G.stop)) return;
     unsigned long long v[8];
 #pragma unroll
     for (int a = 0; a < 8; ++a)
@@ -631,6 +632,7 @@ int stage_permute(Ctx* c, bh_particles* p) {
                                    (unsigned long long*)p->m,  (unsigned long long*)p->id};
     const uint32_t* perm = c->idx[c->key_cur].p;
     Gather8 G = {};
+    G.stop = c->dev_build ? nullptr : c->d_status;
     for (int a = 0; a < 8; ++a)
         if (arrs[a]) {
             G.dst[G.na] = arrs[a];

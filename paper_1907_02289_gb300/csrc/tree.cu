@@ -600,7 +600,8 @@ int grow_nodes(Ctx* c, size_t need) {
 int64_t tree_count_words(int64_t n) { return kTreeRows * ((n + kTreeTile - 1) / kTreeTile); }
 
 // Nodes and groups.  Eager: the counts are read back once, to size the
-// arrays.  Device-sized (c->dev_build): the arrays hold c->cap_nodes nodes and
+// arrays, together with the status word of the keys (with an error in it the
+// particles were left as they were).  Device-sized (c->dev_build): the arrays hold c->cap_nodes nodes and
 // one group per particle; c->n_nodes and c->n_groups are those bounds until
 // the sizes are read back.
 int stage_octree(Ctx* c) {
@@ -614,7 +615,7 @@ int stage_octree(Ctx* c) {
     k_tree_count<<<(unsigned)ntiles, kTreeThreads, 0, c->stream>>>(key, n, c->d_off.p, np, n_leaf, n_g, ntiles,
                                                                  c->tree_range.p, cnt);
     BH_LAUNCH(c);
-    BH_TRY(scan_u32(c, cnt, cnt, tree_count_words(n), c->d_small));
+    BH_TRY(scan_u32(c, cnt, tree_count_words(n), c->d_small));
     k_tree_sizes<<<1, 32, 0, c->stream>>>(cnt, ntiles, c->d_small, dev ? (unsigned long long)c->cap_nodes : ~0ull,
                                           c->d_sz);
     BH_LAUNCH(c);
@@ -622,9 +623,9 @@ int stage_octree(Ctx* c) {
         c->n_nodes = c->cap_nodes;
         c->n_groups = n;
     } else {
-        unsigned long long sz[kSzWords];
-        BH_CUDA(c, cudaMemcpyAsync(sz, c->d_sz, sizeof(sz), cudaMemcpyDeviceToHost, c->stream));
-        BH_CUDA(c, cudaStreamSynchronize(c->stream));
+        const unsigned long long* sz = c->h_pin;
+        BH_CUDA(c, cudaMemcpyAsync(c->h_pin, c->d_sz, kSzWords * sizeof(*sz), cudaMemcpyDeviceToHost, c->stream));
+        BH_TRY(read_status(c));  // non-finite coordinates; a particle on the axis of the cylindrical frame
         c->n_nodes = (int64_t)sz[kSzLvl + kLevels + 2];
         c->n_groups = (int64_t)sz[kSzNg];
         c->lvl_start.assign(1, 0);

@@ -545,10 +545,6 @@ __global__ void k_unstash(int64_t ng, const unsigned long long* __restrict__ dng
     }
 }
 
-__global__ void k_set_last(int64_t* off, int64_t ng, const unsigned long long* dng, const unsigned long long* total) {
-    off[dng ? min(ng, (int64_t)*dng) : ng] = (int64_t)*total;
-}
-
 // Walk thresholds per patch from its key grid (S = 2^21 / L).  Contact
 // reach in grid units: Cartesian r_coll S; cylindrical (phi, r, z): two
 // particles within r_coll have |dr|, |dz| <= r_coll and a phi difference of
@@ -670,11 +666,8 @@ int launch_walk(Ctx* c, const WalkArgs& A, const WalkParams& wp, int64_t groups)
 int expand_lists(Ctx* c, const WalkParams& wp, const unsigned long long* dng, unsigned grid) {
     const int64_t ng = c->n_groups;
     const bool split = c->prm.precision == BH_PREC_FP32;
-    unsigned long long* n_far = c->d_small + 10;
-    if (split) {
-        BH_TRY(grow(c, c->cnt_jm, (size_t)ng + 1, "list split points"));
-        BH_CUDA(c, cudaMemsetAsync(n_far, 0, sizeof(unsigned long long), c->stream));
-    }
+    unsigned long long* n_far = c->d_small + 10;  // (cleared before the walk)
+    if (split) BH_TRY(grow(c, c->cnt_jm, (size_t)ng + 1, "list split points"));
     auto expand = split ? k_expand<true> : k_expand<false>;
     expand<<<grid, 256, 0, c->stream>>>(ng, dng, c->groups.p, c->cnt_p.p, c->P.p, c->begin.p, c->end.p, c->wnode.p,
                                         wp, c->cnt_j.p, c->JJ.p, split ? c->cnt_jm.p : nullptr, n_far);
@@ -714,14 +707,10 @@ int stage_lists(Ctx* c) {
     } else {
         BH_TRY(launch_walk<kWalkCount>(c, A, wp, ng));
     }
-    DBuf<int64_t>* arr[3] = {&c->cnt_p, &c->cnt_c, &c->cnt_j};
-    for (int a = 0; a < 3; ++a) {
-        BH_TRY(scan_i64(c, arr[a]->p, arr[a]->p, ng, c->d_small + a));
-        k_set_last<<<1, 1, 0, c->stream>>>(arr[a]->p, ng, nullptr, c->d_small + a);
-        BH_LAUNCH(c);
-    }
-    unsigned long long h[16];
-    BH_CUDA(c, cudaMemcpyAsync(h, c->d_small, sizeof(h), cudaMemcpyDeviceToHost, c->stream));
+    int64_t* const arr[3] = {c->cnt_p.p, c->cnt_c.p, c->cnt_j.p};
+    BH_TRY(scan3_i64(c, arr, ng, c->d_small, nullptr));
+    const unsigned long long* h = c->h_pin;
+    BH_CUDA(c, cudaMemcpyAsync(c->h_pin, c->d_small, 16 * sizeof(*h), cudaMemcpyDeviceToHost, c->stream));
     BH_CUDA(c, cudaStreamSynchronize(c->stream));
     c->n_pp = (int64_t)h[0];
     c->n_pc = (int64_t)h[1];
@@ -760,13 +749,8 @@ int stage_lists(Ctx* c) {
     c->walk_cap_c = (int64_t)(((h[13] + h[13] / 4 + 4) + 3) & ~3ull);
     BH_TRY(expand_lists(c, wp, nullptr, blocks_for(ng * 32, 256)));
     c->n_int_pp_far = 0;
-    if (c->prm.precision == BH_PREC_FP32) {
-        unsigned long long hf = 0;
-        BH_CUDA(c, cudaMemcpyAsync(&hf, c->d_small + 10, sizeof(hf), cudaMemcpyDeviceToHost, c->stream));
-        BH_CUDA(c, cudaStreamSynchronize(c->stream));
-        c->n_int_pp_far = (int64_t)hf;
-        BH_TRY(build_order32(c));
-    }
+    c->far_pending = c->prm.precision == BH_PREC_FP32;  // its count is read when asked for
+    if (c->prm.precision == BH_PREC_FP32) BH_TRY(build_order32(c));
     return BH_OK;
 }
 
@@ -794,12 +778,8 @@ int stage_lists_dev_walk(Ctx* c) {
     A.capP = capP;
     A.capC = capC;
     BH_TRY(launch_walk<kWalkStash>(c, A, wp, std::max<int64_t>(slots, 1)));
-    DBuf<int64_t>* arr[3] = {&c->cnt_p, &c->cnt_c, &c->cnt_j};
-    for (int a = 0; a < 3; ++a) {
-        BH_TRY(scan_i64(c, arr[a]->p, arr[a]->p, ng, c->d_small + a, dng));
-        k_set_last<<<1, 1, 0, c->stream>>>(arr[a]->p, ng, dng, c->d_small + a);
-        BH_LAUNCH(c);
-    }
+    int64_t* const arr[3] = {c->cnt_p.p, c->cnt_c.p, c->cnt_j.p};
+    BH_TRY(scan3_i64(c, arr, ng, c->d_small, dng));
     k_list_room<<<1, 32, 0, c->stream>>>(c->d_small, (long long)c->P.cap - 1, (long long)c->C.cap - 1,
                                          (long long)c->JJ.cap - 1, c->d_sz);
     BH_LAUNCH(c);
