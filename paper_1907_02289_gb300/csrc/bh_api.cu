@@ -519,6 +519,7 @@ int size_dev_build(Ctx* c, const int64_t cap[5]) {
     BH_TRY(grow(c, c->wnode, (size_t)nodes, "walk records"));
     BH_TRY(grow(c, c->tree_cnt, (size_t)tree_count_words(n), "node counts"));
     BH_TRY(grow(c, c->tree_range, (size_t)n, "node ranges"));
+    BH_TRY(grow(c, c->tree_top, (size_t)n, "first nodes"));
     if (f32) {
         BH_TRY(grow(c, c->cell32, 3 * (size_t)nodes, "FP32 cell records"));
         BH_TRY(grow(c, c->cell32lo, (size_t)nodes, "FP32 cell mass corrections"));
@@ -527,6 +528,7 @@ int size_dev_build(Ctx* c, const int64_t cap[5]) {
         BH_TRY(grow(c, c->Q, 6 * (size_t)nodes, "moments Q"));
     }
     BH_TRY(grow(c, c->groups, (size_t)n + 1, "groups"));
+    BH_TRY(grow(c, c->leaves, (size_t)nodes, "leaves"));
     for (auto* b : {&c->cnt_p, &c->cnt_c, &c->cnt_j, &c->cnt_jm})
         BH_TRY(grow(c, *b, (size_t)n + 1, "list offsets"));
     BH_TRY(grow(c, c->order, (size_t)n + 1, "group order"));
@@ -676,6 +678,7 @@ int graph_rebuild_step(Ctx* c, bh_particles* p) {
     for (int l = 0; l <= kLevels && sz[kSzLvl + l + 1] > sz[kSzLvl + l]; ++l)
         c->lvl_start.push_back((int64_t)sz[kSzLvl + l + 1]);
     c->n_groups = (int64_t)sz[kSzNg];
+    c->n_leaves = (int64_t)sz[kSzNl];
     c->n_pp = (int64_t)sm[0];
     c->n_pc = (int64_t)sm[1];
     c->n_jj = (int64_t)sm[2];
@@ -1005,10 +1008,10 @@ int bh_destroy(bh_ctx* ctx) {
     }
     release(c->sort_scratch); release(c->pscratch); release(c->scan_tmp);
     release(c->level); release(c->nchild); release(c->begin); release(c->end); release(c->parent);
-    release(c->first_child); release(c->qlo); release(c->qhi); release(c->wnode); release(c->tree_range); release(c->tree_cnt);
+    release(c->first_child); release(c->qlo); release(c->qhi); release(c->wnode); release(c->tree_range); release(c->tree_top); release(c->tree_cnt);
     release(c->M); release(c->cx); release(c->cy);
     release(c->cz); release(c->Q); release(c->cell32); release(c->cell32lo); release(c->refine); release(c->cbnd); release(c->cslot); release(c->cflag); release(c->phi); release(c->plo); release(c->contacts);
-    release(c->groups); release(c->order); release(c->cnt_p);
+    release(c->groups); release(c->leaves); release(c->order); release(c->cnt_p);
     release(c->cnt_c); release(c->cnt_j); release(c->cnt_jm); release(c->stash_p); release(c->stash_c); release(c->P); release(c->C); release(c->JJ); release(c->ipp);
     release(c->hbuf); release(c->hid);
     for (auto& pr : c->ev_force) {

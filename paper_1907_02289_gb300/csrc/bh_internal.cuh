@@ -30,6 +30,7 @@ constexpr int kSzLvl = 0;                   // kLevels + 3 words: first node of 
 constexpr int kSzNg = kLevels + 3;          // group count
 constexpr int kSzOvf = kSzNg + 1;           // overflow bits
 constexpr int kSzNeedNodes = kSzOvf + 1;    // nodes wanted when the node capacity ran out (a lower bound)
+constexpr int kSzNl = kSzNeedNodes + 1;     // leaf count
 constexpr int kSzWords = 32;
 constexpr unsigned long long kOvfNodes = 1, kOvfLists = 2;
 
@@ -151,6 +152,7 @@ struct Ctx {
     DBuf<uint32_t> qlo, qhi;         // 3 per node
     DBuf<WalkNode> wnode;
     DBuf<uint16_t> tree_range;       // per particle: levels of the nodes that begin there
+    DBuf<int32_t> tree_top;          // per particle at which nodes begin: the highest of them
     DBuf<uint32_t> tree_cnt;         // per (level, particle tile): nodes that begin there, then first ids
 
     // moments
@@ -174,6 +176,8 @@ struct Ctx {
     // groups
     int64_t n_groups = 0;
     DBuf<int32_t> groups;            // node ids ordered by begin
+    int64_t n_leaves = 0;
+    DBuf<int32_t> leaves;            // node ids ordered by begin
     DBuf<int32_t> order;             // force-kernel processing order of groups
     DBuf<unsigned long long> order_cnt;  // order buckets: counts/starts and cursors
     DBuf<uint64_t> ord_key[2];           // windowed order: sort keys
@@ -312,7 +316,6 @@ int stage_lists_dev_walk(Ctx* c);                  // device-sized: walk, offset
 int stage_lists_dev_fill(Ctx* c);                  // device-sized: lists, expansion, group order
 
 // force.cu
-int stage_split(Ctx* c, const bh_particles* p);    // FP32 hi/lo split of particles
 int build_order32(Ctx* c);                         // FP32 kernel's group order (per list build)
 int stage_force(Ctx* c, bh_particles* p, bool add_central);
 int stage_potential(Ctx* c, const bh_particles* p, double* phi, double* W);  // self-gravity potential (FP64)

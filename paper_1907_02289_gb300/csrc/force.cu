@@ -8,8 +8,8 @@
 //                   traceless quadrupole about the centre of mass.
 //
 // This file: the plain FP64 kernels (absolute coordinates) of the force and
-// of the self-gravity potential, the per-evaluation FP32 hi/lo split used by
-// the FP32 kernel (force32.cu), and the dispatcher.  Pairs that may be in
+// of the self-gravity potential, the FP32 hi/lo split on its own
+// (bh_split_f32), and the dispatcher.  Pairs that may be in
 // contact (r^2 <= r_coll^2 up to rounding) are re-evaluated in the oracle's
 // exact operation order, so the r <= r_coll decision is the oracle's.
 #include <algorithm>
@@ -356,20 +356,6 @@ __global__ void k_wsum_final(const double* __restrict__ part, double* out) {
     *out = s;
 }
 
-__global__ void k_split_particles(const double* __restrict__ x, const double* __restrict__ y,
-                                  const double* __restrict__ z, const double* __restrict__ m, int64_t n,
-                                  float4* __restrict__ phi, float4* __restrict__ plo) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const double v[3] = {x[i], y[i], z[i]};
-    float h[3], l[3], mh, ml;
-#pragma unroll
-    for (int a = 0; a < 3; ++a) split_f32(v[a], h[a], l[a]);
-    split_f32(m[i], mh, ml);
-    phi[i] = make_float4(h[0], h[1], h[2], mh);
-    plo[i] = make_float4(l[0], l[1], l[2], ml);
-}
-
 // The split alone, for callers and tests of it (bh_split_f32).
 __global__ void k_split_values(const double* __restrict__ v, int64_t n, float* __restrict__ hi,
                                float* __restrict__ lo) {
@@ -402,15 +388,6 @@ ForceParams force_params(const Ctx* c) {
     fp.Gf = (float)p.G;
     fp.order = p.order;
     return fp;
-}
-
-int stage_split(Ctx* c, const bh_particles* p) {
-    BH_TRY(grow(c, c->phi, (size_t)c->n, "FP32 positions hi"));
-    BH_TRY(grow(c, c->plo, (size_t)c->n, "FP32 positions lo"));
-    k_split_particles<<<blocks_for(c->n, 256), 256, 0, c->stream>>>(p->x, p->y, p->z, p->m, c->n, c->phi.p,
-                                                                    c->plo.p);
-    BH_LAUNCH(c);
-    return BH_OK;
 }
 
 namespace {

@@ -14,6 +14,7 @@
 
 #include "bh_internal.cuh"
 #include "dfloat.cuh"
+#include "split32.cuh"
 
 namespace bh {
 namespace {
@@ -28,12 +29,37 @@ __device__ __forceinline__ uint32_t compact3(uint64_t x) {
     return (uint32_t)x;
 }
 
-// Node range of one level: [ls, ls + cnt) as given, or from the device
-// level bounds lvl[lev], lvl[lev + 1] (device-sized builds).
-__device__ __forceinline__ void level_range(int64_t& ls, int64_t& cnt, const unsigned long long* lvl, int lev) {
-    if (lvl) {
-        ls = (int64_t)lvl[lev];
-        cnt = (int64_t)lvl[lev + 1] - ls;
+// ---- bottom-up passes ------------------------------------------------------
+// Boxes and moments take the levels from the deepest up.  A level with many
+// nodes is a launch of its own; a run of levels with few is one launch of one
+// thread block cluster, whose hardware barrier (arrive with release, wait
+// with acquire, which makes the children's records visible) stands between
+// two levels: a launch costs 3 to 5 us with its gap, the barrier well under
+// one.  The span_nodes of each pass is where the cluster's 2048 threads, on 8
+// SMs, start to take longer over a level than a launch of its own (the FP64
+// moments early: 8 SMs have 16 FP64 lanes).  A node's particles or children
+// are loaded several at a time before any of them is used.  Measured with the
+// leaf pass below: force evaluation on kept lists of a 20,000-particle ring 124
+// -> 95 us, evaluation of a 65,537-particle ring 624 -> 540 us, 4 graph steps of
+// 64 patches 22.32 -> 22.03 ms.
+constexpr int kSpanBlocks = 8, kSpanThreads = 256;
+constexpr int64_t kSpanBoxes = 4096, kSpanMoments32 = 4096, kSpanMoments64 = 256;
+
+__device__ __forceinline__ void cluster_barrier() {
+    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+
+// node(k) for every node of the levels hi, hi - 1, ..., lo (first nodes in
+// lvl); hi > lo only in a one-cluster launch.
+template <class F>
+__device__ __forceinline__ void for_levels(const unsigned long long* lvl, int hi, int lo, F node) {
+    for (int lev = hi;; --lev) {
+        const int64_t le = (int64_t)lvl[lev + 1];
+        for (int64_t k = (int64_t)lvl[lev] + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < le;
+             k += (int64_t)gridDim.x * blockDim.x)
+            node(k);
+        if (lev == lo) break;
+        cluster_barrier();
     }
 }
 
@@ -48,19 +74,21 @@ __device__ __forceinline__ void level_range(int64_t& ls, int64_t& cnt, const uns
 //   so the nodes that begin at i are, if the level-c cell around i splits
 //     (more than n_leaf particles), those of levels c + 1 to
 //     max(c, min(common(i, i + n_leaf), 20)) + 1, a chain of first children;
+//   the deepest of them is a leaf;
 //   and the group that begins at i, if there is one, is the highest of them
 //     with at most n_g particles (or the leaf).
-// One pass counts the nodes per level (and the groups) of each tile of
-// particles, a scan over (level, tile) turns the counts into node ids (breadth
+// One pass counts the nodes per level, the groups and the leaves of each tile
+// of particles, a scan over (level, tile) turns the counts into node ids (breadth
 // first, key order within a level), a second pass writes the nodes and the
-// group list, and a pass over the nodes links each to its children.  Against
+// lists of groups and leaves, and a pass over the nodes links each to its children.  Against
 // one counting, scanning and writing round per level, with binary searches
 // for the children (each of a top level's a serial chain through memory), and
 // a host wait per level for the eager build: a list-constructing evaluation
 // of a 65,537-particle ring 1.49 -> 1.00 ms, 4 graph steps of 64 patches 23.2
 // -> 22.7 ms, of the 2^26 ring 543.8 -> 542.8 ms.
 constexpr int kTreeThreads = 256, kTreeItems = 4, kTreeTile = kTreeThreads * kTreeItems;
-constexpr int kTreeRows = kLevels + 2;  // levels 0..21, then the groups
+constexpr int kRowGroups = kLevels + 1, kRowLeaves = kLevels + 2;
+constexpr int kTreeRows = kLevels + 3;  // levels 0..21, the groups, the leaves
 static_assert(kTreeItems * (kTreeThreads / 32) == 32, "one lane per (round, warp) when ranks are scanned");
 
 // Levels at which two keys lie in the same cell: the deepest (0..21).
@@ -165,36 +193,41 @@ __global__ void __launch_bounds__(kTreeThreads) k_tree_count(const uint64_t* __r
             if (lane == 0 && m) atomicAdd(&h[l], (uint32_t)__popc(m));
         }
         const unsigned mg = __ballot_sync(0xffffffffu, q.lg != kNoGroup);
-        if (lane == 0 && mg) atomicAdd(&h[kLevels + 1], (uint32_t)__popc(mg));
+        if (lane == 0 && mg) atomicAdd(&h[kRowGroups], (uint32_t)__popc(mg));
+        const unsigned ml = __ballot_sync(0xffffffffu, q.l1 >= 0);
+        if (lane == 0 && ml) atomicAdd(&h[kRowLeaves], (uint32_t)__popc(ml));
     }
     __syncthreads();
     if (threadIdx.x < kTreeRows) cnt[(int64_t)threadIdx.x * ntiles + blockIdx.x] = h[threadIdx.x];
 }
 
-// The level bounds, the node and group counts from the scanned counts: sz
-// words kSzLvl.. and kSzNg, cut at the node capacity (overflow flagged).
+// The level bounds and the node, group and leaf counts from the scanned
+// counts: sz words kSzLvl.., kSzNg and kSzNl, cut at the node capacity (overflow flagged).
 __global__ void k_tree_sizes(const uint32_t* __restrict__ scan, int64_t ntiles,
                              const unsigned long long* __restrict__ total, unsigned long long cap,
                              unsigned long long* sz) {
     const int l = threadIdx.x;
-    const unsigned long long nodes = scan[(int64_t)(kLevels + 1) * ntiles];
+    const unsigned long long nodes = scan[(int64_t)kRowGroups * ntiles], leaf0 = scan[(int64_t)kRowLeaves * ntiles];
     if (l < kLevels + 3) {
         const unsigned long long v = l <= kLevels ? (unsigned long long)scan[(int64_t)l * ntiles] : nodes;
         sz[kSzLvl + l] = v < cap ? v : cap;
     }
     if (l == 0) {
-        sz[kSzNg] = *total - nodes;
+        sz[kSzNg] = leaf0 - nodes;
+        sz[kSzNl] = *total - leaf0;
         sz[kSzOvf] = nodes > cap ? kOvfNodes : 0ull;
         sz[kSzNeedNodes] = nodes > cap ? nodes : 0ull;
     }
 }
 
-// Nodes (level, begin, first child; end and parent of the roots) and groups.
+// Nodes (level, begin, first child; end and parent of the roots), groups and
+// leaves (by first particle), and the highest node that begins at a particle.
 __global__ void __launch_bounds__(kTreeThreads) k_tree_write(
     const uint16_t* __restrict__ range, int64_t n, const int64_t* __restrict__ off, int np, int64_t ntiles,
     const uint32_t* __restrict__ scan, int64_t cap, uint8_t* __restrict__ level,
     uint32_t* __restrict__ begin, uint32_t* __restrict__ end, int32_t* __restrict__ parent,
-    int32_t* __restrict__ first_child, uint8_t* __restrict__ nchild, int32_t* __restrict__ groups) {
+    int32_t* __restrict__ first_child, uint8_t* __restrict__ nchild, int32_t* __restrict__ groups,
+    int32_t* __restrict__ leaves, int32_t* __restrict__ top) {
     __shared__ uint32_t base[kTreeRows][32];  // per (round, warp): nodes of the row before it in the tile, then ids
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const unsigned lt = (1u << lane) - 1u;
@@ -211,7 +244,9 @@ __global__ void __launch_bounds__(kTreeThreads) k_tree_write(
             if (lane == 0) base[l][r * (kTreeThreads / 32) + w] = __popc(m);
         }
         const unsigned mg = __ballot_sync(0xffffffffu, q[r].lg != kNoGroup);
-        if (lane == 0) base[kLevels + 1][r * (kTreeThreads / 32) + w] = __popc(mg);
+        if (lane == 0) base[kRowGroups][r * (kTreeThreads / 32) + w] = __popc(mg);
+        const unsigned ml = __ballot_sync(0xffffffffu, q[r].l1 >= 0);
+        if (lane == 0) base[kRowLeaves][r * (kTreeThreads / 32) + w] = __popc(ml);
     }
     __syncthreads();
     for (int row = w; row < kTreeRows; row += kTreeThreads / 32) {  // counts -> ids
@@ -225,7 +260,7 @@ __global__ void __launch_bounds__(kTreeThreads) k_tree_write(
         base[row][lane] = scan[(int64_t)row * ntiles + blockIdx.x] + x - v;
     }
     __syncthreads();
-    const uint32_t nodes = scan[(int64_t)(kLevels + 1) * ntiles];
+    const uint32_t nodes = scan[(int64_t)kRowGroups * ntiles], leaf0 = scan[(int64_t)kRowLeaves * ntiles];
 #pragma unroll
     for (int r = 0; r < kTreeItems; ++r) {
         const int64_t i = (int64_t)blockIdx.x * kTreeTile + r * kTreeThreads + threadIdx.x;
@@ -238,6 +273,7 @@ __global__ void __launch_bounds__(kTreeThreads) k_tree_write(
             if (!has) continue;
             const int64_t id = (int64_t)base[l][slot] + __popc(m & lt);
             if (l == q[r].lg) gnode = id;
+            if (l == q[r].l0) top[i] = (int32_t)id;
             if (prev >= 0 && prev < cap) first_child[prev] = (int32_t)id;
             if (id < cap) {
                 level[id] = (uint8_t)l;
@@ -254,7 +290,10 @@ __global__ void __launch_bounds__(kTreeThreads) k_tree_write(
             prev = id;
         }
         const unsigned mg = __ballot_sync(0xffffffffu, q[r].lg != kNoGroup);
-        if (q[r].lg != kNoGroup) groups[(int64_t)base[kLevels + 1][slot] + __popc(mg & lt) - nodes] = (int32_t)gnode;
+        if (q[r].lg != kNoGroup) groups[(int64_t)base[kRowGroups][slot] + __popc(mg & lt) - nodes] = (int32_t)gnode;
+        const unsigned ml = __ballot_sync(0xffffffffu, q[r].l1 >= 0);
+        const int64_t lf = (int64_t)base[kRowLeaves][slot] + __popc(ml & lt) - leaf0;
+        if (q[r].l1 >= 0 && lf < cap) leaves[lf] = (int32_t)prev;
     }
 }
 
@@ -314,55 +353,61 @@ __global__ void __launch_bounds__(128) k_tree_link(const uint64_t* __restrict__ 
     }
 }
 
-// Depth-first successor of node u's subtree: the node a pre-order walk
-// visits after u when it does not descend into u.  Children of a node are
-// consecutive ids, so that is u + 1 unless u is its parent's last child, in
-// which case it is the parent's successor; a root has none (-1), which ends
-// the walk of its patch.
-__device__ __forceinline__ int32_t skip_of(int64_t u, const int32_t* __restrict__ parent,
-                                           const int32_t* __restrict__ first_child,
-                                           const uint8_t* __restrict__ nchild, int* status) {
-    int64_t v = u;
-    for (int up = 0; up <= kLevels + 1; ++up) {
-        const int32_t p = parent[v];
-        if (p < 0) return -1;
-        if (v + 1 < (int64_t)first_child[p] + nchild[p]) return (int32_t)(v + 1);
-        v = p;
-    }
-    atomicOr(status, kStatBounds);  // deeper than the key grid: never for a valid tree
-    return -1;
+// Depth-first successor of a node's subtree: the node a pre-order walk visits
+// after it when it does not descend into it, which is the highest node that
+// begins at the particle past the subtree's last; none (-1) past a patch's
+// last particle, where the next patch's root (one of nodes 0..np - 1) or
+// nothing begins.
+__device__ __forceinline__ int32_t skip_of(uint32_t e, int64_t n, int np, const int32_t* __restrict__ top) {
+    if ((int64_t)e >= n) return -1;
+    const int32_t t = top[e];
+    return t < np ? -1 : t;
 }
 
 // Integer tight boxes (grid coordinates recovered from the keys) and the
 // packed records the walk reads (WalkNode).
-__global__ void k_boxes(const uint64_t* __restrict__ key, int64_t ls, int64_t cnt,
-                        const unsigned long long* __restrict__ lvl, int lev,
-                        const uint8_t* __restrict__ level, const uint32_t* __restrict__ begin,
-                        const uint32_t* __restrict__ end, const int32_t* __restrict__ parent,
-                        const int32_t* __restrict__ first_child, const uint8_t* __restrict__ nchild,
-                        uint32_t* qlo, uint32_t* qhi, WalkNode* wnode, int* status) {
-    level_range(ls, cnt, lvl, lev);
-    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < cnt; t += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t k = ls + t;
+__global__ void __launch_bounds__(kSpanThreads) k_boxes(
+    const uint64_t* __restrict__ key, int64_t n, int np, const uint8_t* __restrict__ level,
+    const uint32_t* __restrict__ begin, const uint32_t* __restrict__ end, const int32_t* __restrict__ first_child,
+    const uint8_t* __restrict__ nchild, const int32_t* __restrict__ top, uint32_t* qlo, uint32_t* qhi,
+    WalkNode* wnode, const unsigned long long* __restrict__ lvl, int lev_hi, int lev_lo) {
+    for_levels(lvl, lev_hi, lev_lo, [&](int64_t k) {
+        const uint32_t e = end[k];
+        const int32_t skip = skip_of(e, n, np, top);
         uint32_t lo[3] = {kQMax, kQMax, kQMax}, hi[3] = {0, 0, 0};
         const int nc = nchild[k];
         if (nc == 0) {
-            for (uint32_t i = begin[k]; i < end[k]; ++i) {
-                uint64_t kk = key[i];
-                uint32_t q[3] = {compact3(kk >> 2), compact3(kk >> 1), compact3(kk)};
+            for (uint32_t p = begin[k]; p < e; p += 8) {
+                uint64_t kk[8];
 #pragma unroll
-                for (int a = 0; a < 3; ++a) {
-                    lo[a] = min(lo[a], q[a]);
-                    hi[a] = max(hi[a], q[a]);
+                for (int u = 0; u < 8; ++u) kk[u] = key[min(p + u, e - 1u)];  // (a repeated key changes nothing)
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    const uint32_t q[3] = {compact3(kk[u] >> 2), compact3(kk[u] >> 1), compact3(kk[u])};
+#pragma unroll
+                    for (int a = 0; a < 3; ++a) {
+                        lo[a] = min(lo[a], q[a]);
+                        hi[a] = max(hi[a], q[a]);
+                    }
                 }
             }
         } else {
             const int64_t f = first_child[k];
-            for (int c = 0; c < nc; ++c)
+            uint32_t cl[8][3], ch[8][3];
+#pragma unroll
+            for (int c = 0; c < 8; ++c)
 #pragma unroll
                 for (int a = 0; a < 3; ++a) {
-                    lo[a] = min(lo[a], qlo[3 * (f + c) + a]);
-                    hi[a] = max(hi[a], qhi[3 * (f + c) + a]);
+                    const int64_t at = 3 * (f + min(c, nc - 1)) + a;  // (a repeated child changes nothing)
+                    cl[c][a] = qlo[at];
+                    ch[c][a] = qhi[at];
+                }
+#pragma unroll
+            for (int c = 0; c < 8; ++c)
+#pragma unroll
+                for (int a = 0; a < 3; ++a) {
+                    lo[a] = min(lo[a], cl[c][a]);
+                    hi[a] = max(hi[a], ch[c][a]);
                 }
         }
 #pragma unroll
@@ -373,60 +418,83 @@ __global__ void k_boxes(const uint64_t* __restrict__ key, int64_t ls, int64_t cn
         WalkNode w;
         // a leaf carries its first particle and (up to kWalkCntMax - 1) its
         // particle count instead of a first child and the child count
-        const uint32_t cnt = nc == 0 ? min(end[k] - begin[k], kWalkCntMax) : (uint32_t)nc;
+        const uint32_t cnt = nc == 0 ? min(e - begin[k], kWalkCntMax) : (uint32_t)nc;
         w.a = make_uint4(lo[0] | ((uint32_t)level[k] << kLevels) | (nc == 0 ? kWalkLeaf : 0u),
                          lo[1] | (cnt << kLevels), lo[2],
-                         (uint32_t)skip_of(k, parent, first_child, nchild, status));
+                         (uint32_t)skip);
         w.b = make_uint4(hi[0], hi[1], hi[2], nc == 0 ? begin[k] : (uint32_t)first_child[k]);
         wnode[k] = w;
-    }
+    });
 }
 
-// Moments of the nodes of one level (children already done).
+// Moments of the nodes (children already done).
 template <int ORDER>
-__global__ void k_moments(int64_t ls, int64_t cnt, const unsigned long long* __restrict__ lvl, int lev,
-                          const uint32_t* __restrict__ begin,
-                          const uint32_t* __restrict__ end, const int32_t* __restrict__ first_child,
-                          const uint8_t* __restrict__ nchild, const double* __restrict__ x,
-                          const double* __restrict__ y, const double* __restrict__ z,
-                          const double* __restrict__ m, double* M, double* cx, double* cy,
-                          double* cz, double* Q) {
-    level_range(ls, cnt, lvl, lev);
-    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < cnt; t += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t k = ls + t;
+__global__ void __launch_bounds__(kSpanThreads) k_moments(
+    const uint32_t* __restrict__ begin, const uint32_t* __restrict__ end, const int32_t* __restrict__ first_child,
+    const uint8_t* __restrict__ nchild, const double* __restrict__ x, const double* __restrict__ y,
+    const double* __restrict__ z, const double* __restrict__ m, double* M, double* cx, double* cy, double* cz,
+    double* Q, const unsigned long long* __restrict__ lvl, int lev_hi, int lev_lo) {
+    for_levels(lvl, lev_hi, lev_lo, [&](int64_t k) {
         const int nc = nchild[k];
         double Mk = 0.0, sx = 0.0, sy = 0.0, sz = 0.0, c0, c1, c2;
         double q[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
         if (nc == 0) {
             const uint32_t b = begin[k], e = end[k];
-            for (uint32_t i = b; i < e; ++i) {
-                const double mi = m[i];
-                Mk = __dadd_rn(Mk, mi);
-                sx = __dadd_rn(sx, __dmul_rn(mi, x[i]));
-                sy = __dadd_rn(sy, __dmul_rn(mi, y[i]));
-                sz = __dadd_rn(sz, __dmul_rn(mi, z[i]));
+            double px[8], py[8], pz[8], pm[8];
+            uint32_t have = b;
+            auto load = [&](uint32_t p) {
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    const uint32_t i = min(p + u, e - 1u);
+                    px[u] = x[i];
+                    py[u] = y[i];
+                    pz[u] = z[i];
+                    pm[u] = m[i];
+                }
+                have = p;
+            };
+            load(b);
+            const double x0 = px[0], y0 = py[0], z0 = pz[0];
+            for (uint32_t p = b; p < e; p += 8) {
+                if (p != have) load(p);
+#pragma unroll
+                for (int u = 0; u < 8; ++u)
+                    if (p + u < e) {
+                        const double mi = pm[u];
+                        Mk = __dadd_rn(Mk, mi);
+                        sx = __dadd_rn(sx, __dmul_rn(mi, px[u]));
+                        sy = __dadd_rn(sy, __dmul_rn(mi, py[u]));
+                        sz = __dadd_rn(sz, __dmul_rn(mi, pz[u]));
+                    }
             }
             if (Mk > 0.0) {
                 c0 = __ddiv_rn(sx, Mk);
                 c1 = __ddiv_rn(sy, Mk);
                 c2 = __ddiv_rn(sz, Mk);
             } else {
-                c0 = x[b];
-                c1 = y[b];
-                c2 = z[b];
+                c0 = x0;
+                c1 = y0;
+                c2 = z0;
             }
             if (ORDER >= 2)
-                for (uint32_t i = b; i < e; ++i) {
-                    const double mi = m[i];
-                    const double dx = __dsub_rn(x[i], c0), dy = __dsub_rn(y[i], c1), dz = __dsub_rn(z[i], c2);
-                    const double d2 = __dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz));
-                    const double tx = __dmul_rn(3.0, dx), ty = __dmul_rn(3.0, dy), tz = __dmul_rn(3.0, dz);
-                    q[0] = __dadd_rn(q[0], __dmul_rn(mi, __dsub_rn(__dmul_rn(tx, dx), d2)));
-                    q[1] = __dadd_rn(q[1], __dmul_rn(mi, __dsub_rn(__dmul_rn(ty, dy), d2)));
-                    q[2] = __dadd_rn(q[2], __dmul_rn(mi, __dsub_rn(__dmul_rn(tz, dz), d2)));
-                    q[3] = __dadd_rn(q[3], __dmul_rn(mi, __dmul_rn(tx, dy)));
-                    q[4] = __dadd_rn(q[4], __dmul_rn(mi, __dmul_rn(tx, dz)));
-                    q[5] = __dadd_rn(q[5], __dmul_rn(mi, __dmul_rn(ty, dz)));
+                for (uint32_t p = b; p < e; p += 8) {
+                    if (p != have) load(p);
+#pragma unroll
+                    for (int u = 0; u < 8; ++u)
+                        if (p + u < e) {
+                            const double mi = pm[u];
+                            const double dx = __dsub_rn(px[u], c0), dy = __dsub_rn(py[u], c1),
+                                         dz = __dsub_rn(pz[u], c2);
+                            const double d2 =
+                                __dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz));
+                            const double tx = __dmul_rn(3.0, dx), ty = __dmul_rn(3.0, dy), tz = __dmul_rn(3.0, dz);
+                            q[0] = __dadd_rn(q[0], __dmul_rn(mi, __dsub_rn(__dmul_rn(tx, dx), d2)));
+                            q[1] = __dadd_rn(q[1], __dmul_rn(mi, __dsub_rn(__dmul_rn(ty, dy), d2)));
+                            q[2] = __dadd_rn(q[2], __dmul_rn(mi, __dsub_rn(__dmul_rn(tz, dz), d2)));
+                            q[3] = __dadd_rn(q[3], __dmul_rn(mi, __dmul_rn(tx, dy)));
+                            q[4] = __dadd_rn(q[4], __dmul_rn(mi, __dmul_rn(tx, dz)));
+                            q[5] = __dadd_rn(q[5], __dmul_rn(mi, __dmul_rn(ty, dz)));
+                        }
                 }
         } else {
             const int64_t f = first_child[k];
@@ -468,7 +536,7 @@ __global__ void k_moments(int64_t ls, int64_t cnt, const unsigned long long* __r
         cz[k] = c2;
 #pragma unroll
         for (int a = 0; a < 6; ++a) Q[6 * k + a] = q[a];
-    }
+    });
 }
 
 // Moments for the FP32 force path, all in FP32: offsets from a reference
@@ -480,29 +548,83 @@ __device__ __forceinline__ float dsub(float ah, float al, float bh, float bl) {
     return __fadd_rn(__fsub_rn(ah, bh), __fsub_rn(al, bl));
 }
 
+// A node's record from its mass, reference point, centre offset and quadrupole.
+__device__ __forceinline__ void put_moments32(int64_t k, float Mk, df Md, const float (&rh)[3], const float (&rl)[3],
+                                              const float (&dc)[3], const float (&q)[6], float4* cell32,
+                                              float* __restrict__ mlo) {
+    // centre = reference + offset, renormalised into a hi/lo pair
+    float ch[3], cl[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        const float lo = __fadd_rn(rl[a], dc[a]);
+        const float hi = __fadd_rn(rh[a], lo);
+        ch[a] = hi;
+        cl[a] = __fsub_rn(lo, __fsub_rn(hi, rh[a]));
+    }
+    mlo[k] = __fadd_rn(__fsub_rn(Md.hi, Mk), Md.lo);
+    cell32[3 * k + 0] = make_float4(ch[0], ch[1], ch[2], Mk);
+    cell32[3 * k + 1] = make_float4(cl[0], cl[1], cl[2], q[0]);
+    cell32[3 * k + 2] = make_float4(q[3], q[4], q[1], q[5]);
+}
+
+// The FP32 hi/lo split of the particles and the leaves' moments in one pass:
+// a block takes kLeafTile consecutive leaves, whose particles are consecutive
+// too; it splits them with coalesced loads, writes the split and keeps it in
+// shared memory, from which a thread per leaf sums the moments (more particles
+// than fit are read back from memory).  Bound by HBM: 32 B read and 32 B
+// written per particle and 52 B per leaf, where a pass of its own re-read the
+// 32 B with a leaf's stride between the lanes.  Split and moments of the 2^24
+// ring, per evaluation: 0.65 -> 0.54 ms.
+constexpr int kLeafTile = 128, kLeafCap = 768;
+
 template <int ORDER>
-__global__ void k_moments32(int64_t ls, int64_t cnt, const unsigned long long* __restrict__ lvl, int lev,
-                            const uint32_t* __restrict__ begin,
-                            const uint32_t* __restrict__ end, const int32_t* __restrict__ first_child,
-                            const uint8_t* __restrict__ nchild, const float4* __restrict__ phi,
-                            const float4* __restrict__ plo, float4* cell32, float* __restrict__ mlo) {
-    level_range(ls, cnt, lvl, lev);
-    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < cnt; t += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t k = ls + t;
-        const int nc = nchild[k];
-        float rh[3], rl[3];  // reference point (hi/lo)
-        float Mk = 0.f, s[3] = {0.f, 0.f, 0.f}, q[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-        // the mass also as a compensated sum of the (hi + lo) masses: the record
-        // keeps Mk, mlo[k] the difference (for the refinement of the FP32 kernel)
-        df Md = {0.f, 0.f};
-        if (nc == 0) {
-            const uint32_t b = begin[k], e = end[k];
-            const float4 h0 = phi[b], l0 = plo[b];
-            rh[0] = h0.x; rh[1] = h0.y; rh[2] = h0.z;
-            rl[0] = l0.x; rl[1] = l0.y; rl[2] = l0.z;
-            for (uint32_t i = b; i < e; ++i) {
-                const float4 h = phi[i], l = plo[i];
-                const float d[3] = {dsub(h.x, l.x, rh[0], rl[0]), dsub(h.y, l.y, rh[1], rl[1]), dsub(h.z, l.z, rh[2], rl[2])};
+__global__ void __launch_bounds__(kLeafTile) k_leaf32(const int32_t* __restrict__ leaves,
+                                                      const unsigned long long* __restrict__ dnl,
+                                                      const uint32_t* __restrict__ begin,
+                                                      const uint32_t* __restrict__ end,
+                                                      const double* __restrict__ x, const double* __restrict__ y,
+                                                      const double* __restrict__ z, const double* __restrict__ m,
+                                                      float4* phi, float4* plo, float4* cell32,
+                                                      float* __restrict__ mlo) {
+    __shared__ float4 sh[kLeafCap], sl[kLeafCap];
+    const int64_t nl = (int64_t)*dnl;
+    for (int64_t t0 = (int64_t)blockIdx.x * kLeafTile; t0 < nl; t0 += (int64_t)gridDim.x * kLeafTile) {
+        const int64_t t1 = min(t0 + kLeafTile, nl);
+        const uint32_t p0 = begin[leaves[t0]], p1 = end[leaves[t1 - 1]];
+        const bool mine = t0 + threadIdx.x < t1;
+        const int64_t k = mine ? leaves[t0 + threadIdx.x] : 0;
+        const uint32_t b = mine ? begin[k] : 0u, e = mine ? end[k] : 0u;
+#pragma unroll 2
+        for (uint32_t i = p0 + threadIdx.x; i < p1; i += kLeafTile) {
+            const double v[3] = {x[i], y[i], z[i]}, mi = m[i];
+            float h[3], l[3], mh, ml;
+#pragma unroll
+            for (int a = 0; a < 3; ++a) split_f32(v[a], h[a], l[a]);
+            split_f32(mi, mh, ml);
+            const float4 H = make_float4(h[0], h[1], h[2], mh), L = make_float4(l[0], l[1], l[2], ml);
+            phi[i] = H;
+            plo[i] = L;
+            if (i - p0 < kLeafCap) {
+                sh[i - p0] = H;
+                sl[i - p0] = L;
+            }
+        }
+        __syncthreads();
+        if (mine) {
+            const bool in = e - p0 <= kLeafCap;
+            const float4* H = in ? sh : phi + p0;
+            const float4* L = in ? sl : plo + p0;
+            const uint32_t i0 = b - p0, i1 = e - p0;
+            const float4 h0 = H[i0], l0 = L[i0];
+            const float rh[3] = {h0.x, h0.y, h0.z}, rl[3] = {l0.x, l0.y, l0.z};
+            float Mk = 0.f, s[3] = {0.f, 0.f, 0.f}, q[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+            // the mass also as a compensated sum of the (hi + lo) masses: the record
+            // keeps Mk, mlo[k] the difference (for the refinement of the FP32 kernel)
+            df Md = {0.f, 0.f};
+            for (uint32_t i = i0; i < i1; ++i) {
+                const float4 h = H[i], l = L[i];
+                const float d[3] = {dsub(h.x, l.x, rh[0], rl[0]), dsub(h.y, l.y, rh[1], rl[1]),
+                                    dsub(h.z, l.z, rh[2], rl[2])};
                 Mk += h.w;
                 Md = df_add(Md, {h.w, l.w});
 #pragma unroll
@@ -511,8 +633,8 @@ __global__ void k_moments32(int64_t ls, int64_t cnt, const unsigned long long* _
             const float inv = Mk > 0.f ? 1.f / Mk : 0.f;
             const float dc[3] = {s[0] * inv, s[1] * inv, s[2] * inv};
             if (ORDER >= 2)
-                for (uint32_t i = b; i < e; ++i) {
-                    const float4 h = phi[i], l = plo[i];
+                for (uint32_t i = i0; i < i1; ++i) {
+                    const float4 h = H[i], l = L[i];
                     const float d[3] = {dsub(h.x, l.x, rh[0], rl[0]) - dc[0], dsub(h.y, l.y, rh[1], rl[1]) - dc[1],
                                         dsub(h.z, l.z, rh[2], rl[2]) - dc[2]};
                     const float d2 = fmaf(d[0], d[0], fmaf(d[1], d[1], d[2] * d[2]));
@@ -524,63 +646,112 @@ __global__ void k_moments32(int64_t ls, int64_t cnt, const unsigned long long* _
                     q[4] = fmaf(m3 * d[0], d[2], q[4]);
                     q[5] = fmaf(m3 * d[1], d[2], q[5]);
                 }
-#pragma unroll
-            for (int a = 0; a < 3; ++a) s[a] = dc[a];
-        } else {
-            const int64_t f = first_child[k];
-            const float4 c0h = cell32[3 * f], c0l = cell32[3 * f + 1];
-            rh[0] = c0h.x; rh[1] = c0h.y; rh[2] = c0h.z;
-            rl[0] = c0l.x; rl[1] = c0l.y; rl[2] = c0l.z;
-            for (int cc = 0; cc < nc; ++cc) {
-                const float4 h = cell32[3 * (f + cc)], l = cell32[3 * (f + cc) + 1];
-                const float d[3] = {dsub(h.x, l.x, rh[0], rl[0]), dsub(h.y, l.y, rh[1], rl[1]), dsub(h.z, l.z, rh[2], rl[2])};
-                Mk += h.w;
-                Md = df_add(Md, {h.w, mlo[f + cc]});
-#pragma unroll
-                for (int a = 0; a < 3; ++a) s[a] = fmaf(h.w, d[a], s[a]);
-            }
-            const float inv = Mk > 0.f ? 1.f / Mk : 0.f;
-            const float dc[3] = {s[0] * inv, s[1] * inv, s[2] * inv};
-            if (ORDER >= 2)
-                for (int cc = 0; cc < nc; ++cc) {
-                    const float4 h = cell32[3 * (f + cc)], l = cell32[3 * (f + cc) + 1], u = cell32[3 * (f + cc) + 2];
-                    const float D[3] = {dsub(h.x, l.x, rh[0], rl[0]) - dc[0], dsub(h.y, l.y, rh[1], rl[1]) - dc[1],
-                                        dsub(h.z, l.z, rh[2], rl[2]) - dc[2]};
-                    const float D2 = fmaf(D[0], D[0], fmaf(D[1], D[1], D[2] * D[2]));
-                    const float Mc = h.w, m3 = 3.f * Mc;
-                    q[0] += l.w + Mc * fmaf(3.f * D[0], D[0], -D2);
-                    q[1] += u.z + Mc * fmaf(3.f * D[1], D[1], -D2);
-                    q[2] += -(l.w + u.z) + Mc * fmaf(3.f * D[2], D[2], -D2);
-                    q[3] += u.x + m3 * D[0] * D[1];
-                    q[4] += u.y + m3 * D[0] * D[2];
-                    q[5] += u.w + m3 * D[1] * D[2];
-                }
-#pragma unroll
-            for (int a = 0; a < 3; ++a) s[a] = dc[a];
+            put_moments32(k, Mk, Md, rh, rl, dc, q, cell32, mlo);
         }
-        // centre = reference + offset, renormalised into a hi/lo pair
-        float ch[3], cl[3];
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            const float lo = __fadd_rn(rl[a], s[a]);
-            const float hi = __fadd_rn(rh[a], lo);
-            ch[a] = hi;
-            cl[a] = __fsub_rn(lo, __fsub_rn(hi, rh[a]));
-        }
-        mlo[k] = __fadd_rn(__fsub_rn(Md.hi, Mk), Md.lo);
-        cell32[3 * k + 0] = make_float4(ch[0], ch[1], ch[2], Mk);
-        cell32[3 * k + 1] = make_float4(cl[0], cl[1], cl[2], q[0]);
-        cell32[3 * k + 2] = make_float4(q[3], q[4], q[1], q[5]);
+        __syncthreads();
     }
 }
 
-// Grid of a device-sized level launch: enough blocks for the previous
-// build's nodes on that level with the build's room to grow (the kernels
-// stride, so any count is covered; this only sets the parallelism).
-unsigned dev_level_grid(const Ctx* c, int lev, int threads) {
+// Moments of the inner nodes, from their children's.
+template <int ORDER>
+__global__ void __launch_bounds__(kSpanThreads) k_moments32(
+    const int32_t* __restrict__ first_child, const uint8_t* __restrict__ nchild, float4* cell32, float* mlo,
+    const unsigned long long* __restrict__ lvl, int lev_hi, int lev_lo) {
+    for_levels(lvl, lev_hi, lev_lo, [&](int64_t k) {
+        const int nc = nchild[k];
+        if (nc == 0) return;
+        const int64_t f = first_child[k];
+        float4 H[4], L[4], U[4];
+        float ml[4];
+        auto load = [&](int c0) {  // children c0..c0 + 3 (the last one again past the end)
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int64_t j = f + min(c0 + u, nc - 1);
+                H[u] = cell32[3 * j];
+                L[u] = cell32[3 * j + 1];
+                if (ORDER >= 2) U[u] = cell32[3 * j + 2];
+                ml[u] = mlo[j];
+            }
+        };
+        load(0);
+        const float rh[3] = {H[0].x, H[0].y, H[0].z}, rl[3] = {L[0].x, L[0].y, L[0].z};
+        float Mk = 0.f, s[3] = {0.f, 0.f, 0.f}, q[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+        df Md = {0.f, 0.f};
+        for (int c0 = 0; c0 < nc; c0 += 4) {
+            if (c0 > 0) load(c0);
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (c0 + u < nc) {
+                    const float4 h = H[u], l = L[u];
+                    const float d[3] = {dsub(h.x, l.x, rh[0], rl[0]), dsub(h.y, l.y, rh[1], rl[1]),
+                                        dsub(h.z, l.z, rh[2], rl[2])};
+                    Mk += h.w;
+                    Md = df_add(Md, {h.w, ml[u]});
+#pragma unroll
+                    for (int a = 0; a < 3; ++a) s[a] = fmaf(h.w, d[a], s[a]);
+                }
+        }
+        const float inv = Mk > 0.f ? 1.f / Mk : 0.f;
+        const float dc[3] = {s[0] * inv, s[1] * inv, s[2] * inv};
+        if (ORDER >= 2)
+            for (int c0 = 0; c0 < nc; c0 += 4) {
+                if (nc > 4) load(c0);
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    if (c0 + u < nc) {
+                        const float4 h = H[u], l = L[u], v = U[u];
+                        const float D[3] = {dsub(h.x, l.x, rh[0], rl[0]) - dc[0], dsub(h.y, l.y, rh[1], rl[1]) - dc[1],
+                                            dsub(h.z, l.z, rh[2], rl[2]) - dc[2]};
+                        const float D2 = fmaf(D[0], D[0], fmaf(D[1], D[1], D[2] * D[2]));
+                        const float Mc = h.w, m3 = 3.f * Mc;
+                        q[0] += l.w + Mc * fmaf(3.f * D[0], D[0], -D2);
+                        q[1] += v.z + Mc * fmaf(3.f * D[1], D[1], -D2);
+                        q[2] += -(l.w + v.z) + Mc * fmaf(3.f * D[2], D[2], -D2);
+                        q[3] += v.x + m3 * D[0] * D[1];
+                        q[4] += v.y + m3 * D[0] * D[2];
+                        q[5] += v.w + m3 * D[1] * D[2];
+                    }
+            }
+        put_moments32(k, Mk, Md, rh, rl, dc, q, cell32, mlo);
+    });
+}
+
+// Issue a bottom-up pass over all levels: kern(args..., lvl, hi, lo).  The
+// level sizes that choose the launches are the tree's, or, in a device-sized
+// build, the previous build's with its room to grow (every size is covered;
+// they only set the parallelism), with all 22 levels issued.
+template <class... KA, class... A>
+int launch_levels(Ctx* c, int64_t span_nodes, void (*kern)(KA...), A... args) {
     const auto& ls = c->lvl_start;
-    const int64_t prev = lev + 1 < (int)ls.size() ? ls[lev + 1] - ls[lev] : 0;
-    return blocks_for(prev + prev * c->tune.graph_room / 100 + 64, threads);
+    auto nodes = [&](int l) -> int64_t {
+        const int64_t v = l + 1 < (int)ls.size() ? ls[l + 1] - ls[l] : 0;
+        return c->dev_build ? v + v * c->tune.graph_room / 100 + 64 : v;
+    };
+    const unsigned long long* lvl = c->d_sz + kSzLvl;
+    int hi = c->dev_build ? kLevels : (int)ls.size() - 2;
+    while (hi >= 0) {
+        int lo = hi;
+        cudaLaunchConfig_t cfg = {};
+        cudaLaunchAttribute at = {};
+        cfg.stream = c->stream;
+        if (nodes(hi) <= span_nodes) {
+            while (lo > 0 && nodes(lo - 1) <= span_nodes) --lo;
+            cfg.gridDim = dim3(kSpanBlocks);
+            cfg.blockDim = dim3(kSpanThreads);
+            at.id = cudaLaunchAttributeClusterDimension;
+            at.val.clusterDim.x = kSpanBlocks;
+            at.val.clusterDim.y = at.val.clusterDim.z = 1;
+            cfg.attrs = &at;
+            cfg.numAttrs = 1;
+        } else {
+            cfg.gridDim = dim3(blocks_for(nodes(hi), 128));
+            cfg.blockDim = dim3(128);
+        }
+        BH_CUDA(c, cudaLaunchKernelEx(&cfg, kern, args..., lvl, hi, lo));
+        BH_LAUNCH(c);
+        hi = lo - 1;
+    }
+    return BH_OK;
 }
 
 int grow_nodes(Ctx* c, size_t need) {
@@ -602,7 +773,7 @@ int64_t tree_count_words(int64_t n) { return kTreeRows * ((n + kTreeTile - 1) / 
 // Nodes and groups.  Eager: the counts are read back once, to size the
 // arrays, together with the status word of the keys (with an error in it the
 // particles were left as they were).  Device-sized (c->dev_build): the arrays hold c->cap_nodes nodes and
-// one group per particle; c->n_nodes and c->n_groups are those bounds until
+// leaves and one group per particle; c->n_nodes and c->n_groups are those bounds until
 // the sizes are read back.
 int stage_octree(Ctx* c) {
     const int64_t n = c->n, ntiles = (n + kTreeTile - 1) / kTreeTile;
@@ -611,6 +782,7 @@ int stage_octree(Ctx* c) {
     const uint64_t* key = c->key[c->key_cur].p;
     BH_TRY(grow(c, c->tree_cnt, (size_t)tree_count_words(n), "node counts"));
     BH_TRY(grow(c, c->tree_range, (size_t)n, "node ranges"));
+    BH_TRY(grow(c, c->tree_top, (size_t)n, "first nodes"));
     uint32_t* cnt = c->tree_cnt.p;
     k_tree_count<<<(unsigned)ntiles, kTreeThreads, 0, c->stream>>>(key, n, c->d_off.p, np, n_leaf, n_g, ntiles,
                                                                  c->tree_range.p, cnt);
@@ -621,22 +793,24 @@ int stage_octree(Ctx* c) {
     BH_LAUNCH(c);
     if (dev) {
         c->n_nodes = c->cap_nodes;
-        c->n_groups = n;
+        c->n_groups = n;  // (c->n_leaves stays the previous build's)
     } else {
         const unsigned long long* sz = c->h_pin;
         BH_CUDA(c, cudaMemcpyAsync(c->h_pin, c->d_sz, kSzWords * sizeof(*sz), cudaMemcpyDeviceToHost, c->stream));
         BH_TRY(read_status(c));  // non-finite coordinates; a particle on the axis of the cylindrical frame
         c->n_nodes = (int64_t)sz[kSzLvl + kLevels + 2];
         c->n_groups = (int64_t)sz[kSzNg];
+        c->n_leaves = (int64_t)sz[kSzNl];
         c->lvl_start.assign(1, 0);
         for (int l = 0; l <= kLevels && sz[kSzLvl + l + 1] > sz[kSzLvl + l]; ++l)
             c->lvl_start.push_back((int64_t)sz[kSzLvl + l + 1]);
         BH_TRY(grow_nodes(c, (size_t)c->n_nodes));
         BH_TRY(grow(c, c->groups, (size_t)c->n_groups + 1, "groups"));
+        BH_TRY(grow(c, c->leaves, (size_t)c->n_leaves, "leaves"));
     }
     k_tree_write<<<(unsigned)ntiles, kTreeThreads, 0, c->stream>>>(
         c->tree_range.p, n, c->d_off.p, np, ntiles, cnt, c->n_nodes, c->level.p, c->begin.p, c->end.p, c->parent.p,
-        c->first_child.p, c->nchild.p, c->groups.p);
+        c->first_child.p, c->nchild.p, c->groups.p, c->leaves.p, c->tree_top.p);
     BH_LAUNCH(c);
     k_tree_link<<<blocks_for(c->n_nodes, 128), 128, 0, c->stream>>>(key, c->d_off.p, np, c->d_sz, c->level.p,
                                                                     c->begin.p, c->end.p, c->parent.p,
@@ -650,75 +824,47 @@ int stage_boxes(Ctx* c) {
     BH_TRY(grow(c, c->qlo, (size_t)nn * 3, "node qlo"));
     BH_TRY(grow(c, c->qhi, (size_t)nn * 3, "node qhi"));
     BH_TRY(grow(c, c->wnode, (size_t)nn, "walk records"));
-    const unsigned long long* lvl = c->dev_build ? c->d_sz + kSzLvl : nullptr;
-    const int depth = c->dev_build ? kLevels + 1 : (int)c->lvl_start.size() - 1;
-    for (int lev = depth - 1; lev >= 0; --lev) {
-        const int64_t ls = lvl ? 0 : c->lvl_start[lev], cnt = lvl ? 0 : c->lvl_start[lev + 1] - ls;
-        k_boxes<<<lvl ? dev_level_grid(c, lev, 128) : blocks_for(cnt, 128), 128, 0, c->stream>>>(
-            c->key[c->key_cur].p, ls, cnt, lvl, lev, c->level.p, c->begin.p, c->end.p, c->parent.p,
-            c->first_child.p, c->nchild.p, c->qlo.p, c->qhi.p, c->wnode.p, c->d_status);
-        BH_LAUNCH(c);
-    }
-    return BH_OK;
+    return launch_levels(c, kSpanBoxes, k_boxes, c->key[c->key_cur].p, c->n, c->n_patches, c->level.p, c->begin.p,
+                         c->end.p, c->first_child.p, c->nchild.p, c->tree_top.p, c->qlo.p, c->qhi.p, c->wnode.p);
 }
 
 int stage_moments(Ctx* c, const bh_particles* p) {
     const int64_t nn = c->n_nodes;
-    const bool f32 = c->prm.precision == BH_PREC_FP32;
-    const unsigned long long* lvl = c->dev_build ? c->d_sz + kSzLvl : nullptr;
-    const int depth = c->dev_build ? kLevels + 1 : (int)c->lvl_start.size() - 1;
-    if (f32) {
-        // FP32 path: hi/lo split of the particles, then FP32 moments with a
-        // hi/lo centre (no FP64 arithmetic per node)
-        BH_TRY(grow(c, c->cell32, (size_t)nn * 3, "FP32 cell records"));
-        BH_TRY(grow(c, c->cell32lo, (size_t)nn, "FP32 cell mass corrections"));
-        BH_TRY(stage_begin(c, BH_STAGE_SPLIT));
-        BH_TRY(stage_split(c, p));
-        BH_TRY(stage_end(c));
-        BH_TRY(stage_begin(c, BH_STAGE_MOMENTS));
-        for (int lev = depth - 1; lev >= 0; --lev) {
-            const int64_t ls = lvl ? 0 : c->lvl_start[lev], cnt = lvl ? 0 : c->lvl_start[lev + 1] - ls;
-            const unsigned nb = lvl ? dev_level_grid(c, lev, 128) : blocks_for(cnt, 128);
-            if (c->prm.order >= 2)
-                k_moments32<2><<<nb, 128, 0, c->stream>>>(ls, cnt, lvl, lev, c->begin.p, c->end.p, c->first_child.p,
-                                                          c->nchild.p, c->phi.p, c->plo.p, c->cell32.p,
-                                                          c->cell32lo.p);
-            else
-                k_moments32<1><<<nb, 128, 0, c->stream>>>(ls, cnt, lvl, lev, c->begin.p, c->end.p, c->first_child.p,
-                                                          c->nchild.p, c->phi.p, c->plo.p, c->cell32.p,
-                                                          c->cell32lo.p);
-            BH_LAUNCH(c);
-        }
-        return stage_end(c);
-    }
-    return stage_moments64(c, p);
+    if (c->prm.precision != BH_PREC_FP32) return stage_moments64(c, p);
+    // FP32 path: hi/lo split of the particles with the leaves' moments, then
+    // the inner nodes', all in FP32 with a hi/lo centre (no FP64 arithmetic)
+    BH_TRY(grow(c, c->cell32, (size_t)nn * 3, "FP32 cell records"));
+    BH_TRY(grow(c, c->cell32lo, (size_t)nn, "FP32 cell mass corrections"));
+    BH_TRY(grow(c, c->phi, (size_t)c->n, "FP32 positions hi"));
+    BH_TRY(grow(c, c->plo, (size_t)c->n, "FP32 positions lo"));
+    const bool quad = c->prm.order >= 2;
+    BH_TRY(stage_begin(c, BH_STAGE_SPLIT));
+    // (device-sized: the previous build's leaves with its room to grow; strided)
+    const int64_t nl = c->dev_build ? c->n_leaves + c->n_leaves * c->tune.graph_room / 100 + 64 : c->n_leaves;
+    auto leaf = quad ? k_leaf32<2> : k_leaf32<1>;
+    leaf<<<blocks_for(nl, kLeafTile), kLeafTile, 0, c->stream>>>(c->leaves.p, c->d_sz + kSzNl, c->begin.p, c->end.p,
+                                                                 p->x, p->y, p->z, p->m, c->phi.p, c->plo.p,
+                                                                 c->cell32.p, c->cell32lo.p);
+    BH_LAUNCH(c);
+    BH_TRY(stage_end(c));
+    BH_TRY(stage_begin(c, BH_STAGE_MOMENTS));
+    BH_TRY(launch_levels(c, kSpanMoments32, quad ? k_moments32<2> : k_moments32<1>, c->first_child.p, c->nchild.p,
+                         c->cell32.p, c->cell32lo.p));
+    return stage_end(c);
 }
 
 // FP64 node moments (the FP64 path's records; the FP32 path's potential
 // diagnostic also uses them).
 int stage_moments64(Ctx* c, const bh_particles* p) {
     const int64_t nn = c->n_nodes;
-    const unsigned long long* lvl = c->dev_build ? c->d_sz + kSzLvl : nullptr;
-    const int depth = c->dev_build ? kLevels + 1 : (int)c->lvl_start.size() - 1;
     BH_TRY(grow(c, c->M, (size_t)nn, "moments M"));
     BH_TRY(grow(c, c->cx, (size_t)nn, "moments cx"));
     BH_TRY(grow(c, c->cy, (size_t)nn, "moments cy"));
     BH_TRY(grow(c, c->cz, (size_t)nn, "moments cz"));
     BH_TRY(grow(c, c->Q, (size_t)nn * 6, "moments Q"));
     BH_TRY(stage_begin(c, BH_STAGE_MOMENTS));
-    for (int lev = depth - 1; lev >= 0; --lev) {
-        const int64_t ls = lvl ? 0 : c->lvl_start[lev], cnt = lvl ? 0 : c->lvl_start[lev + 1] - ls;
-        const unsigned nb = lvl ? dev_level_grid(c, lev, 128) : blocks_for(cnt, 128);
-#define BH_MOM(O)                                                                                              \
-    k_moments<O><<<nb, 128, 0, c->stream>>>(ls, cnt, lvl, lev, c->begin.p, c->end.p, c->first_child.p, c->nchild.p, \
-                                            p->x, p->y, p->z, p->m, c->M.p, c->cx.p, c->cy.p, c->cz.p, c->Q.p)
-        if (c->prm.order >= 2)
-            BH_MOM(2);
-        else
-            BH_MOM(1);
-#undef BH_MOM
-        BH_LAUNCH(c);
-    }
+    BH_TRY(launch_levels(c, kSpanMoments64, c->prm.order >= 2 ? k_moments<2> : k_moments<1>, c->begin.p, c->end.p, c->first_child.p,
+                         c->nchild.p, p->x, p->y, p->z, p->m, c->M.p, c->cx.p, c->cy.p, c->cz.p, c->Q.p));
     return stage_end(c);
 }
 
