@@ -323,8 +323,9 @@ typedef struct {
     int order_by_cost; /* 0 or 1 */
     int graph;         /* 1: bh_step issues every step as one CUDA graph launch.
                           A list-reusing step (kick-drift, moment refresh,
-                          force kernel, contact pass, kick) is captured after
-                          each list build.  A list-constructing step (kick-
+                          force kernel, contact pass, kick) is captured once
+                          and again when buffers moved or sizes outgrew its
+                          grids.  A list-constructing step (kick-
                           drift, keys, sort, reordering, tree, moments,
                           groups, walk, lists, forces, kick) reads no size
                           back while it runs: its buffers are sized from the

@@ -47,6 +47,7 @@ int grow_raw(Ctx* c, void** p, size_t* cap, size_t need, const char* what, bool 
     }
     *p = q;
     *cap = bytes;
+    ++c->buf_gen;
     return BH_OK;
 }
 
@@ -276,7 +277,6 @@ int make_lists(Ctx* c) {
     if (!c->have_tree) return fail(c, BH_E_STATE, "bh_make_lists needs a tree (call bh_build_tree)");
     BH_STAGE(c, BH_STAGE_LISTS, stage_lists(c));
     c->have_lists = true;
-    c->graph_ok = false;
     c->evals_since_build = 0;
     c->n_rebuilds++;
     return BH_OK;
@@ -354,19 +354,32 @@ bool same_arrays(const bh_particles& a, const bh_particles& b) {
            a.id == b.id && a.ax == b.ax && a.ay == b.ay && a.az == b.az && a.n == b.n;
 }
 
+// The captured list-reusing step reads the group count and the level bounds on
+// the device, so it serves the lists of later builds too, as long as the
+// arrays, the settings and every library buffer are the ones it was captured
+// with and the sizes are within the room its grids were laid out for (and not
+// below half the sizes then).
+bool reuse_graph_fits(const Ctx* c, const bh_particles* p) {
+    if (!c->graph_ok || !same_arrays(c->graph_p, *p) || c->graph_gen != c->buf_gen) return false;
+    const int64_t now[2] = {c->n_groups, c->n_nodes};
+    for (int k = 0; k < 2; ++k)
+        if (now[k] > with_room(c, c->graph_size[k]) || 2 * now[k] < c->graph_size[k]) return false;
+    return true;
+}
+
 // One list-reusing step (kick-drift, moment refresh, forces, kick) as a CUDA
-// graph launch; the graph is captured on the first such step after a list
-// build (or when the arrays change) and updated in place when possible.
+// graph launch; the graph is captured when there is none that fits and updated
+// in place when possible.
 int graph_reuse_step(Ctx* c, bh_particles* p) {
     const double dt = c->prm.dt;
-    if (!c->graph_ok || !same_arrays(c->graph_p, *p)) {
-        // inside the graph the contact pass cannot grow its buffer: leave room
-        // for twice the candidates of the last eager evaluation
-        if (c->prm.precision == BH_PREC_FP32 && c->prm.r_coll > 0.0) {
-            const size_t want = c->tune.graph_contact_room > 0 ? (size_t)c->tune.graph_contact_room
-                                                               : (size_t)(2 * c->n_contacts + 65536);
-            if (c->contacts.cap < want) BH_TRY(grow(c, c->contacts, want, "contact pairs"));
-        }
+    // inside the graph the contact pass cannot grow its buffer: leave room for
+    // twice the candidates of the last evaluation whose count was read
+    if (c->prm.precision == BH_PREC_FP32 && c->prm.r_coll > 0.0) {
+        const size_t want = c->tune.graph_contact_room > 0 ? (size_t)c->tune.graph_contact_room
+                                                           : (size_t)(2 * c->n_contacts + 65536);
+        if (c->contacts.cap < want) BH_TRY(grow(c, c->contacts, want, "contact pairs"));
+    }
+    if (!reuse_graph_fits(c, p)) {
         // capture on a private stream (the legacy default stream cannot be
         // captured); the graph is then launched on the context's stream
         if (!c->cap_stream) BH_CUDA(c, cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking));
@@ -383,13 +396,13 @@ int graph_reuse_step(Ctx* c, bh_particles* p) {
                 BH_CUDA(c, eb);
             }
         }
-        c->capturing = true;
+        c->capturing = c->dev_sizes = true;
         const int64_t l0 = c->n_launches;
         int rc = stage_kick_drift(c, p, 0.5 * dt, dt);
         if (rc == BH_OK) rc = stage_moments(c, p);
         if (rc == BH_OK) rc = stage_force(c, p, true);
         if (rc == BH_OK) rc = stage_kick(c, p, 0.5 * dt);
-        c->capturing = false;
+        c->capturing = c->dev_sizes = false;
         c->gt_cur = nullptr;
         const cudaError_t ec = cudaStreamEndCapture(c->stream, &g);
         c->stream = s0;
@@ -426,6 +439,9 @@ int graph_reuse_step(Ctx* c, bh_particles* p) {
         }
         c->graph_ok = true;
         c->graph_p = *p;
+        c->graph_gen = c->buf_gen;
+        c->graph_size[0] = c->n_groups;
+        c->graph_size[1] = c->n_nodes;
         ++c->n_graph_captures;
     }
     BH_TRY(launch_graph(c, c->graph_exec, c->gt_reuse));
@@ -578,7 +594,7 @@ int capture_rebuild(Ctx* c, bh_particles* p) {
             BH_CUDA(c, eb);
         }
     }
-    c->capturing = true;
+    c->capturing = c->dev_sizes = true;
     c->dev_build = true;
     const int64_t l0 = c->n_launches;
     int rc = stage_kick_drift(c, p, 0.5 * dt, dt);
@@ -601,7 +617,7 @@ int capture_rebuild(Ctx* c, bh_particles* p) {
     if (rc == BH_OK) rc = stage_force(c, p, true);
     if (rc == BH_OK) rc = stage_kick(c, p, 0.5 * dt);
     c->abort = nullptr;
-    c->capturing = false;
+    c->capturing = c->dev_sizes = false;
     c->dev_build = false;
     c->gt_cur = nullptr;
     cudaGraph_t g = nullptr;
@@ -637,14 +653,15 @@ int capture_rebuild(Ctx* c, bh_particles* p) {
     c->rgraph_walk_cap[0] = c->walk_cap_p;
     c->rgraph_walk_cap[1] = c->walk_cap_c;
     c->rgraph_ok = true;
+    c->rgraph_gen = c->buf_gen;
     c->rgraph_p = *p;
     return BH_OK;
 }
 
 // The captured step still leaves the last build at least half its room (and
-// slot sizes within a tenth), on the same arrays.
+// slot sizes within a tenth), on the same arrays and library buffers.
 bool rebuild_graph_fits(const Ctx* c, const bh_particles* p) {
-    if (!c->rgraph_ok || !c->rgraph_exec || !same_arrays(c->rgraph_p, *p)) return false;
+    if (!c->rgraph_ok || !c->rgraph_exec || !same_arrays(c->rgraph_p, *p) || c->rgraph_gen != c->buf_gen) return false;
     const int64_t now[5] = {c->n_nodes, c->n_groups, c->n_pp, c->n_pc, c->n_jj};
     for (int k = 0; k < 5; ++k)
         if (now[k] + now[k] * c->tune.graph_room / 200 > c->rgraph_cap[k]) return false;
@@ -692,7 +709,6 @@ int graph_rebuild_step(Ctx* c, bh_particles* p) {
     if (c->prm.precision == BH_PREC_FP32 && c->prm.r_coll > 0.0) c->n_contacts = (int64_t)sm[16];
     c->have_tree = c->have_lists = true;
     c->list_overflowed = false;
-    c->graph_ok = false;  // the list-reusing graph follows the new lists
     c->n_rebuilds++;
     c->evals_since_build = 1;
     c->k_eval++;

@@ -203,7 +203,13 @@ struct Ctx {
     const bh_particles* early_src = nullptr;  // device arrays it copies from
     bool early_ids = true;               // the early copy includes masses and ids
     int64_t h2d_bytes = 0, d2h_bytes = 0;  // copied by bh_step_host so far
-    bool graph_ok = false;               // graph_exec matches the current lists and arrays
+    // sizes of the step being issued are read on the device, within bounds that
+    // outlive the current lists (captured steps of either kind)
+    bool dev_sizes = false;
+    int64_t buf_gen = 0;                 // library buffers (re)allocated so far
+    bool graph_ok = false;               // graph_exec matches the current arrays and settings,
+    int64_t graph_gen = 0;               // the buffers,
+    int64_t graph_size[2] = {};          // and about the sizes: groups and nodes it was captured with
     bh_particles graph_p{};              // particle arrays the graph was captured with
     int64_t graph_launches = 0;          // kernels in the graph
 
@@ -217,6 +223,7 @@ struct Ctx {
     int64_t dev_slots = 0;               // groups with a list slot in it
     cudaGraphExec_t rgraph_exec = nullptr;  // the captured list-constructing step
     bool rgraph_ok = false;              // rgraph_exec matches the arrays and capacities
+    int64_t rgraph_gen = 0;
     bh_particles rgraph_p{};
     int64_t rgraph_launches = 0;
     int64_t rgraph_cap[5] = {};          // nodes, slots, P, C, JJ it was captured with
@@ -322,6 +329,27 @@ int stage_potential(Ctx* c, const bh_particles* p, double* phi, double* W);  // 
 
 // bh_api.cu: wait for the stream and report the device status word
 int read_status(Ctx* c);
+
+// Bounds of the step being issued: the sizes themselves, or, with sizes read on
+// the device, the buffers' capacities (bounds of indices) and the sizes with
+// graph_room to grow (for grids; every size is covered).
+inline int64_t with_room(const Ctx* c, int64_t v) { return v + v * c->tune.graph_room / 100 + 64; }
+inline const unsigned long long* dev_groups(const Ctx* c) { return c->dev_sizes ? c->d_sz + kSzNg : nullptr; }
+inline int64_t groups_bound(const Ctx* c) {
+    if (!c->dev_sizes || c->dev_build) return c->n_groups;
+    size_t b = c->groups.cap;
+    for (size_t v : {c->cnt_p.cap, c->cnt_c.cap, c->cnt_j.cap}) b = v < b ? v : b;
+    if (c->prm.precision == BH_PREC_FP32)
+        for (size_t v : {c->cnt_jm.cap, c->order.cap}) b = v < b ? v : b;
+    return (int64_t)b - 1;
+}
+inline int64_t groups_expected(const Ctx* c) {
+    return c->dev_build ? (c->dev_slots > 1 ? c->dev_slots : 1) : c->dev_sizes ? with_room(c, c->n_groups) : c->n_groups;
+}
+inline int64_t nodes_bound(const Ctx* c) {
+    if (!c->dev_sizes || c->dev_build) return c->n_nodes;
+    return (int64_t)(c->prm.precision == BH_PREC_FP32 ? c->cell32lo.cap : c->M.cap);
+}
 
 // bh_api.cu: force-kernel and stage timing (no-ops unless enabled, or while
 // capturing a graph); stage_end closes the innermost stage begun

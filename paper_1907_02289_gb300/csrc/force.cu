@@ -394,7 +394,8 @@ namespace {
 
 Args64 args64(const Ctx* c, const bh_particles* p, const ForceParams& fp) {
     Args64 A = {};
-    A.ng = c->n_groups;
+    A.ng = groups_bound(c);
+    A.dng = dev_groups(c);
     A.groups = c->groups.p;
     A.begin = c->begin.p;
     A.end = c->end.p;
@@ -416,7 +417,7 @@ Args64 args64(const Ctx* c, const bh_particles* p, const ForceParams& fp) {
     A.Q = c->Q.p;
     A.fp = fp;
     A.n = (uint32_t)c->n;
-    A.nn = c->n_nodes;
+    A.nn = nodes_bound(c);
     A.status = c->d_status;
     A.off = c->d_off.p;
     A.np = c->n_patches;
@@ -431,8 +432,7 @@ int launch_sum64(Ctx* c, Args64& A) {
         const int lc = item_lcap(c->h_off[q + 1] - c->h_off[q]);
         A.slots = std::max(A.slots, whole_items(c->prm.n_g, lc) + lc);
     }
-    // (device-sized build: the expected groups; the kernel strides over more)
-    const int64_t ng = A.dng ? std::min(A.ng, std::max<int64_t>(c->dev_slots, 1)) : A.ng;
+    const int64_t ng = std::min(A.ng, groups_expected(c));  // (the kernel strides over more)
     const int64_t nb = (ng * A.slots + kWarps - 1) / kWarps;
     const unsigned grid = (unsigned)std::min<int64_t>(nb, (int64_t)1 << 30);
     const bool eps = A.fp.eps2 != 0.0;
@@ -450,7 +450,6 @@ int stage_force(Ctx* c, bh_particles* p, bool add_central) {
     add_central = add_central && c->prm.M_central != 0.0;
     if (c->prm.precision == BH_PREC_FP64) {
         Args64 A = args64(c, p, fp);
-        A.dng = c->dev_build ? c->d_sz + kSzNg : nullptr;
         A.abort = c->abort;
         A.add_central = add_central;
         A.ax = p->ax;

@@ -1326,8 +1326,8 @@ int contact_pass(Ctx* c, const Args& A, const ForceParams& fp, bh_particles* p) 
 
 int launch_force32(Ctx* c, bh_particles* p, const ForceParams& fp, bool add_central) {
     Args A;
-    A.ng = c->n_groups;
-    A.dng = c->dev_build ? c->d_sz + kSzNg : nullptr;
+    A.ng = groups_bound(c);
+    A.dng = dev_groups(c);
     A.abort = c->abort;
     A.order = c->order.p;
     A.groups = c->groups.p;
@@ -1361,7 +1361,7 @@ int launch_force32(Ctx* c, bh_particles* p, const ForceParams& fp, bool add_cent
     A.ncontact = c->d_small + 16;
     c->contact_stats = contact;
     A.n = (uint32_t)c->n;
-    A.nn = c->n_nodes;
+    A.nn = nodes_bound(c);
     A.status = c->d_status;
     A.fp = fp;
     A.floor2 = (float)(fp.rc2 + fp.eps2);

@@ -53,6 +53,7 @@ __device__ __forceinline__ void cluster_barrier() {
 // lvl); hi > lo only in a one-cluster launch.
 template <class F>
 __device__ __forceinline__ void for_levels(const unsigned long long* lvl, int hi, int lo, F node) {
+    while (hi > lo && lvl[hi + 1] == lvl[hi]) --hi;  // (empty levels, below the tree's depth)
     for (int lev = hi;; --lev) {
         const int64_t le = (int64_t)lvl[lev + 1];
         for (int64_t k = (int64_t)lvl[lev] + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < le;
@@ -717,18 +718,18 @@ __global__ void __launch_bounds__(kSpanThreads) k_moments32(
 }
 
 // Issue a bottom-up pass over all levels: kern(args..., lvl, hi, lo).  The
-// level sizes that choose the launches are the tree's, or, in a device-sized
-// build, the previous build's with its room to grow (every size is covered;
-// they only set the parallelism), with all 22 levels issued.
+// level sizes that choose the launches are the tree's, or, in a captured step,
+// the last build's with room to grow (every size is covered; they only set the
+// parallelism), with all 22 levels issued.
 template <class... KA, class... A>
 int launch_levels(Ctx* c, int64_t span_nodes, void (*kern)(KA...), A... args) {
     const auto& ls = c->lvl_start;
     auto nodes = [&](int l) -> int64_t {
         const int64_t v = l + 1 < (int)ls.size() ? ls[l + 1] - ls[l] : 0;
-        return c->dev_build ? v + v * c->tune.graph_room / 100 + 64 : v;
+        return c->dev_sizes ? with_room(c, v) : v;
     };
     const unsigned long long* lvl = c->d_sz + kSzLvl;
-    int hi = c->dev_build ? kLevels : (int)ls.size() - 2;
+    int hi = c->dev_sizes ? kLevels : (int)ls.size() - 2;
     while (hi >= 0) {
         int lo = hi;
         cudaLaunchConfig_t cfg = {};
@@ -839,8 +840,8 @@ int stage_moments(Ctx* c, const bh_particles* p) {
     BH_TRY(grow(c, c->plo, (size_t)c->n, "FP32 positions lo"));
     const bool quad = c->prm.order >= 2;
     BH_TRY(stage_begin(c, BH_STAGE_SPLIT));
-    // (device-sized: the previous build's leaves with its room to grow; strided)
-    const int64_t nl = c->dev_build ? c->n_leaves + c->n_leaves * c->tune.graph_room / 100 + 64 : c->n_leaves;
+    // (captured: the last build's leaves with room to grow; strided)
+    const int64_t nl = c->dev_sizes ? with_room(c, c->n_leaves) : c->n_leaves;
     auto leaf = quad ? k_leaf32<2> : k_leaf32<1>;
     leaf<<<blocks_for(nl, kLeafTile), kLeafTile, 0, c->stream>>>(c->leaves.p, c->d_sz + kSzNl, c->begin.p, c->end.p,
                                                                  p->x, p->y, p->z, p->m, c->phi.p, c->plo.p,
