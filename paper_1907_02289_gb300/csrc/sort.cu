@@ -63,8 +63,7 @@ __global__ void k_box_partial(const double* __restrict__ x, const double* __rest
         slot = (int64_t)blockIdx.y * gridDim.x + blockIdx.x;
     }
     const int64_t e = off[q + 1];
-    for (int64_t i = off[q] + (int64_t)j * blockDim.x + threadIdx.x; i < e; i += (int64_t)nbq * blockDim.x) {
-        const double v[3] = {x[i], y[i], z[i]};
+    auto take = [&](const double (&v)[3]) {
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
             const unsigned long long b = (unsigned long long)__double_as_longlong(v[a]);
@@ -73,6 +72,23 @@ __global__ void k_box_partial(const double* __restrict__ x, const double* __rest
             mn[a] = min(mn[a], k);
             mx[a] = max(mx[a], k);
         }
+    };
+    const int64_t step = (int64_t)nbq * blockDim.x;
+    int64_t i = off[q] + (int64_t)j * blockDim.x + threadIdx.x;
+    for (; i + 3 * step < e; i += 4 * step) {  // twelve loads in flight
+        double v[4][3];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            v[u][0] = x[i + u * step];
+            v[u][1] = y[i + u * step];
+            v[u][2] = z[i + u * step];
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) take(v[u]);
+    }
+    for (; i < e; i += step) {
+        const double v[3] = {x[i], y[i], z[i]};
+        take(v);
     }
     if (bad) atomicOr(status, kStatNonFinite);
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -103,11 +119,16 @@ __global__ void k_box_final(const unsigned long long* __restrict__ part_all, int
     if (poff) nb = poff[blockIdx.x + 1] - poff[blockIdx.x];
     double* box = box_all + 8 * blockIdx.x;
     __shared__ double r[6];
-    if (threadIdx.x < 6) {
-        unsigned long long v = part[threadIdx.x];
-        for (int b = 1; b < nb; ++b)
-            v = threadIdx.x < 3 ? min(v, part[6 * b + threadIdx.x]) : max(v, part[6 * b + threadIdx.x]);
-        r[threadIdx.x] = val_of(v);
+    {  // a warp per value
+        const int a = threadIdx.x >> 5, lane = threadIdx.x & 31;
+        unsigned long long mn = ~0ull, mx = 0ull;
+        for (int b = lane; b < nb; b += 32) {
+            const unsigned long long v = part[6 * b + a];
+            mn = min(mn, v);
+            mx = max(mx, v);
+        }
+        warp_minmax(mn, mx);
+        if (lane == 0) r[a] = val_of(a < 3 ? mn : mx);
     }
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -614,7 +635,7 @@ int stage_keys(Ctx* c, const bh_particles* p) {
         k_box_partial<<<nbt, kBoxThreads, 0, c->stream>>>(cx, cy, p->z, c->d_off.p, c->box_map.p, c->box_poff.p,
                                                           c->box_part.p, c->d_status);
         BH_LAUNCH(c);
-        k_box_final<<<np, 32, 0, c->stream>>>(c->box_part.p, 0, c->box_poff.p, c->d_box, c->prm.key_frame == 1,
+        k_box_final<<<np, 6 * 32, 0, c->stream>>>(c->box_part.p, 0, c->box_poff.p, c->d_box, c->prm.key_frame == 1,
                                               c->d_status);
         BH_LAUNCH(c);
     } else {
@@ -623,7 +644,7 @@ int stage_keys(Ctx* c, const bh_particles* p) {
         k_box_partial<<<nb, kBoxThreads, 0, c->stream>>>(cx, cy, p->z, c->d_off.p, nullptr, nullptr,
                                                          c->box_part.p, c->d_status);
         BH_LAUNCH(c);
-        k_box_final<<<1, 32, 0, c->stream>>>(c->box_part.p, nb, nullptr, c->d_box, c->prm.key_frame == 1,
+        k_box_final<<<1, 6 * 32, 0, c->stream>>>(c->box_part.p, nb, nullptr, c->d_box, c->prm.key_frame == 1,
                                              c->d_status);
         BH_LAUNCH(c);
     }

@@ -99,12 +99,12 @@ __device__ __forceinline__ int common(uint64_t a, uint64_t b) {
 }
 
 // Whether the level-c cell that holds particle i has more than m particles
-// (patch [ps, pe)).  Most answers come from three keys: yes if i + m is in the
-// cell; no if neither i + m/2 nor i - m/2 is (m + 1 particles in a row that
-// hold i reach m/2 past it on one side); else from the cell's first particle.
+// (patch [ps, pe)), when particle i + m is not in it.  Most answers are no,
+// from two keys: neither i + m/2 nor i - m/2 is in the cell either (m + 1
+// particles in a row that hold i reach m/2 past it on one side); else the
+// cell's first particle decides.
 __device__ __forceinline__ bool cell_above(const uint64_t* __restrict__ key, int64_t i, uint64_t ki, int64_t ps,
                                            int64_t pe, int c, int64_t m) {
-    if (i + m < pe && common(ki, key[i + m]) >= c) return true;
     const int64_t h = m >> 1;
     if (!(i + h < pe && common(ki, key[i + h]) >= c) && !(i - h >= ps && common(key[i - h], ki) >= c)) return false;
     int64_t lo = max(ps, i - m), b = i;
@@ -151,21 +151,39 @@ struct NodeRange {
     }
 };
 
-__device__ __forceinline__ NodeRange node_range(const uint64_t* __restrict__ key, int64_t i,
+// What a particle's node range starts from: its key, its patch [ps, pe), the
+// levels it shares with the particle before it (-1: none in the patch) and with
+// those n_leaf and n_g on.
+struct NodeProbe {
+    uint64_t ki;
+    int64_t ps, pe;
+    int c, d, dg;
+};
+
+__device__ __forceinline__ NodeProbe node_probe(const uint64_t* __restrict__ key, int64_t i,
                                                 const int64_t* __restrict__ off, int np, int n_leaf, int n_g) {
-    NodeRange r;
+    NodeProbe v;
     const int q = patch_at(off, np, i);
-    const int64_t ps = off[q], pe = off[q + 1];
-    const uint64_t ki = key[i];
-    const int c = i > ps ? common(key[i - 1], ki) : -1;
-    if (c >= kLevels || (c >= 0 && !cell_above(key, i, ki, ps, pe, c, n_leaf))) return r;
-    const int d = i + n_leaf < pe ? common(ki, key[i + n_leaf]) : -1;
-    r.l0 = c + 1;
-    r.l1 = max(c, min(d, kLevels - 1)) + 1;
-    const int dg = i + n_g < pe ? common(ki, key[i + n_g]) : -1;
-    if (dg >= r.l0)
-        r.lg = min(dg + 1, r.l1);
-    else if (c < 0 || cell_above(key, i, ki, ps, pe, c, n_g))
+    v.ps = off[q];
+    v.pe = off[q + 1];
+    v.ki = key[i];
+    const bool b = i > v.ps, l = i + n_leaf < v.pe, g = i + n_g < v.pe;
+    const uint64_t kb = key[b ? i - 1 : i], kl = key[l ? i + n_leaf : i], kg = key[g ? i + n_g : i];
+    v.c = b ? common(kb, v.ki) : -1;
+    v.d = l ? common(v.ki, kl) : -1;
+    v.dg = g ? common(v.ki, kg) : -1;
+    return v;
+}
+
+__device__ __forceinline__ NodeRange node_range(const uint64_t* __restrict__ key, int64_t i, const NodeProbe& v,
+                                                int n_leaf, int n_g) {
+    NodeRange r;
+    if (v.c >= kLevels || (v.c >= 0 && v.d < v.c && !cell_above(key, i, v.ki, v.ps, v.pe, v.c, n_leaf))) return r;
+    r.l0 = v.c + 1;
+    r.l1 = max(v.c, min(v.d, kLevels - 1)) + 1;
+    if (v.dg >= r.l0)
+        r.lg = min(v.dg + 1, r.l1);
+    else if (v.c < 0 || v.dg >= v.c || cell_above(key, i, v.ki, v.ps, v.pe, v.c, n_g))
         r.lg = r.l0;
     return r;
 }
@@ -180,12 +198,17 @@ __global__ void __launch_bounds__(kTreeThreads) k_tree_count(const uint64_t* __r
     if (threadIdx.x < kTreeRows) h[threadIdx.x] = 0;
     __syncthreads();
     const int lane = threadIdx.x & 31;
-#pragma unroll 1
+    const int64_t i0 = (int64_t)blockIdx.x * kTreeTile + threadIdx.x;
+    NodeProbe v[kTreeItems];  // (all rounds' loads in flight)
+#pragma unroll
+    for (int r = 0; r < kTreeItems; ++r)
+        v[r] = node_probe(key, min(i0 + r * kTreeThreads, n - 1), off, np, n_leaf, n_g);
+#pragma unroll
     for (int r = 0; r < kTreeItems; ++r) {
-        const int64_t i = (int64_t)blockIdx.x * kTreeTile + r * kTreeThreads + threadIdx.x;
+        const int64_t i = i0 + r * kTreeThreads;
         NodeRange q;
         if (i < n) {
-            q = node_range(key, i, off, np, n_leaf, n_g);
+            q = node_range(key, i, v[r], n_leaf, n_g);
             range[i] = q.code();
         }
         const int l0 = __reduce_min_sync(0xffffffffu, q.l0), l1 = __reduce_max_sync(0xffffffffu, q.l1);
