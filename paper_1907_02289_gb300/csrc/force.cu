@@ -307,6 +307,7 @@ __device__ __forceinline__ void item64(const Args64& A, Smem64& S, int64_t k, ui
 
 template <bool POT, int ORDER, bool EPS>
 __global__ void __launch_bounds__(32 * kWarps) k_sum64(const Args64 A) {
+    launch_wait();
     __shared__ Smem64 sm[kWarps];
     if (A.abort && *A.abort) return;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -348,6 +349,7 @@ constexpr int kWBlocks = 512, kWThreads = 256;
 
 __global__ void __launch_bounds__(kWThreads) k_wsum_partial(int64_t n, const double* __restrict__ m,
                                                             const double* __restrict__ phi, double* part) {
+    launch_wait();
     __shared__ double sh[kWThreads];
     double acc = 0.0;
     for (int64_t i = (int64_t)blockIdx.x * kWThreads + threadIdx.x; i < n; i += (int64_t)kWBlocks * kWThreads)
@@ -362,6 +364,7 @@ __global__ void __launch_bounds__(kWThreads) k_wsum_partial(int64_t n, const dou
 }
 
 __global__ void k_wsum_final(const double* __restrict__ part, double* out) {
+    launch_wait();
     if (threadIdx.x != 0) return;
     double s = 0.0;
     for (int b = 0; b < kWBlocks; ++b) s += part[b];
@@ -450,7 +453,7 @@ int launch_sum64(Ctx* c, Args64& A) {
     const bool eps = A.fp.eps2 != 0.0;
     auto kern = A.fp.order >= 2 ? (eps ? k_sum64<POT, 2, true> : k_sum64<POT, 2, false>)
                                 : (eps ? k_sum64<POT, 1, true> : k_sum64<POT, 1, false>);
-    kern<<<grid, 32 * kWarps, 0, c->stream>>>(A);
+    BH_CUDA(c, launch(c, kern, grid, 32 * kWarps, 0, A));
     BH_LAUNCH(c);
     return BH_OK;
 }
@@ -489,9 +492,9 @@ int stage_potential(Ctx* c, const bh_particles* p, double* phi, double* W) {
     BH_TRY(launch_sum64<true>(c, A));
     if (W) {
         BH_TRY(grow(c, c->diag, (size_t)kWBlocks + 1, "potential energy sums"));
-        k_wsum_partial<<<kWBlocks, kWThreads, 0, c->stream>>>(c->n, p->m, phi, c->diag.p);
+        BH_CUDA(c, launch(c, k_wsum_partial, kWBlocks, kWThreads, 0, c->n, p->m, phi, c->diag.p));
         BH_LAUNCH(c);
-        k_wsum_final<<<1, 32, 0, c->stream>>>(c->diag.p, c->diag.p + kWBlocks);
+        BH_CUDA(c, launch(c, k_wsum_final, 1, 32, 0, c->diag.p, c->diag.p + kWBlocks));
         BH_LAUNCH(c);
         BH_CUDA(c, cudaMemcpyAsync(W, c->diag.p + kWBlocks, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
         BH_CUDA(c, cudaStreamSynchronize(c->stream));

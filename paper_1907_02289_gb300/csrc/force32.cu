@@ -808,6 +808,7 @@ __device__ __forceinline__ void force_group(const Args& A, Smem32& S, int64_t sl
 // Warps per block = blockDim.x / 32 (at most BH_F32_MAXW); one Smem32 per warp.
 template <int ORDER, int MODE>
 __global__ void __launch_bounds__(32 * BH_F32_MAXW, 2) k_force32(const Args A) {
+    launch_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     Smem32* sm = reinterpret_cast<Smem32*>(smem_raw);
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
@@ -878,6 +879,7 @@ __global__ void k_order_hist(int64_t ng, const unsigned long long* __restrict__ 
                              const uint32_t* __restrict__ end, const int64_t* __restrict__ jj_off,
                              const int64_t* __restrict__ pc_off, uint32_t chunk, bool by_cost,
                              unsigned long long* cnt) {
+    launch_wait();
     if (dng) ng = min(ng, (int64_t)*dng);
     for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < ng; k += (int64_t)gridDim.x * blockDim.x)
         atomicAdd(&cnt[order_bucket(k, groups, begin, end, jj_off, pc_off, chunk, by_cost)], 1ull);
@@ -891,6 +893,7 @@ __global__ void k_order_keys(int64_t ng, const int32_t* __restrict__ groups, con
                              const uint32_t* __restrict__ end, const int64_t* __restrict__ jj_off,
                              const int64_t* __restrict__ pc_off, uint32_t chunk, bool by_cost, int64_t window,
                              uint64_t* __restrict__ keys) {
+    launch_wait();
     const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= ng) return;
     keys[k] = ((uint64_t)(k / window) << 8) | (uint64_t)order_bucket(k, groups, begin, end, jj_off, pc_off, chunk, by_cost);
@@ -902,6 +905,7 @@ __global__ void k_order_scatter(int64_t ng, const unsigned long long* __restrict
                                 const int64_t* __restrict__ pc_off, uint32_t chunk, bool by_cost,
                                 const unsigned long long* __restrict__ cnt, unsigned long long* cursor,
                                 int32_t* __restrict__ order) {
+    launch_wait();
     if (dng) ng = min(ng, (int64_t)*dng);
     // exclusive prefix of the bucket counts, by the block's first warp
     __shared__ unsigned long long start[kOrderBuckets];
@@ -961,6 +965,7 @@ __global__ void k_contacts64(const uint2* __restrict__ pairs, const unsigned lon
                              const double* __restrict__ vz, const double* __restrict__ m,
                              unsigned long long* __restrict__ acc, unsigned long long* n_touch, int* status,
                              bool flag) {
+    launch_wait();
     const int64_t np = contact_count(count, cap, status, flag);
     unsigned long long touching = 0;
     for (int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; u < np; u += (int64_t)gridDim.x * blockDim.x) {
@@ -1069,6 +1074,7 @@ __device__ __forceinline__ void ref_pc(const Args& A, const RefineConsts& K, flo
 // gravity and contact, is small against its FP32 bound.
 __global__ void k_contacts_apply(const Args A, const uint2* __restrict__ pairs, const unsigned long long* count,
                                  int64_t cap, unsigned long long* __restrict__ acc) {
+    launch_wait();
     int64_t np = (int64_t)*count;
     if (np > cap) np = cap;
     const double kg = A.kref * A.fp.G;
@@ -1103,6 +1109,7 @@ __global__ void k_contacts_apply(const Args A, const uint2* __restrict__ pairs, 
 // 2^26 ring in 6.1 ms against 6.6 ms at 16 warps (97 registers).
 __global__ void __launch_bounds__(256, 4) k_refine32(const Args A, const RefineConsts K,
                                                      const float* __restrict__ mlo, int64_t cap) {
+    launch_wait();
     const int lane = threadIdx.x & 31;
     const int64_t wid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -1263,9 +1270,8 @@ int build_order32(Ctx* c) {
             BH_TRY(grow(c, c->ord_idx[b], (size_t)ng, "group order indices"));
         }
         BH_TRY(grow(c, c->ord_scratch, (size_t)sort_scratch_words(ng), "group order sort scratch"));
-        k_order_keys<<<blocks_for(ng, 256), 256, 0, c->stream>>>(ng, c->groups.p, c->begin.p, c->end.p, c->cnt_j.p,
-                                                                 c->cnt_c.p, chunk, by_cost, c->tune.order_window,
-                                                                 c->ord_key[0].p);
+        BH_CUDA(c, launch(c, k_order_keys, blocks_for(ng, 256), 256, 0, ng, c->groups.p, c->begin.p,
+                          c->end.p, c->cnt_j.p, c->cnt_c.p, chunk, by_cost, c->tune.order_window, c->ord_key[0].p));
         BH_LAUNCH(c);
         if (c->sort_attr_device != c->device) {
             BH_CUDA(c, sort_setup_device());
@@ -1282,11 +1288,11 @@ int build_order32(Ctx* c) {
     const unsigned long long* dng = c->dev_build ? c->d_sz + kSzNg : nullptr;
     const unsigned nb = dng ? (unsigned)(4 * c->num_sms) : blocks_for(ng, 256);
     BH_CUDA(c, cudaMemsetAsync(cnt, 0, 2 * kOrderBuckets * sizeof(unsigned long long), c->stream));
-    k_order_hist<<<nb, 256, 0, c->stream>>>(ng, dng, c->groups.p, c->begin.p, c->end.p, c->cnt_j.p, c->cnt_c.p, chunk,
-                                            by_cost, cnt);
+    BH_CUDA(c, launch(c, k_order_hist, nb, 256, 0, ng, dng, c->groups.p, c->begin.p, c->end.p, c->cnt_j.p,
+                      c->cnt_c.p, chunk, by_cost, cnt));
     BH_LAUNCH(c);
-    k_order_scatter<<<nb, 256, 0, c->stream>>>(ng, dng, c->groups.p, c->begin.p, c->end.p, c->cnt_j.p, c->cnt_c.p,
-                                               chunk, by_cost, cnt, cnt + kOrderBuckets, c->order.p);
+    BH_CUDA(c, launch(c, k_order_scatter, nb, 256, 0, ng, dng, c->groups.p, c->begin.p, c->end.p,
+                      c->cnt_j.p, c->cnt_c.p, chunk, by_cost, cnt, cnt + kOrderBuckets, c->order.p));
     BH_LAUNCH(c);
     return BH_OK;
 }
@@ -1304,8 +1310,8 @@ RefineConsts refine_consts(const ForceParams& fp) {
 // read on the device, so it can run inside a captured graph).
 int refine_pass(Ctx* c, const Args& A, const ForceParams& fp) {
     BH_TRY(stage_begin(c, BH_STAGE_REFINE));
-    k_refine32<<<(unsigned)(c->num_sms * 4), 256, 0, c->stream>>>(A, refine_consts(fp), c->cell32lo.p,
-                                                                   (int64_t)c->refine.cap);
+    BH_CUDA(c, launch(c, k_refine32, (unsigned)(c->num_sms * 4), 256, 0, A, refine_consts(fp),
+                      c->cell32lo.p, (int64_t)c->refine.cap));
     BH_LAUNCH(c);
     return stage_end(c);
 }
@@ -1315,10 +1321,10 @@ int contact_pass(Ctx* c, const Args& A, const ForceParams& fp, bh_particles* p) 
     unsigned long long* acc = c->contact_acc.p;
     BH_TRY(stage_begin(c, BH_STAGE_CONTACTS));
     // (an overflow is flagged in a captured step; eagerly the host sees the count)
-    k_contacts64<<<nb, 128, 0, c->stream>>>(A.contacts, A.ncontact, A.contact_cap, fp, p->x, p->y, p->z, p->vx, p->vy,
-                                            p->vz, p->m, acc, c->d_small + 18, c->d_status, c->capturing);
+    BH_CUDA(c, launch(c, k_contacts64, nb, 128, 0, A.contacts, A.ncontact, A.contact_cap, fp, p->x, p->y,
+                      p->z, p->vx, p->vy, p->vz, p->m, acc, c->d_small + 18, c->d_status, c->capturing));
     BH_LAUNCH(c);
-    k_contacts_apply<<<nb, 128, 0, c->stream>>>(A, A.contacts, A.ncontact, A.contact_cap, acc);
+    BH_CUDA(c, launch(c, k_contacts_apply, nb, 128, 0, A, A.contacts, A.ncontact, A.contact_cap, acc));
     BH_LAUNCH(c);
     return stage_end(c);
 }
@@ -1426,7 +1432,7 @@ int launch_force32(Ctx* c, bh_particles* p, const ForceParams& fp, bool add_cent
         BH_CUDA(c, cudaMemsetAsync(c->d_small + 16, 0, 5 * sizeof(unsigned long long), c->stream));
         BH_TRY(timing_begin(c));
         BH_TRY(stage_begin(c, BH_STAGE_FORCE));
-        kern<<<nb, 32 * W, smem, c->stream>>>(A);
+        BH_CUDA(c, launch(c, kern, nb, 32 * W, smem, A));
         BH_LAUNCH(c);
         BH_TRY(stage_end(c));
         BH_TRY(timing_end(c));

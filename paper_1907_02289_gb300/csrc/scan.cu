@@ -58,6 +58,7 @@ struct ScanArrays {
 template <typename T>
 __global__ void k_reduce(ScanArrays<T> a, int64_t n, const unsigned long long* dn, T* __restrict__ sums,
                          int64_t stride) {
+    launch_wait();
     __shared__ T wt[kThreads / 32];
     __shared__ T tot;
     const T* __restrict__ in = a.in[blockIdx.y];
@@ -82,6 +83,7 @@ __global__ void k_reduce(ScanArrays<T> a, int64_t n, const unsigned long long* d
 template <typename T>
 __global__ void k_scan_sums(ScanArrays<T> a, T* sums, int64_t stride, int64_t n, const unsigned long long* dn,
                             unsigned long long* d_total, bool close) {
+    launch_wait();
     __shared__ T wt[kThreads / 32];
     __shared__ T tot;
     sums += blockIdx.y * stride;
@@ -104,6 +106,7 @@ __global__ void k_scan_sums(ScanArrays<T> a, T* sums, int64_t stride, int64_t n,
 template <typename T>
 __global__ void k_scan_apply(ScanArrays<T> a, int64_t n, const unsigned long long* dn, const T* __restrict__ sums,
                              int64_t stride) {
+    launch_wait();
     __shared__ T wt[kThreads / 32];
     __shared__ T tot;
     __shared__ T stage[kTile];
@@ -149,11 +152,11 @@ int scan_impl(Ctx* c, const ScanArrays<T>& a, int na, int64_t n, unsigned long l
     BH_TRY(grow(c, c->scan_tmp, (size_t)(na * nb) * sizeof(T), "scan block sums"));
     T* sums = (T*)c->scan_tmp.p;
     const dim3 grid(dn ? (unsigned)std::min<int64_t>(nb, 4 * (int64_t)c->num_sms) : (unsigned)nb, na);
-    k_reduce<T><<<grid, kThreads, 0, c->stream>>>(a, n, dn, sums, nb);
+    BH_CUDA(c, launch(c, k_reduce<T>, grid, kThreads, 0, a, n, dn, sums, nb));
     BH_LAUNCH(c);
-    k_scan_sums<T><<<dim3(1, na), kThreads, 0, c->stream>>>(a, sums, nb, n, dn, d_total, close);
+    BH_CUDA(c, launch(c, k_scan_sums<T>, dim3(1, na), kThreads, 0, a, sums, nb, n, dn, d_total, close));
     BH_LAUNCH(c);
-    k_scan_apply<T><<<grid, kThreads, 0, c->stream>>>(a, n, dn, sums, nb);
+    BH_CUDA(c, launch(c, k_scan_apply<T>, grid, kThreads, 0, a, n, dn, sums, nb));
     BH_LAUNCH(c);
     return BH_OK;
 }

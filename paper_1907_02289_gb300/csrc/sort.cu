@@ -45,6 +45,7 @@ __global__ void k_box_partial(const double* __restrict__ x, const double* __rest
                               const double* __restrict__ z, const int64_t* __restrict__ off,
                               const uint2* __restrict__ map, const int* __restrict__ poff,
                               unsigned long long* __restrict__ part, int* status) {
+    launch_wait();
     __shared__ unsigned long long s[6][kBoxThreads / 32];
     unsigned long long mn[3] = {~0ull, ~0ull, ~0ull}, mx[3] = {0ull, 0ull, 0ull};
     bool bad = false;
@@ -115,6 +116,7 @@ __global__ void k_box_partial(const double* __restrict__ x, const double* __rest
 // kStatAxis.
 __global__ void k_box_final(const unsigned long long* __restrict__ part_all, int nb, const int* __restrict__ poff,
                             double* box_all, int cyl, int* status) {
+    launch_wait();
     const unsigned long long* part = part_all + 6 * (poff ? (int64_t)poff[blockIdx.x] : (int64_t)blockIdx.x * nb);
     if (poff) nb = poff[blockIdx.x + 1] - poff[blockIdx.x];
     double* box = box_all + 8 * blockIdx.x;
@@ -174,6 +176,7 @@ __device__ __forceinline__ float atan01(float t) {
 
 __global__ void k_cyl(const double* __restrict__ x, const double* __restrict__ y, int64_t n,
                       double* __restrict__ phi, double* __restrict__ r) {
+    launch_wait();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     const float X = __double2float_rn(x[i]), Y = __double2float_rn(y[i]);
@@ -216,6 +219,7 @@ __device__ __forceinline__ uint32_t quantise(double v, double lo, double S) {
 __global__ void k_keys(const double* __restrict__ x, const double* __restrict__ y,
                        const double* __restrict__ z, int64_t n, const int64_t* __restrict__ off, int np,
                        const double* __restrict__ boxes, uint64_t* __restrict__ key) {
+    launch_wait();
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     int q = 0;
@@ -306,6 +310,7 @@ __device__ __forceinline__ TileInfo tile_info(const uint32_t* __restrict__ tmeta
 template <int ITEMS>
 __global__ void __launch_bounds__(256) k_digit_hist(const uint64_t* __restrict__ key, int64_t n, int ntiles,
                                                     const uint32_t* __restrict__ tmeta, uint32_t* __restrict__ hist) {
+    launch_wait();
     __shared__ uint32_t h[8][kRadix];
     const int per = (ntiles + gridDim.x - 1) / gridDim.x;
     const int t0 = blockIdx.x * per, t1 = min(t0 + per, ntiles);
@@ -375,6 +380,7 @@ __global__ void __launch_bounds__(kSortThreads, 3) k_sweep(
     const uint64_t* __restrict__ kin, const uint32_t* __restrict__ iin, int64_t n, int pass, int ntiles,
     const uint32_t* __restrict__ tmeta, const uint32_t* __restrict__ hist, W* words, uint32_t* ticket,
     uint64_t* __restrict__ kout, uint32_t* __restrict__ iout, int* status) {
+    launch_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     SweepSmem<ITEMS>& S = *reinterpret_cast<SweepSmem<ITEMS>*>(smem_raw);
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, shift = 8 * pass;
@@ -533,7 +539,7 @@ int64_t sort_tiles(int64_t n) {  // of one set
 // Sort (key[0]) into (key[0], idx[0]): eight passes, the first one numbering
 // the keys by position.
 template <class W, int ITEMS>
-cudaError_t sort_passes(cudaStream_t s, uint64_t* const (&kb)[2], uint32_t* const (&ib)[2], int64_t n,
+cudaError_t sort_passes(cudaStream_t s, bool early, uint64_t* const (&kb)[2], uint32_t* const (&ib)[2], int64_t n,
                         const uint32_t* tmeta, int ntiles, int nslots, int num_sms, uint32_t* scratch, int* status) {
     const SortScratch z = sort_scratch(n, ntiles, nslots);
     W* words = reinterpret_cast<W*>(scratch);
@@ -543,24 +549,26 @@ cudaError_t sort_passes(cudaStream_t s, uint64_t* const (&kb)[2], uint32_t* cons
     if (e != cudaSuccess) return e;
     if (nslots > 0) {
         const int nb = std::min(ntiles, 4 * num_sms);
-        k_digit_hist<ITEMS><<<nb, 256, 0, s>>>(kb[0], n, ntiles, tmeta, hist);
+        e = launch_on(s, early, k_digit_hist<ITEMS>, nb, 256, 0, kb[0], n, ntiles, tmeta, hist);
+        if (e != cudaSuccess) return e;
     }
     const int smem = (int)sizeof(SweepSmem<ITEMS>);
     for (int pass = 0; pass < 8; ++pass) {
         const int a = pass & 1, b = 1 - a;
         auto kern = pass == 0 ? k_sweep<W, true, ITEMS> : k_sweep<W, false, ITEMS>;
-        kern<<<ntiles, kSortThreads, smem, s>>>(kb[a], ib[a], n, pass, ntiles, tmeta, hist, words, ticket + pass, kb[b],
-                                                ib[b], status);
+        e = launch_on(s, early, kern, ntiles, kSortThreads, smem, kb[a], ib[a], n, pass, ntiles, tmeta, hist, words,
+                      ticket + pass, kb[b], ib[b], status);
+        if (e != cudaSuccess) return e;
     }
-    return cudaGetLastError();
+    return cudaSuccess;
 }
 
-cudaError_t sort_any(cudaStream_t s, uint64_t* const (&kb)[2], uint32_t* const (&ib)[2], int64_t n,
+cudaError_t sort_any(cudaStream_t s, bool early, uint64_t* const (&kb)[2], uint32_t* const (&ib)[2], int64_t n,
                      const uint32_t* tmeta, int ntiles, int nslots, int num_sms, uint32_t* scratch, int* status) {
     auto run = !tmeta && n < kSortSmall ? sort_passes<uint32_t, kSortSmallItems>
                : n < kSort32            ? sort_passes<uint32_t, kSortItems>
                                         : sort_passes<unsigned long long, kSortItems>;
-    return run(s, kb, ib, n, tmeta, ntiles, nslots, num_sms, scratch, status);
+    return run(s, early, kb, ib, n, tmeta, ntiles, nslots, num_sms, scratch, status);
 }
 constexpr int kSortLaunches = 9;  // kernels of one sort
 
@@ -576,6 +584,7 @@ struct Gather8 {
 
 __global__ void k_gather_all(Gather8 G, unsigned long long* __restrict__ scratch, const uint32_t* __restrict__ perm,
                              int64_t n, int* status) {
+    launch_wait();
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n || (G.stop && *G.stop)) return;
     const uint32_t j = perm[i];
@@ -595,6 +604,7 @@ __global__ void k_gather_all(Gather8 G, unsigned long long* __restrict__ scratch
 // The gathered arrays back into place (one launch; eight copies of a small
 // set's arrays cost their launches).
 __global__ void k_copy_back(Gather8 G, const unsigned long long* __restrict__ scratch, int64_t n) {
+    launch_wait();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n || (G.stop && *G.stop)) return;
     unsigned long long v[8];
@@ -621,7 +631,7 @@ int stage_keys(Ctx* c, const bh_particles* p) {
     const double *cx = p->x, *cy = p->y;
     if (c->prm.key_frame == 1) {
         BH_TRY(grow(c, c->cyl, 2 * (size_t)n, "cylindrical coordinates"));
-        k_cyl<<<blocks_for(n, 256), 256, 0, c->stream>>>(p->x, p->y, n, c->cyl.p, c->cyl.p + n);
+        BH_CUDA(c, launch(c, k_cyl, blocks_for(n, 256), 256, 0, p->x, p->y, n, c->cyl.p, c->cyl.p + n));
         BH_LAUNCH(c);
         cx = c->cyl.p;
         cy = c->cyl.p + n;
@@ -632,23 +642,24 @@ int stage_keys(Ctx* c, const bh_particles* p) {
     if (np > 1) {
         const int nbt = c->n_box_blocks;
         BH_TRY(grow(c, c->box_part, 6 * (size_t)nbt, "box partials"));
-        k_box_partial<<<nbt, kBoxThreads, 0, c->stream>>>(cx, cy, p->z, c->d_off.p, c->box_map.p, c->box_poff.p,
-                                                          c->box_part.p, c->d_status);
+        BH_CUDA(c, launch(c, k_box_partial, nbt, kBoxThreads, 0, cx, cy, p->z, c->d_off.p, c->box_map.p,
+                          c->box_poff.p, c->box_part.p, c->d_status));
         BH_LAUNCH(c);
-        k_box_final<<<np, 6 * 32, 0, c->stream>>>(c->box_part.p, 0, c->box_poff.p, c->d_box, c->prm.key_frame == 1,
-                                              c->d_status);
+        BH_CUDA(c, launch(c, k_box_final, np, 6 * 32, 0, c->box_part.p, 0, c->box_poff.p, c->d_box,
+                          c->prm.key_frame == 1, c->d_status));
         BH_LAUNCH(c);
     } else {
         const int nb = (int)std::max<int64_t>(1, std::min<int64_t>(nbmax, blocks_for(n, 4 * kBoxThreads)));
         BH_TRY(grow(c, c->box_part, 6 * (size_t)nb, "box partials"));
-        k_box_partial<<<nb, kBoxThreads, 0, c->stream>>>(cx, cy, p->z, c->d_off.p, nullptr, nullptr,
-                                                         c->box_part.p, c->d_status);
+        BH_CUDA(c, launch(c, k_box_partial, nb, kBoxThreads, 0, cx, cy, p->z, c->d_off.p, nullptr, nullptr,
+                          c->box_part.p, c->d_status));
         BH_LAUNCH(c);
-        k_box_final<<<1, 6 * 32, 0, c->stream>>>(c->box_part.p, nb, nullptr, c->d_box, c->prm.key_frame == 1,
-                                             c->d_status);
+        BH_CUDA(c, launch(c, k_box_final, 1, 6 * 32, 0, c->box_part.p, nb, nullptr, c->d_box,
+                          c->prm.key_frame == 1, c->d_status));
         BH_LAUNCH(c);
     }
-    k_keys<<<blocks_for(n, 256), 256, 0, c->stream>>>(cx, cy, p->z, n, c->d_off.p, np, c->d_box, c->key[0].p);
+    BH_CUDA(c, launch(c, k_keys, blocks_for(n, 256), 256, 0, cx, cy, p->z, n, c->d_off.p, np, c->d_box,
+                      c->key[0].p));
     BH_LAUNCH(c);
     c->key_cur = 0;
     return BH_OK;
@@ -667,7 +678,7 @@ int stage_sort(Ctx* c) {
     }
     uint64_t* const kb[2] = {c->key[0].p, c->key[1].p};
     uint32_t* const ib[2] = {c->idx[0].p, c->idx[1].p};
-    BH_CUDA(c, sort_any(c->stream, kb, ib, n, tmeta, ntiles, nslots, c->num_sms, c->sort_scratch.p, c->d_status));
+    BH_CUDA(c, sort_any(c->stream, !c->capturing, kb, ib, n, tmeta, ntiles, nslots, c->num_sms, c->sort_scratch.p, c->d_status));
     c->n_launches += kSortLaunches - (nslots > 0 ? 0 : 1);
     c->key_cur = 0;
     return BH_OK;
@@ -689,9 +700,9 @@ int stage_permute(Ctx* c, bh_particles* p) {
             G.src[G.na++] = arrs[a];
         }
     unsigned long long* scratch = (unsigned long long*)c->pscratch.p;
-    k_gather_all<<<blocks_for(n, 256), 256, 0, c->stream>>>(G, scratch, perm, n, c->d_status);
+    BH_CUDA(c, launch(c, k_gather_all, blocks_for(n, 256), 256, 0, G, scratch, perm, n, c->d_status));
     BH_LAUNCH(c);
-    k_copy_back<<<blocks_for(n, 256), 256, 0, c->stream>>>(G, scratch, n);
+    BH_CUDA(c, launch(c, k_copy_back, blocks_for(n, 256), 256, 0, G, scratch, n));
     BH_LAUNCH(c);
     return BH_OK;
 }
@@ -742,7 +753,11 @@ cudaError_t sort_pairs_with(cudaStream_t s, uint64_t* keys, uint32_t* idx, uint6
     const int ntiles = (int)sort_tiles(n);
     uint64_t* const kb[2] = {keys, ktmp};
     uint32_t* const ib[2] = {idx, itmp};
-    return sort_any(s, kb, ib, n, nullptr, ntiles, ntiles > 1 ? 1 : 0, num_sms, scratch, status);
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;  // (a caller may be capturing its stream)
+    const cudaError_t e = cudaStreamIsCapturing(s, &st);
+    if (e != cudaSuccess) return e;
+    return sort_any(s, st == cudaStreamCaptureStatusNone, kb, ib, n, nullptr, ntiles, ntiles > 1 ? 1 : 0, num_sms,
+                    scratch, status);
 }
 int sort_launches() { return kSortLaunches; }
 

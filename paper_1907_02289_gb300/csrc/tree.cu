@@ -194,6 +194,7 @@ __global__ void __launch_bounds__(kTreeThreads) k_tree_count(const uint64_t* __r
                                                              const int64_t* __restrict__ off, int np, int n_leaf,
                                                              int n_g, int64_t ntiles, uint16_t* __restrict__ range,
                                                              uint32_t* __restrict__ cnt) {
+    launch_wait();
     __shared__ uint32_t h[kTreeRows];
     if (threadIdx.x < kTreeRows) h[threadIdx.x] = 0;
     __syncthreads();
@@ -230,6 +231,7 @@ __global__ void __launch_bounds__(kTreeThreads) k_tree_count(const uint64_t* __r
 __global__ void k_tree_sizes(const uint32_t* __restrict__ scan, int64_t ntiles,
                              const unsigned long long* __restrict__ total, unsigned long long cap,
                              unsigned long long* sz) {
+    launch_wait();
     const int l = threadIdx.x;
     const unsigned long long nodes = scan[(int64_t)kRowGroups * ntiles], leaf0 = scan[(int64_t)kRowLeaves * ntiles];
     if (l < kLevels + 3) {
@@ -252,6 +254,7 @@ __global__ void __launch_bounds__(kTreeThreads) k_tree_write(
     uint32_t* __restrict__ begin, uint32_t* __restrict__ end, int32_t* __restrict__ parent,
     int32_t* __restrict__ first_child, uint8_t* __restrict__ nchild, int32_t* __restrict__ groups,
     int32_t* __restrict__ leaves, int32_t* __restrict__ top) {
+    launch_wait();
     __shared__ uint32_t base[kTreeRows][32];  // per (round, warp): nodes of the row before it in the tile, then ids
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const unsigned lt = (1u << lane) - 1u;
@@ -330,6 +333,7 @@ __global__ void __launch_bounds__(128) k_tree_link(const uint64_t* __restrict__ 
                                                    int32_t* __restrict__ parent,
                                                    const int32_t* __restrict__ first_child,
                                                    uint8_t* __restrict__ nchild) {
+    launch_wait();
     if (sz[kSzOvf]) return;  // (a device-sized build that outgrew its nodes)
     const int64_t nn = (int64_t)sz[kSzLvl + kLevels + 2];
     for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < nn; k += (int64_t)gridDim.x * blockDim.x) {
@@ -395,6 +399,7 @@ __global__ void __launch_bounds__(kSpanThreads) k_boxes(
     const uint32_t* __restrict__ begin, const uint32_t* __restrict__ end, const int32_t* __restrict__ first_child,
     const uint8_t* __restrict__ nchild, const int32_t* __restrict__ top, uint32_t* qlo, uint32_t* qhi,
     WalkNode* wnode, const unsigned long long* __restrict__ lvl, int lev_hi, int lev_lo) {
+    launch_wait();
     for_levels(lvl, lev_hi, lev_lo, [&](int64_t k) {
         const uint32_t e = end[k];
         const int32_t skip = skip_of(e, n, np, top);
@@ -458,6 +463,7 @@ __global__ void __launch_bounds__(kSpanThreads) k_moments(
     const uint8_t* __restrict__ nchild, const double* __restrict__ x, const double* __restrict__ y,
     const double* __restrict__ z, const double* __restrict__ m, double* M, double* cx, double* cy, double* cz,
     double* Q, const unsigned long long* __restrict__ lvl, int lev_hi, int lev_lo) {
+    launch_wait();
     for_levels(lvl, lev_hi, lev_lo, [&](int64_t k) {
         const int nc = nchild[k];
         double Mk = 0.0, sx = 0.0, sy = 0.0, sz = 0.0, c0, c1, c2;
@@ -610,6 +616,7 @@ __global__ void __launch_bounds__(kLeafTile) k_leaf32(const int32_t* __restrict_
                                                       const double* __restrict__ z, const double* __restrict__ m,
                                                       float4* phi, float4* plo, float4* cell32,
                                                       float* __restrict__ mlo) {
+    launch_wait();
     __shared__ float4 sh[kLeafCap], sl[kLeafCap];
     const int64_t nl = (int64_t)*dnl;
     for (int64_t t0 = (int64_t)blockIdx.x * kLeafTile; t0 < nl; t0 += (int64_t)gridDim.x * kLeafTile) {
@@ -681,6 +688,7 @@ template <int ORDER>
 __global__ void __launch_bounds__(kSpanThreads) k_moments32(
     const int32_t* __restrict__ first_child, const uint8_t* __restrict__ nchild, float4* cell32, float* mlo,
     const unsigned long long* __restrict__ lvl, int lev_hi, int lev_lo) {
+    launch_wait();
     for_levels(lvl, lev_hi, lev_lo, [&](int64_t k) {
         const int nc = nchild[k];
         if (nc == 0) return;
@@ -756,17 +764,19 @@ int launch_levels(Ctx* c, int64_t span_nodes, void (*kern)(KA...), A... args) {
     while (hi >= 0) {
         int lo = hi;
         cudaLaunchConfig_t cfg = {};
-        cudaLaunchAttribute at = {};
+        cudaLaunchAttribute at[2] = {};
         cfg.stream = c->stream;
+        at[0] = early_attribute(!c->capturing);
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
         if (nodes(hi) <= span_nodes) {
             while (lo > 0 && nodes(lo - 1) <= span_nodes) --lo;
             cfg.gridDim = dim3(kSpanBlocks);
             cfg.blockDim = dim3(kSpanThreads);
-            at.id = cudaLaunchAttributeClusterDimension;
-            at.val.clusterDim.x = kSpanBlocks;
-            at.val.clusterDim.y = at.val.clusterDim.z = 1;
-            cfg.attrs = &at;
-            cfg.numAttrs = 1;
+            at[1].id = cudaLaunchAttributeClusterDimension;
+            at[1].val.clusterDim.x = kSpanBlocks;
+            at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
+            cfg.numAttrs = 2;
         } else {
             cfg.gridDim = dim3(blocks_for(nodes(hi), 128));
             cfg.blockDim = dim3(128);
@@ -808,12 +818,12 @@ int stage_octree(Ctx* c) {
     BH_TRY(grow(c, c->tree_range, (size_t)n, "node ranges"));
     BH_TRY(grow(c, c->tree_top, (size_t)n, "first nodes"));
     uint32_t* cnt = c->tree_cnt.p;
-    k_tree_count<<<(unsigned)ntiles, kTreeThreads, 0, c->stream>>>(key, n, c->d_off.p, np, n_leaf, n_g, ntiles,
-                                                                 c->tree_range.p, cnt);
+    BH_CUDA(c, launch(c, k_tree_count, (unsigned)ntiles, kTreeThreads, 0, key, n, c->d_off.p, np, n_leaf,
+                      n_g, ntiles, c->tree_range.p, cnt));
     BH_LAUNCH(c);
     BH_TRY(scan_u32(c, cnt, tree_count_words(n), c->d_small));
-    k_tree_sizes<<<1, 32, 0, c->stream>>>(cnt, ntiles, c->d_small, dev ? (unsigned long long)c->cap_nodes : ~0ull,
-                                          c->d_sz);
+    BH_CUDA(c, launch(c, k_tree_sizes, 1, 32, 0, cnt, ntiles, c->d_small, dev ? (unsigned long
+                      long)c->cap_nodes : ~0ull, c->d_sz));
     BH_LAUNCH(c);
     if (dev) {
         c->n_nodes = c->cap_nodes;
@@ -832,13 +842,12 @@ int stage_octree(Ctx* c) {
         BH_TRY(grow(c, c->groups, (size_t)c->n_groups + 1, "groups"));
         BH_TRY(grow(c, c->leaves, (size_t)c->n_leaves, "leaves"));
     }
-    k_tree_write<<<(unsigned)ntiles, kTreeThreads, 0, c->stream>>>(
-        c->tree_range.p, n, c->d_off.p, np, ntiles, cnt, c->n_nodes, c->level.p, c->begin.p, c->end.p, c->parent.p,
-        c->first_child.p, c->nchild.p, c->groups.p, c->leaves.p, c->tree_top.p);
+    BH_CUDA(c, launch(c, k_tree_write, (unsigned)ntiles, kTreeThreads, 0, c->tree_range.p, n, c->d_off.p,
+                      np, ntiles, cnt, c->n_nodes, c->level.p, c->begin.p, c->end.p, c->parent.p, c->first_child.p,
+                      c->nchild.p, c->groups.p, c->leaves.p, c->tree_top.p));
     BH_LAUNCH(c);
-    k_tree_link<<<blocks_for(c->n_nodes, 128), 128, 0, c->stream>>>(key, c->d_off.p, np, c->d_sz, c->level.p,
-                                                                    c->begin.p, c->end.p, c->parent.p,
-                                                                    c->first_child.p, c->nchild.p);
+    BH_CUDA(c, launch(c, k_tree_link, blocks_for(c->n_nodes, 128), 128, 0, key, c->d_off.p, np, c->d_sz,
+                      c->level.p, c->begin.p, c->end.p, c->parent.p, c->first_child.p, c->nchild.p));
     BH_LAUNCH(c);
     return BH_OK;
 }
@@ -866,9 +875,9 @@ int stage_moments(Ctx* c, const bh_particles* p) {
     // (captured: the last build's leaves with room to grow; strided)
     const int64_t nl = c->dev_sizes ? with_room(c, c->n_leaves) : c->n_leaves;
     auto leaf = quad ? k_leaf32<2> : k_leaf32<1>;
-    leaf<<<blocks_for(nl, kLeafTile), kLeafTile, 0, c->stream>>>(c->leaves.p, c->d_sz + kSzNl, c->begin.p, c->end.p,
-                                                                 p->x, p->y, p->z, p->m, c->phi.p, c->plo.p,
-                                                                 c->cell32.p, c->cell32lo.p);
+    BH_CUDA(c, launch(c, leaf, blocks_for(nl, kLeafTile), kLeafTile, 0, c->leaves.p, c->d_sz + kSzNl,
+                      c->begin.p, c->end.p, p->x, p->y, p->z, p->m, c->phi.p, c->plo.p, c->cell32.p,
+                      c->cell32lo.p));
     BH_LAUNCH(c);
     BH_TRY(stage_end(c));
     BH_TRY(stage_begin(c, BH_STAGE_MOMENTS));

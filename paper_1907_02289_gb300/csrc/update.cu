@@ -13,6 +13,7 @@ namespace {
 __global__ void k_kick(int64_t n, double h, const double* __restrict__ ax, const double* __restrict__ ay,
                        const double* __restrict__ az, double* __restrict__ vx, double* __restrict__ vy,
                        double* __restrict__ vz, const unsigned long long* __restrict__ abort) {
+    launch_wait();
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n || (abort && *abort)) return;
     vx[i] += h * ax[i];
@@ -29,6 +30,7 @@ __global__ void k_kick_drift(int64_t n, double h, double dt, const double* __res
                              double* __restrict__ vx, double* __restrict__ vy, double* __restrict__ vz,
                              double* __restrict__ x, double* __restrict__ y, double* __restrict__ z, double c,
                              double s) {
+    launch_wait();
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     const double ux = vx[i] + h * ax[i], uy = vy[i] + h * ay[i], uz = vz[i] + h * az[i];
@@ -58,6 +60,7 @@ __global__ void __launch_bounds__(kDiagThreads) k_diag_partial(
     int64_t n, double GMc, const double* __restrict__ x, const double* __restrict__ y, const double* __restrict__ z,
     const double* __restrict__ vx, const double* __restrict__ vy, const double* __restrict__ vz,
     const double* __restrict__ m, double* __restrict__ part) {
+    launch_wait();
     __shared__ double sh[kDiagSums][kDiagThreads];
     double acc[kDiagSums];
 #pragma unroll
@@ -88,6 +91,7 @@ __global__ void __launch_bounds__(kDiagThreads) k_diag_partial(
 }
 
 __global__ void k_diag_final(const double* __restrict__ part, double* out) {
+    launch_wait();
     const int q = threadIdx.x;
     if (q >= kDiagSums) return;
     double s = 0.0;
@@ -101,10 +105,10 @@ int stage_diagnostics(Ctx* c, const bh_particles* p, double* host_out) {
     BH_TRY(grow(c, c->diag, (size_t)kDiagBlocks * kDiagSums + kDiagSums, "diagnostic sums"));
     double* part = c->diag.p;
     double* out = part + (size_t)kDiagBlocks * kDiagSums;
-    k_diag_partial<<<kDiagBlocks, kDiagThreads, 0, c->stream>>>(p->n, c->prm.G * c->prm.M_central, p->x, p->y, p->z,
-                                                                 p->vx, p->vy, p->vz, p->m, part);
+    BH_CUDA(c, launch(c, k_diag_partial, kDiagBlocks, kDiagThreads, 0, p->n, c->prm.G * c->prm.M_central,
+                      p->x, p->y, p->z, p->vx, p->vy, p->vz, p->m, part));
     BH_LAUNCH(c);
-    k_diag_final<<<1, 32, 0, c->stream>>>(part, out);
+    BH_CUDA(c, launch(c, k_diag_final, 1, 32, 0, part, out));
     BH_LAUNCH(c);
     BH_CUDA(c, cudaMemcpyAsync(host_out, out, kDiagSums * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
     BH_CUDA(c, cudaStreamSynchronize(c->stream));
@@ -113,8 +117,8 @@ int stage_diagnostics(Ctx* c, const bh_particles* p, double* host_out) {
 
 int stage_kick(Ctx* c, bh_particles* p, double h) {
     BH_TRY(stage_begin(c, BH_STAGE_UPDATE));
-    k_kick<<<blocks_for(c->n, 256), 256, 0, c->stream>>>(c->n, h, p->ax, p->ay, p->az, p->vx, p->vy, p->vz,
-                                                         c->abort);
+    BH_CUDA(c, launch(c, k_kick, blocks_for(c->n, 256), 256, 0, c->n, h, p->ax, p->ay, p->az, p->vx, p->vy,
+                      p->vz, c->abort));
     BH_LAUNCH(c);
     return stage_end(c);
 }
@@ -123,8 +127,8 @@ int stage_kick_drift(Ctx* c, bh_particles* p, double h, double dt) {
     BH_TRY(stage_begin(c, BH_STAGE_UPDATE));
     const double om = c->prm.omega * dt;
     auto kern = om != 0.0 ? k_kick_drift<true> : k_kick_drift<false>;
-    kern<<<blocks_for(c->n, 256), 256, 0, c->stream>>>(c->n, h, dt, p->ax, p->ay, p->az, p->vx, p->vy, p->vz, p->x,
-                                                       p->y, p->z, std::cos(om), std::sin(om));
+    BH_CUDA(c, launch(c, kern, blocks_for(c->n, 256), 256, 0, c->n, h, dt, p->ax, p->ay, p->az, p->vx,
+                      p->vy, p->vz, p->x, p->y, p->z, std::cos(om), std::sin(om)));
     BH_LAUNCH(c);
     return stage_end(c);
 }

@@ -250,6 +250,7 @@ __device__ __forceinline__ void walk_counts(const WalkArgs& A, int64_t k, const 
 // same path and the SMs are full.
 template <int MODE>
 __global__ void __launch_bounds__(128) k_walk(const WalkArgs A, const WalkParams wp) {
+    launch_wait();
     const int64_t ng = A.dng ? min(A.ng, (int64_t)*A.dng) : A.ng;
     for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < ng; base += (int64_t)gridDim.x * blockDim.x) {
         const int64_t k = base + threadIdx.x;
@@ -311,6 +312,7 @@ __device__ __forceinline__ uint32_t warp_exclusive(uint32_t v, int lane, uint32_
 
 template <int MODE>
 __global__ void __launch_bounds__(32 * kCoopWarps) k_walk_coop(const WalkArgs A, const WalkParams wp) {
+    launch_wait();
     __shared__ uint32_t buf[kCoopWarps][kCoopCap];
     const int lane = threadIdx.x & 31;
     uint32_t* E = buf[threadIdx.x >> 5];
@@ -430,6 +432,7 @@ __global__ void k_expand(int64_t ng, const unsigned long long* __restrict__ dng,
                          const uint32_t* __restrict__ end, const WalkNode* __restrict__ wn, WalkParams wp,
                          const int64_t* __restrict__ jj_off, uint32_t* __restrict__ JJ, int64_t* __restrict__ jm,
                          unsigned long long* n_far) {
+    launch_wait();
     if (dng) ng = min(ng, (int64_t)*dng);
     const int lane = threadIdx.x & 31;
     const int64_t wstride = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -518,6 +521,7 @@ __global__ void k_unstash(int64_t ng, const unsigned long long* __restrict__ dng
                           const int64_t* __restrict__ pp_off, const int64_t* __restrict__ pc_off,
                           const int32_t* __restrict__ sP, const int32_t* __restrict__ sC, int64_t capP,
                           int64_t capC, int32_t* __restrict__ P, int32_t* __restrict__ C) {
+    launch_wait();
     if (dng) ng = min(ng, (int64_t)*dng);
     const int lane = threadIdx.x & 31;
     const int64_t wstride = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -557,6 +561,7 @@ __global__ void k_unstash(int64_t ng, const unsigned long long* __restrict__ dng
 __global__ void k_walk_thresholds(const double* __restrict__ box, int np, double r_coll, int cyl,
                                   long long* __restrict__ rcq, long long* __restrict__ rfar,
                                   long long* __restrict__ period) {
+    launch_wait();
     const int q = blockIdx.x * blockDim.x + threadIdx.x;
     if (q >= np) return;
     const double S = __ddiv_rn(2097152.0, box[8 * q + 3]);
@@ -581,6 +586,7 @@ __global__ void k_walk_thresholds(const double* __restrict__ box, int np, double
 // Device-sized build: the list totals against the buffers' room.
 __global__ void k_list_room(const unsigned long long* __restrict__ tot, long long roomP, long long roomC,
                             long long roomJ, unsigned long long* sz) {
+    launch_wait();
     if (threadIdx.x != 0) return;
     if ((long long)tot[0] > roomP || (long long)tot[1] > roomC || (long long)tot[2] > roomJ) sz[kSzOvf] |= kOvfLists;
 }
@@ -624,8 +630,8 @@ int walk_thresholds(Ctx* c) {
     BH_TRY(grow(c, c->d_rcq, (size_t)np, "walk contact thresholds"));
     BH_TRY(grow(c, c->d_rfar, (size_t)np, "far thresholds"));
     BH_TRY(grow(c, c->d_period, (size_t)np, "walk periods"));
-    k_walk_thresholds<<<blocks_for(np, 64), 64, 0, c->stream>>>(c->d_box, np, c->prm.r_coll, c->prm.key_frame == 1,
-                                                                c->d_rcq.p, c->d_rfar.p, c->d_period.p);
+    BH_CUDA(c, launch(c, k_walk_thresholds, blocks_for(np, 64), 64, 0, c->d_box, np, c->prm.r_coll,
+                      c->prm.key_frame == 1, c->d_rcq.p, c->d_rfar.p, c->d_period.p));
     BH_LAUNCH(c);
     return BH_OK;
 }
@@ -654,9 +660,9 @@ WalkArgs walk_args(const Ctx* c, const unsigned long long* dng, int64_t slots) {
 template <int MODE>
 int launch_walk(Ctx* c, const WalkArgs& A, const WalkParams& wp, int64_t groups) {
     if (groups <= kCoopGroups && A.nn <= (int64_t)1 << kEntBits)
-        k_walk_coop<MODE><<<blocks_for(groups, kCoopWarps), 32 * kCoopWarps, 0, c->stream>>>(A, wp);
+        BH_CUDA(c, launch(c, k_walk_coop<MODE>, blocks_for(groups, kCoopWarps), 32 * kCoopWarps, 0, A, wp));
     else
-        k_walk<MODE><<<blocks_for(groups, 128), 128, 0, c->stream>>>(A, wp);
+        BH_CUDA(c, launch(c, k_walk<MODE>, blocks_for(groups, 128), 128, 0, A, wp));
     BH_LAUNCH(c);
     return BH_OK;
 }
@@ -669,8 +675,8 @@ int expand_lists(Ctx* c, const WalkParams& wp, const unsigned long long* dng, un
     unsigned long long* n_far = c->d_small + 10;  // (cleared before the walk)
     if (split) BH_TRY(grow(c, c->cnt_jm, (size_t)ng + 1, "list split points"));
     auto expand = split ? k_expand<true> : k_expand<false>;
-    expand<<<grid, 256, 0, c->stream>>>(ng, dng, c->groups.p, c->cnt_p.p, c->P.p, c->begin.p, c->end.p, c->wnode.p,
-                                        wp, c->cnt_j.p, c->JJ.p, split ? c->cnt_jm.p : nullptr, n_far);
+    BH_CUDA(c, launch(c, expand, grid, 256, 0, ng, dng, c->groups.p, c->cnt_p.p, c->P.p, c->begin.p,
+                      c->end.p, c->wnode.p, wp, c->cnt_j.p, c->JJ.p, split ? c->cnt_jm.p : nullptr, n_far));
     BH_LAUNCH(c);
     return BH_OK;
 }
@@ -732,9 +738,8 @@ int stage_lists(Ctx* c) {
     BH_TRY(grow(c, c->C, (size_t)c->n_pc + 1, "cell lists"));
     BH_TRY(grow(c, c->JJ, (size_t)c->n_jj + 1, "list particle indices"));
     if (stash && h[11] == 0) {
-        k_unstash<<<blocks_for(ng * 32, 256), 256, 0, c->stream>>>(ng, nullptr, -1, c->cnt_p.p, c->cnt_c.p,
-                                                                   c->stash_p.p, c->stash_c.p, capP, capC, c->P.p,
-                                                                   c->C.p);
+        BH_CUDA(c, launch(c, k_unstash, blocks_for(ng * 32, 256), 256, 0, ng, nullptr, -1, c->cnt_p.p,
+                          c->cnt_c.p, c->stash_p.p, c->stash_c.p, capP, capC, c->P.p, c->C.p));
         BH_LAUNCH(c);
         ++c->n_one_walk_builds;
     } else {
@@ -780,8 +785,8 @@ int stage_lists_dev_walk(Ctx* c) {
     BH_TRY(launch_walk<kWalkStash>(c, A, wp, std::max<int64_t>(slots, 1)));
     int64_t* const arr[3] = {c->cnt_p.p, c->cnt_c.p, c->cnt_j.p};
     BH_TRY(scan3_i64(c, arr, ng, c->d_small, dng));
-    k_list_room<<<1, 32, 0, c->stream>>>(c->d_small, (long long)c->P.cap - 1, (long long)c->C.cap - 1,
-                                         (long long)c->JJ.cap - 1, c->d_sz);
+    BH_CUDA(c, launch(c, k_list_room, 1, 32, 0, c->d_small, (long long)c->P.cap - 1, (long long)c->C.cap -
+                      1, (long long)c->JJ.cap - 1, c->d_sz));
     BH_LAUNCH(c);
     return BH_OK;
 }
@@ -795,8 +800,8 @@ int stage_lists_dev_fill(Ctx* c) {
     const WalkParams wp = walk_params(c);
     const int64_t slots = c->dev_slots, capP = c->walk_cap_p, capC = c->walk_cap_c;
     const unsigned grid = blocks_for(std::max<int64_t>(slots, 1) * 32, 256);  // a warp per expected group
-    k_unstash<<<grid, 256, 0, c->stream>>>(ng, dng, slots, c->cnt_p.p, c->cnt_c.p, c->stash_p.p, c->stash_c.p, capP,
-                                           capC, c->P.p, c->C.p);
+    BH_CUDA(c, launch(c, k_unstash, grid, 256, 0, ng, dng, slots, c->cnt_p.p, c->cnt_c.p, c->stash_p.p,
+                      c->stash_c.p, capP, capC, c->P.p, c->C.p));
     BH_LAUNCH(c);
     WalkArgs A = walk_args(c, dng, slots);
     A.P = c->P.p;
