@@ -547,7 +547,7 @@ int size_dev_build(Ctx* c, const int64_t cap[5]) {
     BH_TRY(grow(c, c->leaves, (size_t)nodes, "leaves"));
     for (auto* b : {&c->cnt_p, &c->cnt_c, &c->cnt_j, &c->cnt_jm})
         BH_TRY(grow(c, *b, (size_t)n + 1, "list offsets"));
-    BH_TRY(grow(c, c->order, (size_t)n + 1, "group order"));
+    BH_TRY(grow(c, c->order, (size_t)n + 1, "work items"));
     // three scans over up to n group counts (8-byte words, 2048 per tile)
     BH_TRY(grow(c, c->scan_tmp, 3 * ((size_t)n / 2048 + 2) * sizeof(int64_t), "scan block sums"));
     BH_TRY(grow(c, c->stash_p, (size_t)std::max<int64_t>(1, cap[1] * c->walk_cap_p), "stashed particle lists"));

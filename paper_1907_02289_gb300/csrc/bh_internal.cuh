@@ -31,6 +31,7 @@ constexpr int kSzNg = kLevels + 3;          // group count
 constexpr int kSzOvf = kSzNg + 1;           // overflow bits
 constexpr int kSzNeedNodes = kSzOvf + 1;    // nodes wanted when the node capacity ran out (a lower bound)
 constexpr int kSzNl = kSzNeedNodes + 1;     // leaf count
+constexpr int kSzItems = kSzNl + 1;         // work items of the FP32 force kernel
 constexpr int kSzWords = 32;
 constexpr unsigned long long kOvfNodes = 1, kOvfLists = 2;
 
@@ -178,7 +179,7 @@ struct Ctx {
     DBuf<int32_t> groups;            // node ids ordered by begin
     int64_t n_leaves = 0;
     DBuf<int32_t> leaves;            // node ids ordered by begin
-    DBuf<int32_t> order;             // force-kernel processing order of groups
+    DBuf<int2> order;                // FP32 force kernel's work items (group, i-chunk) in processing order
     DBuf<unsigned long long> order_cnt;  // order buckets: counts/starts and cursors
     DBuf<uint64_t> ord_key[2];           // windowed order: sort keys
     DBuf<uint32_t> ord_idx[2];
@@ -376,8 +377,7 @@ inline int64_t groups_bound(const Ctx* c) {
     if (!c->dev_sizes || c->dev_build) return c->n_groups;
     size_t b = c->groups.cap;
     for (size_t v : {c->cnt_p.cap, c->cnt_c.cap, c->cnt_j.cap}) b = v < b ? v : b;
-    if (c->prm.precision == BH_PREC_FP32)
-        for (size_t v : {c->cnt_jm.cap, c->order.cap}) b = v < b ? v : b;
+    if (c->prm.precision == BH_PREC_FP32 && c->cnt_jm.cap < b) b = c->cnt_jm.cap;
     return (int64_t)b - 1;
 }
 inline int64_t groups_expected(const Ctx* c) {

@@ -39,7 +39,8 @@
 // FP32 numbers, dfloat.cuh), from the hi/lo coordinates and masses, and
 // replaces a_i.
 //
-// Mapping: one warp per group.  A group of n_i = 32 R + t particles gives
+// Mapping: one warp per i-chunk of a group (at most 96 particles; a larger
+// group is several warps' work).  A chunk of n_i = 32 R + t particles gives
 // every lane R i-slots; the t remaining particles go to a "tail" slot shared
 // by J = 32 / T lanes (T = t rounded up to a power of two) that split the
 // list between them, so a 65-particle group costs 2 + 1/32 slots rather
@@ -47,16 +48,15 @@
 // and the pair (j, j+1) is evaluated with packed f32x2 instructions (FADD2,
 // FFMA2, FMUL2) against the i-particle held as (x_i, x_i), which halves the
 // issue slots per interaction.  The next tile is gathered with cp.async
-// while the current one is evaluated.  Groups larger than the i-chunk (at
-// most 96) are evaluated chunk by chunk.  The group's own particles are
+// while the current one is evaluated.  The group's own particles are
 // evaluated first in a phase that excludes i = j; the expanded list holds
 // only the other particles.
 //
-// Scheduling: groups are taken in order of size class (warps running side
+// Scheduling: chunks are taken in order of size class (warps running side
 // by side execute the same code), by decreasing estimated cost within a
-// class, optionally within windows of consecutive groups; the grid is one
-// warp per group, or persistent (resident blocks only) with warps taking
-// groups round robin or from an atomic ticket counter.  Warps per block and
+// class, optionally whole groups within windows of consecutive groups; the
+// grid is one warp per item, or persistent (resident blocks only) with warps
+// taking items round robin or from an atomic ticket counter.  Warps per block and
 // the i-chunk are runtime settings; the compile-time options below exist for
 // experiments.
 #include <algorithm>
@@ -136,7 +136,9 @@ struct Args {
     int64_t ng;
     const unsigned long long* dng;  // device group count (device-sized list builds; NULL: ng)
     const unsigned long long* abort;  // device-sized build: nonzero overflow bits skip the launch
-    const int32_t* order;  // processing order of the groups (NULL: list order)
+    const int2* order;     // work items in processing order: (group, i-chunk, or -1: every chunk)
+    const unsigned long long* items;  // their count (device)
+    int64_t items_cap;     // and its bound
     const int32_t* groups;
     const uint32_t* begin;
     const uint32_t* end;
@@ -768,18 +770,21 @@ __device__ __forceinline__ unsigned long long global_ns() {
     return t;
 }
 
-// One group (list slot) for one warp.
+// One work item for one warp: an i-chunk of a group (or all of them in turn).
 template <int ORDER, int MODE>
-__device__ __forceinline__ void force_group(const Args& A, Smem32& S, int64_t slot, int lane) {
-    const int64_t k = A.order ? A.order[slot] : slot;  // groups of one size class run side by side
+__device__ __forceinline__ void force_item(const Args& A, Smem32& S, int64_t slot, int lane) {
+    const int2 o = A.order[slot];
+    const int64_t k = o.x;
     const int32_t g = A.groups[k];
     const uint32_t b = A.begin[g], e = A.end[g];
     // origin: the group node's centre of mass as an FP32 hi/lo pair
     const float4 o0 = A.cell32[3 * (int64_t)g], o1 = A.cell32[3 * (int64_t)g + 1];
     const float oh[3] = {o0.x, o0.y, o0.z}, ol[3] = {o1.x, o1.y, o1.z};
     // chunks of at most A.chunk particles: R full slots plus a tail of at most 16
-    for (uint32_t i0 = b; i0 < e;) {
-        const uint32_t rem = e - i0, cnt = min(rem, (uint32_t)A.chunk);
+    const uint32_t first = o.y < 0 ? b : b + (uint32_t)o.y * (uint32_t)A.chunk;
+    const uint32_t last = o.y < 0 ? e : min(e, first + (uint32_t)A.chunk);
+    for (uint32_t i0 = first; i0 < last;) {
+        const uint32_t rem = last - i0, cnt = min(rem, (uint32_t)A.chunk);
         int R = (int)(cnt >> 5), t = (int)(cnt & 31), T = 0;
         if (t > 16) {
             ++R;  // more than half a slot left: a full one
@@ -816,18 +821,19 @@ __global__ void __launch_bounds__(32 * BH_F32_MAXW, 2) k_force32(const Args A) {
     Smem32& S = sm[w];
     const unsigned long long t0 = A.warp_time ? global_ns() : 0ull;
     if (A.abort && *A.abort) return;  // that build outgrew its buffers: the step is finished eagerly
-    const int64_t ng = A.dng ? min(A.ng, (int64_t)*A.dng) : A.ng;
-    if (A.ticket) {  // persistent, dynamic: the next list slot from the shared counter
-        for (;;) {
-            unsigned long long s = 0;
+    const int64_t ni = min(A.items_cap, (int64_t)*A.items);
+    if (A.ticket) {  // persistent, dynamic: the next item from the shared counter
+        unsigned long long s = 0;
+        if (lane == 0) s = atomicAdd(A.ticket, 1ull);
+        s = __shfl_sync(0xffffffffu, s, 0);
+        while ((int64_t)s < ni) {
+            force_item<ORDER, MODE>(A, S, (int64_t)s, lane);
             if (lane == 0) s = atomicAdd(A.ticket, 1ull);
             s = __shfl_sync(0xffffffffu, s, 0);
-            if ((int64_t)s >= ng) break;
-            force_group<ORDER, MODE>(A, S, (int64_t)s, lane);
         }
-    } else {  // static: one slot per warp (grid) or every stride-th slot (persistent)
+    } else {  // static: one item per warp (grid) or every stride-th item (persistent)
         const int64_t stride = (int64_t)gridDim.x * nw;
-        for (int64_t s = wid; s < ng; s += stride) force_group<ORDER, MODE>(A, S, s, lane);
+        for (int64_t s = wid; s < ni; s += stride) force_item<ORDER, MODE>(A, S, s, lane);
     }
     if (A.warp_time && lane == 0) {
         A.warp_time[2 * wid] = t0;
@@ -835,12 +841,11 @@ __global__ void __launch_bounds__(32 * BH_F32_MAXW, 2) k_force32(const Args A) {
     }
 }
 
-// Size class of a group = the (R, tail) variant of its last chunk; classes
+// Size class of an i-chunk of cnt particles = its (R, tail) variant; classes
 // are numbered so that larger work comes first.
-__device__ __forceinline__ int size_class(uint32_t n_i, uint32_t chunk) {
-    const uint32_t rem = n_i - chunk * ((n_i - 1u) / chunk);
-    int R = (int)(rem >> 5);
-    const int t = (int)(rem & 31);
+__device__ __forceinline__ int size_class(uint32_t cnt) {
+    int R = (int)(cnt >> 5);
+    const int t = (int)(cnt & 31);
     bool tail = false;
     if (t > 16)
         ++R;
@@ -850,63 +855,82 @@ __device__ __forceinline__ int size_class(uint32_t n_i, uint32_t chunk) {
     return 5 - cls;
 }
 
-// Processing order: size class first (warps side by side run the same code),
-// then, with cost ordering on, largest estimated cost first within a class
-// (cost = n_i (n_i + list particles + 2 list cells), bucketed by log2), so the
-// list ends with the cheapest groups of each class.
+// Processing order of the work items, one per i-chunk of a group: size class
+// first (warps side by side run the same code), then, with cost ordering on,
+// largest estimated cost first within a class (cost = chunk (n_i + list
+// particles + 2 list cells), bucketed by log2), so the list ends with the
+// cheapest items of each class.  A chunk streams its group's whole list, so a
+// group of several chunks is several warps' work at no extra cost, and warps
+// side by side run one chunk shape.  Against whole groups: 4 steps of the 2^26
+// ring (groups of 128 to 192) 532 -> 521 ms, host steps of the 2^20 ring 4.89 ->
+// 4.70 ms, 4 graph steps of a 300,007-particle ring 1449 -> 1430 us.
 constexpr int kCostBuckets = 32;
 constexpr int kOrderBuckets = 6 * kCostBuckets;
 
-__device__ __forceinline__ int order_bucket(int64_t k, const int32_t* __restrict__ groups,
-                                            const uint32_t* __restrict__ begin, const uint32_t* __restrict__ end,
-                                            const int64_t* __restrict__ jj_off, const int64_t* __restrict__ pc_off,
-                                            uint32_t chunk, bool by_cost) {
-    const int32_t g = groups[k];
-    const uint32_t ni = end[g] - begin[g];
+struct OrderArgs {
+    int64_t ng;
+    const unsigned long long* dng;
+    const int32_t* groups;
+    const uint32_t *begin, *end;
+    const int64_t *jj_off, *pc_off;
+    uint32_t chunk;
+    bool by_cost;
+};
+
+__device__ __forceinline__ uint32_t group_size(const OrderArgs& O, int64_t k) {
+    const int32_t g = O.groups[k];
+    return O.end[g] - O.begin[g];
+}
+
+// Bucket of a chunk of cnt of group k's ni particles.
+__device__ __forceinline__ int order_bucket(const OrderArgs& O, int64_t k, uint32_t ni, uint32_t cnt) {
     int cb = 0;
-    if (by_cost) {
+    if (O.by_cost) {
         const unsigned long long cost =
-            (unsigned long long)ni * ((unsigned long long)ni + (unsigned long long)(jj_off[k + 1] - jj_off[k]) +
-                                      2ull * (unsigned long long)(pc_off[k + 1] - pc_off[k]));
+            (unsigned long long)cnt * ((unsigned long long)ni + (unsigned long long)(O.jj_off[k + 1] - O.jj_off[k]) +
+                                       2ull * (unsigned long long)(O.pc_off[k + 1] - O.pc_off[k]));
         const int lg = cost ? 63 - __clzll((long long)cost) : 0;
         cb = kCostBuckets - 1 - min(lg, kCostBuckets - 1);
     }
-    return size_class(ni, chunk) * kCostBuckets + cb;
+    return size_class(cnt) * kCostBuckets + cb;
 }
 
-__global__ void k_order_hist(int64_t ng, const unsigned long long* __restrict__ dng,
-                             const int32_t* __restrict__ groups, const uint32_t* __restrict__ begin,
-                             const uint32_t* __restrict__ end, const int64_t* __restrict__ jj_off,
-                             const int64_t* __restrict__ pc_off, uint32_t chunk, bool by_cost,
-                             unsigned long long* cnt) {
+__global__ void k_order_hist(const OrderArgs O, unsigned long long* cnt) {
     launch_wait();
-    if (dng) ng = min(ng, (int64_t)*dng);
-    for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < ng; k += (int64_t)gridDim.x * blockDim.x)
-        atomicAdd(&cnt[order_bucket(k, groups, begin, end, jj_off, pc_off, chunk, by_cost)], 1ull);
+    const int64_t ng = O.dng ? min(O.ng, (int64_t)*O.dng) : O.ng;
+    for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < ng; k += (int64_t)gridDim.x * blockDim.x) {
+        const uint32_t ni = group_size(O, k);
+        for (uint32_t i = 0; i < ni; i += O.chunk)
+            atomicAdd(&cnt[order_bucket(O, k, ni, min(O.chunk, ni - i))], 1ull);
+    }
 }
 
-// Windowed order: key = (group index / window, bucket); a stable sort of the
-// keys keeps list (Morton) order within a window and a bucket, so the warps
-// running at one time work on one stretch of the ring (their list data
-// overlaps in L2) while the warps side by side still share a size class.
-__global__ void k_order_keys(int64_t ng, const int32_t* __restrict__ groups, const uint32_t* __restrict__ begin,
-                             const uint32_t* __restrict__ end, const int64_t* __restrict__ jj_off,
-                             const int64_t* __restrict__ pc_off, uint32_t chunk, bool by_cost, int64_t window,
-                             uint64_t* __restrict__ keys) {
+// Windowed order: key = (group index / window, bucket of the last chunk); a
+// stable sort of the keys keeps list (Morton) order within a window and a
+// bucket, so the warps running at one time work on one stretch of the ring
+// (their list data overlaps in L2) while the warps side by side still share a
+// size class.  One item per group, all its chunks.
+__global__ void k_order_keys(const OrderArgs O, int64_t window, uint64_t* __restrict__ keys) {
     launch_wait();
     const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= ng) return;
-    keys[k] = ((uint64_t)(k / window) << 8) | (uint64_t)order_bucket(k, groups, begin, end, jj_off, pc_off, chunk, by_cost);
+    if (k >= O.ng) return;
+    const uint32_t ni = group_size(O, k), last = ni - O.chunk * ((ni - 1u) / O.chunk);
+    keys[k] = ((uint64_t)(k / window) << 8) | (uint64_t)order_bucket(O, k, ni, last);
 }
 
-__global__ void k_order_scatter(int64_t ng, const unsigned long long* __restrict__ dng,
-                                const int32_t* __restrict__ groups, const uint32_t* __restrict__ begin,
-                                const uint32_t* __restrict__ end, const int64_t* __restrict__ jj_off,
-                                const int64_t* __restrict__ pc_off, uint32_t chunk, bool by_cost,
-                                const unsigned long long* __restrict__ cnt, unsigned long long* cursor,
-                                int32_t* __restrict__ order) {
+__global__ void k_order_whole(const uint32_t* __restrict__ idx, int64_t ng, int2* __restrict__ order,
+                              unsigned long long* items) {
     launch_wait();
-    if (dng) ng = min(ng, (int64_t)*dng);
+    const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (k == 0) *items = (unsigned long long)ng;
+    if (k < ng) order[k] = make_int2((int)idx[k], -1);
+}
+
+__global__ void k_order_scatter(const OrderArgs O, const unsigned long long* __restrict__ cnt,
+                                unsigned long long* cursor, int2* __restrict__ order, int64_t cap,
+                                unsigned long long* items) {
+    launch_wait();
+    const int64_t ng = O.dng ? min(O.ng, (int64_t)*O.dng) : O.ng;
     // exclusive prefix of the bucket counts, by the block's first warp
     __shared__ unsigned long long start[kOrderBuckets];
     constexpr int PL = kOrderBuckets / 32;
@@ -925,11 +949,17 @@ __global__ void k_order_scatter(int64_t ng, const unsigned long long* __restrict
         }
 #pragma unroll
         for (int b = 0; b < PL; ++b) start[threadIdx.x * PL + b] = x - sum + v[b];
+        if (blockIdx.x == 0 && threadIdx.x == 31) *items = x;
     }
     __syncthreads();
     for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < ng; k += (int64_t)gridDim.x * blockDim.x) {
-        const int b = order_bucket(k, groups, begin, end, jj_off, pc_off, chunk, by_cost);
-        order[start[b] + atomicAdd(&cursor[b], 1ull)] = (int32_t)k;
+        const uint32_t ni = group_size(O, k);
+        int c = 0;
+        for (uint32_t i = 0; i < ni; i += O.chunk, ++c) {
+            const int b = order_bucket(O, k, ni, min(O.chunk, ni - i));
+            const int64_t at = (int64_t)(start[b] + atomicAdd(&cursor[b], 1ull));
+            if (at < cap) order[at] = make_int2((int)k, c);
+        }
     }
 }
 
@@ -1256,22 +1286,28 @@ int resident_blocks(Force32Fn kern, int warps) {
 
 }  // namespace
 
-// Processing order of the groups for the FP32 kernel (once per list build).
+// Work items of the FP32 kernel in processing order (once per list build).
 int build_order32(Ctx* c) {
     const int64_t ng = c->n_groups;
-    BH_TRY(grow(c, c->order, (size_t)ng + 1, "group order"));
+    const int chunk = std::min(c->tune.chunk, 32 * BH_F32_MAXR);
+    // (device-sized: sized before capture, at most one item per particle)
+    if (!c->dev_build) BH_TRY(grow(c, c->order, (size_t)(ng + c->n / chunk + 1), "work items"));
     BH_TRY(grow(c, c->order_cnt, 2 * (size_t)kOrderBuckets, "group order buckets"));
     unsigned long long* cnt = c->order_cnt.p;
-    const uint32_t chunk = (uint32_t)std::min(c->tune.chunk, 32 * BH_F32_MAXR);
-    const bool by_cost = c->tune.order_by_cost != 0;
+    unsigned long long* items = c->d_sz + kSzItems;
+    const OrderArgs O{ng,         c->dev_build ? c->d_sz + kSzNg : nullptr,
+                      c->groups.p, c->begin.p,
+                      c->end.p,    c->cnt_j.p,
+                      c->cnt_c.p,  (uint32_t)chunk,
+                      c->tune.order_by_cost != 0};
     if (c->tune.order_window > 0 && ng > c->tune.order_window && !c->dev_build) {  // (device-sized: plain order)
         for (int b = 0; b < 2; ++b) {
             BH_TRY(grow(c, c->ord_key[b], (size_t)ng, "group order keys"));
             BH_TRY(grow(c, c->ord_idx[b], (size_t)ng, "group order indices"));
         }
         BH_TRY(grow(c, c->ord_scratch, (size_t)sort_scratch_words(ng), "group order sort scratch"));
-        BH_CUDA(c, launch(c, k_order_keys, blocks_for(ng, 256), 256, 0, ng, c->groups.p, c->begin.p,
-                          c->end.p, c->cnt_j.p, c->cnt_c.p, chunk, by_cost, c->tune.order_window, c->ord_key[0].p));
+        BH_CUDA(c, launch(c, k_order_keys, blocks_for(ng, 256), 256, 0, O, c->tune.order_window,
+                          c->ord_key[0].p));
         BH_LAUNCH(c);
         if (c->sort_attr_device != c->device) {
             BH_CUDA(c, sort_setup_device());
@@ -1280,19 +1316,17 @@ int build_order32(Ctx* c) {
         BH_CUDA(c, sort_pairs_with(c->stream, c->ord_key[0].p, c->ord_idx[0].p, c->ord_key[1].p, c->ord_idx[1].p, ng,
                                    c->num_sms, c->ord_scratch.p, c->d_status));
         c->n_launches += sort_launches();
-        BH_CUDA(c, cudaMemcpyAsync(c->order.p, c->ord_idx[0].p, ng * sizeof(int32_t), cudaMemcpyDeviceToDevice,
-                                   c->stream));
+        BH_CUDA(c, launch(c, k_order_whole, blocks_for(ng, 256), 256, 0, c->ord_idx[0].p, ng, c->order.p,
+                          items));
+        BH_LAUNCH(c);
         return BH_OK;
     }
-    // device-sized build: the group count is read on the device
-    const unsigned long long* dng = c->dev_build ? c->d_sz + kSzNg : nullptr;
-    const unsigned nb = dng ? (unsigned)(4 * c->num_sms) : blocks_for(ng, 256);
+    const unsigned nb = c->dev_build ? (unsigned)(4 * c->num_sms) : blocks_for(ng, 256);
     BH_CUDA(c, cudaMemsetAsync(cnt, 0, 2 * kOrderBuckets * sizeof(unsigned long long), c->stream));
-    BH_CUDA(c, launch(c, k_order_hist, nb, 256, 0, ng, dng, c->groups.p, c->begin.p, c->end.p, c->cnt_j.p,
-                      c->cnt_c.p, chunk, by_cost, cnt));
+    BH_CUDA(c, launch(c, k_order_hist, nb, 256, 0, O, cnt));
     BH_LAUNCH(c);
-    BH_CUDA(c, launch(c, k_order_scatter, nb, 256, 0, ng, dng, c->groups.p, c->begin.p, c->end.p,
-                      c->cnt_j.p, c->cnt_c.p, chunk, by_cost, cnt, cnt + kOrderBuckets, c->order.p));
+    BH_CUDA(c, launch(c, k_order_scatter, nb, 256, 0, O, cnt, cnt + kOrderBuckets, c->order.p,
+                      (int64_t)c->order.cap, items));
     BH_LAUNCH(c);
     return BH_OK;
 }
@@ -1336,6 +1370,8 @@ int launch_force32(Ctx* c, bh_particles* p, const ForceParams& fp, bool add_cent
     A.dng = dev_groups(c);
     A.abort = c->abort;
     A.order = c->order.p;
+    A.items = c->d_sz + kSzItems;
+    A.items_cap = (int64_t)c->order.cap;
     A.groups = c->groups.p;
     A.begin = c->begin.p;
     A.end = c->end.p;
@@ -1410,11 +1446,12 @@ int launch_force32(Ctx* c, bh_particles* p, const ForceParams& fp, bool add_cent
         A.cflag = c->cflag.p;
     }
     unsigned nb;
+    const int64_t items = std::min(A.items_cap, groups_expected(c) + c->n / A.chunk + 1);  // about (a bound, eagerly)
     if (c->tune.sched == BH_SCHED_GRID && !A.dng) {
-        nb = blocks_for(A.ng, W);
+        nb = blocks_for(items, W);
     } else {  // (a device-sized build runs the grid schedule as a persistent static one)
         nb = (unsigned)(c->num_sms * resident_blocks(kern, W));
-        const int64_t need = (A.ng + W - 1) / W;
+        const int64_t need = (items + W - 1) / W;
         if ((int64_t)nb > need) nb = (unsigned)(need > 0 ? need : 1);
         if (c->tune.sched == BH_SCHED_DYNAMIC) {
             A.ticket = c->d_small + 17;
