@@ -264,9 +264,10 @@ int build_tree(Ctx* c, bh_particles* p) {
     BH_STAGE(c, BH_STAGE_SORT, stage_sort(c));
     BH_STAGE(c, BH_STAGE_PERMUTE, stage_permute(c, p));
     BH_TRY(stage_begin(c, BH_STAGE_TREE));
-    BH_TRY(stage_octree(c));
-    BH_TRY(stage_boxes(c));
+    int rc = stage_octree(c);  // (reports the keys' errors too: the stage is closed either way)
+    if (rc == BH_OK) rc = stage_boxes(c);
     BH_TRY(stage_end(c));
+    BH_TRY(rc);
     BH_TRY(stage_moments(c, p));
     BH_STAGE(c, BH_STAGE_GROUPS, BH_OK);  // (found with the octree: the stage takes no time of its own)
     c->have_tree = true;

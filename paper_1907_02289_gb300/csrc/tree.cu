@@ -41,7 +41,8 @@ __device__ __forceinline__ uint32_t compact3(uint64_t x) {
 // are loaded several at a time before any of them is used.  Measured with the
 // leaf pass below: force evaluation on kept lists of a 20,000-particle ring 124
 // -> 95 us, evaluation of a 65,537-particle ring 624 -> 540 us, 4 graph steps of
-// 64 patches 22.32 -> 22.03 ms.
+// 64 patches 22.32 -> 22.03 ms; with the next level's fixed fields loaded before
+// the barrier 89 -> 82 us, 415 -> 402 us and 21.81 -> 21.74 ms.
 constexpr int kSpanBlocks = 8, kSpanThreads = 256;
 constexpr int64_t kSpanBoxes = 4096, kSpanMoments32 = 4096, kSpanMoments64 = 256;
 
@@ -49,17 +50,26 @@ __device__ __forceinline__ void cluster_barrier() {
     asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
 }
 
-// node(k) for every node of the levels hi, hi - 1, ..., lo (first nodes in
-// lvl); hi > lo only in a one-cluster launch.
-template <class F>
-__device__ __forceinline__ void for_levels(const unsigned long long* lvl, int hi, int lo, F node) {
+// node(k, pre(k)) for every node k of the levels hi, hi - 1, ..., lo (first
+// nodes in lvl); hi > lo only in a one-cluster launch.  pre loads what does not
+// depend on the level below: the next level's while this one is waited for.
+template <class P, class F>
+__device__ __forceinline__ void for_levels(const unsigned long long* __restrict__ lvl, int hi, int lo, P pre, F node) {
     while (hi > lo && lvl[hi + 1] == lvl[hi]) --hi;  // (empty levels, below the tree's depth)
+    const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, stride = (int64_t)gridDim.x * blockDim.x;
+    int64_t ls = (int64_t)lvl[hi], le = (int64_t)lvl[hi + 1], k = ls + tid;
+    auto q = pre(min(k, le - 1));
     for (int lev = hi;; --lev) {
-        const int64_t le = (int64_t)lvl[lev + 1];
-        for (int64_t k = (int64_t)lvl[lev] + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < le;
-             k += (int64_t)gridDim.x * blockDim.x)
-            node(k);
+        while (k < le) {
+            node(k, q);
+            k += stride;
+            if (k < le) q = pre(k);
+        }
         if (lev == lo) break;
+        le = ls;
+        ls = (int64_t)lvl[lev - 1];
+        k = ls + tid;
+        q = pre(min(k, le - 1));
         cluster_barrier();
     }
 }
@@ -400,13 +410,22 @@ __global__ void __launch_bounds__(kSpanThreads) k_boxes(
     const uint8_t* __restrict__ nchild, const int32_t* __restrict__ top, uint32_t* qlo, uint32_t* qhi,
     WalkNode* wnode, const unsigned long long* __restrict__ lvl, int lev_hi, int lev_lo) {
     launch_wait();
-    for_levels(lvl, lev_hi, lev_lo, [&](int64_t k) {
-        const uint32_t e = end[k];
-        const int32_t skip = skip_of(e, n, np, top);
+    struct Pre {
+        uint32_t b, e;
+        int32_t f, skip;
+        int nc, lev;
+    };
+    auto pre = [&](int64_t k) {
+        Pre v{begin[k], end[k], first_child[k], 0, nchild[k], level[k]};
+        v.skip = skip_of(v.e, n, np, top);
+        return v;
+    };
+    for_levels(lvl, lev_hi, lev_lo, pre, [&](int64_t k, const Pre& v) {
+        const uint32_t b = v.b, e = v.e;
         uint32_t lo[3] = {kQMax, kQMax, kQMax}, hi[3] = {0, 0, 0};
-        const int nc = nchild[k];
+        const int nc = v.nc;
         if (nc == 0) {
-            for (uint32_t p = begin[k]; p < e; p += 8) {
+            for (uint32_t p = b; p < e; p += 8) {
                 uint64_t kk[8];
 #pragma unroll
                 for (int u = 0; u < 8; ++u) kk[u] = key[min(p + u, e - 1u)];  // (a repeated key changes nothing)
@@ -421,7 +440,7 @@ __global__ void __launch_bounds__(kSpanThreads) k_boxes(
                 }
             }
         } else {
-            const int64_t f = first_child[k];
+            const int64_t f = v.f;
             uint32_t cl[8][3], ch[8][3];
 #pragma unroll
             for (int c = 0; c < 8; ++c)
@@ -447,11 +466,11 @@ __global__ void __launch_bounds__(kSpanThreads) k_boxes(
         WalkNode w;
         // a leaf carries its first particle and (up to kWalkCntMax - 1) its
         // particle count instead of a first child and the child count
-        const uint32_t cnt = nc == 0 ? min(e - begin[k], kWalkCntMax) : (uint32_t)nc;
-        w.a = make_uint4(lo[0] | ((uint32_t)level[k] << kLevels) | (nc == 0 ? kWalkLeaf : 0u),
+        const uint32_t cnt = nc == 0 ? min(e - b, kWalkCntMax) : (uint32_t)nc;
+        w.a = make_uint4(lo[0] | ((uint32_t)v.lev << kLevels) | (nc == 0 ? kWalkLeaf : 0u),
                          lo[1] | (cnt << kLevels), lo[2],
-                         (uint32_t)skip);
-        w.b = make_uint4(hi[0], hi[1], hi[2], nc == 0 ? begin[k] : (uint32_t)first_child[k]);
+                         (uint32_t)v.skip);
+        w.b = make_uint4(hi[0], hi[1], hi[2], nc == 0 ? b : (uint32_t)v.f);
         wnode[k] = w;
     });
 }
@@ -464,12 +483,18 @@ __global__ void __launch_bounds__(kSpanThreads) k_moments(
     const double* __restrict__ z, const double* __restrict__ m, double* M, double* cx, double* cy, double* cz,
     double* Q, const unsigned long long* __restrict__ lvl, int lev_hi, int lev_lo) {
     launch_wait();
-    for_levels(lvl, lev_hi, lev_lo, [&](int64_t k) {
-        const int nc = nchild[k];
+    struct Pre {
+        uint32_t b, e;
+        int32_t f;
+        int nc;
+    };
+    auto pre = [&](int64_t k) { return Pre{begin[k], end[k], first_child[k], nchild[k]}; };
+    for_levels(lvl, lev_hi, lev_lo, pre, [&](int64_t k, const Pre& v) {
+        const int nc = v.nc;
         double Mk = 0.0, sx = 0.0, sy = 0.0, sz = 0.0, c0, c1, c2;
         double q[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
         if (nc == 0) {
-            const uint32_t b = begin[k], e = end[k];
+            const uint32_t b = v.b, e = v.e;
             double px[8], py[8], pz[8], pm[8];
             uint32_t have = b;
             auto load = [&](uint32_t p) {
@@ -527,7 +552,7 @@ __global__ void __launch_bounds__(kSpanThreads) k_moments(
                         }
                 }
         } else {
-            const int64_t f = first_child[k];
+            const int64_t f = v.f;
             for (int c = 0; c < nc; ++c) {
                 const double Mc = M[f + c];
                 Mk = __dadd_rn(Mk, Mc);
@@ -689,10 +714,15 @@ __global__ void __launch_bounds__(kSpanThreads) k_moments32(
     const int32_t* __restrict__ first_child, const uint8_t* __restrict__ nchild, float4* cell32, float* mlo,
     const unsigned long long* __restrict__ lvl, int lev_hi, int lev_lo) {
     launch_wait();
-    for_levels(lvl, lev_hi, lev_lo, [&](int64_t k) {
-        const int nc = nchild[k];
+    struct Pre {
+        int32_t f;
+        int nc;
+    };
+    auto pre = [&](int64_t k) { return Pre{first_child[k], nchild[k]}; };
+    for_levels(lvl, lev_hi, lev_lo, pre, [&](int64_t k, const Pre& v) {
+        const int nc = v.nc;
         if (nc == 0) return;
-        const int64_t f = first_child[k];
+        const int64_t f = v.f;
         float4 H[4], L[4], U[4];
         float ml[4];
         auto load = [&](int c0) {  // children c0..c0 + 3 (the last one again past the end)
@@ -731,17 +761,17 @@ __global__ void __launch_bounds__(kSpanThreads) k_moments32(
 #pragma unroll
                 for (int u = 0; u < 4; ++u)
                     if (c0 + u < nc) {
-                        const float4 h = H[u], l = L[u], v = U[u];
+                        const float4 h = H[u], l = L[u], t = U[u];
                         const float D[3] = {dsub(h.x, l.x, rh[0], rl[0]) - dc[0], dsub(h.y, l.y, rh[1], rl[1]) - dc[1],
                                             dsub(h.z, l.z, rh[2], rl[2]) - dc[2]};
                         const float D2 = fmaf(D[0], D[0], fmaf(D[1], D[1], D[2] * D[2]));
                         const float Mc = h.w, m3 = 3.f * Mc;
                         q[0] += l.w + Mc * fmaf(3.f * D[0], D[0], -D2);
-                        q[1] += v.z + Mc * fmaf(3.f * D[1], D[1], -D2);
-                        q[2] += -(l.w + v.z) + Mc * fmaf(3.f * D[2], D[2], -D2);
-                        q[3] += v.x + m3 * D[0] * D[1];
-                        q[4] += v.y + m3 * D[0] * D[2];
-                        q[5] += v.w + m3 * D[1] * D[2];
+                        q[1] += t.z + Mc * fmaf(3.f * D[1], D[1], -D2);
+                        q[2] += -(l.w + t.z) + Mc * fmaf(3.f * D[2], D[2], -D2);
+                        q[3] += t.x + m3 * D[0] * D[1];
+                        q[4] += t.y + m3 * D[0] * D[2];
+                        q[5] += t.w + m3 * D[1] * D[2];
                     }
             }
         put_moments32(k, Mk, Md, rh, rl, dc, q, cell32, mlo);
