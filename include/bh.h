@@ -23,7 +23,8 @@
  *    the context; they are allocated with cudaMalloc and grown on demand.
  *  - Work is issued on the CUDA stream given to bh_create.  Calls that must
  *    size buffers (building trees and lists) synchronise that stream; force
- *    and step calls do not, except where stated.  Device-side error words are
+ *    and step calls do not, except where stated (on the FP32 path with
+ *    contacts an eager evaluation waits for its contact count).  Device-side error words are
  *    checked at the next synchronising call (or bh_sync).
  *  - bh_get_* read-back functions copy into CALLER-OWNED HOST buffers sized
  *    from bh_get_sizes, and synchronise the stream.
@@ -126,11 +127,12 @@ typedef struct {
  *  KEYS      cylindrical coordinates (key_frame 1), root box, Morton keys   (a1)
  *  SORT      stable radix sort of (key, index)                              (a2)
  *  PERMUTE   gather of the particle arrays into key order                   (a2)
- *  TREE      octree levels, integer node boxes and walk records             (a3)
- *  MOMENTS   node moments (every evaluation)                                (a4)
- *  GROUPS    groups                                                         (a5)
+ *  TREE      octree and groups, integer node boxes and walk records    (a3, a5)
+ *  MOMENTS   node moments (every evaluation; FP32 path: the inner nodes)    (a4)
+ *  GROUPS    found with the octree: timed, but no work of its own           (a5)
  *  LISTS     tree walk, list expansion and the FP32 kernel's group order (a6, a7)
- *  SPLIT     FP32 path: hi/lo split of the particles (every evaluation)
+ *  SPLIT     FP32 path: hi/lo split of the particles and the leaves' moments
+ *            (every evaluation)
  *  FORCE     force kernel                                                   (a8)
  *  CONTACTS  FP32 path: the FP64 contact pass after the force kernel        (a8)
  *  UPDATE    leapfrog kicks and drift                                       (a9)
@@ -303,15 +305,16 @@ int bh_get_timing(bh_ctx* ctx, double* force_ms, int64_t* force_launches, int re
 
 /* Launch tuning (the persistent-kernel schedule of Sec. 4.6's load balance,
  * and the knobs the autotuner searches).  Schedules of the FP32 force kernel:
- *  BH_SCHED_GRID     one warp per group, grid sized to the groups;
+ *  BH_SCHED_GRID     one warp per work item, grid sized to the items;
  *  BH_SCHED_STATIC   persistent grid (as many blocks as fit on the GPU), each
- *                    warp takes every (warps in grid)-th group of the order;
- *  BH_SCHED_DYNAMIC  persistent grid, each warp draws its next group from an
+ *                    warp takes every (warps in grid)-th item of the order;
+ *  BH_SCHED_DYNAMIC  persistent grid, each warp draws its next item from an
  *                    atomic ticket counter (dynamic longest-first when
  *                    order_by_cost is set).
- * Groups are taken in order of size class, and, with order_by_cost, by
- * decreasing estimated cost n_i (n_i + list particles + 2 list cells) within
- * a class. */
+ * A work item is an i-chunk of a group (a whole group with order_window).
+ * Items are taken in order of size class, and, with order_by_cost, by
+ * decreasing estimated cost n (n_i + list particles + 2 list cells) within a
+ * class (n: the chunk's particles, n_i: its group's). */
 #define BH_SCHED_GRID 0
 #define BH_SCHED_STATIC 1
 #define BH_SCHED_DYNAMIC 2
