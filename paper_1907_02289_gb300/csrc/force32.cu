@@ -71,12 +71,6 @@ namespace {
 #ifndef BH_F32_MAXW
 #define BH_F32_MAXW 8  // most warps per block (the register budget is sized for 2 such blocks per SM)
 #endif
-#ifndef BH_F32_UNROLL
-#define BH_F32_UNROLL 1  // list pairs per iteration of the particle loop
-#endif
-#ifndef BH_F32_PCUNROLL
-#define BH_F32_PCUNROLL 1  // list pairs per iteration of the cell loop
-#endif
 #ifndef BH_F32_MAXR
 #define BH_F32_MAXR 3  // most full i-slots per lane (chunks of up to 32 x this particles)
 #endif
@@ -92,7 +86,15 @@ namespace {
 constexpr int kTileJ = 64 * BH_F32_TILE;  // list particles per tile (2 per lane per 64)
 constexpr int kTileC = 32 * BH_F32_TILE;  // list cells per tile (1 per lane per 32)
 constexpr int kSlots = 3;                 // i-slots per lane (full slots + tail)
-constexpr int kUnrollPP = BH_F32_UNROLL, kUnrollPC = BH_F32_PCUNROLL;
+// List pairs per iteration of the far-particle and cell loops.  A chunk with
+// one full slot has one chain dx -> r^2 -> rsqrt -> f -> g per lane and
+// iteration, so two list pairs run side by side (groups of 33 to 63: the
+// 100,003-particle cube's evaluation 623 -> 595 us, the 64 patches' four
+// steps 21.71 -> 21.35 ms).  With two and three slots the slots are the
+// independent chains and a second copy of the body costs instruction
+// fetches: two pairs at R <= 2 give -0.4% on the 2^26 ring but +0.4% on the
+// 2^24 one, four pairs at R = 1 +3.5% on the patches.
+__host__ __device__ constexpr int list_unroll(int R) { return R == 1 ? 2 : 1; }
 constexpr int kQueueCap = 32 + 2 * kSlots * 32;
 constexpr uint32_t kNone = 0xffffffffu;
 
@@ -503,7 +505,7 @@ __device__ __forceinline__ void pp_tile(const Args& A, Smem32& S, Chunk<R, TAIL>
                                         int& qn, int lane) {
     if constexpr (R > 0) {
         uint32_t hit = 0;
-#pragma unroll kUnrollPP
+#pragma unroll 1
         for (int q = 0; q < npair; ++q) {
             const JPair P = S.t.p.jp[q];
             const uint32_t* jid = &S.t.p.jid[2 * q];
@@ -554,7 +556,7 @@ template <int R, bool TAIL>
 __device__ __forceinline__ void pp_far_tile(const Args& A, Smem32& S, Chunk<R, TAIL>& K, int npair, int J, int tj) {
     const float2 eps2 = f2(A.fp.eps2f);
     if constexpr (R > 0)
-#pragma unroll kUnrollPP
+#pragma unroll list_unroll(R)
         for (int q = 0; q < npair; ++q) {
             const JPair& P = S.t.p.jp[q];
 #pragma unroll
@@ -569,7 +571,7 @@ template <int R, bool TAIL, int ORDER>
 __device__ __forceinline__ void pc_tile(const Args& A, Smem32& S, Chunk<R, TAIL>& K, int npair, int J, int tj) {
     const float2 eps2 = f2(A.fp.eps2f);
     if constexpr (R > 0)
-#pragma unroll kUnrollPC
+#pragma unroll list_unroll(R)
         for (int q = 0; q < npair; ++q) {
             const CPair& Cp = S.t.cp[q];
 #pragma unroll

@@ -1,0 +1,31 @@
+"""The FP32 force kernel's list loops at the sizes that pick their variants:
+chunks of 1 to 3 slots with and without a tail and odd counts of list pairs.
+Tolerance: the FP32 gate, 1e-5 (each term rounds by a few units of 6e-8)."""
+import pytest
+
+import oracle as orc
+from paper_1907_02289_gb300 import synth
+from _common import accel_of, assert_force_close, gpu_build, orc_params
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import __graft_entry__
+    __graft_entry__.build()
+
+
+def check(P, prm):
+    op = orc_params(prm)
+    ctx, D = gpu_build(P, prm, precision=1)
+    assert_force_close(accel_of(D), orc.tree_forces(orc.rebuild(P, op), op), 1e-5)
+    ctx.close()
+
+
+@pytest.mark.parametrize("n_g", [8, 31, 32, 33, 47, 48, 63, 64, 95, 97, 130])
+def test_chunk_sizes(n_g):
+    check(synth.uniform_cube(3001, n_g), dict(synth.PRESETS["cube4k"]["params"], n_g=n_g, theta=0.6))
