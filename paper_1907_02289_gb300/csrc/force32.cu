@@ -108,8 +108,8 @@ __host__ __device__ constexpr bool has_contact(int mode) { return mode == kConta
 struct __align__(16) JPair {  // two list particles relative to the origin (hi/lo)
     float2 x, y, z, m, xl, yl, zl, pad;
 };
-struct CPair {  // two cells: centre relative to the origin, mass, negated quadrupole
-    float2 x, y, z, m, qxx, qxy, qxz, qyy, qyz, qzz;
+struct CPair {  // two cells: centre relative to the origin, mass, -3/2 Nxx, N - Nxx I (see pc_body)
+    float2 x, y, z, m, e, qxy, qxz, qyy, qyz, qzz;
 };
 
 struct Smem32 {
@@ -331,7 +331,22 @@ __device__ __forceinline__ void pp_far_body(const JPair& P, const float2 (&nh)[3
     g[2] = __ffma2_rn(f, dz, g[2]);
 }
 
-template <int ORDER>
+// Cell term of one pair of list cells for one slot (G-free).  The
+// quadrupole is N = -Q (Q traceless), and only its action on d is needed:
+// N d = (N - Nxx I) d + Nxx d, so the kernel keeps N - Nxx I, whose xx entry
+// is 0, and the part along d joins the monopole's coefficient of d:
+//   (M R^2 - 5/2 d.N d / R^2) d + N d
+//     = (M R^2 - 3/2 Nxx - 5/2 (d.q - Nxx eps^2) / R^2) d + q,  q = (N - Nxx I) d
+// with R^2 = d.d + eps^2; all of it over R^5.  29 FMA-pipe operations per
+// pair without softening (30 with it, and 30 for N d as it stands): four
+// steps of the 2^24 ring 66.04 -> 65.07 ms, of the 2^26 ring 518.0 -> 512.2,
+// of the 64 patches 21.35 -> 21.19.  Of the
+// three axes x is taken because a ring lies across z: its cells are flat
+// discs with Nxx ~ Nyy, so taking Nxx out leaves little of the matrix
+// (rounding error of the term against 64 bits, 4e5 random cells each at
+// theta 0.5: cubic cells 1.532e-7 rms before and after, discs across z
+// 1.523e-7 -> 1.517e-7; taking Nzz out would give 1.540e-7).
+template <int ORDER, bool EPS>
 __device__ __forceinline__ void pc_body(const CPair& Cp, const float2 (&nh)[3], float2 (&g)[3], float2 eps2) {
     const float2 dx = __fadd2_rn(Cp.x, nh[0]);
     const float2 dy = __fadd2_rn(Cp.y, nh[1]);
@@ -341,14 +356,14 @@ __device__ __forceinline__ void pc_body(const CPair& Cp, const float2 (&nh)[3], 
     const float2 ri2 = __fmul2_rn(ri, ri);
     const float2 ri3 = __fmul2_rn(ri, ri2);
     if (ORDER >= 2) {
-        // q = -Q d, dqd = d.(-Q d); a += (M R^2 - 5/2 dqd / R^2) d / R^5 + q / R^5
-        const float2 qx = __ffma2_rn(Cp.qxx, dx, __ffma2_rn(Cp.qxy, dy, __fmul2_rn(Cp.qxz, dz)));
+        const float2 qx = __ffma2_rn(Cp.qxy, dy, __fmul2_rn(Cp.qxz, dz));
         const float2 qy = __ffma2_rn(Cp.qxy, dx, __ffma2_rn(Cp.qyy, dy, __fmul2_rn(Cp.qyz, dz)));
         const float2 qz = __ffma2_rn(Cp.qxz, dx, __ffma2_rn(Cp.qyz, dy, __fmul2_rn(Cp.qzz, dz)));
-        const float2 dqd = __ffma2_rn(dx, qx, __ffma2_rn(dy, qy, __fmul2_rn(dz, qz)));
+        float2 dqd = __ffma2_rn(dx, qx, __ffma2_rn(dy, qy, __fmul2_rn(dz, qz)));
+        if (EPS) dqd = __ffma2_rn(Cp.e, __fmul2_rn(eps2, f2(2.f / 3.f)), dqd);
         const float2 ri4 = __fmul2_rn(ri2, ri2);
         const float2 ri5 = __fmul2_rn(ri4, ri);
-        const float2 s = __ffma2_rn(__fmul2_rn(dqd, ri2), f2(-2.5f), __fmul2_rn(Cp.m, R2));
+        const float2 s = __ffma2_rn(__fmul2_rn(dqd, ri2), f2(-2.5f), __ffma2_rn(Cp.m, R2, Cp.e));
         g[0] = __ffma2_rn(ri5, __ffma2_rn(s, dx, qx), g[0]);
         g[1] = __ffma2_rn(ri5, __ffma2_rn(s, dy, qy), g[1]);
         g[2] = __ffma2_rn(ri5, __ffma2_rn(s, dz, qz), g[2]);
@@ -475,13 +490,13 @@ __device__ __forceinline__ void put_cell(Smem32& S, int u, bool real, const floa
         v[1] = rel(r0.y, r1.y, oh[1], ol[1]);
         v[2] = rel(r0.z, r1.z, oh[2], ol[2]);
         v[3] = r0.w;
-        if (ORDER >= 2) {  // stored negated; Qzz = -(Qxx + Qyy)
-            v[4] = -r1.w;
+        if (ORDER >= 2) {  // N = -Q, Qzz = -(Qxx + Qyy)
+            v[4] = 1.5f * r1.w;
             v[5] = -r2v.x;
             v[6] = -r2v.y;
-            v[7] = -r2v.z;
+            v[7] = r1.w - r2v.z;
             v[8] = -r2v.w;
-            v[9] = r1.w + r2v.z;
+            v[9] = __fadd_rn(__fadd_rn(r1.w, r2v.z), r1.w);
         }
     } else {  // padding entry: far away, massless
         v[0] = v[1] = v[2] = 1e15f;
@@ -567,7 +582,7 @@ __device__ __forceinline__ void pp_far_tile(const Args& A, Smem32& S, Chunk<R, T
         for (int q = tj; q < npair; q += J) pp_far_body(S.t.p.jp[q], K.nh[R], K.g[R], eps2);
 }
 
-template <int R, bool TAIL, int ORDER>
+template <int R, bool TAIL, int ORDER, bool EPS>
 __device__ __forceinline__ void pc_tile(const Args& A, Smem32& S, Chunk<R, TAIL>& K, int npair, int J, int tj) {
     const float2 eps2 = f2(A.fp.eps2f);
     if constexpr (R > 0)
@@ -575,11 +590,11 @@ __device__ __forceinline__ void pc_tile(const Args& A, Smem32& S, Chunk<R, TAIL>
         for (int q = 0; q < npair; ++q) {
             const CPair& Cp = S.t.cp[q];
 #pragma unroll
-            for (int r = 0; r < R; ++r) pc_body<ORDER>(Cp, K.nh[r], K.g[r], eps2);
+            for (int r = 0; r < R; ++r) pc_body<ORDER, EPS>(Cp, K.nh[r], K.g[r], eps2);
         }
     if constexpr (TAIL)
 #pragma unroll 1
-        for (int q = tj; q < npair; q += J) pc_body<ORDER>(S.t.cp[q], K.nh[R], K.g[R], eps2);
+        for (int q = tj; q < npair; q += J) pc_body<ORDER, EPS>(S.t.cp[q], K.nh[R], K.g[R], eps2);
 }
 
 template <int MODE, int R, bool TAIL, int ORDER>
@@ -719,7 +734,7 @@ __device__ __forceinline__ void group_chunk(const Args& A, Smem32& S, int64_t k,
                 cb[s] = cell_index(A, t0 + 2 * kTileC + lane + 32 * s, c1);
             }
             cp_async_commit();
-            pc_tile<R, TAIL, ORDER>(A, S, K, npair, J, tj);
+            pc_tile<R, TAIL, ORDER, MODE == kContact || MODE == kPlain>(A, S, K, npair, J, tj);
             fold_all<R, TAIL>(S, K, lane);
             __syncwarp();
         }

@@ -1,6 +1,10 @@
 """The FP32 force kernel's list loops at the sizes that pick their variants:
-chunks of 1 to 3 slots with and without a tail and odd counts of list pairs.
-Tolerance: the FP32 gate, 1e-5 (each term rounds by a few units of 6e-8)."""
+chunks of 1 to 3 slots with and without a tail, odd counts of list pairs,
+and cells flat along each axis (the kernel takes the quadrupole's xx entry
+out of the matrix), with and without softening.  Tolerance: the FP32 gate,
+1e-5 (rounding of ~30 units of 6e-8 per term, ~1e-6 of a sum of ~1e3 terms;
+the quadrupole terms are 1e-3 to 1e-2 of the pull, so that a wrong entry is
+100 times the gate)."""
 import pytest
 
 import oracle as orc
@@ -28,4 +32,12 @@ def check(P, prm):
 
 @pytest.mark.parametrize("n_g", [8, 31, 32, 33, 47, 48, 63, 64, 95, 97, 130])
 def test_chunk_sizes(n_g):
-    check(synth.uniform_cube(3001, n_g), dict(synth.PRESETS["cube4k"]["params"], n_g=n_g, theta=0.6))
+    check(synth.uniform_cube(3001, n_g), dict(synth.PRESETS["cube4k"]["params"], order=2, n_g=n_g, theta=0.6))
+
+
+@pytest.mark.parametrize("axis", ["x", "y", "z"])
+@pytest.mark.parametrize("eps", [0.0, 0.05])
+def test_flat_cells(axis, eps):
+    P = synth.uniform_cube(4000, 11)
+    P[axis] = 0.5 + 0.02 * (P[axis] - 0.5)
+    check(P, dict(synth.PRESETS["cube4k"]["params"], order=2, eps=eps, n_g=48, theta=0.8))
