@@ -311,7 +311,7 @@ int bh_get_timing(bh_ctx* ctx, double* force_ms, int64_t* force_launches, int re
  *  BH_SCHED_DYNAMIC  persistent grid, each warp draws its next item from an
  *                    atomic ticket counter (dynamic longest-first when
  *                    order_by_cost is set).
- * A work item is an i-chunk of a group (a whole group with order_window).
+ * A work item is an i-chunk of a group.
  * Items are taken in order of size class, and, with order_by_cost, by
  * decreasing estimated cost n (n_i + list particles + 2 list cells) within a
  * class (n: the chunk's particles, n_i: its group's). */
@@ -346,8 +346,9 @@ typedef struct {
                           synchronising call */
     int order_window;  /* 0: one global size-class order; w > 0: the size-class
                           order is applied within windows of w consecutive
-                          groups (list order = Morton order), so the warps in
-                          flight work on nearby groups whose list data share L2 */
+                          groups (w below 64: 64; list order = Morton order),
+                          so the warps in flight work on nearby groups whose
+                          list data share L2 */
     int graph_contact_room; /* contact candidates a graph step may hold: 0 = twice
                           the last eager evaluation's count + 65536; n > 0 = n.
                           More candidates than that in a graph step are

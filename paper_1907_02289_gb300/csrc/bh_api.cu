@@ -1014,11 +1014,7 @@ int bh_destroy(bh_ctx* ctx) {
     if (c->count_event) cudaEventDestroy(c->count_event);
     using bh::release;
     release(c->d_off); release(c->tile_meta); release(c->box_map); release(c->box_poff); release(c->d_rcq); release(c->d_rfar); release(c->d_period); release(c->cyl); release(c->box_part); release(c->order_cnt); release(c->warp_time); release(c->contact_acc); release(c->diag); release(c->pot);
-    for (int b = 0; b < 2; ++b) {
-        release(c->ord_key[b]);
-        release(c->ord_idx[b]);
-    }
-    release(c->ord_scratch);
+    release(c->ord_cnt);
     for (int b = 0; b < 2; ++b) {
         release(c->key[b]);
         release(c->idx[b]);

@@ -181,9 +181,7 @@ struct Ctx {
     DBuf<int32_t> leaves;            // node ids ordered by begin
     DBuf<int2> order;                // FP32 force kernel's work items (group, i-chunk) in processing order
     DBuf<unsigned long long> order_cnt;  // order buckets: counts/starts and cursors
-    DBuf<uint64_t> ord_key[2];           // windowed order: sort keys
-    DBuf<uint32_t> ord_idx[2];
-    DBuf<uint32_t> ord_scratch;
+    DBuf<uint32_t> ord_cnt;              // windowed order: bucket counts, then cursors, per window
     int sort_attr_device = -1;           // device the sort kernel's smem limit was raised on
     int f32_attr_device = -1;            // device the FP32 kernels' smem limit was raised on
     unsigned f32_blocks = 0;             // grid of the last FP32 force launch

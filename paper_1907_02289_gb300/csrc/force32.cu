@@ -54,7 +54,7 @@
 //
 // Scheduling: chunks are taken in order of size class (warps running side
 // by side execute the same code), by decreasing estimated cost within a
-// class, optionally whole groups within windows of consecutive groups; the
+// class, optionally within windows of consecutive groups; the
 // grid is one warp per item, or persistent (resident blocks only) with warps
 // taking items round robin or from an atomic ticket counter.  Warps per block and
 // the i-chunk are runtime settings; the compile-time options below exist for
@@ -138,7 +138,7 @@ struct Args {
     int64_t ng;
     const unsigned long long* dng;  // device group count (device-sized list builds; NULL: ng)
     const unsigned long long* abort;  // device-sized build: nonzero overflow bits skip the launch
-    const int2* order;     // work items in processing order: (group, i-chunk, or -1: every chunk)
+    const int2* order;     // work items in processing order: (group, i-chunk)
     const unsigned long long* items;  // their count (device)
     int64_t items_cap;     // and its bound
     const int32_t* groups;
@@ -798,10 +798,9 @@ __device__ __forceinline__ void force_item(const Args& A, Smem32& S, int64_t slo
     const float4 o0 = A.cell32[3 * (int64_t)g], o1 = A.cell32[3 * (int64_t)g + 1];
     const float oh[3] = {o0.x, o0.y, o0.z}, ol[3] = {o1.x, o1.y, o1.z};
     // chunks of at most A.chunk particles: R full slots plus a tail of at most 16
-    const uint32_t first = o.y < 0 ? b : b + (uint32_t)o.y * (uint32_t)A.chunk;
-    const uint32_t last = o.y < 0 ? e : min(e, first + (uint32_t)A.chunk);
-    for (uint32_t i0 = first; i0 < last;) {
-        const uint32_t rem = last - i0, cnt = min(rem, (uint32_t)A.chunk);
+    const uint32_t i0 = b + (uint32_t)o.y * (uint32_t)A.chunk;
+    {
+        const uint32_t cnt = min(e - i0, (uint32_t)A.chunk);
         int R = (int)(cnt >> 5), t = (int)(cnt & 31), T = 0;
         if (t > 16) {
             ++R;  // more than half a slot left: a full one
@@ -823,7 +822,6 @@ __device__ __forceinline__ void force_item(const Args& A, Smem32& S, int64_t slo
                 default: group_chunk<MODE, BH_F32_MAXR, false, ORDER>(A, S, k, b, e, i0, ce, 0, oh, ol, lane); break;
             }
         }
-        i0 += cnt;
     }
 }
 
@@ -883,6 +881,7 @@ __device__ __forceinline__ int size_class(uint32_t cnt) {
 // 4.70 ms, 4 graph steps of a 300,007-particle ring 1449 -> 1430 us.
 constexpr int kCostBuckets = 32;
 constexpr int kOrderBuckets = 6 * kCostBuckets;
+constexpr int64_t kLeastWindow = 64;  // smaller windows are rounded up: 3 bucket words per group at most
 
 struct OrderArgs {
     int64_t ng;
@@ -892,6 +891,7 @@ struct OrderArgs {
     const int64_t *jj_off, *pc_off;
     uint32_t chunk;
     bool by_cost;
+    int64_t window;  // groups per window (0: one order over all)
 };
 
 __device__ __forceinline__ uint32_t group_size(const OrderArgs& O, int64_t k) {
@@ -912,6 +912,37 @@ __device__ __forceinline__ int order_bucket(const OrderArgs& O, int64_t k, uint3
     return size_class(cnt) * kCostBuckets + cb;
 }
 
+// Windowed order: every window of consecutive groups (list order is Morton
+// order) has buckets of its own, so the warps running at one time work on one
+// stretch of the ring (their list data overlaps in L2) while the warps side by
+// side still share a size class.  The items are i-chunks, as in the plain
+// order; with whole groups sorted by a key (window, bucket) a step of the 2^26
+// ring took 145.7 ms at groups of up to 192 and windows of 8192, now 131.1
+// (plain order 131.3; groups of up to 128 with chunks of 64: 136.9, plain 139.4).
+// Windows below a few thousand groups put several size classes side by side
+// and lose more than the L2 gives: 530 -> 686 ms for four steps at 1024.
+__global__ void k_order_hist_windows(const OrderArgs O, uint32_t* cnt) {
+    launch_wait();
+    const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= O.ng) return;
+    uint32_t* mine = cnt + (k / O.window) * kOrderBuckets;
+    const uint32_t ni = group_size(O, k);
+    for (uint32_t i = 0; i < ni; i += O.chunk) atomicAdd(&mine[order_bucket(O, k, ni, min(O.chunk, ni - i))], 1u);
+}
+
+__global__ void k_order_scatter_windows(const OrderArgs O, uint32_t* cursor, int2* __restrict__ order, int64_t cap) {
+    launch_wait();
+    const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= O.ng) return;
+    uint32_t* mine = cursor + (k / O.window) * kOrderBuckets;
+    const uint32_t ni = group_size(O, k);
+    int c = 0;
+    for (uint32_t i = 0; i < ni; i += O.chunk, ++c) {
+        const int64_t at = atomicAdd(&mine[order_bucket(O, k, ni, min(O.chunk, ni - i))], 1u);
+        if (at < cap) order[at] = make_int2((int)k, c);
+    }
+}
+
 __global__ void k_order_hist(const OrderArgs O, unsigned long long* cnt) {
     launch_wait();
     const int64_t ng = O.dng ? min(O.ng, (int64_t)*O.dng) : O.ng;
@@ -920,27 +951,6 @@ __global__ void k_order_hist(const OrderArgs O, unsigned long long* cnt) {
         for (uint32_t i = 0; i < ni; i += O.chunk)
             atomicAdd(&cnt[order_bucket(O, k, ni, min(O.chunk, ni - i))], 1ull);
     }
-}
-
-// Windowed order: key = (group index / window, bucket of the last chunk); a
-// stable sort of the keys keeps list (Morton) order within a window and a
-// bucket, so the warps running at one time work on one stretch of the ring
-// (their list data overlaps in L2) while the warps side by side still share a
-// size class.  One item per group, all its chunks.
-__global__ void k_order_keys(const OrderArgs O, int64_t window, uint64_t* __restrict__ keys) {
-    launch_wait();
-    const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= O.ng) return;
-    const uint32_t ni = group_size(O, k), last = ni - O.chunk * ((ni - 1u) / O.chunk);
-    keys[k] = ((uint64_t)(k / window) << 8) | (uint64_t)order_bucket(O, k, ni, last);
-}
-
-__global__ void k_order_whole(const uint32_t* __restrict__ idx, int64_t ng, int2* __restrict__ order,
-                              unsigned long long* items) {
-    launch_wait();
-    const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k == 0) *items = (unsigned long long)ng;
-    if (k < ng) order[k] = make_int2((int)idx[k], -1);
 }
 
 __global__ void k_order_scatter(const OrderArgs O, const unsigned long long* __restrict__ cnt,
@@ -1316,25 +1326,17 @@ int build_order32(Ctx* c) {
                       c->groups.p, c->begin.p,
                       c->end.p,    c->cnt_j.p,
                       c->cnt_c.p,  (uint32_t)chunk,
-                      c->tune.order_by_cost != 0};
+                      c->tune.order_by_cost != 0,
+                      std::max<int64_t>(c->tune.order_window, kLeastWindow)};
     if (c->tune.order_window > 0 && ng > c->tune.order_window && !c->dev_build) {  // (device-sized: plain order)
-        for (int b = 0; b < 2; ++b) {
-            BH_TRY(grow(c, c->ord_key[b], (size_t)ng, "group order keys"));
-            BH_TRY(grow(c, c->ord_idx[b], (size_t)ng, "group order indices"));
-        }
-        BH_TRY(grow(c, c->ord_scratch, (size_t)sort_scratch_words(ng), "group order sort scratch"));
-        BH_CUDA(c, launch(c, k_order_keys, blocks_for(ng, 256), 256, 0, O, c->tune.order_window,
-                          c->ord_key[0].p));
+        const int64_t words = (ng + O.window - 1) / O.window * kOrderBuckets;
+        BH_TRY(grow(c, c->ord_cnt, (size_t)words, "group order buckets of the windows"));
+        BH_CUDA(c, cudaMemsetAsync(c->ord_cnt.p, 0, (size_t)words * sizeof(uint32_t), c->stream));
+        BH_CUDA(c, launch(c, k_order_hist_windows, blocks_for(ng, 256), 256, 0, O, c->ord_cnt.p));
         BH_LAUNCH(c);
-        if (c->sort_attr_device != c->device) {
-            BH_CUDA(c, sort_setup_device());
-            c->sort_attr_device = c->device;
-        }
-        BH_CUDA(c, sort_pairs_with(c->stream, c->ord_key[0].p, c->ord_idx[0].p, c->ord_key[1].p, c->ord_idx[1].p, ng,
-                                   c->num_sms, c->ord_scratch.p, c->d_status));
-        c->n_launches += sort_launches();
-        BH_CUDA(c, launch(c, k_order_whole, blocks_for(ng, 256), 256, 0, c->ord_idx[0].p, ng, c->order.p,
-                          items));
+        BH_TRY(scan_u32(c, c->ord_cnt.p, words, items));
+        BH_CUDA(c, launch(c, k_order_scatter_windows, blocks_for(ng, 256), 256, 0, O, c->ord_cnt.p, c->order.p,
+                          (int64_t)c->order.cap));
         BH_LAUNCH(c);
         return BH_OK;
     }

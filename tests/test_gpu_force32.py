@@ -1,10 +1,12 @@
 """The FP32 force kernel's list loops at the sizes that pick their variants:
 chunks of 1 to 3 slots with and without a tail, odd counts of list pairs,
-and cells flat along each axis (the kernel takes the quadrupole's xx entry
-out of the matrix), with and without softening.  Tolerance: the FP32 gate,
+cells flat along each axis (the kernel takes the quadrupole's xx entry out
+of the matrix), with and without softening, and the windowed order of the
+work items.  Tolerance: the FP32 gate,
 1e-5 (rounding of ~30 units of 6e-8 per term, ~1e-6 of a sum of ~1e3 terms;
 the quadrupole terms are 1e-3 to 1e-2 of the pull, so that a wrong entry is
 100 times the gate)."""
+import numpy as np
 import pytest
 
 import oracle as orc
@@ -41,3 +43,19 @@ def test_flat_cells(axis, eps):
     P = synth.uniform_cube(4000, 11)
     P[axis] = 0.5 + 0.02 * (P[axis] - 0.5)
     check(P, dict(synth.PRESETS["cube4k"]["params"], order=2, eps=eps, n_g=48, theta=0.8))
+
+
+@pytest.mark.parametrize("chunk", [32, 96])
+@pytest.mark.parametrize("window", [1, 63, 65, 91, 10000])
+def test_windowed_items(window, chunk):
+    """Groups of one to five chunks; the order of the items changes no bit."""
+    P, prm = synth.uniform_cube(9001, 5), dict(synth.PRESETS["cube4k"]["params"], order=2, n_g=130)
+    a = []
+    for w in (0, window):
+        ctx, D = gpu_build(P, prm, precision=1, forces=False)
+        ctx.bh_set_tuning(chunk=chunk, order_window=w)
+        ctx.bh_make_lists()
+        ctx.bh_compute_forces(D, 1)
+        a.append(accel_of(D))
+        ctx.close()
+    assert np.array_equal(a[0], a[1])
