@@ -44,9 +44,6 @@ __device__ __forceinline__ df df_add(df a, df b) {
     return fast_two_sum(s.hi, s.lo);
 }
 
-__device__ __forceinline__ df df_neg(df a) { return {-a.hi, -a.lo}; }
-__device__ __forceinline__ df df_sub(df a, df b) { return df_add(a, df_neg(b)); }
-
 __device__ __forceinline__ df df_mul(df a, df b) {
     df p = two_prod(a.hi, b.hi);
     p.lo = __fmaf_rn(a.hi, b.lo, p.lo);
@@ -54,10 +51,36 @@ __device__ __forceinline__ df df_mul(df a, df b) {
     return fast_two_sum(p.hi, p.lo);
 }
 
-__device__ __forceinline__ df df_mul_f(df a, float b) {
-    df p = two_prod(a.hi, b);
-    p.lo = __fmaf_rn(a.lo, b, p.lo);
+// a * b without the last renormalisation (|lo| up to a few ulp(hi)): a factor
+// of a product that is summed with df_accumulate
+__device__ __forceinline__ df df_mul_loose(df a, df b) {
+    df p = two_prod(a.hi, b.hi);
+    p.lo = __fmaf_rn(a.hi, b.lo, p.lo);
+    p.lo = __fmaf_rn(a.lo, b.hi, p.lo);
+    return p;
+}
+
+__device__ __forceinline__ df df_sqr(df a) {
+    df p = two_prod(a.hi, a.hi);
+    p.lo = __fmaf_rn(__fadd_rn(a.hi, a.hi), a.lo, p.lo);
     return fast_two_sum(p.hi, p.lo);
+}
+
+// One term of a running sum: the high parts are added exactly, the errors
+// and low parts in FP32.  Every rounding is 2^-24 of a low part, 2^-48 of the
+// larger of sum and term, as for df_add -- but where the two cancel, df_add
+// keeps the bits of the low parts' own rounding, which a sum of many terms
+// does not have.  8 operations instead of 20; renormalise with fast_two_sum.
+__device__ __forceinline__ void df_accumulate(df& sum, df t) {
+    const df s = two_sum(sum.hi, t.hi);
+    sum.hi = s.hi;
+    sum.lo = __fadd_rn(sum.lo, __fadd_rn(s.lo, t.lo));
+}
+
+__device__ __forceinline__ void df_accumulate(df& sum, float t) {
+    const df s = two_sum(sum.hi, t);
+    sum.hi = s.hi;
+    sum.lo = __fadd_rn(sum.lo, s.lo);
 }
 
 // (x_hi + x_lo) - (y_hi + y_lo) for two hi/lo splits of FP64 values
@@ -67,16 +90,24 @@ __device__ __forceinline__ df df_diff(float xh, float xl, float yh, float yl) {
     return fast_two_sum(d.hi, d.lo);
 }
 
-__device__ __forceinline__ df df_dot3(df x, df y, df z) { return df_add(df_add(df_mul(x, x), df_mul(y, y)), df_mul(z, z)); }
+// x^2 + y^2 + z^2: nothing cancels, so the low parts are summed in FP32
+__device__ __forceinline__ df df_norm2(df x, df y, df z) {
+    const df px = two_prod(x.hi, x.hi), py = two_prod(y.hi, y.hi), pz = two_prod(z.hi, z.hi);
+    const df s = two_sum(px.hi, py.hi), t = two_sum(s.hi, pz.hi);
+    const float ex = __fmaf_rn(__fadd_rn(x.hi, x.hi), x.lo, px.lo);
+    const float ey = __fmaf_rn(__fadd_rn(y.hi, y.hi), y.lo, py.lo);
+    const float ez = __fmaf_rn(__fadd_rn(z.hi, z.hi), z.lo, pz.lo);
+    return fast_two_sum(t.hi, __fadd_rn(__fadd_rn(s.lo, t.lo), __fadd_rn(__fadd_rn(ex, ey), ez)));
+}
 
-// 1 / sqrt(s), s > 0: an FP32 estimate y0 and one Newton step carried out in
-// df, y = y0 + y0 (1 - s y0^2) / 2 (the residual in df; the step squares the
-// estimate's relative error).
+// 1 / sqrt(s), s > 0: an FP32 estimate y0 and one Newton step,
+// y = y0 + y0 (1 - s y0^2) / 2 (the step squares the estimate's relative
+// error).  s y0^2 is within a few 2^-23 of 1, so 1 - its high part is exact.
 __device__ __forceinline__ df df_rsqrt(df s) {
     const float y0 = rsqrtf(s.hi);
-    const df y2 = two_prod(y0, y0);
-    const df r = df_sub(df_make(1.f), df_mul(s, y2));
-    return fast_two_sum(y0, __fmul_rn(__fmul_rn(y0, 0.5f), r.hi));
+    const df p = df_mul_loose(s, two_prod(y0, y0));
+    const float r = __fsub_rn(__fsub_rn(1.f, p.hi), p.lo);
+    return fast_two_sum(y0, __fmul_rn(__fmul_rn(y0, 0.5f), r));
 }
 
 __device__ __forceinline__ bool df_gt(df a, df b) { return a.hi > b.hi || (a.hi == b.hi && a.lo > b.lo); }

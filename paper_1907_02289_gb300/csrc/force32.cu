@@ -1060,6 +1060,7 @@ __global__ void k_contacts64(const uint2* __restrict__ pairs, const unsigned lon
 // the pull of the neighbour it touches.
 struct RefineConsts {
     df rc2, eps2, rc2eps2;  // r_coll^2, eps^2, r_coll^2 + eps^2
+    bool soft;              // eps^2 > 0
 };
 
 __device__ __forceinline__ df df_of(double v) {
@@ -1071,16 +1072,16 @@ __device__ __forceinline__ void ref_pp(const Args& A, const RefineConsts& K, flo
                                        float zh, float zl, uint32_t i, uint32_t j, const float4 h, const float4 l,
                                        df (&acc)[3], double (&ac)[3]) {
     const df d[3] = {df_diff(h.x, l.x, xh, xl), df_diff(h.y, l.y, yh, yl), df_diff(h.z, l.z, zh, zl)};
-    const df r2 = df_dot3(d[0], d[1], d[2]);
+    const df r2 = df_norm2(d[0], d[1], d[2]);
     if (r2.hi == 0.f) return;  // coincident pair: no term
     if (r2.hi < A.rc2chk)  // the contact term of the FP64 pass, decided and evaluated as there
         contact_term64(A.fp, A.x[i], A.y[i], A.z[i], A.vx[i], A.vy[i], A.vz[i], A.m[i], A.x[j], A.y[j], A.z[j],
                        A.vx[j], A.vy[j], A.vz[j], A.m[j], ac);
-    const df s2 = df_gt(r2, K.rc2) ? df_add(r2, K.eps2) : K.rc2eps2;
+    const df s2 = df_gt(r2, K.rc2) ? (K.soft ? df_add(r2, K.eps2) : r2) : K.rc2eps2;
     const df y = df_rsqrt(s2);
-    const df f = df_mul(df_mul(fast_two_sum(h.w, l.w), y), df_mul(y, y));  // m / s^3
+    const df f = df_mul(df_mul({h.w, l.w}, y), df_sqr(y));  // m / s^3
 #pragma unroll
-    for (int c = 0; c < 3; ++c) acc[c] = df_add(acc[c], df_mul(f, d[c]));
+    for (int c = 0; c < 3; ++c) df_accumulate(acc[c], df_mul_loose(f, d[c]));
 }
 
 struct CellRec {
@@ -1097,15 +1098,13 @@ __device__ __forceinline__ void ref_pc(const Args& A, const RefineConsts& K, flo
     const float4 r0 = cr.r0, r1 = cr.r1;
     // R = x_i - c (the oracle's sign); a = -M R / R^3 + Q R / R^5 - 5/2 (R.Q.R) R / R^7 (G-free)
     const df R[3] = {df_diff(xh, xl, r0.x, r1.x), df_diff(yh, yl, r0.y, r1.y), df_diff(zh, zl, r0.z, r1.z)};
-    const df R2 = df_add(df_dot3(R[0], R[1], R[2]), K.eps2);
+    df R2 = df_norm2(R[0], R[1], R[2]);
+    if (K.soft) R2 = df_add(R2, K.eps2);
     const df y = df_rsqrt(R2);
-    const df y2 = df_mul(y, y);
-    const df y3 = df_mul(y2, y);
-    const df M = fast_two_sum(r0.w, cr.mlo);
-    const df mono = df_neg(df_mul(M, y3));
-    df t[3];
+    const df y3 = df_mul(df_sqr(y), y);
+    const df mono = df_mul(fast_two_sum(-r0.w, -cr.mlo), y3);
 #pragma unroll
-    for (int c = 0; c < 3; ++c) t[c] = df_mul(mono, R[c]);
+    for (int c = 0; c < 3; ++c) df_accumulate(acc[c], df_mul_loose(mono, R[c]));
     if (A.fp.order >= 2) {
         // the quadrupole part, at most about theta^2 of the monopole, in FP32
         // from the df separation (its FP32 rounding stays far below the
@@ -1118,12 +1117,10 @@ __device__ __forceinline__ void ref_pc(const Args& A, const RefineConsts& K, flo
         const float rqr = Rx * qx + Ry * qy + Rz * qz;
         const float yf = y.hi, y2f = yf * yf, y5f = y2f * y2f * yf;
         const float w = -2.5f * rqr * y5f * y2f;  // -5/2 (R.Q.R) / R^7
-        t[0] = df_add(t[0], df_make(y5f * qx + w * Rx));
-        t[1] = df_add(t[1], df_make(y5f * qy + w * Ry));
-        t[2] = df_add(t[2], df_make(y5f * qz + w * Rz));
+        df_accumulate(acc[0], y5f * qx + w * Rx);
+        df_accumulate(acc[1], y5f * qy + w * Ry);
+        df_accumulate(acc[2], y5f * qz + w * Rz);
     }
-#pragma unroll
-    for (int c = 0; c < 3; ++c) acc[c] = df_add(acc[c], t[c]);
 }
 
 // After the contact terms: each particle with a contact candidate (claimed
@@ -1163,7 +1160,12 @@ __global__ void k_contacts_apply(const Args A, const uint2* __restrict__ pairs, 
 
 // Launch bounds for 4 blocks of 8 warps per SM (64 registers, a few small
 // spills): the df chains are latency-bound, and 32 warps per SM refine a
-// 2^26 ring in 6.1 ms against 6.6 ms at 16 warps (97 registers).
+// 2^26 ring in 6.1 ms against 6.6 ms at 16 warps (97 registers).  Bound by
+// the FMA pipe and those chains: about 135 operations per list particle and
+// 190 per cell since sums and squares keep only what their own rounding
+// carries (250 and 345 before).  With every particle of the 2^24 ring refined
+// a step takes 177 ms against 242, with the same errors against FP64 (median
+// 3.07e-9, from the FP32 quadrupole).
 __global__ void __launch_bounds__(256, 4) k_refine32(const Args A, const RefineConsts K,
                                                      const float* __restrict__ mlo, int64_t cap) {
     launch_wait();
@@ -1263,6 +1265,8 @@ __global__ void __launch_bounds__(256, 4) k_refine32(const Args A, const RefineC
             }
         }
 #pragma unroll
+        for (int c = 0; c < 3; ++c) acc[c] = fast_two_sum(acc[c].hi, acc[c].lo);
+#pragma unroll
         for (int o = 16; o > 0; o >>= 1)
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
@@ -1356,7 +1360,7 @@ RefineConsts refine_consts(const ForceParams& fp) {
         const float h = (float)v;
         return df{h, (float)(v - (double)h)};
     };
-    return RefineConsts{split(fp.rc2), split(fp.eps2), split(fp.rc2 + fp.eps2)};
+    return RefineConsts{split(fp.rc2), split(fp.eps2), split(fp.rc2 + fp.eps2), fp.eps2 > 0.0};
 }
 
 // The refinement pass over the particles the force kernel queued (count
