@@ -717,6 +717,15 @@ int graph_rebuild_step(Ctx* c, bh_particles* p) {
     return BH_OK;
 }
 
+// How bh_step issues the next step.
+bool reuse_by_graph(const Ctx* c) {
+    return c->tune.graph && c->have_lists && c->k_eval % c->prm.rebuild_every != 0;
+}
+// (a list capacity needs the eager build's exact sizes)
+bool rebuild_by_graph(const Ctx* c) {
+    return c->tune.graph == 1 && c->have_lists && c->prm.list_capacity == 0;
+}
+
 int check_tuning(Ctx* c, const bh_tuning* t) {
     if (!t) return fail(c, BH_E_INVAL, "tuning is NULL");
     if (t->n_g < c->prm.n_leaf) return fail(c, BH_E_INVAL, "n_g must be >= n_leaf");
@@ -1084,20 +1093,28 @@ int bh_step(bh_ctx* ctx, bh_particles* p, int nsteps) {
         BH_TRY(bh::evaluate(c, p));
         c->have_acc = true;
     }
+    // between two eager steps the closing kick and the next kick-drift are one
+    // pass over the particles (stage timing keeps them apart)
+    bool kicked = false;
     for (int s = 0; s < nsteps; ++s) {
         c->early_now = s == nsteps - 1;  // only the last step's evaluation counts
-        if (c->tune.graph && c->have_lists && c->k_eval % c->prm.rebuild_every != 0) {
-            BH_TRY(bh::graph_reuse_step(c, p));
-            continue;
+        if (!kicked) {
+            if (bh::reuse_by_graph(c)) {
+                BH_TRY(bh::graph_reuse_step(c, p));
+                continue;
+            }
+            if (bh::rebuild_by_graph(c)) {
+                BH_TRY(bh::graph_rebuild_step(c, p));
+                continue;
+            }
+            BH_TRY(bh::stage_kick_drift(c, p, 0.5 * dt, dt));
         }
-        // a list capacity needs the eager build's exact sizes
-        if (c->tune.graph == 1 && c->have_lists && c->prm.list_capacity == 0) {
-            BH_TRY(bh::graph_rebuild_step(c, p));
-            continue;
-        }
-        BH_TRY(bh::stage_kick_drift(c, p, 0.5 * dt, dt));
         BH_TRY(bh::evaluate(c, p));
-        BH_TRY(bh::stage_kick(c, p, 0.5 * dt));
+        kicked = s + 1 < nsteps && !c->timing && !bh::reuse_by_graph(c) && !bh::rebuild_by_graph(c);
+        if (kicked)
+            BH_TRY(bh::stage_kick_drift(c, p, 0.5 * dt, dt, true));
+        else
+            BH_TRY(bh::stage_kick(c, p, 0.5 * dt));
     }
     return BH_OK;
 }

@@ -395,7 +395,7 @@ int stage_end(Ctx* c);
 
 // update.cu
 int stage_kick(Ctx* c, bh_particles* p, double h);
-int stage_kick_drift(Ctx* c, bh_particles* p, double h, double dt);
+int stage_kick_drift(Ctx* c, bh_particles* p, double h, double dt, bool twice = false);
 int stage_diagnostics(Ctx* c, const bh_particles* p, double* host_out);  // 11 sums to the host
 
 }  // namespace bh
