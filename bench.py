@@ -62,19 +62,23 @@ HBM_FALLBACK_GBS = 6800.0  # the profiling recipe's fallback copy bandwidth
 
 # Algorithmic HBM bytes of the HBM-bound stages (per particle; per node where
 # stated), for their GB/s against the measured copy bandwidth:
-#  keys      x, y, z read for the root box and again for the keys, key + index
-#            written (24 + 24 + 12); the cylindrical frame first reads x, y and
+#  keys      x, y, z read for the root box and again for the keys, keys
+#            written (24 + 24 + 8); the cylindrical frame first reads x, y and
 #            writes phi, r (+32)
-#  sort      8 passes of 8 bits, each reading and writing key + index (8 x 24)
+#  sort      the keys read for the digit counts (8), then 8 passes of 8 bits,
+#            each reading and writing key + index (8 x 24; the first reads no
+#            index)
 #  permute   index read, 8 particle arrays read and written (4 + 8 x 16)
-#  moments   x, y, z, m (FP64 path) or the hi/lo float4 pair (FP32 path) read
-#            per particle; per node its record written and read once more by
-#            its parent (FP64: 2 x 80; FP32: 2 x 48 + 4)
-#  split     x, y, z, m read, two float4 written (32 + 32)
+#  moments   FP64 path: x, y, z, m read per particle, per node its record
+#            written and read once more by its parent (2 x 80).  FP32 path:
+#            the inner nodes, every record read by its parent (52 per node;
+#            the inner nodes' own records are not counted)
+#  split     FP32 path, with the leaves' moments: x, y, z, m read, two float4
+#            written (32 + 32; the leaves' records are not counted)
 #  update    per step: kick-drift reads a, v, x and writes v, x (72 + 48), the
 #            closing kick reads a, v and writes v (48 + 24)
-STAGE_BYTES = {"keys": 60, "keys_cyl_extra": 32, "sort": 192, "permute": 132, "split": 64, "update": 192}
-MOMENT_BYTES = {0: (32, 160), 1: (32, 100)}  # precision -> (per particle, per node)
+STAGE_BYTES = {"keys": 56, "keys_cyl_extra": 32, "sort": 196, "permute": 132, "split": 64, "update": 192}
+MOMENT_BYTES = {0: (32, 160), 1: (0, 52)}  # precision -> (per particle, per node)
 
 
 def fp32_peak_tflops(mhz: float) -> float:

@@ -866,7 +866,11 @@ int autotune(Ctx* c, bh_particles* p, double* best_ms) {
     } else {
         BH_TRY(try_force(best));  // the FP64 kernel has no launch settings
     }
-    // (2) n_g by the cost of a step: force time + list-build time / rebuild_every
+    // (2) n_g by the cost of a step: force time + list-build time /
+    // rebuild_every, each with the chunk found and with the largest (groups of
+    // 128 favour chunks of 64, groups of 192 and 256 chunks of 96: at 2^26 a
+    // step takes 137.3, 131.1 and 128.4 ms with 96, 137.0, 135.6 and 132.7 with
+    // 64, and the best of the latter alone need not be the best of all)
     {
         double best_step = 1e300;
         bh_tuning best_ng = best;
@@ -879,15 +883,24 @@ int autotune(Ctx* c, bh_particles* p, double* best_ms) {
             double b = 0.0, f = 1e300;
             BH_TRY(time_ms(c, build, &b));
             BH_TRY(settle());
-            for (int rep = 0; rep < 3; ++rep) {
-                double m = 0.0;
-                BH_TRY(time_ms(c, force, &m));
-                if (m < f) f = m;
-            }
-            const double step = f + b / c->prm.rebuild_every;
-            if (step < best_step) {
-                best_step = step;
-                best_ng = t;
+            const bool both = c->prm.precision == BH_PREC_FP32 && best.chunk != 96;
+            for (int ch = 0; ch < (both ? 2 : 1); ++ch) {
+                if (ch == 1) {
+                    t.chunk = 96;
+                    apply_tuning(c, &t);
+                    BH_TRY(build_order32(c));
+                }
+                f = 1e300;
+                for (int rep = 0; rep < 3; ++rep) {
+                    double m = 0.0;
+                    BH_TRY(time_ms(c, force, &m));
+                    if (m < f) f = m;
+                }
+                const double step = f + b / c->prm.rebuild_every;
+                if (step < best_step) {
+                    best_step = step;
+                    best_ng = t;
+                }
             }
         }
         best = best_ng;
