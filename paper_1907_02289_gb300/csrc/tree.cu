@@ -629,8 +629,12 @@ __device__ __forceinline__ void put_moments32(int64_t k, float Mk, df Md, const 
 // than fit are read back from memory).  Bound by HBM: 32 B read and 32 B
 // written per particle and 52 B per leaf, where a pass of its own re-read the
 // 32 B with a leaf's stride between the lanes.  Split and moments of the 2^24
-// ring, per evaluation: 0.65 -> 0.54 ms.
-constexpr int kLeafTile = 128, kLeafCap = 768;
+// ring, per evaluation: 0.65 -> 0.54 ms.  Room for 640 particles (5 per leaf)
+// lets 10 blocks share an SM, and the masses are summed with the short form of
+// the hi/lo addition (here and in k_moments32), which is a chain per particle:
+// evaluation of a 100,003-particle cube 592 -> 586 us, of a 65,537-particle
+// ring 403 -> 399, four steps of the 2^24 ring 64.1 -> 64.0 ms.
+constexpr int kLeafTile = 128, kLeafCap = 640;
 
 template <int ORDER>
 __global__ void __launch_bounds__(kLeafTile) k_leaf32(const int32_t* __restrict__ leaves,
@@ -682,7 +686,7 @@ __global__ void __launch_bounds__(kLeafTile) k_leaf32(const int32_t* __restrict_
                 const float d[3] = {dsub(h.x, l.x, rh[0], rl[0]), dsub(h.y, l.y, rh[1], rl[1]),
                                     dsub(h.z, l.z, rh[2], rl[2])};
                 Mk += h.w;
-                Md = df_add(Md, {h.w, l.w});
+                df_accumulate(Md, {h.w, l.w});
 #pragma unroll
                 for (int a = 0; a < 3; ++a) s[a] = fmaf(h.w, d[a], s[a]);
             }
@@ -748,7 +752,7 @@ __global__ void __launch_bounds__(kSpanThreads) k_moments32(
                     const float d[3] = {dsub(h.x, l.x, rh[0], rl[0]), dsub(h.y, l.y, rh[1], rl[1]),
                                         dsub(h.z, l.z, rh[2], rl[2])};
                     Mk += h.w;
-                    Md = df_add(Md, {h.w, ml[u]});
+                    df_accumulate(Md, {h.w, ml[u]});
 #pragma unroll
                     for (int a = 0; a < 3; ++a) s[a] = fmaf(h.w, d[a], s[a]);
                 }
