@@ -138,7 +138,7 @@ struct Args {
     int64_t ng;
     const unsigned long long* dng;  // device group count (device-sized list builds; NULL: ng)
     const unsigned long long* abort;  // device-sized build: nonzero overflow bits skip the launch
-    const int2* order;     // work items in processing order: (group, i-chunk)
+    const int2* order;     // work items in processing order: (group, item_code of the i-chunk)
     const unsigned long long* items;  // their count (device)
     int64_t items_cap;     // and its bound
     const int32_t* groups;
@@ -166,7 +166,6 @@ struct Args {
     bool add_central;
     // schedule: warps take list slots slot0, slot0 + stride, ... (grid or
     // persistent static), or draw them from *ticket (persistent dynamic)
-    int chunk;                     // largest i-chunk (32, 64 or 96 particles)
     unsigned long long* ticket;    // NULL: static
     unsigned long long* warp_time; // optional: per warp (start, end) %globaltimer
     // refinement: particle i of list slot k is queued as (i, k) when
@@ -797,10 +796,10 @@ __device__ __forceinline__ void force_item(const Args& A, Smem32& S, int64_t slo
     // origin: the group node's centre of mass as an FP32 hi/lo pair
     const float4 o0 = A.cell32[3 * (int64_t)g], o1 = A.cell32[3 * (int64_t)g + 1];
     const float oh[3] = {o0.x, o0.y, o0.z}, ol[3] = {o1.x, o1.y, o1.z};
-    // chunks of at most A.chunk particles: R full slots plus a tail of at most 16
-    const uint32_t i0 = b + (uint32_t)o.y * (uint32_t)A.chunk;
+    // R full slots plus a tail of at most 16
+    const uint32_t i0 = b + 32u * ((uint32_t)o.y >> 2);
     {
-        const uint32_t cnt = min(e - i0, (uint32_t)A.chunk);
+        const uint32_t cnt = min(e - i0, 32u * ((uint32_t)o.y & 3u));
         int R = (int)(cnt >> 5), t = (int)(cnt & 31), T = 0;
         if (t > 16) {
             ++R;  // more than half a slot left: a full one
@@ -889,10 +888,27 @@ struct OrderArgs {
     const int32_t* groups;
     const uint32_t *begin, *end;
     const int64_t *jj_off, *pc_off;
-    uint32_t chunk;
+    uint32_t chunk;  // largest i-chunk (32, 64 or 96 particles)
     bool by_cost;
     int64_t window;  // groups per window (0: one order over all)
+    int64_t few;     // up to this many groups the i-chunks are of 32
 };
+
+// With hardly more groups than warps in flight (fewer than 1.5 per warp) the
+// launch lasts as long as its longest item and warps stay idle, so the items
+// are single slots: the same bits (a particle's sum does not depend on the
+// chunk it is in), the lists staged more often.  Measured with chunks of 96 and
+// of 32, 2432 warps in flight: evaluation of a 65,537-particle ring (1163
+// groups) 401 and 361 us, forces of 20,000 particles (831) 83.5 and 80.7, of
+// 65,537 (2492) 125 and 100, of 131,072 (4420) 141.0 and 140.8, of 262,144
+// (10,503) 232 and 236, 100,003-particle cube (4096) 584 and 586.
+__host__ __device__ __forceinline__ uint32_t item_chunk(int64_t ng, int64_t few, uint32_t chunk) {
+    return ng <= few ? 32u : chunk;
+}
+
+// An item's i-chunk: its first particle (in slots of 32 from the group's
+// first) and its slots.
+__device__ __forceinline__ int item_code(uint32_t i, uint32_t chunk) { return (int)((i / 32u) << 2 | chunk / 32u); }
 
 __device__ __forceinline__ uint32_t group_size(const OrderArgs& O, int64_t k) {
     const int32_t g = O.groups[k];
@@ -927,7 +943,8 @@ __global__ void k_order_hist_windows(const OrderArgs O, uint32_t* cnt) {
     if (k >= O.ng) return;
     uint32_t* mine = cnt + (k / O.window) * kOrderBuckets;
     const uint32_t ni = group_size(O, k);
-    for (uint32_t i = 0; i < ni; i += O.chunk) atomicAdd(&mine[order_bucket(O, k, ni, min(O.chunk, ni - i))], 1u);
+    const uint32_t chunk = item_chunk(O.ng, O.few, O.chunk);
+    for (uint32_t i = 0; i < ni; i += chunk) atomicAdd(&mine[order_bucket(O, k, ni, min(chunk, ni - i))], 1u);
 }
 
 __global__ void k_order_scatter_windows(const OrderArgs O, uint32_t* cursor, int2* __restrict__ order, int64_t cap) {
@@ -936,20 +953,20 @@ __global__ void k_order_scatter_windows(const OrderArgs O, uint32_t* cursor, int
     if (k >= O.ng) return;
     uint32_t* mine = cursor + (k / O.window) * kOrderBuckets;
     const uint32_t ni = group_size(O, k);
-    int c = 0;
-    for (uint32_t i = 0; i < ni; i += O.chunk, ++c) {
-        const int64_t at = atomicAdd(&mine[order_bucket(O, k, ni, min(O.chunk, ni - i))], 1u);
-        if (at < cap) order[at] = make_int2((int)k, c);
+    const uint32_t chunk = item_chunk(O.ng, O.few, O.chunk);
+    for (uint32_t i = 0; i < ni; i += chunk) {
+        const int64_t at = atomicAdd(&mine[order_bucket(O, k, ni, min(chunk, ni - i))], 1u);
+        if (at < cap) order[at] = make_int2((int)k, item_code(i, chunk));
     }
 }
 
 __global__ void k_order_hist(const OrderArgs O, unsigned long long* cnt) {
     launch_wait();
     const int64_t ng = O.dng ? min(O.ng, (int64_t)*O.dng) : O.ng;
+    const uint32_t chunk = item_chunk(ng, O.few, O.chunk);
     for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < ng; k += (int64_t)gridDim.x * blockDim.x) {
         const uint32_t ni = group_size(O, k);
-        for (uint32_t i = 0; i < ni; i += O.chunk)
-            atomicAdd(&cnt[order_bucket(O, k, ni, min(O.chunk, ni - i))], 1ull);
+        for (uint32_t i = 0; i < ni; i += chunk) atomicAdd(&cnt[order_bucket(O, k, ni, min(chunk, ni - i))], 1ull);
     }
 }
 
@@ -958,6 +975,7 @@ __global__ void k_order_scatter(const OrderArgs O, const unsigned long long* __r
                                 unsigned long long* items) {
     launch_wait();
     const int64_t ng = O.dng ? min(O.ng, (int64_t)*O.dng) : O.ng;
+    const uint32_t chunk = item_chunk(ng, O.few, O.chunk);
     // exclusive prefix of the bucket counts, by the block's first warp
     __shared__ unsigned long long start[kOrderBuckets];
     constexpr int PL = kOrderBuckets / 32;
@@ -981,11 +999,10 @@ __global__ void k_order_scatter(const OrderArgs O, const unsigned long long* __r
     __syncthreads();
     for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < ng; k += (int64_t)gridDim.x * blockDim.x) {
         const uint32_t ni = group_size(O, k);
-        int c = 0;
-        for (uint32_t i = 0; i < ni; i += O.chunk, ++c) {
-            const int b = order_bucket(O, k, ni, min(O.chunk, ni - i));
+        for (uint32_t i = 0; i < ni; i += chunk) {
+            const int b = order_bucket(O, k, ni, min(chunk, ni - i));
             const int64_t at = (int64_t)(start[b] + atomicAdd(&cursor[b], 1ull));
-            if (at < cap) order[at] = make_int2((int)k, c);
+            if (at < cap) order[at] = make_int2((int)k, item_code(i, chunk));
         }
     }
 }
@@ -1062,11 +1079,6 @@ struct RefineConsts {
     df rc2, eps2, rc2eps2;  // r_coll^2, eps^2, r_coll^2 + eps^2
     bool soft;              // eps^2 > 0
 };
-
-__device__ __forceinline__ df df_of(double v) {
-    const float h = __double2float_rn(v);
-    return {h, __double2float_rn(v - (double)h)};
-}
 
 __device__ __forceinline__ void ref_pp(const Args& A, const RefineConsts& K, float xh, float xl, float yh, float yl,
                                        float zh, float zl, uint32_t i, uint32_t j, const float4 h, const float4 l,
@@ -1317,21 +1329,26 @@ int resident_blocks(Force32Fn kern, int warps) {
 
 }  // namespace
 
+// Groups up to which the items are single slots (16 warps per SM in flight).
+static int64_t few_groups(const Ctx* c) { return 24 * (int64_t)c->num_sms; }
+
 // Work items of the FP32 kernel in processing order (once per list build).
 int build_order32(Ctx* c) {
     const int64_t ng = c->n_groups;
-    const int chunk = std::min(c->tune.chunk, 32 * BH_F32_MAXR);
+    const uint32_t chunk = (uint32_t)std::min(c->tune.chunk, 32 * BH_F32_MAXR);
+    const int64_t few = few_groups(c);
     // (device-sized: sized before capture, at most one item per particle)
-    if (!c->dev_build) BH_TRY(grow(c, c->order, (size_t)(ng + c->n / chunk + 1), "work items"));
+    if (!c->dev_build) BH_TRY(grow(c, c->order, (size_t)(ng + c->n / item_chunk(ng, few, chunk) + 1), "work items"));
     BH_TRY(grow(c, c->order_cnt, 2 * (size_t)kOrderBuckets, "group order buckets"));
     unsigned long long* cnt = c->order_cnt.p;
     unsigned long long* items = c->d_sz + kSzItems;
     const OrderArgs O{ng,         c->dev_build ? c->d_sz + kSzNg : nullptr,
                       c->groups.p, c->begin.p,
                       c->end.p,    c->cnt_j.p,
-                      c->cnt_c.p,  (uint32_t)chunk,
+                      c->cnt_c.p,  chunk,
                       c->tune.order_by_cost != 0,
-                      std::max<int64_t>(c->tune.order_window, kLeastWindow)};
+                      std::max<int64_t>(c->tune.order_window, kLeastWindow),
+                      few};
     if (c->tune.order_window > 0 && ng > c->tune.order_window && !c->dev_build) {  // (device-sized: plain order)
         const int64_t words = (ng + O.window - 1) / O.window * kOrderBuckets;
         BH_TRY(grow(c, c->ord_cnt, (size_t)words, "group order buckets of the windows"));
@@ -1444,7 +1461,6 @@ int launch_force32(Ctx* c, bh_particles* p, const ForceParams& fp, bool add_cent
                                                 smax));
         c->f32_attr_device = c->device;
     }
-    A.chunk = std::min(c->tune.chunk, 32 * BH_F32_MAXR);
     A.ticket = nullptr;
     A.warp_time = nullptr;
     A.kref = BH_REFINE_K;
@@ -1469,7 +1485,9 @@ int launch_force32(Ctx* c, bh_particles* p, const ForceParams& fp, bool add_cent
         A.cflag = c->cflag.p;
     }
     unsigned nb;
-    const int64_t items = std::min(A.items_cap, groups_expected(c) + c->n / A.chunk + 1);  // about (a bound, eagerly)
+    const uint32_t chunk =
+        item_chunk(groups_expected(c), few_groups(c), (uint32_t)std::min(c->tune.chunk, 32 * BH_F32_MAXR));
+    const int64_t items = std::min(A.items_cap, groups_expected(c) + c->n / chunk + 1);  // about (a bound, eagerly)
     if (c->tune.sched == BH_SCHED_GRID && !A.dng) {
         nb = blocks_for(items, W);
     } else {  // (a device-sized build runs the grid schedule as a persistent static one)

@@ -1,8 +1,8 @@
 """The FP32 force kernel's list loops at the sizes that pick their variants:
 chunks of 1 to 3 slots with and without a tail, odd counts of list pairs,
 cells flat along each axis (the kernel takes the quadrupole's xx entry out
-of the matrix), with and without softening, and the windowed order of the
-work items.  Tolerance: the FP32 gate,
+of the matrix), with and without softening, and the work items: windowed
+order, and chunk sizes (32 where the groups are few), which change no bit.  Tolerance: the FP32 gate,
 1e-5 (rounding of ~30 units of 6e-8 per term, ~1e-6 of a sum of ~1e3 terms;
 the quadrupole terms are 1e-3 to 1e-2 of the pull, so that a wrong entry is
 100 times the gate)."""
@@ -59,3 +59,22 @@ def test_windowed_items(window, chunk):
         a.append(accel_of(D))
         ctx.close()
     assert np.array_equal(a[0], a[1])
+
+
+@pytest.mark.parametrize("shape", ["ring", "cube"])
+def test_chunks_same_bits(shape):
+    """Many groups of one to three slots and contacts; few groups take 32."""
+    if shape == "ring":
+        P, prm = synth.ring(400000, 3, phi_max=0.05), dict(synth.PRESETS["ring16m_fp32"]["params"], n_g=100)
+    else:
+        P, prm = synth.uniform_cube(400000, 3), dict(synth.PRESETS["cube4k"]["params"], order=2, n_g=100)
+    a = []
+    for chunk in (96, 64, 32):
+        ctx, D = gpu_build(P, prm, precision=1, forces=False)
+        ctx.bh_set_tuning(chunk=chunk)
+        ctx.bh_make_lists()
+        ctx.bh_compute_forces(D, 1)
+        a.append(accel_of(D))
+        assert ctx.bh_get_sizes()["n_groups"] > 3648
+        ctx.close()
+    assert np.array_equal(a[0], a[1]) and np.array_equal(a[0], a[2])
