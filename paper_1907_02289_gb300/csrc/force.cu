@@ -347,8 +347,8 @@ __global__ void __launch_bounds__(32 * kWarps) k_sum64(const Args64 A) {
 // block tree, one final pass), so repeated calls give the same bits.
 constexpr int kWBlocks = 512, kWThreads = 256;
 
-__global__ void __launch_bounds__(kWThreads) k_wsum_partial(int64_t n, const double* __restrict__ m,
-                                                            const double* __restrict__ phi, double* part) {
+__global__ void __launch_bounds__(kWThreads) k_wsum_partial(int64_t n, const double* m,
+                                                            const double* phi, double* part) {
     launch_wait();
     __shared__ double sh[kWThreads];
     double acc = 0.0;
@@ -363,7 +363,7 @@ __global__ void __launch_bounds__(kWThreads) k_wsum_partial(int64_t n, const dou
     if (threadIdx.x == 0) part[blockIdx.x] = sh[0];
 }
 
-__global__ void k_wsum_final(const double* __restrict__ part, double* out) {
+__global__ void k_wsum_final(const double* part, double* out) {
     launch_wait();
     if (threadIdx.x != 0) return;
     double s = 0.0;

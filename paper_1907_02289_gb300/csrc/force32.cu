@@ -947,7 +947,7 @@ __global__ void k_order_hist_windows(const OrderArgs O, uint32_t* cnt) {
     for (uint32_t i = 0; i < ni; i += chunk) atomicAdd(&mine[order_bucket(O, k, ni, min(chunk, ni - i))], 1u);
 }
 
-__global__ void k_order_scatter_windows(const OrderArgs O, uint32_t* cursor, int2* __restrict__ order, int64_t cap) {
+__global__ void k_order_scatter_windows(const OrderArgs O, uint32_t* cursor, int2* order, int64_t cap) {
     launch_wait();
     const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= O.ng) return;
@@ -970,8 +970,8 @@ __global__ void k_order_hist(const OrderArgs O, unsigned long long* cnt) {
     }
 }
 
-__global__ void k_order_scatter(const OrderArgs O, const unsigned long long* __restrict__ cnt,
-                                unsigned long long* cursor, int2* __restrict__ order, int64_t cap,
+__global__ void k_order_scatter(const OrderArgs O, const unsigned long long* cnt,
+                                unsigned long long* cursor, int2* order, int64_t cap,
                                 unsigned long long* items) {
     launch_wait();
     const int64_t ng = O.dng ? min(O.ng, (int64_t)*O.dng) : O.ng;
@@ -1032,12 +1032,12 @@ __device__ __forceinline__ int64_t contact_count(const unsigned long long* count
     return np;
 }
 
-__global__ void k_contacts64(const uint2* __restrict__ pairs, const unsigned long long* __restrict__ count,
-                             int64_t cap, ForceParams fp, const double* __restrict__ x,
-                             const double* __restrict__ y, const double* __restrict__ z,
-                             const double* __restrict__ vx, const double* __restrict__ vy,
-                             const double* __restrict__ vz, const double* __restrict__ m,
-                             unsigned long long* __restrict__ acc, unsigned long long* n_touch, int* status,
+__global__ void k_contacts64(const uint2* pairs, const unsigned long long* count,
+                             int64_t cap, ForceParams fp, const double* x,
+                             const double* y, const double* z,
+                             const double* vx, const double* vy,
+                             const double* vz, const double* m,
+                             unsigned long long* acc, unsigned long long* n_touch, int* status,
                              bool flag) {
     launch_wait();
     const int64_t np = contact_count(count, cap, status, flag);
@@ -1101,7 +1101,7 @@ struct CellRec {
     float mlo;
 };
 
-__device__ __forceinline__ CellRec load_cell(const Args& A, const float* __restrict__ mlo, int32_t cc) {
+__device__ __forceinline__ CellRec load_cell(const Args& A, const float* mlo, int32_t cc) {
     return {A.cell32[3 * (int64_t)cc], A.cell32[3 * (int64_t)cc + 1], A.cell32[3 * (int64_t)cc + 2], mlo[cc]};
 }
 
@@ -1138,8 +1138,8 @@ __device__ __forceinline__ void ref_pc(const Args& A, const RefineConsts& K, flo
 // After the contact terms: each particle with a contact candidate (claimed
 // once through its flag) gets their sum, and is queued when its tree part,
 // gravity and contact, is small against its FP32 bound.
-__global__ void k_contacts_apply(const Args A, const uint2* __restrict__ pairs, const unsigned long long* count,
-                                 int64_t cap, unsigned long long* __restrict__ acc) {
+__global__ void k_contacts_apply(const Args A, const uint2* pairs, const unsigned long long* count,
+                                 int64_t cap, unsigned long long* acc) {
     launch_wait();
     int64_t np = (int64_t)*count;
     if (np > cap) np = cap;
@@ -1179,7 +1179,7 @@ __global__ void k_contacts_apply(const Args A, const uint2* __restrict__ pairs, 
 // a step takes 177 ms against 242, with the same errors against FP64 (median
 // 3.07e-9, from the FP32 quadrupole).
 __global__ void __launch_bounds__(256, 4) k_refine32(const Args A, const RefineConsts K,
-                                                     const float* __restrict__ mlo, int64_t cap) {
+                                                     const float* mlo, int64_t cap) {
     launch_wait();
     const int lane = threadIdx.x & 31;
     const int64_t wid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;

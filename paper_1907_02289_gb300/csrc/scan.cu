@@ -56,12 +56,12 @@ struct ScanArrays {
 };
 
 template <typename T>
-__global__ void k_reduce(ScanArrays<T> a, int64_t n, const unsigned long long* dn, T* __restrict__ sums,
+__global__ void k_reduce(ScanArrays<T> a, int64_t n, const unsigned long long* dn, T* sums,
                          int64_t stride) {
     launch_wait();
     __shared__ T wt[kThreads / 32];
     __shared__ T tot;
-    const T* __restrict__ in = a.in[blockIdx.y];
+    const T* in = a.in[blockIdx.y];
     sums += blockIdx.y * stride;
     n = count_of(n, dn);
     const int64_t nt = (n + kTile - 1) / kTile;
@@ -104,7 +104,7 @@ __global__ void k_scan_sums(ScanArrays<T> a, T* sums, int64_t stride, int64_t n,
 
 // Blocked arrangement: thread t owns items [t*kItems, (t+1)*kItems) of the tile.
 template <typename T>
-__global__ void k_scan_apply(ScanArrays<T> a, int64_t n, const unsigned long long* dn, const T* __restrict__ sums,
+__global__ void k_scan_apply(ScanArrays<T> a, int64_t n, const unsigned long long* dn, const T* sums,
                              int64_t stride) {
     launch_wait();
     __shared__ T wt[kThreads / 32];

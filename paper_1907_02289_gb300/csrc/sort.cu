@@ -41,10 +41,10 @@ __device__ __forceinline__ void warp_minmax(unsigned long long& mn, unsigned lon
 // patches of uneven sizes): block b works on patch map[b].x as its map[b].y-th
 // of poff[q + 1] - poff[q] blocks (blocks in proportion to the patch sizes),
 // partials at b.
-__global__ void k_box_partial(const double* __restrict__ x, const double* __restrict__ y,
-                              const double* __restrict__ z, const int64_t* __restrict__ off,
-                              const uint2* __restrict__ map, const int* __restrict__ poff,
-                              unsigned long long* __restrict__ part, int* status) {
+__global__ void k_box_partial(const double* x, const double* y,
+                              const double* z, const int64_t* off,
+                              const uint2* map, const int* poff,
+                              unsigned long long* part, int* status) {
     launch_wait();
     __shared__ unsigned long long s[6][kBoxThreads / 32];
     unsigned long long mn[3] = {~0ull, ~0ull, ~0ull}, mx[3] = {0ull, 0ull, 0ull};
@@ -114,7 +114,7 @@ __global__ void k_box_partial(const double* __restrict__ x, const double* __rest
 // blocks poff[q] .. poff[q + 1] - 1): {lo_x, lo_y, lo_z, L, S} at box + 8 q.
 // Cylindrical frame (cyl): every particle must be off the axis (r > 0), else
 // kStatAxis.
-__global__ void k_box_final(const unsigned long long* __restrict__ part_all, int nb, const int* __restrict__ poff,
+__global__ void k_box_final(const unsigned long long* part_all, int nb, const int* poff,
                             double* box_all, int cyl, int* status) {
     launch_wait();
     const unsigned long long* part = part_all + 6 * (poff ? (int64_t)poff[blockIdx.x] : (int64_t)blockIdx.x * nb);
@@ -174,8 +174,8 @@ __device__ __forceinline__ float atan01(float t) {
     return __fadd_rn(base, __fmul_rn(u, p));
 }
 
-__global__ void k_cyl(const double* __restrict__ x, const double* __restrict__ y, int64_t n,
-                      double* __restrict__ phi, double* __restrict__ r) {
+__global__ void k_cyl(const double* x, const double* y, int64_t n,
+                      double* phi, double* r) {
     launch_wait();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
@@ -216,9 +216,9 @@ __device__ __forceinline__ uint32_t quantise(double v, double lo, double S) {
 
 // Keys of every particle on its patch's grid (patch by binary search of the
 // offsets).
-__global__ void k_keys(const double* __restrict__ x, const double* __restrict__ y,
-                       const double* __restrict__ z, int64_t n, const int64_t* __restrict__ off, int np,
-                       const double* __restrict__ boxes, uint64_t* __restrict__ key) {
+__global__ void k_keys(const double* x, const double* y,
+                       const double* z, int64_t n, const int64_t* off, int np,
+                       const double* boxes, uint64_t* key) {
     launch_wait();
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
@@ -308,8 +308,8 @@ __device__ __forceinline__ TileInfo tile_info(const uint32_t* __restrict__ tmeta
 
 // Digit counts of every pass, per patch of more than one tile: hist[slot][pass][digit].
 template <int ITEMS>
-__global__ void __launch_bounds__(256) k_digit_hist(const uint64_t* __restrict__ key, int64_t n, int ntiles,
-                                                    const uint32_t* __restrict__ tmeta, uint32_t* __restrict__ hist) {
+__global__ void __launch_bounds__(256) k_digit_hist(const uint64_t* key, int64_t n, int ntiles,
+                                                    const uint32_t* tmeta, uint32_t* hist) {
     launch_wait();
     __shared__ uint32_t h[8][kRadix];
     const int per = (ntiles + gridDim.x - 1) / gridDim.x;
@@ -377,9 +377,9 @@ struct SweepSmem {
 // FIRST: the index of a key is its position (iin is not read).
 template <class W, bool FIRST, int ITEMS>
 __global__ void __launch_bounds__(kSortThreads, 3) k_sweep(
-    const uint64_t* __restrict__ kin, const uint32_t* __restrict__ iin, int64_t n, int pass, int ntiles,
-    const uint32_t* __restrict__ tmeta, const uint32_t* __restrict__ hist, W* words, uint32_t* ticket,
-    uint64_t* __restrict__ kout, uint32_t* __restrict__ iout, int* status) {
+    const uint64_t* kin, const uint32_t* iin, int64_t n, int pass, int ntiles,
+    const uint32_t* tmeta, const uint32_t* hist, W* words, uint32_t* ticket,
+    uint64_t* kout, uint32_t* iout, int* status) {
     launch_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     SweepSmem<ITEMS>& S = *reinterpret_cast<SweepSmem<ITEMS>*>(smem_raw);
@@ -582,7 +582,7 @@ struct Gather8 {
     const int* stop;  // status word: with an error in it the particles stay as they are (NULL: not asked)
 };
 
-__global__ void k_gather_all(Gather8 G, unsigned long long* __restrict__ scratch, const uint32_t* __restrict__ perm,
+__global__ void k_gather_all(Gather8 G, unsigned long long* scratch, const uint32_t* perm,
                              int64_t n, int* status) {
     launch_wait();
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -603,7 +603,7 @@ __global__ void k_gather_all(Gather8 G, unsigned long long* __restrict__ scratch
 
 // The gathered arrays back into place (one launch; eight copies of a small
 // set's arrays cost their launches).
-__global__ void k_copy_back(Gather8 G, const unsigned long long* __restrict__ scratch, int64_t n) {
+__global__ void k_copy_back(Gather8 G, const unsigned long long* scratch, int64_t n) {
     launch_wait();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n || (G.stop && *G.stop)) return;

@@ -200,10 +200,10 @@ __device__ __forceinline__ NodeRange node_range(const uint64_t* __restrict__ key
 
 // Each particle's node range, and the nodes per level, and groups, of each
 // tile: cnt[row * ntiles + tile].
-__global__ void __launch_bounds__(kTreeThreads) k_tree_count(const uint64_t* __restrict__ key, int64_t n,
-                                                             const int64_t* __restrict__ off, int np, int n_leaf,
-                                                             int n_g, int64_t ntiles, uint16_t* __restrict__ range,
-                                                             uint32_t* __restrict__ cnt) {
+__global__ void __launch_bounds__(kTreeThreads) k_tree_count(const uint64_t* key, int64_t n,
+                                                             const int64_t* off, int np, int n_leaf,
+                                                             int n_g, int64_t ntiles, uint16_t* range,
+                                                             uint32_t* cnt) {
     launch_wait();
     __shared__ uint32_t h[kTreeRows];
     if (threadIdx.x < kTreeRows) h[threadIdx.x] = 0;
@@ -238,8 +238,8 @@ __global__ void __launch_bounds__(kTreeThreads) k_tree_count(const uint64_t* __r
 
 // The level bounds and the node, group and leaf counts from the scanned
 // counts: sz words kSzLvl.., kSzNg and kSzNl, cut at the node capacity (overflow flagged).
-__global__ void k_tree_sizes(const uint32_t* __restrict__ scan, int64_t ntiles,
-                             const unsigned long long* __restrict__ total, unsigned long long cap,
+__global__ void k_tree_sizes(const uint32_t* scan, int64_t ntiles,
+                             const unsigned long long* total, unsigned long long cap,
                              unsigned long long* sz) {
     launch_wait();
     const int l = threadIdx.x;
@@ -259,11 +259,11 @@ __global__ void k_tree_sizes(const uint32_t* __restrict__ scan, int64_t ntiles,
 // Nodes (level, begin, first child; end and parent of the roots), groups and
 // leaves (by first particle), and the highest node that begins at a particle.
 __global__ void __launch_bounds__(kTreeThreads) k_tree_write(
-    const uint16_t* __restrict__ range, int64_t n, const int64_t* __restrict__ off, int np, int64_t ntiles,
-    const uint32_t* __restrict__ scan, int64_t cap, uint8_t* __restrict__ level,
-    uint32_t* __restrict__ begin, uint32_t* __restrict__ end, int32_t* __restrict__ parent,
-    int32_t* __restrict__ first_child, uint8_t* __restrict__ nchild, int32_t* __restrict__ groups,
-    int32_t* __restrict__ leaves, int32_t* __restrict__ top) {
+    const uint16_t* range, int64_t n, const int64_t* off, int np, int64_t ntiles,
+    const uint32_t* scan, int64_t cap, uint8_t* level,
+    uint32_t* begin, uint32_t* end, int32_t* parent,
+    int32_t* first_child, uint8_t* nchild, int32_t* groups,
+    int32_t* leaves, int32_t* top) {
     launch_wait();
     __shared__ uint32_t base[kTreeRows][32];  // per (round, warp): nodes of the row before it in the tile, then ids
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -336,13 +336,13 @@ __global__ void __launch_bounds__(kTreeThreads) k_tree_write(
 
 // Children of every node that splits: parent links, child count, and each
 // child's end (the next one's begin; the last one's by a search forward).
-__global__ void __launch_bounds__(128) k_tree_link(const uint64_t* __restrict__ key, const int64_t* __restrict__ off,
-                                                   int np, const unsigned long long* __restrict__ sz,
-                                                   const uint8_t* __restrict__ level,
-                                                   const uint32_t* __restrict__ begin, uint32_t* __restrict__ end,
-                                                   int32_t* __restrict__ parent,
-                                                   const int32_t* __restrict__ first_child,
-                                                   uint8_t* __restrict__ nchild) {
+__global__ void __launch_bounds__(128) k_tree_link(const uint64_t* key, const int64_t* off,
+                                                   int np, const unsigned long long* sz,
+                                                   const uint8_t* level,
+                                                   const uint32_t* begin, uint32_t* end,
+                                                   int32_t* parent,
+                                                   const int32_t* first_child,
+                                                   uint8_t* nchild) {
     launch_wait();
     if (sz[kSzOvf]) return;  // (a device-sized build that outgrew its nodes)
     const int64_t nn = (int64_t)sz[kSzLvl + kLevels + 2];
@@ -405,10 +405,10 @@ __device__ __forceinline__ int32_t skip_of(uint32_t e, int64_t n, int np, const 
 // Integer tight boxes (grid coordinates recovered from the keys) and the
 // packed records the walk reads (WalkNode).
 __global__ void __launch_bounds__(kSpanThreads) k_boxes(
-    const uint64_t* __restrict__ key, int64_t n, int np, const uint8_t* __restrict__ level,
-    const uint32_t* __restrict__ begin, const uint32_t* __restrict__ end, const int32_t* __restrict__ first_child,
-    const uint8_t* __restrict__ nchild, const int32_t* __restrict__ top, uint32_t* qlo, uint32_t* qhi,
-    WalkNode* wnode, const unsigned long long* __restrict__ lvl, int lev_hi, int lev_lo) {
+    const uint64_t* key, int64_t n, int np, const uint8_t* level,
+    const uint32_t* begin, const uint32_t* end, const int32_t* first_child,
+    const uint8_t* nchild, const int32_t* top, uint32_t* qlo, uint32_t* qhi,
+    WalkNode* wnode, const unsigned long long* lvl, int lev_hi, int lev_lo) {
     launch_wait();
     struct Pre {
         uint32_t b, e;
@@ -478,10 +478,10 @@ __global__ void __launch_bounds__(kSpanThreads) k_boxes(
 // Moments of the nodes (children already done).
 template <int ORDER>
 __global__ void __launch_bounds__(kSpanThreads) k_moments(
-    const uint32_t* __restrict__ begin, const uint32_t* __restrict__ end, const int32_t* __restrict__ first_child,
-    const uint8_t* __restrict__ nchild, const double* __restrict__ x, const double* __restrict__ y,
-    const double* __restrict__ z, const double* __restrict__ m, double* M, double* cx, double* cy, double* cz,
-    double* Q, const unsigned long long* __restrict__ lvl, int lev_hi, int lev_lo) {
+    const uint32_t* begin, const uint32_t* end, const int32_t* first_child,
+    const uint8_t* nchild, const double* x, const double* y,
+    const double* z, const double* m, double* M, double* cx, double* cy, double* cz,
+    double* Q, const unsigned long long* lvl, int lev_hi, int lev_lo) {
     launch_wait();
     struct Pre {
         uint32_t b, e;
@@ -606,7 +606,7 @@ __device__ __forceinline__ float dsub(float ah, float al, float bh, float bl) {
 // A node's record from its mass, reference point, centre offset and quadrupole.
 __device__ __forceinline__ void put_moments32(int64_t k, float Mk, df Md, const float (&rh)[3], const float (&rl)[3],
                                               const float (&dc)[3], const float (&q)[6], float4* cell32,
-                                              float* __restrict__ mlo) {
+                                              float* mlo) {
     // centre = reference + offset, renormalised into a hi/lo pair
     float ch[3], cl[3];
 #pragma unroll
@@ -637,14 +637,14 @@ __device__ __forceinline__ void put_moments32(int64_t k, float Mk, df Md, const 
 constexpr int kLeafTile = 128, kLeafCap = 640;
 
 template <int ORDER>
-__global__ void __launch_bounds__(kLeafTile) k_leaf32(const int32_t* __restrict__ leaves,
-                                                      const unsigned long long* __restrict__ dnl,
-                                                      const uint32_t* __restrict__ begin,
-                                                      const uint32_t* __restrict__ end,
-                                                      const double* __restrict__ x, const double* __restrict__ y,
-                                                      const double* __restrict__ z, const double* __restrict__ m,
+__global__ void __launch_bounds__(kLeafTile) k_leaf32(const int32_t* leaves,
+                                                      const unsigned long long* dnl,
+                                                      const uint32_t* begin,
+                                                      const uint32_t* end,
+                                                      const double* x, const double* y,
+                                                      const double* z, const double* m,
                                                       float4* phi, float4* plo, float4* cell32,
-                                                      float* __restrict__ mlo) {
+                                                      float* mlo) {
     launch_wait();
     __shared__ float4 sh[kLeafCap], sl[kLeafCap];
     const int64_t nl = (int64_t)*dnl;
@@ -654,20 +654,23 @@ __global__ void __launch_bounds__(kLeafTile) k_leaf32(const int32_t* __restrict_
         const bool mine = t0 + threadIdx.x < t1;
         const int64_t k = mine ? leaves[t0 + threadIdx.x] : 0;
         const uint32_t b = mine ? begin[k] : 0u, e = mine ? end[k] : 0u;
-#pragma unroll 2
-        for (uint32_t i = p0 + threadIdx.x; i < p1; i += kLeafTile) {
-            const double v[3] = {x[i], y[i], z[i]}, mi = m[i];
-            float h[3], l[3], mh, ml;
+        auto put = [&](uint32_t i, const double (&v)[4]) {
+            float h[4], l[4];
 #pragma unroll
-            for (int a = 0; a < 3; ++a) split_f32(v[a], h[a], l[a]);
-            split_f32(mi, mh, ml);
-            const float4 H = make_float4(h[0], h[1], h[2], mh), L = make_float4(l[0], l[1], l[2], ml);
+            for (int a = 0; a < 4; ++a) split_f32(v[a], h[a], l[a]);
+            const float4 H = make_float4(h[0], h[1], h[2], h[3]), L = make_float4(l[0], l[1], l[2], l[3]);
             phi[i] = H;
             plo[i] = L;
             if (i - p0 < kLeafCap) {
                 sh[i - p0] = H;
                 sl[i - p0] = L;
             }
+        };
+        for (uint32_t i = p0 + threadIdx.x; i < p1; i += 2 * kLeafTile) {  // two particles' loads in flight
+            const uint32_t j = min(i + kLeafTile, p1 - 1u);
+            const double v[4] = {x[i], y[i], z[i], m[i]}, w[4] = {x[j], y[j], z[j], m[j]};
+            put(i, v);
+            if (i + kLeafTile < p1) put(j, w);
         }
         __syncthreads();
         if (mine) {
@@ -715,8 +718,8 @@ __global__ void __launch_bounds__(kLeafTile) k_leaf32(const int32_t* __restrict_
 // Moments of the inner nodes, from their children's.
 template <int ORDER>
 __global__ void __launch_bounds__(kSpanThreads) k_moments32(
-    const int32_t* __restrict__ first_child, const uint8_t* __restrict__ nchild, float4* cell32, float* mlo,
-    const unsigned long long* __restrict__ lvl, int lev_hi, int lev_lo) {
+    const int32_t* first_child, const uint8_t* nchild, float4* cell32, float* mlo,
+    const unsigned long long* lvl, int lev_hi, int lev_lo) {
     launch_wait();
     struct Pre {
         int32_t f;

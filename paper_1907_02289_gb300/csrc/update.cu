@@ -10,15 +10,16 @@ namespace {
 
 // abort (a list-constructing graph step): nonzero overflow bits mean the
 // step's forces were not computed, so the kick is skipped.
-__global__ void k_kick(int64_t n, double h, const double* __restrict__ ax, const double* __restrict__ ay,
-                       const double* __restrict__ az, double* __restrict__ vx, double* __restrict__ vy,
-                       double* __restrict__ vz, const unsigned long long* __restrict__ abort) {
+__global__ void k_kick(int64_t n, double h, const double* ax, const double* ay,
+                       const double* az, double* vx, double* vy,
+                       double* vz, const unsigned long long* abort) {
     launch_wait();
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n || (abort && *abort)) return;
-    vx[i] += h * ax[i];
-    vy[i] += h * ay[i];
-    vz[i] += h * az[i];
+    const double ux = vx[i] + h * ax[i], uy = vy[i] + h * ay[i], uz = vz[i] + h * az[i];
+    vx[i] = ux;
+    vy[i] = uy;
+    vz[i] = uz;
 }
 
 // Kick and drift; with ROT the frame then turns by omega dt (Sec. 4.4): x, y
@@ -29,10 +30,10 @@ __global__ void k_kick(int64_t n, double h, const double* __restrict__ ax, const
 // pass of 120 B per particle where the two move 192 B (four steps of the 2^24
 // ring 64.58 -> 64.07 ms, of the 2^26 ring 508.2 -> 506.1).
 template <bool ROT, bool TWICE>
-__global__ void k_kick_drift(int64_t n, double h, double dt, const double* __restrict__ ax,
-                             const double* __restrict__ ay, const double* __restrict__ az,
-                             double* __restrict__ vx, double* __restrict__ vy, double* __restrict__ vz,
-                             double* __restrict__ x, double* __restrict__ y, double* __restrict__ z, double c,
+__global__ void k_kick_drift(int64_t n, double h, double dt, const double* ax,
+                             const double* ay, const double* az,
+                             double* vx, double* vy, double* vz,
+                             double* x, double* y, double* z, double c,
                              double s) {
     launch_wait();
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -67,9 +68,9 @@ __global__ void k_kick_drift(int64_t n, double h, double dt, const double* __res
 constexpr int kDiagSums = 11, kDiagBlocks = 512, kDiagThreads = 256;
 
 __global__ void __launch_bounds__(kDiagThreads) k_diag_partial(
-    int64_t n, double GMc, const double* __restrict__ x, const double* __restrict__ y, const double* __restrict__ z,
-    const double* __restrict__ vx, const double* __restrict__ vy, const double* __restrict__ vz,
-    const double* __restrict__ m, double* __restrict__ part) {
+    int64_t n, double GMc, const double* x, const double* y, const double* z,
+    const double* vx, const double* vy, const double* vz,
+    const double* m, double* part) {
     launch_wait();
     __shared__ double sh[kDiagSums][kDiagThreads];
     double acc[kDiagSums];
@@ -100,7 +101,7 @@ __global__ void __launch_bounds__(kDiagThreads) k_diag_partial(
     if (threadIdx.x < kDiagSums) part[(int64_t)blockIdx.x * kDiagSums + threadIdx.x] = sh[threadIdx.x][0];
 }
 
-__global__ void k_diag_final(const double* __restrict__ part, double* out) {
+__global__ void k_diag_final(const double* part, double* out) {
     launch_wait();
     const int q = threadIdx.x;
     if (q >= kDiagSums) return;

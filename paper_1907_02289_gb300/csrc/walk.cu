@@ -427,10 +427,10 @@ __global__ void __launch_bounds__(32 * kCoopWarps) k_walk_coop(const WalkArgs A,
 // (each run in list order); jm[k] = index of the first far particle, and
 // the far interactions n_i x (far particles) are summed into *n_far.
 template <bool SPLIT>
-__global__ void k_expand(int64_t ng, const unsigned long long* __restrict__ dng, const int32_t* __restrict__ groups,
-                         const int64_t* __restrict__ pp_off, const int32_t* __restrict__ P, const uint32_t* __restrict__ begin,
-                         const uint32_t* __restrict__ end, const WalkNode* __restrict__ wn, WalkParams wp,
-                         const int64_t* __restrict__ jj_off, uint32_t* __restrict__ JJ, int64_t* __restrict__ jm,
+__global__ void k_expand(int64_t ng, const unsigned long long* dng, const int32_t* groups,
+                         const int64_t* pp_off, const int32_t* P, const uint32_t* begin,
+                         const uint32_t* end, const WalkNode* wn, WalkParams wp,
+                         const int64_t* jj_off, uint32_t* JJ, int64_t* jm,
                          unsigned long long* n_far) {
     launch_wait();
     if (dng) ng = min(ng, (int64_t)*dng);
@@ -517,10 +517,10 @@ __global__ void k_expand(int64_t ng, const unsigned long long* __restrict__ dng,
 // One warp per group: the group's stashed lists (slots of capP / capC
 // entries) to their places in the packed lists.  slots >= 0 (device-sized
 // build): only the groups below slots whose lists fit their slot.
-__global__ void k_unstash(int64_t ng, const unsigned long long* __restrict__ dng, int64_t slots,
-                          const int64_t* __restrict__ pp_off, const int64_t* __restrict__ pc_off,
-                          const int32_t* __restrict__ sP, const int32_t* __restrict__ sC, int64_t capP,
-                          int64_t capC, int32_t* __restrict__ P, int32_t* __restrict__ C) {
+__global__ void k_unstash(int64_t ng, const unsigned long long* dng, int64_t slots,
+                          const int64_t* pp_off, const int64_t* pc_off,
+                          const int32_t* sP, const int32_t* sC, int64_t capP,
+                          int64_t capC, int32_t* P, int32_t* C) {
     launch_wait();
     if (dng) ng = min(ng, (int64_t)*dng);
     const int lane = threadIdx.x & 31;
@@ -529,7 +529,7 @@ __global__ void k_unstash(int64_t ng, const unsigned long long* __restrict__ dng
         const int64_t p0 = pp_off[k], np = pp_off[k + 1] - p0, c0 = pc_off[k], nc = pc_off[k + 1] - c0;
         if (slots >= 0 && !(k < slots && np <= capP && nc <= capC)) continue;
         // four loads in flight per lane
-        auto copy = [&](int32_t* __restrict__ dst, const int32_t* __restrict__ src, int64_t cnt) {
+        auto copy = [&](int32_t* dst, const int32_t* src, int64_t cnt) {
             for (int64_t t0 = 0; t0 < cnt; t0 += 128) {
                 int32_t v[4];
 #pragma unroll
@@ -558,9 +558,9 @@ __global__ void k_unstash(int64_t ng, const unsigned long long* __restrict__ dng
 // of the split expansion widens the reach by 1e-5 of itself plus two cells,
 // so that no rounding of a coordinate into its cell can put a touching pair
 // into a far leaf.  Round-to-nearest operations throughout (no contraction).
-__global__ void k_walk_thresholds(const double* __restrict__ box, int np, double r_coll, int cyl,
-                                  long long* __restrict__ rcq, long long* __restrict__ rfar,
-                                  long long* __restrict__ period) {
+__global__ void k_walk_thresholds(const double* box, int np, double r_coll, int cyl,
+                                  long long* rcq, long long* rfar,
+                                  long long* period) {
     launch_wait();
     const int q = blockIdx.x * blockDim.x + threadIdx.x;
     if (q >= np) return;
@@ -584,7 +584,7 @@ __global__ void k_walk_thresholds(const double* __restrict__ box, int np, double
 }
 
 // Device-sized build: the list totals against the buffers' room.
-__global__ void k_list_room(const unsigned long long* __restrict__ tot, long long roomP, long long roomC,
+__global__ void k_list_room(const unsigned long long* tot, long long roomP, long long roomC,
                             long long roomJ, unsigned long long* sz) {
     launch_wait();
     if (threadIdx.x != 0) return;
