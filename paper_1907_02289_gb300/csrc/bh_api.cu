@@ -249,6 +249,11 @@ int read_status(Ctx* c) {
 
 namespace {
 
+int ensure_copy_stream(Ctx* c) {
+    if (!c->copy_stream) BH_CUDA(c, cudaStreamCreateWithFlags(&c->copy_stream, cudaStreamNonBlocking));
+    return BH_OK;
+}
+
 int build_tree(Ctx* c, bh_particles* p) {
     BH_TRY(check_particles(c, p, true));
     if (c->n_patches > 1 && p->n != c->h_off.back())
@@ -981,6 +986,7 @@ static int create_ctx(const char* who, const bh_params* p, int n_patches, const 
     if (e == cudaSuccess) e = cudaMalloc(&c->d_sz, bh::kSzWords * sizeof(unsigned long long));
     if (e == cudaSuccess) e = cudaHostAlloc(&c->h_pin, 64 * sizeof(unsigned long long), cudaHostAllocDefault);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->count_event, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->lists_event, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->d_sz, 0, bh::kSzWords * sizeof(unsigned long long), c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->d_status, 0, sizeof(int), c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
@@ -1034,6 +1040,7 @@ int bh_destroy(bh_ctx* ctx) {
     cudaFree(c->d_sz);
     if (c->h_pin) cudaFreeHost(c->h_pin);
     if (c->count_event) cudaEventDestroy(c->count_event);
+    if (c->lists_event) cudaEventDestroy(c->lists_event);
     using bh::release;
     release(c->d_off); release(c->tile_meta); release(c->box_map); release(c->box_poff); release(c->d_rcq); release(c->d_rfar); release(c->d_period); release(c->cyl); release(c->box_part); release(c->order_cnt); release(c->warp_time); release(c->contact_acc); release(c->diag); release(c->pot);
     release(c->ord_cnt);
@@ -1238,7 +1245,7 @@ int bh_step_host(bh_ctx* ctx, bh_particles* h, int nsteps) {
         BH_CUDA(c, cudaMemcpyAsync(d.id, h->id, n * sizeof(int64_t), cudaMemcpyHostToDevice, c->stream));
         c->h2d_bytes += n * (int64_t)sizeof(int64_t);
     }
-    if (!c->copy_stream) BH_CUDA(c, cudaStreamCreateWithFlags(&c->copy_stream, cudaStreamNonBlocking));
+    BH_TRY(bh::ensure_copy_stream(c));
     if (!c->pos_event) BH_CUDA(c, cudaEventCreateWithFlags(&c->pos_event, cudaEventDisableTiming));
     c->want_pos_event = true;
     c->pos_event_recorded = false;
@@ -1414,10 +1421,12 @@ int bh_get_counters(bh_ctx* ctx, bh_counters* out) {
     out->n_rebuilds = c->n_rebuilds;
     out->n_launches = c->n_launches;
     out->n_contacts = c->n_contacts;
-    if (c->far_pending) {  // an eager list build since: read its count now
+    if (c->far_pending) {  // an eager list build since: wait for it (not for what follows it) and read its count
         unsigned long long hf = 0;
-        BH_CUDA(c, cudaMemcpyAsync(&hf, c->d_small + 10, sizeof(hf), cudaMemcpyDeviceToHost, c->stream));
-        BH_CUDA(c, cudaStreamSynchronize(c->stream));
+        BH_TRY(bh::ensure_copy_stream(c));
+        BH_CUDA(c, cudaStreamWaitEvent(c->copy_stream, c->lists_event, 0));
+        BH_CUDA(c, cudaMemcpyAsync(&hf, c->d_small + 10, sizeof(hf), cudaMemcpyDeviceToHost, c->copy_stream));
+        BH_CUDA(c, cudaStreamSynchronize(c->copy_stream));
         c->n_int_pp_far = (int64_t)hf;
         c->far_pending = false;
     }

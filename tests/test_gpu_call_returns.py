@@ -1,0 +1,43 @@
+"""What a call has done by the time it returns.  Work of the test's own, of a
+tenth of a second, is put on the context's stream, so that a call that waits for the
+stream, or returns before work that it should have waited for, is seen."""
+import pytest
+
+from paper_1907_02289_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+SLEEP = 200_000_000  # GPU clock cycles, about 0.1 s
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import __graft_entry__
+    __graft_entry__.build()
+
+
+def context(P, precision=1, stream=None, **kw):
+    from paper_1907_02289_gb300 import bh
+    _, prm = synth.make("ring1m_fp64", 16)
+    ctx = bh.Context(stream=stream, **dict(prm, precision=precision, **kw))
+    return ctx, bh.Particles(P)
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+def test_counters_do_not_wait_after_a_list_build(precision):
+    import torch
+    P = synth.ring(20000, 5, phi_max=0.2)
+    s = torch.cuda.Stream()
+    ctx, D = context(P, precision, s.cuda_stream, n_g=64)
+    torch.cuda.synchronize()
+    ctx.bh_build_tree(D)
+    ctx.bh_make_lists()
+    with torch.cuda.stream(s):
+        torch.cuda._sleep(SLEEP)
+    far = ctx.bh_get_counters()["n_pp_far"]
+    assert not s.query(), "the counters waited for the stream"
+    s.synchronize()
+    assert far > 0 if precision else far == 0
+    ctx.close()
