@@ -22,9 +22,11 @@
  *  - Tree, list and scratch buffers are LIBRARY-OWNED device memory inside
  *    the context; they are allocated with cudaMalloc and grown on demand.
  *  - Work is issued on the CUDA stream given to bh_create.  Calls that must
- *    size buffers (building trees and lists) synchronise that stream; force
- *    and step calls do not, except where stated (on the FP32 path with
- *    contacts an eager evaluation waits for its contact count).  Device-side error words are
+ *    size buffers (building trees and lists) wait for those sizes; force
+ *    and step calls do not wait, except where stated (on the FP32 path with
+ *    contacts an eager evaluation waits for its contact count).  On return
+ *    from any call but bh_sync and the read-backs the stream may still be
+ *    busy.  Device-side error words are
  *    checked at the next synchronising call (or bh_sync).
  *  - bh_get_* read-back functions copy into CALLER-OWNED HOST buffers sized
  *    from bh_get_sizes, and synchronise the stream.
@@ -223,15 +225,18 @@ int bh_set_stream(bh_ctx* ctx, void* stream);
 
 /* Sec. 4.2 step 3a (list-constructing step): root box and Morton keys,
  * stable radix sort, in-place permutation of the particle arrays into key
- * order, level-by-level octree (BFS numbering), integer node boxes, node
- * moments and groups.  Synchronises.  Errors: BH_E_INVAL for n < 1 or
+ * order, octree (BFS numbering), integer node boxes, node
+ * moments and groups.  Waits for the tree's sizes and, at the end, until
+ * nothing uses the particle arrays any more (the last passes over the
+ * library's own tree may still run).  Errors: BH_E_INVAL for n < 1 or
  * n >= 2^31 or a non-finite coordinate. */
 int bh_build_tree(bh_ctx* ctx, bh_particles* p);
 
 /* Sec. 4.2 step 3d, first half: one depth-first walk per group builds its
  * particle list (opened leaves) and cell list (accepted nodes), both in
  * order of first particle, and the list-reuse schedule starts.
- * Synchronises.  BH_E_STATE without a tree. */
+ * Waits for the lists' sizes; they may still be written on return.
+ * BH_E_STATE without a tree. */
 int bh_make_lists(bh_ctx* ctx);
 
 /* Sec. 4.2 step 3d, second half (and the list-reusing step): refresh node

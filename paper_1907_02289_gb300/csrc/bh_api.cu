@@ -254,7 +254,11 @@ int ensure_copy_stream(Ctx* c) {
     return BH_OK;
 }
 
-int build_tree(Ctx* c, bh_particles* p) {
+// hand_back: return when the caller's arrays are no longer used.  The moments
+// are the last to read them; the boxes, which come from the keys, are then
+// issued behind them and keep the GPU busy through the wait (stage timing
+// keeps them where they belong).
+int build_tree(Ctx* c, bh_particles* p, bool hand_back = false) {
     BH_TRY(check_particles(c, p, true));
     if (c->n_patches > 1 && p->n != c->h_off.back())
         return fail(c, BH_E_INVAL, "n = %lld but the patches hold %lld particles", (long long)p->n,
@@ -269,11 +273,15 @@ int build_tree(Ctx* c, bh_particles* p) {
     BH_STAGE(c, BH_STAGE_SORT, stage_sort(c));
     BH_STAGE(c, BH_STAGE_PERMUTE, stage_permute(c, p));
     BH_TRY(stage_begin(c, BH_STAGE_TREE));
+    const bool boxes_last = hand_back && !c->timing;
     int rc = stage_octree(c);  // (reports the keys' errors too: the stage is closed either way)
-    if (rc == BH_OK) rc = stage_boxes(c);
+    if (rc == BH_OK && !boxes_last) rc = stage_boxes(c);
     BH_TRY(stage_end(c));
     BH_TRY(rc);
     BH_TRY(stage_moments(c, p));
+    if (hand_back) BH_CUDA(c, cudaEventRecord(c->read_event, c->stream));
+    if (boxes_last) BH_TRY(stage_boxes(c));
+    if (hand_back) BH_CUDA(c, cudaEventSynchronize(c->read_event));
     BH_STAGE(c, BH_STAGE_GROUPS, BH_OK);  // (found with the octree: the stage takes no time of its own)
     c->have_tree = true;
     return BH_OK;
@@ -985,7 +993,7 @@ static int create_ctx(const char* who, const bh_params* p, int n_patches, const 
     if (e == cudaSuccess) e = cudaMalloc(&c->d_small, 64 * sizeof(unsigned long long));
     if (e == cudaSuccess) e = cudaMalloc(&c->d_sz, bh::kSzWords * sizeof(unsigned long long));
     if (e == cudaSuccess) e = cudaHostAlloc(&c->h_pin, 64 * sizeof(unsigned long long), cudaHostAllocDefault);
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->count_event, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->read_event, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->lists_event, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->d_sz, 0, bh::kSzWords * sizeof(unsigned long long), c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->d_status, 0, sizeof(int), c->stream);
@@ -1039,7 +1047,7 @@ int bh_destroy(bh_ctx* ctx) {
     cudaFree(c->d_small);
     cudaFree(c->d_sz);
     if (c->h_pin) cudaFreeHost(c->h_pin);
-    if (c->count_event) cudaEventDestroy(c->count_event);
+    if (c->read_event) cudaEventDestroy(c->read_event);
     if (c->lists_event) cudaEventDestroy(c->lists_event);
     using bh::release;
     release(c->d_off); release(c->tile_meta); release(c->box_map); release(c->box_poff); release(c->d_rcq); release(c->d_rfar); release(c->d_period); release(c->cyl); release(c->box_part); release(c->order_cnt); release(c->warp_time); release(c->contact_acc); release(c->diag); release(c->pot);
@@ -1080,7 +1088,7 @@ int bh_set_stream(bh_ctx* ctx, void* stream) {
 int bh_build_tree(bh_ctx* ctx, bh_particles* p) {
     Ctx* c = (Ctx*)ctx;
     if (!c) return BH_E_INVAL;
-    return bh::build_tree(c, p);
+    return bh::build_tree(c, p, true);
 }
 
 int bh_make_lists(bh_ctx* ctx) {

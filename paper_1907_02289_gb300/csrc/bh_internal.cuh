@@ -132,7 +132,7 @@ struct Ctx {
     double* d_box = nullptr;   // per patch: lo[3], L, S, spare x3 (8 doubles)
     unsigned long long* d_small = nullptr;  // scan totals etc. (64 words)
     unsigned long long* h_pin = nullptr;    // page-locked words for size read-backs (64)
-    cudaEvent_t count_event = nullptr;      // the contact count has been copied to h_pin
+    cudaEvent_t read_event = nullptr;       // what the host waits for: a copied count, the last read of an array
 
     // keys and sort
     DBuf<uint64_t> key[2];

@@ -1519,7 +1519,7 @@ int launch_force32(Ctx* c, bh_particles* p, const ForceParams& fp, bool add_cent
         if (read) {
             BH_CUDA(c, cudaMemcpyAsync(c->h_pin, A.ncontact, sizeof(unsigned long long), cudaMemcpyDeviceToHost,
                                        c->stream));
-            BH_CUDA(c, cudaEventRecord(c->count_event, c->stream));
+            BH_CUDA(c, cudaEventRecord(c->read_event, c->stream));
         }
         if (contact) BH_TRY(contact_pass(c, A, fp, p));
         BH_TRY(refine_pass(c, A, fp));
@@ -1527,7 +1527,7 @@ int launch_force32(Ctx* c, bh_particles* p, const ForceParams& fp, bool add_cent
         // the host waits for the count alone (the passes run on); on overflow
         // it grows the list and evaluates again.  Inside a captured graph
         // nothing is read back: an overflow is flagged in the status word.
-        BH_CUDA(c, cudaEventSynchronize(c->count_event));
+        BH_CUDA(c, cudaEventSynchronize(c->read_event));
         const int64_t np = (int64_t)c->h_pin[0];
         c->n_contacts = np;
         if (np <= A.contact_cap) break;

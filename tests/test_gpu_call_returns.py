@@ -41,3 +41,25 @@ def test_counters_do_not_wait_after_a_list_build(precision):
     s.synchronize()
     assert far > 0 if precision else far == 0
     ctx.close()
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("order", [1, 2])
+def test_build_tree_hands_the_arrays_back(precision, order):
+    """The particles may be written from another stream once bh_build_tree has
+    returned: nothing of it still reads them (its moments did)."""
+    import torch
+    P = synth.ring(1 << 21, 7)
+    ctx, D = context(P, precision, torch.cuda.Stream().cuda_stream, order=order)
+    other = torch.cuda.Stream()
+    got = []
+    for spoil in (False, True):
+        ctx.bh_build_tree(D)
+        if spoil:
+            with torch.cuda.stream(other):
+                D.t["x"].add_(1.0)
+        got.append({f: v.copy() for f, v in ctx.bh_get_moments().items()})
+        torch.cuda.synchronize()
+    for f, v in got[0].items():
+        assert (v == got[1][f]).all(), f
+    ctx.close()
