@@ -363,7 +363,8 @@ int stage_lists_dev_walk(Ctx* c);                  // device-sized: walk, offset
 int stage_lists_dev_fill(Ctx* c);                  // device-sized: lists, expansion, group order
 
 // force.cu
-int build_order32(Ctx* c);                         // FP32 kernel's group order (per list build)
+int build_order32(Ctx* c);                         // FP32 kernel's work items (per list build)
+int reserve_force32(Ctx* c);                       // its buffers
 int stage_force(Ctx* c, bh_particles* p, bool add_central);
 int stage_potential(Ctx* c, const bh_particles* p, double* phi, double* W);  // self-gravity potential (FP64)
 

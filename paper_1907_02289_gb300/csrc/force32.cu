@@ -1404,6 +1404,27 @@ int contact_pass(Ctx* c, const Args& A, const ForceParams& fp, bh_particles* p) 
 }
 }  // namespace
 
+// Buffers of an evaluation, made with the lists: the first evaluation of a
+// context spent 120 us of its 190 (20,000-particle ring) on their allocation.
+int reserve_force32(Ctx* c) {
+    const size_t n = (size_t)c->n;
+    BH_TRY(grow(c, c->refine, n, "refinement queue"));
+    if (!(c->prm.r_coll > 0.0)) return BH_OK;
+    const size_t cap = n > 65536 ? n : 65536;
+    if (c->contacts.cap < cap) BH_TRY(grow(c, c->contacts, cap, "contact pairs"));
+    if (c->contact_acc.cap < 3 * n) {  // zero between evaluations
+        BH_TRY(grow(c, c->contact_acc, 3 * n, "contact sums"));
+        BH_CUDA(c, cudaMemsetAsync(c->contact_acc.p, 0, c->contact_acc.cap * sizeof(unsigned long long), c->stream));
+    }
+    BH_TRY(grow(c, c->cbnd, n, "contact-particle bounds"));
+    BH_TRY(grow(c, c->cslot, n, "contact-particle list slots"));
+    if (c->cflag.cap < n) {  // (likewise)
+        BH_TRY(grow(c, c->cflag, n, "contact-particle flags"));
+        BH_CUDA(c, cudaMemsetAsync(c->cflag.p, 0, c->cflag.cap * sizeof(unsigned), c->stream));
+    }
+    return BH_OK;
+}
+
 int launch_force32(Ctx* c, bh_particles* p, const ForceParams& fp, bool add_central) {
     Args A;
     A.ng = groups_bound(c);
@@ -1430,12 +1451,7 @@ int launch_force32(Ctx* c, bh_particles* p, const ForceParams& fp, bool add_cent
     A.ay = p->ay;
     A.az = p->az;
     const bool contact = c->prm.r_coll > 0.0;
-    const int64_t cap = c->n > 65536 ? c->n : 65536;
-    if (contact && c->contacts.cap < (size_t)cap) BH_TRY(grow(c, c->contacts, (size_t)cap, "contact pairs"));
-    if (contact && c->contact_acc.cap < 3 * (size_t)c->n) {  // zero between evaluations
-        BH_TRY(grow(c, c->contact_acc, 3 * (size_t)c->n, "contact sums"));
-        BH_CUDA(c, cudaMemsetAsync(c->contact_acc.p, 0, c->contact_acc.cap * sizeof(unsigned long long), c->stream));
-    }
+    BH_TRY(reserve_force32(c));
     A.contacts = reinterpret_cast<uint2*>(c->contacts.p);
     A.contact_cap = (int64_t)c->contacts.cap;
     if (c->capturing && c->tune.graph_contact_room > 0)  // the room a graph step may use
@@ -1472,14 +1488,8 @@ int launch_force32(Ctx* c, bh_particles* p, const ForceParams& fp, bool add_cent
     A.vy = p->vy;
     A.vz = p->vz;
     A.m = p->m;
-    BH_TRY(grow(c, c->refine, (size_t)c->n, "refinement queue"));
     A.refine = c->refine.p;
     if (contact) {
-        const bool fresh = c->cflag.cap < (size_t)c->n;
-        BH_TRY(grow(c, c->cbnd, (size_t)c->n, "contact-particle bounds"));
-        BH_TRY(grow(c, c->cslot, (size_t)c->n, "contact-particle list slots"));
-        BH_TRY(grow(c, c->cflag, (size_t)c->n, "contact-particle flags"));
-        if (fresh) BH_CUDA(c, cudaMemsetAsync(c->cflag.p, 0, c->cflag.cap * sizeof(unsigned), c->stream));
         A.cbnd = c->cbnd.p;
         A.cslot = c->cslot.p;
         A.cflag = c->cflag.p;

@@ -758,6 +758,8 @@ int stage_lists(Ctx* c) {
     if (c->far_pending) {                               // from here on
         BH_TRY(build_order32(c));
         BH_CUDA(c, cudaEventRecord(c->lists_event, c->stream));
+        const int rc = reserve_force32(c);  // (while the lists are written; the evaluation reports a lack of memory)
+        if (rc != BH_E_NOMEM) BH_TRY(rc);
     }
     return BH_OK;
 }

@@ -63,3 +63,23 @@ def test_build_tree_hands_the_arrays_back(precision, order):
     for f, v in got[0].items():
         assert (v == got[1][f]).all(), f
     ctx.close()
+
+
+@pytest.mark.parametrize("contacts", [False, True])
+def test_first_forces_allocate_nothing(contacts):
+    """The first evaluation finds its buffers: they are made with the lists."""
+    import torch
+    from paper_1907_02289_gb300 import bh
+    kw = {} if contacts else {"r_coll": 0.0}
+    small, D = context(synth.ring(1000, 9), **kw)  # (loads the kernels)
+    small.bh_step(D, 0)
+    small.bh_sync()
+    ctx, D = context(synth.ring(1 << 20, 9), **kw)
+    ctx.bh_build_tree(D)
+    ctx.bh_make_lists()
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    ctx.bh_compute_forces(D, bh.BH_FORCE_TREE_ONLY)
+    torch.cuda.synchronize()
+    assert torch.cuda.mem_get_info()[0] == free
+    ctx.close()
