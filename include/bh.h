@@ -221,6 +221,10 @@ int bh_create(const bh_params* p, void* stream, bh_ctx** out);
 int bh_batch_create(const bh_params* p, int n_patches, const int64_t* offsets, void* stream, bh_ctx** out);
 int bh_destroy(bh_ctx* ctx);
 const char* bh_last_error(const bh_ctx* ctx);
+/* Issue the calls that follow on another stream, which is made to wait for the
+ * last tree or list build (not when it is being captured: then the caller
+ * orders the two).  Other work of the caller's on either stream, and the
+ * particle arrays, are the caller's to order. */
 int bh_set_stream(bh_ctx* ctx, void* stream);
 
 /* Sec. 4.2 step 3a (list-constructing step): root box and Morton keys,

@@ -281,7 +281,10 @@ int build_tree(Ctx* c, bh_particles* p, bool hand_back = false) {
     BH_TRY(stage_moments(c, p));
     if (hand_back) BH_CUDA(c, cudaEventRecord(c->read_event, c->stream));
     if (boxes_last) BH_TRY(stage_boxes(c));
-    if (hand_back) BH_CUDA(c, cudaEventSynchronize(c->read_event));
+    if (hand_back) {
+        BH_CUDA(c, cudaEventRecord(c->build_event, c->stream));
+        BH_CUDA(c, cudaEventSynchronize(c->read_event));
+    }
     BH_STAGE(c, BH_STAGE_GROUPS, BH_OK);  // (found with the octree: the stage takes no time of its own)
     c->have_tree = true;
     return BH_OK;
@@ -994,7 +997,7 @@ static int create_ctx(const char* who, const bh_params* p, int n_patches, const 
     if (e == cudaSuccess) e = cudaMalloc(&c->d_sz, bh::kSzWords * sizeof(unsigned long long));
     if (e == cudaSuccess) e = cudaHostAlloc(&c->h_pin, 64 * sizeof(unsigned long long), cudaHostAllocDefault);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->read_event, cudaEventDisableTiming);
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->lists_event, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->build_event, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->d_sz, 0, bh::kSzWords * sizeof(unsigned long long), c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->d_status, 0, sizeof(int), c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
@@ -1048,7 +1051,7 @@ int bh_destroy(bh_ctx* ctx) {
     cudaFree(c->d_sz);
     if (c->h_pin) cudaFreeHost(c->h_pin);
     if (c->read_event) cudaEventDestroy(c->read_event);
-    if (c->lists_event) cudaEventDestroy(c->lists_event);
+    if (c->build_event) cudaEventDestroy(c->build_event);
     using bh::release;
     release(c->d_off); release(c->tile_meta); release(c->box_map); release(c->box_poff); release(c->d_rcq); release(c->d_rfar); release(c->d_period); release(c->cyl); release(c->box_part); release(c->order_cnt); release(c->warp_time); release(c->contact_acc); release(c->diag); release(c->pot);
     release(c->ord_cnt);
@@ -1081,7 +1084,17 @@ const char* bh_last_error(const bh_ctx* ctx) {
 int bh_set_stream(bh_ctx* ctx, void* stream) {
     Ctx* c = (Ctx*)ctx;
     if (!c) return BH_E_INVAL;
-    c->stream = (cudaStream_t)stream;
+    const cudaStream_t s = (cudaStream_t)stream;
+    // the last tree or list build may still be writing what the calls on the new
+    // stream read (a stream that is being captured cannot be made to wait)
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (s != c->stream) {
+        if (cudaStreamIsCapturing(s, &st) != cudaSuccess)
+            cudaGetLastError();
+        else if (st == cudaStreamCaptureStatusNone)
+            BH_CUDA(c, cudaStreamWaitEvent(s, c->build_event, 0));
+    }
+    c->stream = s;
     return BH_OK;
 }
 
@@ -1432,7 +1445,7 @@ int bh_get_counters(bh_ctx* ctx, bh_counters* out) {
     if (c->far_pending) {  // an eager list build since: wait for it (not for what follows it) and read its count
         unsigned long long hf = 0;
         BH_TRY(bh::ensure_copy_stream(c));
-        BH_CUDA(c, cudaStreamWaitEvent(c->copy_stream, c->lists_event, 0));
+        BH_CUDA(c, cudaStreamWaitEvent(c->copy_stream, c->build_event, 0));
         BH_CUDA(c, cudaMemcpyAsync(&hf, c->d_small + 10, sizeof(hf), cudaMemcpyDeviceToHost, c->copy_stream));
         BH_CUDA(c, cudaStreamSynchronize(c->copy_stream));
         c->n_int_pp_far = (int64_t)hf;

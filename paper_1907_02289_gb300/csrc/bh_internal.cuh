@@ -247,7 +247,7 @@ struct Ctx {
     int64_t n_int_pp = 0, n_int_pc = 0;
     int64_t n_int_pp_far = 0;            // FP32 path: pp interactions with far list particles
     bool far_pending = false;            // a list build ran since n_int_pp_far was read (word 10 of d_small)
-    cudaEvent_t lists_event = nullptr;   // that build's end
+    cudaEvent_t build_event = nullptr;   // end of the last eager tree or list build
     DBuf<int64_t> cnt_p, cnt_c, cnt_j;   // per group counts, then offsets (ng + 1)
     DBuf<int64_t> cnt_jm;                // FP32 path: per group index of the first far list particle
     DBuf<int32_t> stash_p, stash_c;      // per group list slots of the one-walk build

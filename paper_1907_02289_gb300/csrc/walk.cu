@@ -754,10 +754,11 @@ int stage_lists(Ctx* c) {
     c->walk_cap_c = (int64_t)(((h[13] + h[13] / 4 + 4) + 3) & ~3ull);
     BH_TRY(expand_lists(c, wp, nullptr, blocks_for(ng * 32, 256)));
     c->n_int_pp_far = 0;
-    c->far_pending = c->prm.precision == BH_PREC_FP32;  // its count is read when asked for,
-    if (c->far_pending) {                               // from here on
-        BH_TRY(build_order32(c));
-        BH_CUDA(c, cudaEventRecord(c->lists_event, c->stream));
+    const bool f32 = c->prm.precision == BH_PREC_FP32;
+    if (f32) BH_TRY(build_order32(c));
+    BH_CUDA(c, cudaEventRecord(c->build_event, c->stream));
+    c->far_pending = f32;  // its count is read when asked for
+    if (f32) {
         const int rc = reserve_force32(c);  // (while the lists are written; the evaluation reports a lack of memory)
         if (rc != BH_E_NOMEM) BH_TRY(rc);
     }

@@ -83,3 +83,25 @@ def test_first_forces_allocate_nothing(contacts):
     torch.cuda.synchronize()
     assert torch.cuda.mem_get_info()[0] == free
     ctx.close()
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+def test_a_new_stream_waits_for_the_lists(precision):
+    """bh_make_lists may return while its lists are written; calls on a stream set
+    then come after that."""
+    import ctypes
+
+    import torch
+    ctx, D = context(synth.ring(1 << 22, 11), precision, (s := torch.cuda.Stream()).cuda_stream, n_g=64)
+    ctx.bh_build_tree(D)
+    ctx.bh_make_lists()
+    torch.cuda.synchronize()
+    ctx.bh_make_lists()
+    new = torch.cuda.Stream()
+    assert ctx.lib.bh_set_stream(ctx.h, ctypes.c_void_p(new.cuda_stream)) == 0
+    ctx.bh_sync()
+    assert s.query(), "the list build was still running"
+    ctx.bh_compute_forces(D)
+    ctx.bh_sync()
+    assert new.query()
+    ctx.close()
