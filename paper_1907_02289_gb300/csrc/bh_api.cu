@@ -20,7 +20,7 @@ int fail(Ctx* c, int code, const char* fmt, ...) {
     return code;
 }
 
-int grow_raw(Ctx* c, void** p, size_t* cap, size_t need, const char* what, bool keep) {
+int grow_raw(Ctx* c, void** p, size_t* cap, size_t need, const char* what, bool in_steps) {
     if (need <= *cap && *p) return BH_OK;
     // a captured step cannot allocate: its buffers are sized before capture
     if (c->capturing) return fail(c, BH_E_STATE, "%s would have to grow inside a captured step", what);
@@ -37,17 +37,13 @@ int grow_raw(Ctx* c, void** p, size_t* cap, size_t need, const char* what, bool 
                     cudaGetErrorString(e));
     }
     if (*p) {
-        if (keep && *cap) {
-            e = cudaMemcpyAsync(q, *p, *cap, cudaMemcpyDeviceToDevice, c->stream);
-            if (e != cudaSuccess) return fail(c, BH_E_CUDA, "copy while growing %s: %s", what, cudaGetErrorString(e));
-        }
         e = cudaStreamSynchronize(c->stream);
         if (e != cudaSuccess) return fail(c, BH_E_CUDA, "sync while growing %s: %s", what, cudaGetErrorString(e));
         cudaFree(*p);
     }
     *p = q;
     *cap = bytes;
-    ++c->buf_gen;
+    if (in_steps) ++c->buf_gen;
     return BH_OK;
 }
 
@@ -1244,8 +1240,8 @@ int bh_step_host(bh_ctx* ctx, bh_particles* h, int nsteps) {
     BH_TRY(bh::check_particles(c, h, true));
     if (!h->id) return bh::fail(c, BH_E_INVAL, "id must be set");
     const int64_t n = h->n;
-    BH_TRY(bh::grow(c, c->hbuf, (size_t)n * 10, "host-step particle buffers"));
-    BH_TRY(bh::grow(c, c->hid, (size_t)n, "host-step ids"));
+    BH_TRY(bh::grow(c, c->hbuf, (size_t)n * 10, "host-step particle buffers", false));
+    BH_TRY(bh::grow(c, c->hid, (size_t)n, "host-step ids", false));
     double* b = c->hbuf.p;
     bh_particles d;
     d.x = b; d.y = b + n; d.z = b + 2 * n; d.vx = b + 3 * n; d.vy = b + 4 * n; d.vz = b + 5 * n;

@@ -45,12 +45,14 @@ struct DBuf {
 struct Ctx;
 int fail(Ctx* c, int code, const char* fmt, ...);
 
-// cudaMalloc-backed growth; returns BH_OK or BH_E_NOMEM (with message).
-int grow_raw(Ctx* c, void** p, size_t* cap, size_t bytes_needed, const char* what, bool keep);
+// cudaMalloc-backed growth (the contents are not kept); returns BH_OK or
+// BH_E_NOMEM (with message).  in_steps: a captured step may hold the buffer, so
+// that step is captured again once it has moved.
+int grow_raw(Ctx* c, void** p, size_t* cap, size_t bytes_needed, const char* what, bool in_steps);
 template <typename T>
-int grow(Ctx* c, DBuf<T>& b, size_t n, const char* what, bool keep = false) {
+int grow(Ctx* c, DBuf<T>& b, size_t n, const char* what, bool in_steps = true) {
     size_t cap_bytes = b.cap * sizeof(T);
-    int rc = grow_raw(c, (void**)&b.p, &cap_bytes, n * sizeof(T), what, keep);
+    int rc = grow_raw(c, (void**)&b.p, &cap_bytes, n * sizeof(T), what, in_steps);
     b.cap = cap_bytes / sizeof(T);
     return rc;
 }
@@ -205,7 +207,7 @@ struct Ctx {
     // sizes of the step being issued are read on the device, within bounds that
     // outlive the current lists (captured steps of either kind)
     bool dev_sizes = false;
-    int64_t buf_gen = 0;                 // library buffers (re)allocated so far
+    int64_t buf_gen = 0;                 // buffers that a captured step may hold (re)allocated so far
     bool graph_ok = false;               // graph_exec matches the current arrays and settings,
     int64_t graph_gen = 0;               // the buffers,
     int64_t graph_size[2] = {};          // and about the sizes: groups and nodes it was captured with

@@ -483,7 +483,7 @@ int stage_force(Ctx* c, bh_particles* p, bool add_central) {
 int stage_potential(Ctx* c, const bh_particles* p, double* phi, double* W) {
     BH_TRY(stage_moments64(c, p));  // FP64 moments of the current positions, either precision
     if (!phi) {
-        BH_TRY(grow(c, c->pot, (size_t)c->n, "potential"));
+        BH_TRY(grow(c, c->pot, (size_t)c->n, "potential", false));
         phi = c->pot.p;
     }
     const ForceParams fp = force_params(c);
@@ -491,7 +491,7 @@ int stage_potential(Ctx* c, const bh_particles* p, double* phi, double* W) {
     A.phi = phi;
     BH_TRY(launch_sum64<true>(c, A));
     if (W) {
-        BH_TRY(grow(c, c->diag, (size_t)kWBlocks + 1, "potential energy sums"));
+        BH_TRY(grow(c, c->diag, (size_t)kWBlocks + 1, "potential energy sums", false));
         BH_CUDA(c, launch(c, k_wsum_partial, kWBlocks, kWThreads, 0, c->n, p->m, phi, c->diag.p));
         BH_LAUNCH(c);
         BH_CUDA(c, launch(c, k_wsum_final, 1, 32, 0, c->diag.p, c->diag.p + kWBlocks));

@@ -1351,7 +1351,7 @@ int build_order32(Ctx* c) {
                       few};
     if (c->tune.order_window > 0 && ng > c->tune.order_window && !c->dev_build) {  // (device-sized: plain order)
         const int64_t words = (ng + O.window - 1) / O.window * kOrderBuckets;
-        BH_TRY(grow(c, c->ord_cnt, (size_t)words, "group order buckets of the windows"));
+        BH_TRY(grow(c, c->ord_cnt, (size_t)words, "group order buckets of the windows", false));
         BH_CUDA(c, cudaMemsetAsync(c->ord_cnt.p, 0, (size_t)words * sizeof(uint32_t), c->stream));
         BH_CUDA(c, launch(c, k_order_hist_windows, blocks_for(ng, 256), 256, 0, O, c->ord_cnt.p));
         BH_LAUNCH(c);
@@ -1508,7 +1508,7 @@ int launch_force32(Ctx* c, bh_particles* p, const ForceParams& fp, bool add_cent
             A.ticket = c->d_small + 17;
         }
         if (c->timing && !c->capturing) {
-            BH_TRY(grow(c, c->warp_time, 2 * (size_t)nb * W, "warp times"));
+            BH_TRY(grow(c, c->warp_time, 2 * (size_t)nb * W, "warp times", false));
             A.warp_time = c->warp_time.p;
             c->warp_time_n = (int64_t)nb * W;
         }

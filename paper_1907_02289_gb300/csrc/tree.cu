@@ -927,11 +927,9 @@ int stage_moments(Ctx* c, const bh_particles* p) {
 // diagnostic also uses them).
 int stage_moments64(Ctx* c, const bh_particles* p) {
     const int64_t nn = c->n_nodes;
-    BH_TRY(grow(c, c->M, (size_t)nn, "moments M"));
-    BH_TRY(grow(c, c->cx, (size_t)nn, "moments cx"));
-    BH_TRY(grow(c, c->cy, (size_t)nn, "moments cy"));
-    BH_TRY(grow(c, c->cz, (size_t)nn, "moments cz"));
-    BH_TRY(grow(c, c->Q, (size_t)nn * 6, "moments Q"));
+    const bool steps = c->prm.precision == BH_PREC_FP64;
+    for (auto* b : {&c->M, &c->cx, &c->cy, &c->cz}) BH_TRY(grow(c, *b, (size_t)nn, "moments", steps));
+    BH_TRY(grow(c, c->Q, (size_t)nn * 6, "moments Q", steps));
     BH_TRY(stage_begin(c, BH_STAGE_MOMENTS));
     BH_TRY(launch_levels(c, kSpanMoments64, c->prm.order >= 2 ? k_moments<2> : k_moments<1>, c->begin.p, c->end.p, c->first_child.p,
                          c->nchild.p, p->x, p->y, p->z, p->m, c->M.p, c->cx.p, c->cy.p, c->cz.p, c->Q.p));

@@ -113,7 +113,7 @@ __global__ void k_diag_final(const double* part, double* out) {
 }  // namespace
 
 int stage_diagnostics(Ctx* c, const bh_particles* p, double* host_out) {
-    BH_TRY(grow(c, c->diag, (size_t)kDiagBlocks * kDiagSums + kDiagSums, "diagnostic sums"));
+    BH_TRY(grow(c, c->diag, (size_t)kDiagBlocks * kDiagSums + kDiagSums, "diagnostic sums", false));
     double* part = c->diag.p;
     double* out = part + (size_t)kDiagBlocks * kDiagSums;
     BH_CUDA(c, launch(c, k_diag_partial, kDiagBlocks, kDiagThreads, 0, p->n, c->prm.G * c->prm.M_central,

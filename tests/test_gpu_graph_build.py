@@ -189,3 +189,49 @@ def test_force_kernel_timed_in_graph_steps(graph):
     ctx.bh_set_timing(True)
     ms, launches = ctx.bh_get_timing(reset=True)
     assert launches == 0
+
+
+@pytest.mark.parametrize("graph", [1, 2])
+def test_read_backs_leave_the_step_graphs(graph):
+    """The step graphs are kept over list builds, and over calls whose buffers
+    no step holds (diagnostics, the potential, timed launches)."""
+    from paper_1907_02289_gb300 import bh
+    P, prm = synth.ring(20000, 37), _ring_prm()
+    captures, states = [], []
+    for reads in (False, True):
+        ctx = bh.Context(**prm)
+        ctx.bh_set_tuning(graph=graph, sched=2)
+        D = bh.Particles(P)
+        ctx.bh_step(D, 32)  # (buffers of the first sizes have grown once and have room)
+        ctx.bh_sync()
+        first = ctx.bh_get_counters()["n_graph_captures"]
+        for k in range(4):
+            if reads:
+                ctx.bh_set_timing(k % 2 == 0)
+                ctx.bh_compute_potential(D, None)
+                ctx.bh_get_diagnostics(D)
+            ctx.bh_step(D, 8)
+            ctx.bh_sync()
+        captures.append((first, ctx.bh_get_counters()["n_graph_captures"]))
+        states.append(D.numpy())
+        ctx.close()
+    assert captures[0] == captures[1]
+    assert captures[0][0] == captures[0][1], "captured again on a steady ring"
+    for f in states[0]:
+        assert np.array_equal(states[0][f], states[1][f]), f
+
+
+def test_moved_buffers_are_captured_again():
+    """A tree that outgrows its buffers moves them: the kept graphs are made
+    again, and give the bits of the eager steps."""
+    P = synth.uniform_cube(20000, 35)
+    prm = _cube_prm(precision=1, order=2)
+    c0, D0 = _run(P, prm, 0, [3, 4, 4], between=_cluster)
+    c1, D1 = _run(P, prm, 1, [3], tune=dict(graph_room=0))
+    before = c1.bh_get_counters()["n_graph_captures"]
+    _cluster(0, D1)
+    for k in (4, 4):
+        c1.bh_step(D1, k)
+        c1.bh_sync()
+    _same_state(c0, D0, c1, D1)
+    assert c1.bh_get_counters()["n_graph_captures"] >= before + 2
