@@ -290,11 +290,20 @@ __global__ void __launch_bounds__(128) k_walk(const WalkArgs A, const WalkParams
 // untested entries at a time are tested, then every opened inner node is
 // replaced by its children in its place, so the order stays depth first and
 // ends as the lists' order.  An entry is a node id with its state in the top
-// two bits; an opened node becomes (first child, child count - 1).  Groups
-// whose entries outgrow the buffer are walked by one lane.  Measured, the walk
-// by a thread and by a warp per group: 65,537-particle ring (1166 groups) 151
-// and 18 us; 100,003-particle cube (4096 groups of 1300 entries) 865 and 77 us.
-constexpr int kCoopWarps = 4, kCoopCap = 2048;
+// two bits; an opened node becomes (first child, child count - 1).  Measured,
+// the walk by a thread and by a warp per group: 65,537-particle ring (1166
+// groups) 151 and 18 us; 100,003-particle cube (4096 groups of 1300 entries) 865
+// and 77 us.
+//
+// Entries that outgrow the buffer are walked in pieces (coop_pieces): the back
+// of the buffer holds those whose turn has not come, and a piece from their
+// front that fits what is free goes through the same levels in the front of the
+// buffer, its settled entries leaving for the lists.
+constexpr int kCoopWarps = 4;
+constexpr uint32_t kCoopLevel = 2048;  // most entries before a level is taken in pieces
+// room beyond: a piece of one opened node adds at most 7 entries per level
+constexpr uint32_t kCoopSpare = 7 * kLevels + 13, kCoopCap = kCoopLevel + kCoopSpare;
+static_assert(kCoopSpare >= 7 * kLevels + 8, "the last of a chain of opened nodes needs eight places");
 constexpr int64_t kCoopGroups = 40000;  // most groups it is chosen for
 constexpr uint32_t kEntNew = 0u, kEntCell = 1u << 30, kEntLeaf = 2u << 30, kEntOpen = 3u << 30;
 constexpr int kEntBits = 27;  // node id bits beside an opened node's 3 bits of child count
@@ -310,103 +319,210 @@ __device__ __forceinline__ uint32_t warp_exclusive(uint32_t v, int lane, uint32_
     return x - v;
 }
 
+// Places an entry takes once it is opened.
+__device__ __forceinline__ uint32_t places(uint32_t v) {
+    return v >= kEntOpen ? ((v >> kEntBits) & 7u) + 1u : 1u;
+}
+
+// One group's walk by the lanes of a warp (all calls warp-uniform).
 template <int MODE>
-__global__ void __launch_bounds__(32 * kCoopWarps) k_walk_coop(const WalkArgs A, const WalkParams wp) {
+struct CoopWalk {
+    const WalkArgs& A;
+    const WalkParams& wp;
+    const WalkGroup W;
+    uint32_t* E;  // kCoopCap entries
+    int lane;
+    uint32_t nj = 0, nown = 0;  // of this lane's tests
+    int64_t np = 0, nc = 0;     // entries sent to the lists
+
+    // Test the untested entries of E[0, len); whether any was opened, and how
+    // many more places the opened ones need.
+    __device__ __forceinline__ bool test(uint32_t len, uint32_t* more) {
+        uint32_t grow = 0;  // (an opened node with one child is replaced without growth)
+        bool opened = false;
+        for (uint32_t t = lane; t < len; t += 32) {
+            const uint32_t v = E[t];
+            if (v >> 30) continue;
+            const WalkNode R = A.wn[v];
+            const long long d2 = box_gap2(R, W.glo, W.ghi, W.period);
+            uint32_t r = kEntCell | v;
+            if (d2 < wp.D[(R.a.x >> kLevels) & 31u] || d2 <= W.rcq) {
+                const uint32_t c = R.a.y >> kLevels;  // leaf: particles; inner: children
+                if (R.a.x & kWalkLeaf) {
+                    r = kEntLeaf | v;
+                    const uint32_t lb = R.b.w, cnt = c == kWalkCntMax ? A.end[v] - lb : c;
+                    if (lb >= W.gb && lb < W.ge)
+                        nown += cnt;
+                    else
+                        nj += cnt;
+                } else {
+                    r = kEntOpen | (c - 1u) << kEntBits | R.b.w;
+                    grow += c - 1u;
+                    opened = true;
+                }
+            }
+            E[t] = r;
+        }
+        const bool any = __any_sync(0xffffffffu, opened);
+        *more = __reduce_add_sync(0xffffffffu, grow);
+        __syncwarp();
+        return any;
+    }
+
+    // Opened entries of E[0, len) -> their children, untested, in their places;
+    // from the back: an entry never moves to a lower place.
+    __device__ __forceinline__ void expand(uint32_t len, uint32_t more) {
+        uint32_t out = len + more;
+        for (int t0 = (int)((len - 1) & ~31u); t0 >= 0; t0 -= 32) {
+            const uint32_t t = (uint32_t)t0 + lane;
+            const uint32_t v = t < len ? E[t] : 0u;
+            const uint32_t c = t < len ? places(v) : 0u;
+            uint32_t tot;
+            const uint32_t x = warp_exclusive(c, lane, &tot);
+            out -= tot;
+            __syncwarp();
+            if (t < len && v >= kEntOpen) {
+                const uint32_t f = v & ((1u << kEntBits) - 1u);
+                for (uint32_t u = 0; u < c; ++u) E[out + x + u] = kEntNew | (f + u);
+            } else if (t < len) {
+                E[out + x] = v;
+            }
+            __syncwarp();
+        }
+    }
+
+    // The lanes' settled entries v (those that have one) -> the lists.
+    __device__ __forceinline__ void put(uint32_t v, bool has) {
+        const bool isP = has && (v >> 30) == (kEntLeaf >> 30), isC = has && !isP;
+        const unsigned mP = __ballot_sync(0xffffffffu, isP), mC = __ballot_sync(0xffffffffu, isC);
+        if (MODE != kWalkCount) {
+            const unsigned lt = (1u << lane) - 1u;
+            const int64_t p = np + __popc(mP & lt), c = nc + __popc(mC & lt);
+            if (isP && p < W.capP) W.P[W.baseP + p] = (int32_t)(v & 0x3fffffffu);
+            if (isC && c < W.capC) W.C[W.baseC + c] = (int32_t)(v & 0x3fffffffu);
+        }
+        np += __popc(mP);
+        nc += __popc(mC);
+    }
+
+    __device__ __forceinline__ void put_all(uint32_t len) {
+        for (uint32_t t0 = 0; t0 < len; t0 += 32) put(t0 + lane < len ? E[t0 + lane] : 0u, t0 + lane < len);
+    }
+};
+
+// The rest of a walk whose tested entries E[0, len) cannot all be opened in the
+// buffer.  E[at, kCoopCap) are the entries whose turn has not come, in order.
+// Those up to the first opened one go to the lists; then a piece from the
+// front of the rest, opened, moves to E[0, ..): as many entries as a quarter of the
+// free room holds (their children's children need room too; a half or a sixth
+// measures the same), at least one.  It is taken level by level until it is settled, or goes back when it does not
+// fit either, by then at least a level further.  Pieces of more than one entry
+// leave kCoopSpare places free, and those of one, a chain down the levels, add
+// at most 7 entries per level, so there is always room for the next one.
+// Measured, the list build of a 1,000,003-particle cube (32,768 groups) with such
+// groups walked by one lane, with k_walk, and with this: 6.4, 1.6 and 1.0 ms at
+// theta 0.5 (2150 entries a group), 13.7, 2.7 and 1.5 ms at theta 0.4 (3500); of a
+// 100,003-particle cube at theta 0.4 (4096 groups of 2350) 1.45, 1.69 and 0.22 ms.
+// Inlined, or the walk's state goes through memory: 3.5 instead of 1.5 ms.
+template <int MODE>
+__device__ __forceinline__ void coop_pieces(CoopWalk<MODE>& C, uint32_t len) {
+    uint32_t* E = C.E;
+    const int lane = C.lane;
+    uint32_t at = kCoopCap;
+    auto go_back = [&](uint32_t cnt) {  // E[0, cnt) -> in front of E[at, ..), from the back
+        for (int t0 = (int)((cnt - 1) & ~31u); t0 >= 0; t0 -= 32) {
+            const uint32_t t = (uint32_t)t0 + lane;
+            const uint32_t v = t < cnt ? E[t] : 0u;
+            __syncwarp();
+            if (t < cnt) E[at - cnt + t] = v;
+            __syncwarp();
+        }
+        at -= cnt;
+    };
+    go_back(len);
+    for (int64_t rounds = 0;; ++rounds) {
+        for (;;) {  // settled entries up to the first opened one
+            const uint32_t cnt = min(32u, kCoopCap - at);
+            const uint32_t v = (uint32_t)lane < cnt ? E[at + lane] : 0u;
+            const unsigned m = __ballot_sync(0xffffffffu, v >= kEntOpen);
+            const uint32_t k = m ? (uint32_t)(__ffs(m) - 1) : cnt;
+            C.put(v, (uint32_t)lane < k);
+            at += k;
+            if (m || at == kCoopCap) break;
+        }
+        if (at == kCoopCap) return;
+        const uint32_t room = at > kCoopSpare ? (at - kCoopSpare) / 4u : 0u;
+        uint32_t n = 0, need = 0;  // the piece's entries, and their places once opened
+        for (;;) {
+            const uint32_t cnt = min(32u, kCoopCap - at);
+            const uint32_t v = (uint32_t)lane < cnt ? E[at + lane] : 0u;
+            const uint32_t c = (uint32_t)lane < cnt ? places(v) : 0u;
+            uint32_t tot;
+            const uint32_t x = warp_exclusive(c, lane, &tot) + c;
+            const bool in = (uint32_t)lane < cnt && (need + x <= room || (n == 0 && lane == 0));
+            const uint32_t k = (uint32_t)__popc(__ballot_sync(0xffffffffu, in));
+            if (in) E[n + lane] = v;  // (n + lane < at + lane: read by now)
+            if (k > 0) need += __shfl_sync(0xffffffffu, x, (int)k - 1);
+            __syncwarp();
+            n += k;
+            at += k;
+            if (k < 32u) break;
+        }
+        if (need > at || rounds > C.A.nn) {  // never taken for a valid tree
+            if (lane == 0) atomicOr(C.A.status, kStatBounds);
+            return;
+        }
+        for (uint32_t more = need - n;;) {
+            C.expand(n, more);
+            n += more;
+            if (!C.test(n, &more)) {
+                C.put_all(n);
+                break;
+            }
+            if (n + more + kCoopSpare > at) {
+                go_back(n);
+                break;
+            }
+        }
+    }
+}
+
+template <int MODE>
+__global__ void __launch_bounds__(32 * kCoopWarps) k_walk_coop(const __grid_constant__ WalkArgs A,
+                                                             const __grid_constant__ WalkParams wp) {
     launch_wait();
     __shared__ uint32_t buf[kCoopWarps][kCoopCap];
     const int lane = threadIdx.x & 31;
     uint32_t* E = buf[threadIdx.x >> 5];
-    const unsigned lt = (1u << lane) - 1u;
     const int64_t ng = A.dng ? min(A.ng, (int64_t)*A.dng) : A.ng;
     unsigned long long ipp = 0, ipc = 0, lp = 0, lc = 0;
     for (int64_t k = (int64_t)blockIdx.x * kCoopWarps + (threadIdx.x >> 5); k < ng;
          k += (int64_t)gridDim.x * kCoopWarps) {
         if (!walk_wanted<MODE>(A, k)) continue;
-        const WalkGroup W = walk_group<MODE>(A, wp, k);
-        WalkCount n;
-        uint32_t nj = 0, nown = 0, len = 1;
-        bool fits = true;
+        CoopWalk<MODE> C{A, wp, walk_group<MODE>(A, wp, k), E, lane};
         __syncwarp();
-        if (lane == 0) E[0] = kEntNew | (uint32_t)W.root;
+        if (lane == 0) E[0] = kEntNew | (uint32_t)C.W.root;
         __syncwarp();
-        for (int lev = 0; lev <= kLevels; ++lev) {  // untested entries are nodes of level lev
-            uint32_t grow = 0;  // (an opened node with one child is replaced without growth)
-            bool opened = false;
-            for (uint32_t t = lane; t < len; t += 32) {
-                const uint32_t v = E[t];
-                if (v >> 30) continue;
-                const WalkNode R = A.wn[v];
-                const long long d2 = box_gap2(R, W.glo, W.ghi, W.period);
-                uint32_t r = kEntCell | v;
-                if (d2 < wp.D[lev] || d2 <= W.rcq) {
-                    const uint32_t c = R.a.y >> kLevels;  // leaf: particles; inner: children
-                    if (R.a.x & kWalkLeaf) {
-                        r = kEntLeaf | v;
-                        const uint32_t lb = R.b.w, cnt = c == kWalkCntMax ? A.end[v] - lb : c;
-                        if (lb >= W.gb && lb < W.ge)
-                            nown += cnt;
-                        else
-                            nj += cnt;
-                    } else {
-                        r = kEntOpen | (c - 1u) << kEntBits | R.b.w;
-                        grow += c - 1u;
-                        opened = true;
-                    }
-                }
-                E[t] = r;
-            }
-            if (!__any_sync(0xffffffffu, opened)) break;
-            const uint32_t more = __reduce_add_sync(0xffffffffu, grow);
-            if (len + more > (uint32_t)kCoopCap) {
-                fits = false;
+        // (untested entries are nodes of one level; the last level's are leaves)
+        for (uint32_t len = 1, more;; len += more) {
+            if (!C.test(len, &more)) {
+                C.put_all(len);
                 break;
             }
-            __syncwarp();
-            // in place from the back: an entry never moves to a lower place
-            uint32_t out = len + more;
-            for (int t0 = (int)((len - 1) & ~31u); t0 >= 0; t0 -= 32) {
-                const uint32_t t = (uint32_t)t0 + lane;
-                const uint32_t v = t < len ? E[t] : 0u;
-                const bool op = t < len && v >= kEntOpen;
-                const uint32_t c = t < len ? (op ? ((v >> kEntBits) & 7u) + 1u : 1u) : 0u;
-                uint32_t tot;
-                const uint32_t x = warp_exclusive(c, lane, &tot);
-                out -= tot;
-                __syncwarp();
-                if (op) {
-                    const uint32_t f = v & ((1u << kEntBits) - 1u);
-                    for (uint32_t u = 0; u < c; ++u) E[out + x + u] = kEntNew | (f + u);
-                } else if (t < len) {
-                    E[out + x] = v;
-                }
-                __syncwarp();
+            if (len + more > kCoopLevel) {
+                coop_pieces<MODE>(C, len);
+                break;
             }
-            len += more;
+            C.expand(len, more);
         }
-        if (fits) {
-            // (the last level's nodes are leaves: nothing is left untested)
-            __syncwarp();
-            for (uint32_t t0 = 0; t0 < len; t0 += 32) {
-                const uint32_t t = t0 + lane;
-                const uint32_t v = t < len ? E[t] : 0u;
-                const bool isP = t < len && (v >> 30) == (kEntLeaf >> 30), isC = t < len && !isP;
-                const unsigned mP = __ballot_sync(0xffffffffu, isP), mC = __ballot_sync(0xffffffffu, isC);
-                if (MODE != kWalkCount) {
-                    const int64_t p = n.np + __popc(mP & lt), c = n.nc + __popc(mC & lt);
-                    if (isP && p < W.capP) W.P[W.baseP + p] = (int32_t)(v & 0x3fffffffu);
-                    if (isC && c < W.capC) W.C[W.baseC + c] = (int32_t)(v & 0x3fffffffu);
-                }
-                n.np += __popc(mP);
-                n.nc += __popc(mC);
-            }
-            n.nj = (int64_t)__reduce_add_sync(0xffffffffu, nj);
-            n.nown = (int64_t)__reduce_add_sync(0xffffffffu, nown);
-        } else if (lane == 0) {
-            n = walk_serial<MODE>(A, wp, W);
-        }
+        WalkCount n;
+        n.np = C.np;
+        n.nc = C.nc;
+        n.nj = (int64_t)__reduce_add_sync(0xffffffffu, C.nj);
+        n.nown = (int64_t)__reduce_add_sync(0xffffffffu, C.nown);
         if (lane == 0) {
-            const int64_t ni = (int64_t)(W.ge - W.gb);
-            walk_counts<MODE>(A, k, W, n);
+            const int64_t ni = (int64_t)(C.W.ge - C.W.gb);
+            walk_counts<MODE>(A, k, C.W, n);
             ipp += (unsigned long long)(ni * (n.nj + n.nown));
             ipc += (unsigned long long)(ni * n.nc);
             lp = max(lp, (unsigned long long)n.np);

@@ -124,3 +124,64 @@ def test_leaf_moments(n, n_leaf, n_g):
     ext = max(np.ptp(P[f]) for f in "xyz")
     for f in ("cx", "cy", "cz"):
         assert np.abs(mo[f] - ref.mom[f]).max() <= 32 * 2.0 ** -24 * ext
+
+
+def test_walk_of_longer_lists():
+    """Lists of 2,000 to 16,000 entries, on a tree with chains of opened nodes down
+    to the last level: a warp's buffer takes them in many pieces, down to
+    pieces of one entry.  Twice, and through the step graphs."""
+    from paper_1907_02289_gb300 import bh
+    P = synth.uniform_cube(24000, 8)
+    rng = np.random.default_rng(2)
+    for c in range(40):  # clumps, of two particles in a last-level cell to a few hundred in many levels
+        i = slice(300 * c, 300 * c + 300)
+        for f in ("x", "y", "z"):
+            P[f][i] = P[f][300 * c] + 10.0 ** -(1 + c % 7) * rng.random(300) ** 4
+    prm = dict(synth.PRESETS["cube4k"]["params"], n_leaf=2, n_g=200)
+    for theta in (0.0, 0.02, 0.2):
+        ctx, D, ref = check_build(P, dict(prm, theta=theta))
+        longest = (np.diff(ref.lists["pp_off"]) + np.diff(ref.lists["pc_off"])).max()
+        assert longest > (12000 if theta == 0.0 else 2048)
+        ctx.bh_build_tree(D)
+        ctx.bh_make_lists()
+        L = ctx.bh_get_lists()
+        for f in ("pp_off", "P", "pc_off", "C"):
+            assert np.array_equal(L[f], ref.lists[f]), f
+        ctx.close()
+    got = []
+    for graph in (0, 1):
+        ctx = bh.Context(**dict(prm, theta=0.2, rebuild_every=2))
+        ctx.bh_set_tuning(graph=graph)
+        D = bh.Particles(P)
+        ctx.bh_step(D, 4)
+        ctx.bh_sync()
+        got.append(ctx.bh_get_lists())
+        assert ctx.bh_get_counters()["n_graph_builds"] == 2 * graph
+        ctx.close()
+    for f in got[0]:
+        assert np.array_equal(got[0][f], got[1][f]), f
+
+
+def test_walk_time_of_long_lists():
+    """A list entry costs about as much in lists that outgrow a warp's buffer
+    (5.7 times as much while such a group was walked by one lane)."""
+    from paper_1907_02289_gb300 import bh
+    per = []
+    for theta in (0.7, 0.4):
+        P = synth.uniform_cube(100003, 3)
+        ctx = bh.Context(**dict(synth.PRESETS["cube4k"]["params"], theta=theta, n_g=64, precision=1))
+        D = bh.Particles(P)
+        ctx.bh_set_timing(True)
+        ms = []
+        for _ in range(6):
+            ctx.bh_get_timing(reset=True)
+            ctx.bh_build_tree(D)
+            ctx.bh_make_lists()
+            ctx.bh_sync()
+            ms.append(ctx.bh_get_counters()["stage_ms"]["lists"])
+        L = ctx.bh_get_lists()
+        n = np.diff(L["pp_off"]) + np.diff(L["pc_off"])
+        assert (n.max() < 2048) == (theta == 0.7) and (theta == 0.7 or n.mean() > 2048)
+        per.append(min(ms) / n.sum())
+        ctx.close()
+    assert per[1] < 2.5 * per[0], per
