@@ -330,7 +330,7 @@ int bh_get_timing(bh_ctx* ctx, double* force_ms, int64_t* force_launches, int re
 typedef struct {
     int n_g;           /* group size limit; a change forces a list build at the next evaluation */
     int chunk;         /* particles of a group per work item at most: 32, 64 or 96
-                          (with too few groups to fill the GPU, 32) */
+                          (where that makes too few items to fill the GPU, 32) */
     int warps;         /* warps per block of the FP32 force kernel, 1..8 */
     int sched;         /* BH_SCHED_* */
     int order_by_cost; /* 0 or 1 */

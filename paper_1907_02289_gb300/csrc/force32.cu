@@ -891,19 +891,23 @@ struct OrderArgs {
     uint32_t chunk;  // largest i-chunk (32, 64 or 96 particles)
     bool by_cost;
     int64_t window;  // groups per window (0: one order over all)
-    int64_t few;     // up to this many groups the i-chunks are of 32
+    int64_t n, few;  // particles, and the items up to which the i-chunks are of 32
 };
 
-// With hardly more groups than warps in flight (fewer than 1.5 per warp) the
-// launch lasts as long as its longest item and warps stay idle, so the items
+// With hardly more items than warps in flight (16 per SM; up to 2.25 items a
+// warp) the launch lasts as long as its longest items and warps stay idle, so the items
 // are single slots: the same bits (a particle's sum does not depend on the
-// chunk it is in), the lists staged more often.  Measured with chunks of 96 and
-// of 32, 2432 warps in flight: evaluation of a 65,537-particle ring (1163
-// groups) 401 and 361 us, forces of 20,000 particles (831) 83.5 and 80.7, of
-// 65,537 (2492) 125 and 100, of 131,072 (4420) 141.0 and 140.8, of 262,144
-// (10,503) 232 and 236, 100,003-particle cube (4096) 584 and 586.
-__host__ __device__ __forceinline__ uint32_t item_chunk(int64_t ng, int64_t few, uint32_t chunk) {
-    return ng <= few ? 32u : chunk;
+// chunk it is in), the lists staged more often.  Items are counted with the
+// chunk that is set: groups and n / chunk.  Force kernel in us with chunks of 96
+// and of 32 (2432 warps in flight): ring of 20,000 particles in groups of up to 64
+// (1042 items) 39 and 33; 65,537 in up to 128 (1856) 88 and 51, in up to 256 (1241)
+// 103 and 66; 131,072 in up to 96 (5207) 100 and 80; 262,144 in up to 256 (5321) 208
+// and 200; beyond, 131,072 in up to 64 (5809) 77 and 78; 262,144 in up to 192 (6585)
+// 168 and 168, in up to 96 (7354) 150 and 160; 2^21 in up to 2048 (24,909, of 3064
+// groups) 3566 and 4313; cube of 100,003 (5137) 170 and 169, of 200,000 (6179) 326 and 339.
+constexpr int kFewItems = 36;  // items per SM
+__host__ __device__ __forceinline__ uint32_t item_chunk(int64_t ng, int64_t n, int64_t few, uint32_t chunk) {
+    return ng + n / chunk <= few ? 32u : chunk;
 }
 
 // An item's i-chunk: its first particle (in slots of 32 from the group's
@@ -943,7 +947,7 @@ __global__ void k_order_hist_windows(const OrderArgs O, uint32_t* cnt) {
     if (k >= O.ng) return;
     uint32_t* mine = cnt + (k / O.window) * kOrderBuckets;
     const uint32_t ni = group_size(O, k);
-    const uint32_t chunk = item_chunk(O.ng, O.few, O.chunk);
+    const uint32_t chunk = item_chunk(O.ng, O.n, O.few, O.chunk);
     for (uint32_t i = 0; i < ni; i += chunk) atomicAdd(&mine[order_bucket(O, k, ni, min(chunk, ni - i))], 1u);
 }
 
@@ -953,7 +957,7 @@ __global__ void k_order_scatter_windows(const OrderArgs O, uint32_t* cursor, int
     if (k >= O.ng) return;
     uint32_t* mine = cursor + (k / O.window) * kOrderBuckets;
     const uint32_t ni = group_size(O, k);
-    const uint32_t chunk = item_chunk(O.ng, O.few, O.chunk);
+    const uint32_t chunk = item_chunk(O.ng, O.n, O.few, O.chunk);
     for (uint32_t i = 0; i < ni; i += chunk) {
         const int64_t at = atomicAdd(&mine[order_bucket(O, k, ni, min(chunk, ni - i))], 1u);
         if (at < cap) order[at] = make_int2((int)k, item_code(i, chunk));
@@ -963,7 +967,7 @@ __global__ void k_order_scatter_windows(const OrderArgs O, uint32_t* cursor, int
 __global__ void k_order_hist(const OrderArgs O, unsigned long long* cnt) {
     launch_wait();
     const int64_t ng = O.dng ? min(O.ng, (int64_t)*O.dng) : O.ng;
-    const uint32_t chunk = item_chunk(ng, O.few, O.chunk);
+    const uint32_t chunk = item_chunk(ng, O.n, O.few, O.chunk);
     for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < ng; k += (int64_t)gridDim.x * blockDim.x) {
         const uint32_t ni = group_size(O, k);
         for (uint32_t i = 0; i < ni; i += chunk) atomicAdd(&cnt[order_bucket(O, k, ni, min(chunk, ni - i))], 1ull);
@@ -975,7 +979,7 @@ __global__ void k_order_scatter(const OrderArgs O, const unsigned long long* cnt
                                 unsigned long long* items) {
     launch_wait();
     const int64_t ng = O.dng ? min(O.ng, (int64_t)*O.dng) : O.ng;
-    const uint32_t chunk = item_chunk(ng, O.few, O.chunk);
+    const uint32_t chunk = item_chunk(ng, O.n, O.few, O.chunk);
     // exclusive prefix of the bucket counts, by the block's first warp
     __shared__ unsigned long long start[kOrderBuckets];
     constexpr int PL = kOrderBuckets / 32;
@@ -1329,16 +1333,15 @@ int resident_blocks(Force32Fn kern, int warps) {
 
 }  // namespace
 
-// Groups up to which the items are single slots (16 warps per SM in flight).
-static int64_t few_groups(const Ctx* c) { return 24 * (int64_t)c->num_sms; }
+static int64_t few_items(const Ctx* c) { return kFewItems * (int64_t)c->num_sms; }
 
 // Work items of the FP32 kernel in processing order (once per list build).
 int build_order32(Ctx* c) {
     const int64_t ng = c->n_groups;
     const uint32_t chunk = (uint32_t)std::min(c->tune.chunk, 32 * BH_F32_MAXR);
-    const int64_t few = few_groups(c);
+    const int64_t few = few_items(c);
     // (device-sized: sized before capture, at most one item per particle)
-    if (!c->dev_build) BH_TRY(grow(c, c->order, (size_t)(ng + c->n / item_chunk(ng, few, chunk) + 1), "work items"));
+    if (!c->dev_build) BH_TRY(grow(c, c->order, (size_t)(ng + c->n / item_chunk(ng, c->n, few, chunk) + 1), "work items"));
     BH_TRY(grow(c, c->order_cnt, 2 * (size_t)kOrderBuckets, "group order buckets"));
     unsigned long long* cnt = c->order_cnt.p;
     unsigned long long* items = c->d_sz + kSzItems;
@@ -1348,7 +1351,7 @@ int build_order32(Ctx* c) {
                       c->cnt_c.p,  chunk,
                       c->tune.order_by_cost != 0,
                       std::max<int64_t>(c->tune.order_window, kLeastWindow),
-                      few};
+                      c->n,        few};
     if (c->tune.order_window > 0 && ng > c->tune.order_window && !c->dev_build) {  // (device-sized: plain order)
         const int64_t words = (ng + O.window - 1) / O.window * kOrderBuckets;
         BH_TRY(grow(c, c->ord_cnt, (size_t)words, "group order buckets of the windows", false));
@@ -1496,7 +1499,7 @@ int launch_force32(Ctx* c, bh_particles* p, const ForceParams& fp, bool add_cent
     }
     unsigned nb;
     const uint32_t chunk =
-        item_chunk(groups_expected(c), few_groups(c), (uint32_t)std::min(c->tune.chunk, 32 * BH_F32_MAXR));
+        item_chunk(groups_expected(c), c->n, few_items(c), (uint32_t)std::min(c->tune.chunk, 32 * BH_F32_MAXR));
     const int64_t items = std::min(A.items_cap, groups_expected(c) + c->n / chunk + 1);  // about (a bound, eagerly)
     if (c->tune.sched == BH_SCHED_GRID && !A.dng) {
         nb = blocks_for(items, W);

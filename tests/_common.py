@@ -69,6 +69,13 @@ def gpu_build(P, prm, precision=None, forces=True, flags=None):
     return ctx, D
 
 
+def many_items(n_groups, n, chunk):
+    """Whether the FP32 force kernel's work items are chunks of the size that is
+    set: more than 36 per SM (fewer are cut to one slot of 32)."""
+    import torch
+    return n_groups + n // chunk > 36 * torch.cuda.get_device_properties(0).multi_processor_count
+
+
 def accel_of(D):
     o = D.numpy()
     return np.stack([o["ax"], o["ay"], o["az"]], 1)

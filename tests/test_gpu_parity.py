@@ -8,7 +8,7 @@ import pytest
 
 import oracle as orc
 from paper_1907_02289_gb300 import synth
-from _common import accel_of, assert_force_close, gpu_build, orc_params
+from _common import accel_of, assert_force_close, gpu_build, many_items, orc_params
 
 pytestmark = pytest.mark.gpu
 
@@ -290,11 +290,11 @@ def test_fp32_every_group_size_class(n_g, chunk):
     """Groups from a few particles to several i-chunks (every slot/tail
     variant of the FP32 kernel and multi-chunk groups, at each i-chunk)."""
     from paper_1907_02289_gb300 import bh
-    P = synth.ring(30000, 21, r_in=0.999, r_out=1.001, phi_max=0.05)
+    P = synth.ring(400000, 21, r_in=0.999, r_out=1.001, phi_max=0.67)
     prm = ring_prm(n_g=n_g, n_leaf=min(8, n_g))
     ref = orc.rebuild(P, orc_params(prm))
     sizes = ref.tree["end"][ref.groups].astype(int) - ref.tree["begin"][ref.groups]
-    assert sizes.max() > min(n_g, chunk) // 2
+    assert sizes.max() > min(n_g, chunk) // 2 and many_items(len(sizes), len(P["x"]), chunk)
     aref = orc.tree_forces(ref, orc_params(prm))
     ctx = bh.Context(**dict(prm, precision=1))
     ctx.bh_set_tuning(chunk=chunk)

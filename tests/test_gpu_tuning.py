@@ -10,7 +10,7 @@ import pytest
 
 import oracle as orc
 from paper_1907_02289_gb300 import synth
-from _common import accel_of, assert_force_close, orc_params
+from _common import accel_of, assert_force_close, many_items, orc_params
 
 pytestmark = pytest.mark.gpu
 
@@ -40,6 +40,16 @@ def ring():
     return P, prm, ref, a_ref
 
 
+@pytest.fixture(scope="module")
+def big_ring():
+    """Enough work items for chunks of every size (few are cut to 32)."""
+    P = synth.ring(300011, 22)
+    prm = _prm(n_g=100)
+    ref = orc.rebuild(P, orc_params(prm))
+    assert many_items(len(ref.groups), len(P["x"]), 96)
+    return P, prm, ref, orc.tree_forces(ref, orc_params(prm))
+
+
 def _forces(P, prm, **tune):
     from paper_1907_02289_gb300 import bh
     ctx = bh.Context(**prm)
@@ -64,16 +74,16 @@ def test_schedules_and_block_sizes_agree(ring, sched, warps):
 
 @pytest.mark.parametrize("chunk", [32, 64, 96])
 @pytest.mark.parametrize("by_cost", [0, 1])
-def test_chunks_and_orders_meet_gate(ring, chunk, by_cost):
-    P, prm, ref, a_ref = ring
+def test_chunks_and_orders_meet_gate(big_ring, chunk, by_cost):
+    P, prm, ref, a_ref = big_ring
     _, D = _forces(P, prm, chunk=chunk, order_by_cost=by_cost, sched=2)
     assert_force_close(accel_of(D), a_ref, 1e-5, f"chunk {chunk}")
 
 
 @pytest.mark.parametrize("window", [64, 256, 100000])
-def test_windowed_order_gives_same_forces(ring, window):
+def test_windowed_order_gives_same_forces(big_ring, window):
     """The processing order never changes a group's arithmetic."""
-    P, prm, ref, a_ref = ring
+    P, prm, ref, a_ref = big_ring
     _, D0 = _forces(P, prm)
     _, D1 = _forces(P, prm, order_window=window)
     np.testing.assert_allclose(accel_of(D1), accel_of(D0), rtol=1e-12, atol=1e-30)
