@@ -825,7 +825,8 @@ int autotune(Ctx* c, bh_particles* p, double* best_ms) {
         return stage_force(c, p, false);
     };
     // (1) launch settings on the current n_g, by force-evaluation time, one
-    // knob at a time: schedule, warps per block, i-chunk, order window
+    // knob at a time: schedule, warps per block, i-chunk, order window (settings
+    // that come to what was measured already are not measured again)
     BH_TRY(time_ms(c, build, &tb));
     double best_f = 1e300;
     bh_tuning best = cur;
@@ -863,17 +864,17 @@ int autotune(Ctx* c, bh_particles* p, double* best_ms) {
         for (int q = 0; q < 3; ++q) {
             bh_tuning t = best;
             t.warps = warps[q];
-            BH_TRY(try_force(t));
+            if (t.warps != best.warps) BH_TRY(try_force(t));
         }
         for (int q = 0; q < 3; ++q) {
             bh_tuning t = best;
             t.chunk = chunks[q];
-            BH_TRY(try_force(t));
+            if (!same_items32(c, t, best)) BH_TRY(try_force(t));
         }
         for (int q = 0; q < 3; ++q) {
             bh_tuning t = best;
             t.order_window = windows[q];
-            BH_TRY(try_force(t));
+            if (!same_items32(c, t, best)) BH_TRY(try_force(t));
         }
     } else {
         BH_TRY(try_force(best));  // the FP64 kernel has no launch settings
@@ -895,10 +896,12 @@ int autotune(Ctx* c, bh_particles* p, double* best_ms) {
             double b = 0.0, f = 1e300;
             BH_TRY(time_ms(c, build, &b));
             BH_TRY(settle());
-            const bool both = c->prm.precision == BH_PREC_FP32 && best.chunk != 96;
+            bh_tuning t96 = t;
+            t96.chunk = 96;
+            const bool both = c->prm.precision == BH_PREC_FP32 && !same_items32(c, t, t96);
             for (int ch = 0; ch < (both ? 2 : 1); ++ch) {
                 if (ch == 1) {
-                    t.chunk = 96;
+                    t = t96;
                     apply_tuning(c, &t);
                     BH_TRY(build_order32(c));
                 }
@@ -930,12 +933,16 @@ int autotune(Ctx* c, bh_particles* p, double* best_ms) {
         BH_TRY(try_force(best));
         const double f_best = best_f;
         const int chunks[3] = {32, 64, 96}, windows[3] = {0, 2048, 8192};
-        const bh_tuning base = best;
+        std::vector<bh_tuning> tried{best};
         for (int q = 0; q < 3; ++q)  // all pairs: the best chunk depends on the window
             for (int w = 0; w < 3; ++w) {
-                bh_tuning t = base;
+                bh_tuning t = tried[0];
                 t.chunk = chunks[q];
                 t.order_window = windows[w];
+                bool known = false;
+                for (const bh_tuning& u : tried) known = known || same_items32(c, t, u);
+                if (known) continue;
+                tried.push_back(t);
                 BH_TRY(try_force(t));
             }
         if (best_ms) *best_ms += best_f - f_best;

@@ -366,6 +366,7 @@ int stage_lists_dev_fill(Ctx* c);                  // device-sized: lists, expan
 
 // force.cu
 int build_order32(Ctx* c);                         // FP32 kernel's work items (per list build)
+bool same_items32(const Ctx* c, const bh_tuning& a, const bh_tuning& b);  // the same items with either's chunk and window
 int reserve_force32(Ctx* c);                       // its buffers
 int stage_force(Ctx* c, bh_particles* p, bool add_central);
 int stage_potential(Ctx* c, const bh_particles* p, double* phi, double* W);  // self-gravity potential (FP64)

@@ -1335,6 +1335,13 @@ int resident_blocks(Force32Fn kern, int warps) {
 
 static int64_t few_items(const Ctx* c) { return kFewItems * (int64_t)c->num_sms; }
 
+// What the settings come to on the current lists (as build_order32 takes them).
+bool same_items32(const Ctx* c, const bh_tuning& a, const bh_tuning& b) {
+    auto chunk = [&](const bh_tuning& t) { return item_chunk(c->n_groups, c->n, few_items(c), (uint32_t)t.chunk); };
+    auto window = [&](const bh_tuning& t) { return c->n_groups > t.order_window ? t.order_window : 0; };
+    return chunk(a) == chunk(b) && window(a) == window(b);
+}
+
 // Work items of the FP32 kernel in processing order (once per list build).
 int build_order32(Ctx* c) {
     const int64_t ng = c->n_groups;

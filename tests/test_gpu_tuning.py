@@ -251,3 +251,29 @@ def test_host_steps_copy_ids_only_when_reordering():
     out = D.numpy()
     for f in bh.Particles.FIELDS:
         assert np.array_equal(H.a[f], out[f]), f
+
+
+@pytest.mark.parametrize("n,most", [(20000, 50), (300011, 99)])
+def test_autotune_measures_a_setting_once(n, most):
+    """Force evaluations of bh_autotune, from its launches: with few items every
+    chunk comes to the same, and a window at or above the group count to none."""
+    from paper_1907_02289_gb300 import bh
+    ctx = bh.Context(**_prm())
+    D = bh.Particles(synth.ring(n, 26))
+
+    def launches(f):
+        k = ctx.bh_get_counters()["n_launches"]
+        f()
+        return ctx.bh_get_counters()["n_launches"] - k
+
+    def build():
+        ctx.bh_build_tree(D)
+        ctx.bh_make_lists()
+
+    build()  # (the first one walks twice)
+    b = launches(build)
+    e = launches(lambda: ctx.bh_compute_forces(D, 1))
+    # list builds: the first, one per n_g, one on the chosen n_g, the last
+    evals = (launches(lambda: ctx.bh_autotune(D)) - 8 * b) / e
+    assert evals <= most, evals
+    ctx.close()
