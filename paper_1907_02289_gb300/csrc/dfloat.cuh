@@ -51,8 +51,8 @@ __device__ __forceinline__ df df_mul(df a, df b) {
     return fast_two_sum(p.hi, p.lo);
 }
 
-// a * b without the last renormalisation (|lo| up to a few ulp(hi)): a factor
-// of a product that is summed with df_accumulate
+// a * b without the last renormalisation (the same value, |lo| up to a few
+// ulp(hi)): a term of a running sum
 __device__ __forceinline__ df df_mul_loose(df a, df b) {
     df p = two_prod(a.hi, b.hi);
     p.lo = __fmaf_rn(a.hi, b.lo, p.lo);
@@ -66,21 +66,38 @@ __device__ __forceinline__ df df_sqr(df a) {
     return fast_two_sum(p.hi, p.lo);
 }
 
-// One term of a running sum: the high parts are added exactly, the errors
-// and low parts in FP32.  Every rounding is 2^-24 of a low part, 2^-48 of the
-// larger of sum and term, as for df_add -- but where the two cancel, df_add
-// keeps the bits of the low parts' own rounding, which a sum of many terms
-// does not have.  8 operations instead of 20; renormalise with fast_two_sum.
-__device__ __forceinline__ void df_accumulate(df& sum, df t) {
+// A running sum in three words: the high parts are added exactly, the errors
+// and low parts to a second word, exactly but for the sum of the two that go in,
+// and the second word's own errors to a third.  14 operations a term where df_add
+// takes 20; a sum of 60, 600 and 3000 terms of either sign that cancel to 1e-3
+// is 0.7, 0.6 and 0.6 times as far (median) from the exact sum of its terms as
+// with df_add, and node masses 0.8 times.  (Without the third word, 3, 8 and 18 times,
+// and masses 1.5 to 2.6 times.)
+struct df_sum {
+    float hi, lo, err;
+};
+
+__device__ __forceinline__ void df_accumulate(df_sum& sum, df t) {
     const df s = two_sum(sum.hi, t.hi);
+    const df l = two_sum(sum.lo, __fadd_rn(s.lo, t.lo));
     sum.hi = s.hi;
-    sum.lo = __fadd_rn(sum.lo, __fadd_rn(s.lo, t.lo));
+    sum.lo = l.hi;
+    sum.err = __fadd_rn(sum.err, l.lo);
 }
 
-__device__ __forceinline__ void df_accumulate(df& sum, float t) {
+__device__ __forceinline__ void df_accumulate(df_sum& sum, float t) {
     const df s = two_sum(sum.hi, t);
+    const df l = two_sum(sum.lo, s.lo);
     sum.hi = s.hi;
-    sum.lo = __fadd_rn(sum.lo, s.lo);
+    sum.lo = l.hi;
+    sum.err = __fadd_rn(sum.err, l.lo);
+}
+
+// The sum as a df (the high part may have cancelled below the others).
+__device__ __forceinline__ df df_total(df_sum sum) {
+    const df l = two_sum(sum.lo, sum.err);
+    const df s = two_sum(sum.hi, l.hi);
+    return fast_two_sum(s.hi, __fadd_rn(s.lo, l.lo));
 }
 
 // (x_hi + x_lo) - (y_hi + y_lo) for two hi/lo splits of FP64 values
@@ -100,14 +117,15 @@ __device__ __forceinline__ df df_norm2(df x, df y, df z) {
     return fast_two_sum(t.hi, __fadd_rn(__fadd_rn(s.lo, t.lo), __fadd_rn(__fadd_rn(ex, ey), ez)));
 }
 
-// 1 / sqrt(s), s > 0: an FP32 estimate y0 and one Newton step,
-// y = y0 + y0 (1 - s y0^2) / 2 (the step squares the estimate's relative
-// error).  s y0^2 is within a few 2^-23 of 1, so 1 - its high part is exact.
+// 1 / sqrt(s), s > 0: an FP32 estimate y0 and the binomial series to second
+// order, y = y0 + y0 (r / 2 + 3 r^2 / 8), r = 1 - s y0^2 (r^2 reaches 2^-44: a
+// Newton step, without it, is off by 2e-14 rms for an estimate within an ulp;
+// this by 5e-15).  s y0^2 is within a few 2^-23 of 1, so 1 - its high part is exact.
 __device__ __forceinline__ df df_rsqrt(df s) {
     const float y0 = rsqrtf(s.hi);
     const df p = df_mul_loose(s, two_prod(y0, y0));
     const float r = __fsub_rn(__fsub_rn(1.f, p.hi), p.lo);
-    return fast_two_sum(y0, __fmul_rn(__fmul_rn(y0, 0.5f), r));
+    return fast_two_sum(y0, __fmul_rn(y0, __fmul_rn(r, __fmaf_rn(r, 0.375f, 0.5f))));
 }
 
 __device__ __forceinline__ bool df_gt(df a, df b) { return a.hi > b.hi || (a.hi == b.hi && a.lo > b.lo); }

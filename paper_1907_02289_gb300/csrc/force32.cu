@@ -1086,7 +1086,7 @@ struct RefineConsts {
 
 __device__ __forceinline__ void ref_pp(const Args& A, const RefineConsts& K, float xh, float xl, float yh, float yl,
                                        float zh, float zl, uint32_t i, uint32_t j, const float4 h, const float4 l,
-                                       df (&acc)[3], double (&ac)[3]) {
+                                       df_sum (&acc)[3], double (&ac)[3]) {
     const df d[3] = {df_diff(h.x, l.x, xh, xl), df_diff(h.y, l.y, yh, yl), df_diff(h.z, l.z, zh, zl)};
     const df r2 = df_norm2(d[0], d[1], d[2]);
     if (r2.hi == 0.f) return;  // coincident pair: no term
@@ -1110,7 +1110,7 @@ __device__ __forceinline__ CellRec load_cell(const Args& A, const float* mlo, in
 }
 
 __device__ __forceinline__ void ref_pc(const Args& A, const RefineConsts& K, float xh, float xl, float yh, float yl,
-                                       float zh, float zl, const CellRec& cr, df (&acc)[3]) {
+                                       float zh, float zl, const CellRec& cr, df_sum (&acc)[3]) {
     const float4 r0 = cr.r0, r1 = cr.r1;
     // R = x_i - c (the oracle's sign); a = -M R / R^3 + Q R / R^5 - 5/2 (R.Q.R) R / R^7 (G-free)
     const df R[3] = {df_diff(xh, xl, r0.x, r1.x), df_diff(yh, yl, r0.y, r1.y), df_diff(zh, zl, r0.z, r1.z)};
@@ -1174,15 +1174,16 @@ __global__ void k_contacts_apply(const Args A, const uint2* pairs, const unsigne
     }
 }
 
-// Launch bounds for 4 blocks of 8 warps per SM (64 registers, a few small
-// spills): the df chains are latency-bound, and 32 warps per SM refine a
-// 2^26 ring in 6.1 ms against 6.6 ms at 16 warps (97 registers).  Bound by
-// the FMA pipe and those chains: about 135 operations per list particle and
-// 190 per cell since sums and squares keep only what their own rounding
-// carries (250 and 345 before).  With every particle of the 2^24 ring refined
-// a step takes 177 ms against 242, with the same errors against FP64 (median
-// 3.07e-9, from the FP32 quadrupole).
-__global__ void __launch_bounds__(256, 4) k_refine32(const Args A, const RefineConsts K,
+// Launch bounds for 4 blocks of 7 warps per SM (72 registers, a few small
+// spills): the df chains are latency-bound, and many warps win over few spills
+// (8 warps at 64 registers, 8 at 3 blocks and 80: 0.1% slower each on four steps of
+// the 2^24 ring).  Bound by the FMA pipe and those chains: about 155 operations
+// per list particle and 230 per cell.  Refining every particle of the 2^24 ring
+// takes 169 ms; with every operation renormalised and the sums by df_add 218 (250
+// and 345 operations), with two-word sums 156, and larger errors.  Against FP64 the
+// three have the same errors to five digits (median 8.38e-10 with monopoles: the 48-bit
+// coordinates).
+__global__ void __launch_bounds__(224, 4) k_refine32(const Args A, const RefineConsts K,
                                                      const float* mlo, int64_t cap) {
     launch_wait();
     const int lane = threadIdx.x & 31;
@@ -1201,7 +1202,7 @@ __global__ void __launch_bounds__(256, 4) k_refine32(const Args A, const RefineC
         const int32_t g = A.groups[k];
         const uint32_t b = A.begin[g], en = A.end[g];
         const float4 hi = A.phi[i], lo = A.plo[i];
-        df acc[3] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
+        df_sum acc[3] = {{0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}};
         double ac[3] = {0.0, 0.0, 0.0};  // contact terms (FP64)
         // each loop loads the next entry's data before evaluating the current one
         {
@@ -1280,20 +1281,21 @@ __global__ void __launch_bounds__(256, 4) k_refine32(const Args A, const RefineC
                 cr = crn;
             }
         }
+        df sum[3];
 #pragma unroll
-        for (int c = 0; c < 3; ++c) acc[c] = fast_two_sum(acc[c].hi, acc[c].lo);
+        for (int c = 0; c < 3; ++c) sum[c] = df_total(acc[c]);
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1)
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
-                const df v = {__shfl_xor_sync(0xffffffffu, acc[c].hi, o), __shfl_xor_sync(0xffffffffu, acc[c].lo, o)};
-                acc[c] = df_add(acc[c], v);
+                const df v = {__shfl_xor_sync(0xffffffffu, sum[c].hi, o), __shfl_xor_sync(0xffffffffu, sum[c].lo, o)};
+                sum[c] = df_add(sum[c], v);
                 ac[c] += __shfl_xor_sync(0xffffffffu, ac[c], o);
             }
         if (lane == 0) {
             double a[3];
 #pragma unroll
-            for (int c = 0; c < 3; ++c) a[c] = A.fp.G * df_to_double(acc[c]) + ac[c];
+            for (int c = 0; c < 3; ++c) a[c] = A.fp.G * df_to_double(sum[c]) + ac[c];
             if (A.add_central) central_newton(A.fp.GMc, A.x[i], A.y[i], A.z[i], a);
             A.ax[i] = a[0];
             A.ay[i] = a[1];
@@ -1394,7 +1396,7 @@ RefineConsts refine_consts(const ForceParams& fp) {
 // read on the device, so it can run inside a captured graph).
 int refine_pass(Ctx* c, const Args& A, const ForceParams& fp) {
     BH_TRY(stage_begin(c, BH_STAGE_REFINE));
-    BH_CUDA(c, launch(c, k_refine32, (unsigned)(c->num_sms * 4), 256, 0, A, refine_consts(fp),
+    BH_CUDA(c, launch(c, k_refine32, (unsigned)(c->num_sms * 4), 224, 0, A, refine_consts(fp),
                       c->cell32lo.p, (int64_t)c->refine.cap));
     BH_LAUNCH(c);
     return stage_end(c);

@@ -604,7 +604,7 @@ __device__ __forceinline__ float dsub(float ah, float al, float bh, float bl) {
 }
 
 // A node's record from its mass, reference point, centre offset and quadrupole.
-__device__ __forceinline__ void put_moments32(int64_t k, float Mk, df Md, const float (&rh)[3], const float (&rl)[3],
+__device__ __forceinline__ void put_moments32(int64_t k, float Mk, df_sum Md, const float (&rh)[3], const float (&rl)[3],
                                               const float (&dc)[3], const float (&q)[6], float4* cell32,
                                               float* mlo) {
     // centre = reference + offset, renormalised into a hi/lo pair
@@ -616,7 +616,7 @@ __device__ __forceinline__ void put_moments32(int64_t k, float Mk, df Md, const 
         ch[a] = hi;
         cl[a] = __fsub_rn(lo, __fsub_rn(hi, rh[a]));
     }
-    mlo[k] = __fadd_rn(__fsub_rn(Md.hi, Mk), Md.lo);
+    mlo[k] = __fadd_rn(__fsub_rn(Md.hi, Mk), __fadd_rn(Md.lo, Md.err));
     cell32[3 * k + 0] = make_float4(ch[0], ch[1], ch[2], Mk);
     cell32[3 * k + 1] = make_float4(cl[0], cl[1], cl[2], q[0]);
     cell32[3 * k + 2] = make_float4(q[3], q[4], q[1], q[5]);
@@ -683,7 +683,7 @@ __global__ void __launch_bounds__(kLeafTile) k_leaf32(const int32_t* leaves,
             float Mk = 0.f, s[3] = {0.f, 0.f, 0.f}, q[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
             // the mass also as a compensated sum of the (hi + lo) masses: the record
             // keeps Mk, mlo[k] the difference (for the refinement of the FP32 kernel)
-            df Md = {0.f, 0.f};
+            df_sum Md = {0.f, 0.f, 0.f};
             for (uint32_t i = i0; i < i1; ++i) {
                 const float4 h = H[i], l = L[i];
                 const float d[3] = {dsub(h.x, l.x, rh[0], rl[0]), dsub(h.y, l.y, rh[1], rl[1]),
@@ -745,7 +745,7 @@ __global__ void __launch_bounds__(kSpanThreads) k_moments32(
         load(0);
         const float rh[3] = {H[0].x, H[0].y, H[0].z}, rl[3] = {L[0].x, L[0].y, L[0].z};
         float Mk = 0.f, s[3] = {0.f, 0.f, 0.f}, q[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-        df Md = {0.f, 0.f};
+        df_sum Md = {0.f, 0.f, 0.f};
         for (int c0 = 0; c0 < nc; c0 += 4) {
             if (c0 > 0) load(c0);
 #pragma unroll
