@@ -301,6 +301,18 @@ int bh_get_counters(bh_ctx* ctx, bh_counters* out);
  * Errors: BH_E_INVAL for entries < 0. */
 int bh_set_list_capacity(bh_ctx* ctx, int64_t entries);
 
+/* Bounds of the key sort's look-back (a tile of keys waits for the digit counts
+ * of earlier ones, which running blocks publish).
+ *  wide_from  particles from which the counts have 64 bits, 1..2^27 (the default,
+ *             the least number that 32 bits do not count).
+ *  polls      polls of one tile before it gives up, 0..2^22 (the default).  Then
+ *             the list build fails with BH_E_TIMEOUT: bh_build_tree leaves the
+ *             particles as they were, a step of bh_step ends after its kick and
+ *             drift, not reordered.  It does not happen in a correct run; with 0
+ *             every wait runs out before it begins.
+ * Errors: BH_E_INVAL for values outside those ranges. */
+int bh_set_sort_limits(bh_ctx* ctx, int64_t wide_from, int polls);
+
 /* Measurement hooks.  bh_set_timing(ctx, 1) makes every force-kernel launch,
  * and every stage of the path (BH_STAGE_*), record a pair of CUDA events on
  * the context's stream.  In a step issued as a CUDA graph only the force
@@ -472,10 +484,24 @@ int bh_measure_peak(int kind, double* tflops);
  * array, so calls that can overlap in time (different streams or host
  * threads) race and give wrong results: order them, e.g. on one stream.
  * Errors: BH_E_INVAL (n out of range, NULL or overlapping buffers, device
- * ordinal >= 64), BH_E_CUDA (set-up or launch failure). */
+ * ordinal >= 64), BH_E_CUDA (set-up or launch failure).  A sort that gave up
+ * waiting on the device (see bh_sort_static_status) is not seen by this call. */
 #define BH_SORT_STATIC_MAX_N 4194304
 int bh_sort_keys_static(uint64_t* keys, uint32_t* idx, uint64_t* keys_tmp, uint32_t* idx_tmp, int64_t n,
                         void* stream, char* err, size_t err_len);
+
+/* The same with a bound of the caller's on the sort's waits: polls (0..2^22,
+ * above: 2^22 is bh_sort_keys_static's) of one tile of keys for the counts of an
+ * earlier one before it gives up, which leaves the output incomplete (nothing
+ * is written out of range).  Errors: also BH_E_INVAL for polls out of range. */
+int bh_sort_keys_static_bounded(uint64_t* keys, uint32_t* idx, uint64_t* keys_tmp, uint32_t* idx_tmp, int64_t n,
+                                int polls, void* stream, char* err, size_t err_len);
+
+/* Whether a tile gave up in a sort of the two calls above on the current device
+ * since this was last asked: BH_E_TIMEOUT then (the output of one of them is not
+ * sorted), else BH_OK.  Waits for the stream, which should be the sorts'.
+ * Not for a stream that is being captured.  Errors: also BH_E_CUDA. */
+int bh_sort_static_status(void* stream, char* err, size_t err_len);
 
 /* The FP64 -> FP32 hi/lo split the FP32 path applies to every particle
  * coordinate and mass each evaluation (Sec. 4.7: the single-precision

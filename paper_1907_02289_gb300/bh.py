@@ -23,7 +23,8 @@ SYMBOLS = ("bh_create", "bh_batch_create", "bh_destroy", "bh_last_error", "bh_se
            "bh_get_root", "bh_get_tree", "bh_get_moments", "bh_get_groups", "bh_get_lists",
            "bh_get_counters", "bh_set_timing", "bh_get_timing", "bh_set_tuning", "bh_get_tuning", "bh_autotune",
            "bh_get_balance", "bh_get_diagnostics", "bh_sort_keys_static", "bh_split_f32",
-           "bh_set_list_capacity", "bh_measure_peak", "bh_compute_potential")
+           "bh_set_list_capacity", "bh_measure_peak", "bh_compute_potential", "bh_set_sort_limits",
+           "bh_sort_keys_static_bounded", "bh_sort_static_status")
 BH_SCHED_GRID, BH_SCHED_STATIC, BH_SCHED_DYNAMIC = 0, 1, 2
 BH_SORT_STATIC_MAX_N = 4194304
 STAGES = ("keys", "sort", "permute", "tree", "moments", "groups", "lists", "split", "force", "contacts", "update",
@@ -114,6 +115,10 @@ def load(path: str = LIB_PATH):
     lib.bh_get_balance.argtypes = [P, ctypes.POINTER(ctypes.c_double)]
     lib.bh_get_diagnostics.argtypes = [P, ctypes.POINTER(bh_particles), ctypes.POINTER(bh_diagnostics)]
     lib.bh_sort_keys_static.argtypes = [P, P, P, P, ctypes.c_int64, P, ctypes.c_char_p, ctypes.c_size_t]
+    lib.bh_sort_keys_static_bounded.argtypes = [P, P, P, P, ctypes.c_int64, ctypes.c_int, P, ctypes.c_char_p,
+                                                ctypes.c_size_t]
+    lib.bh_sort_static_status.argtypes = [P, ctypes.c_char_p, ctypes.c_size_t]
+    lib.bh_set_sort_limits.argtypes = [P, ctypes.c_int64, ctypes.c_int]
     lib.bh_split_f32.argtypes = [P, P, P, ctypes.c_int64, P]
     lib.bh_set_list_capacity.argtypes = [P, ctypes.c_int64]
     lib.bh_measure_peak.argtypes = [ctypes.c_int, ctypes.POINTER(ctypes.c_double)]
@@ -168,18 +173,41 @@ def bh_sort_keys_static(keys, idx, keys_tmp, idx_tmp, stream=None):
     elements each.  The call runs with that device current, on the given
     stream (default: that device's current stream).  Nothing is allocated by
     the library; see bh.h for the limits."""
+    return _sort_static("bh_sort_keys_static", keys, idx, keys_tmp, idx_tmp, (), stream)
+
+
+def bh_sort_static_status(stream=None):
+    """Raises BHError (BH_E_TIMEOUT) when a static sort on the current device
+    gave up since this was last asked; waits for the stream."""
+    import torch
+    lib = load()
+    if stream is None:
+        stream = torch.cuda.current_stream().cuda_stream
+    buf = ctypes.create_string_buffer(256)
+    rc = lib.bh_sort_static_status(ctypes.c_void_p(stream), buf, len(buf))
+    if rc != BH_OK:
+        raise BHError(rc, buf.value.decode())
+    return rc
+
+
+def bh_sort_keys_static_bounded(keys, idx, keys_tmp, idx_tmp, polls, stream=None):
+    """bh_sort_keys_static whose tiles give up after the given number of polls
+    (see bh_sort_static_status)."""
+    return _sort_static("bh_sort_keys_static_bounded", keys, idx, keys_tmp, idx_tmp, (int(polls),), stream)
+
+
+def _sort_static(name, keys, idx, keys_tmp, idx_tmp, extra, stream):
     import torch
     n = keys.numel() if isinstance(keys, torch.Tensor) else -1
-    dev = _check_buffers("bh_sort_keys_static", n, [("keys", keys, torch.int64), ("idx", idx, torch.int32),
-                                                     ("keys_tmp", keys_tmp, torch.int64),
-                                                     ("idx_tmp", idx_tmp, torch.int32)])
+    dev = _check_buffers(name, n, [("keys", keys, torch.int64), ("idx", idx, torch.int32),
+                                   ("keys_tmp", keys_tmp, torch.int64), ("idx_tmp", idx_tmp, torch.int32)])
     lib = load()
     with torch.cuda.device(dev):
         if stream is None:
             stream = torch.cuda.current_stream(dev).cuda_stream
         buf = ctypes.create_string_buffer(256)
-        rc = lib.bh_sort_keys_static(keys.data_ptr(), idx.data_ptr(), keys_tmp.data_ptr(), idx_tmp.data_ptr(), n,
-                                     ctypes.c_void_p(stream), buf, len(buf))
+        rc = getattr(lib, name)(keys.data_ptr(), idx.data_ptr(), keys_tmp.data_ptr(), idx_tmp.data_ptr(), n, *extra,
+                                ctypes.c_void_p(stream), buf, len(buf))
     if rc != BH_OK:
         raise BHError(rc, buf.value.decode())
     return rc
@@ -383,6 +411,9 @@ class Context:
 
     def bh_set_list_capacity(self, entries: int):
         return self._chk(self.lib.bh_set_list_capacity(self.h, int(entries)))
+
+    def bh_set_sort_limits(self, wide_from: int = 1 << 27, polls: int = 1 << 22):
+        return self._chk(self.lib.bh_set_sort_limits(self.h, int(wide_from), int(polls)))
 
     def bh_set_timing(self, enable: bool = True):
         return self._chk(self.lib.bh_set_timing(self.h, 1 if enable else 0))

@@ -691,7 +691,9 @@ int graph_rebuild_step(Ctx* c, bh_particles* p) {
     const unsigned long long *sz = c->h_pin, *sm = c->h_pin + kSzWords;  // (24 words)
     BH_CUDA(c, cudaMemcpyAsync(c->h_pin, c->d_sz, kSzWords * sizeof(*sz), cudaMemcpyDeviceToHost, c->stream));
     BH_CUDA(c, cudaMemcpyAsync(c->h_pin + kSzWords, c->d_small, 24 * sizeof(*sm), cudaMemcpyDeviceToHost, c->stream));
-    BH_TRY(read_status(c));
+    const int rc = read_status(c);
+    if (rc == BH_E_TIMEOUT) c->have_tree = c->have_lists = false;  // (the node arrays hold no tree)
+    BH_TRY(rc);
     ++c->n_graph_builds;
     if (sz[kSzOvf] != 0) {
         // a capacity ran out: the step stopped after the kick-drift and the
@@ -1474,6 +1476,16 @@ int bh_get_counters(bh_ctx* ctx, bh_counters* out) {
         out->stage_ms[s] = c->stage_ms[s];
         out->stage_calls[s] = c->stage_calls[s];
     }
+    return BH_OK;
+}
+
+int bh_set_sort_limits(bh_ctx* ctx, int64_t wide_from, int polls) {
+    Ctx* c = (Ctx*)ctx;
+    if (!c) return BH_E_INVAL;
+    if (wide_from < 1 || wide_from > bh::kSortWide) return bh::fail(c, BH_E_INVAL, "wide_from must be in 1..2^27");
+    if (polls < 0 || polls > bh::kSortPolls) return bh::fail(c, BH_E_INVAL, "polls must be in 0..2^22");
+    c->sort_limits = {wide_from, polls};
+    c->rgraph_ok = false;  // (the list-constructing step holds them)
     return BH_OK;
 }
 

@@ -42,6 +42,41 @@ struct DBuf {
     size_t cap = 0;
 };
 
+// ---- sizes of the radix sort (sort.cu) --------------------------------------
+constexpr int kSortThreads = 384;
+constexpr int kSortItems = 12;  // keys per lane of a tile
+// One small particle set is cut into tiles of 4 keys per lane instead, so that
+// more SMs share it and a tile takes less time.  At the line its 391 tiles still
+// run at once (3 blocks on each of 152 SMs).  Sorts of random keys with 4 and with
+// 12 keys per lane: 65,537 keys 75 and 98 us, 400,000 115 and 130, 600,000 134 and
+// 184, 800,000 157 and 193, 1,200,000 204 and 205.
+constexpr int kSortSmallItems = 4;
+constexpr int64_t kSortSmall = 600000;
+constexpr int kRadix = 256;
+constexpr int64_t kSortWide = (int64_t)1 << 27;  // keys from which the look-back words have 64 bits
+constexpr int kSortPolls = 1 << 22;              // look-back polls before a tile gives up
+struct SortLimits {
+    int64_t wide_from;
+    int polls;
+};
+constexpr bool small_tiles(int64_t n, int64_t wide_from) { return n < kSortSmall && n < wide_from; }
+constexpr int64_t sort_tiles(int64_t n, int64_t wide_from) {  // of one set
+    const int64_t tile = kSortThreads * (small_tiles(n, wide_from) ? kSortSmallItems : kSortItems);
+    return (n + tile - 1) / tile;
+}
+// Scratch: look-back words, digit counts and tickets, cleared together at the
+// start of a sort.
+struct SortScratch {
+    int64_t words, total;  // 32-bit words of the look-back part and in all
+};
+constexpr SortScratch sort_scratch(int64_t n, int64_t ntiles, int64_t nslots, int64_t wide_from) {
+    const int64_t words = ntiles * kRadix * (n < wide_from ? 1 : 2);
+    return {words, words + nslots * 8 * kRadix + 8};
+}
+constexpr int64_t sort_scratch_words(int64_t n) {
+    return sort_scratch(n, sort_tiles(n, kSortWide), 1, kSortWide).total;
+}
+
 struct Ctx;
 int fail(Ctx* c, int code, const char* fmt, ...);
 
@@ -141,6 +176,7 @@ struct Ctx {
     DBuf<uint32_t> idx[2];
     int key_cur = 0;           // buffer holding the sorted keys / perm
     DBuf<uint32_t> sort_scratch;  // look-back words, digit counts, tickets
+    SortLimits sort_limits{kSortWide, kSortPolls};
     DBuf<double> pscratch;     // permutation scratch (8 arrays x 8 bytes per particle)
     DBuf<double> cyl;          // cylindrical frame: phi[n], r[n]
     DBuf<unsigned long long> box_part;  // root-box partials (6 per block, as ordered integers)
@@ -346,11 +382,9 @@ int stage_permute(Ctx* c, bh_particles* p);        // gather particle arrays int
 int setup_patches(Ctx* c, int n_patches, const int64_t* off);  // bh_api.cu
 int64_t sort_tiles_for(const std::vector<int64_t>& off, std::vector<uint32_t>* meta, int* nslots);  // sort.cu
 // context-free sort over caller buffers (sort.cu); scratch >= sort_scratch_words(n) words
-int64_t sort_scratch_words(int64_t n);
 cudaError_t sort_setup_device();
 cudaError_t sort_pairs_with(cudaStream_t s, uint64_t* keys, uint32_t* idx, uint64_t* ktmp, uint32_t* itmp,
-                            int64_t n, int num_sms, uint32_t* scratch, int* status);  // (never inside a captured step)
-int sort_launches();                               // kernels of one such sort of more than one tile
+                            int64_t n, int num_sms, uint32_t* scratch, int polls, int* status);
 
 // tree.cu
 int stage_octree(Ctx* c);                          // nodes and groups; sets n_nodes, n_groups

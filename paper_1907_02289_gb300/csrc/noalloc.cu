@@ -12,12 +12,15 @@ namespace bh {
 namespace {
 
 // Largest n this entry point accepts, and the scratch that n needs:
-// 256 look-back words per tile plus the digit counts and tickets (1 MiB holds
-// them, since a tile is more than 4096 keys).
+// look-back words per tile, digit counts and tickets (most at the largest n, or
+// at the largest that small tiles take).
 constexpr int64_t kStaticSortMaxN = BH_SORT_STATIC_MAX_N;
 constexpr int64_t kStaticWords = 256 * (kStaticSortMaxN / 4096) + 128;
+static_assert(sort_scratch_words(kStaticSortMaxN) <= kStaticWords && sort_scratch_words(kSortSmall - 1) <= kStaticWords,
+              "the fixed scratch array holds every sort");
 
 static __device__ __align__(256) uint32_t g_sort_scratch[kStaticWords];
+static __device__ int g_sort_status;  // kStatTimeout once a sort gave up
 
 constexpr int kMaxDevices = 64;
 
@@ -25,6 +28,7 @@ struct DeviceSlot {
     bool ready = false;
     int num_sms = 0;
     uint32_t* scratch = nullptr;
+    int* status = nullptr;
 };
 
 std::mutex g_setup_mu;
@@ -41,12 +45,12 @@ int report(char* err, size_t err_len, int code, const char* fmt, ...) {
 }
 
 // Per-device set-up, done once with the caller's device current: look up the
-// address of g_sort_scratch on that device and raise the downsweep kernel's
-// shared-memory limit there.  A failure is reported and retried next call.
-// The cached address belongs to the device's primary context: it is not valid
+// addresses of g_sort_scratch and g_sort_status on that device and raise the
+// sort kernels' shared-memory limit there.  A failure is reported and retried next call.
+// The cached addresses belong to the device's primary context: they are not valid
 // after that context is destroyed (cudaDeviceReset), after which this entry
 // point must not be called again in the process.
-int device_scratch(uint32_t** out, int* num_sms, char* err, size_t err_len) {
+int device_slot(DeviceSlot* out, char* err, size_t err_len) {
     int dev = -1;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return report(err, err_len, BH_E_CUDA, "cudaGetDevice: %s", cudaGetErrorString(e));
@@ -61,6 +65,11 @@ int device_scratch(uint32_t** out, int* num_sms, char* err, size_t err_len) {
         if (e != cudaSuccess)
             return report(err, err_len, BH_E_CUDA, "cudaGetSymbolAddress(sort scratch) on device %d: %s", dev,
                           cudaGetErrorString(e));
+        void* q = nullptr;
+        e = cudaGetSymbolAddress(&q, g_sort_status);
+        if (e != cudaSuccess)
+            return report(err, err_len, BH_E_CUDA, "cudaGetSymbolAddress(sort status) on device %d: %s", dev,
+                          cudaGetErrorString(e));
         e = sort_setup_device();
         if (e != cudaSuccess)
             return report(err, err_len, BH_E_CUDA, "setting the sort kernel's shared-memory limit on device %d: %s",
@@ -69,10 +78,10 @@ int device_scratch(uint32_t** out, int* num_sms, char* err, size_t err_len) {
         if (e != cudaSuccess)
             return report(err, err_len, BH_E_CUDA, "cudaDeviceGetAttribute: %s", cudaGetErrorString(e));
         s.scratch = static_cast<uint32_t*>(p);
+        s.status = static_cast<int*>(q);
         s.ready = true;
     }
-    *out = s.scratch;
-    *num_sms = s.num_sms;
+    *out = s;
     return BH_OK;
 }
 
@@ -81,12 +90,35 @@ int device_scratch(uint32_t** out, int* num_sms, char* err, size_t err_len) {
 
 extern "C" int bh_sort_keys_static(uint64_t* keys, uint32_t* idx, uint64_t* keys_tmp, uint32_t* idx_tmp, int64_t n,
                                    void* stream, char* err, size_t err_len) {
+    return bh_sort_keys_static_bounded(keys, idx, keys_tmp, idx_tmp, n, bh::kSortPolls, stream, err, err_len);
+}
+
+extern "C" int bh_sort_static_status(void* stream, char* err, size_t err_len) {
+    using namespace bh;
+    if (err && err_len > 0) err[0] = '\0';
+    DeviceSlot slot;
+    const int rc = device_slot(&slot, err, err_len);
+    if (rc != BH_OK) return rc;
+    const cudaStream_t s = (cudaStream_t)stream;
+    int st = 0;
+    cudaError_t e = cudaMemcpyAsync(&st, slot.status, sizeof(int), cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    if (e == cudaSuccess && st) e = cudaMemsetAsync(slot.status, 0, sizeof(int), s);
+    if (e != cudaSuccess) return report(err, err_len, BH_E_CUDA, "sort status: %s", cudaGetErrorString(e));
+    if (st) return report(err, err_len, BH_E_TIMEOUT, "a sort gave up waiting for the counts of a tile");
+    return BH_OK;
+}
+
+extern "C" int bh_sort_keys_static_bounded(uint64_t* keys, uint32_t* idx, uint64_t* keys_tmp, uint32_t* idx_tmp,
+                                           int64_t n, int polls, void* stream, char* err, size_t err_len) {
     using namespace bh;
     if (err && err_len > 0) err[0] = '\0';
     if (n < 0 || n > kStaticSortMaxN)
         return report(err, err_len, BH_E_INVAL,
                       "n = %lld is outside 0..%lld, the largest sort the fixed scratch array holds",
                       (long long)n, (long long)kStaticSortMaxN);
+    if (polls < 0 || polls > kSortPolls)
+        return report(err, err_len, BH_E_INVAL, "polls = %d is outside 0..%d", polls, kSortPolls);
     if (n == 0) return BH_OK;
     if (!keys || !idx || !keys_tmp || !idx_tmp)
         return report(err, err_len, BH_E_INVAL, "null buffer pointer");
@@ -100,16 +132,12 @@ extern "C" int bh_sort_keys_static(uint64_t* keys, uint32_t* idx, uint64_t* keys
                     return report(err, err_len, BH_E_INVAL, "%s and %s overlap (the four buffers must be disjoint)",
                                   name[a], name[b]);
     }
-    if (sort_scratch_words(n) > kStaticWords)
-        return report(err, err_len, BH_E_INVAL, "sort of n = %lld needs %lld scratch words, %lld available",
-                      (long long)n, (long long)sort_scratch_words(n), (long long)kStaticWords);
-    uint32_t* scratch = nullptr;
-    int num_sms = 0;
-    int rc = device_scratch(&scratch, &num_sms, err, err_len);
+    DeviceSlot slot;
+    int rc = device_slot(&slot, err, err_len);
     if (rc != BH_OK) return rc;
-    // (the sort clears the part of the scratch it uses first; no status word:
-    // a look-back that gave up, which cannot happen, would leave keys unsorted)
-    cudaError_t e = sort_pairs_with((cudaStream_t)stream, keys, idx, keys_tmp, idx_tmp, n, num_sms, scratch, nullptr);
+    // (the sort clears the part of the scratch it uses first)
+    cudaError_t e = sort_pairs_with((cudaStream_t)stream, keys, idx, keys_tmp, idx_tmp, n, slot.num_sms, slot.scratch,
+                                    polls, slot.status);
     if (e != cudaSuccess) return report(err, err_len, BH_E_CUDA, "sort launch: %s", cudaGetErrorString(e));
     return BH_OK;
 }

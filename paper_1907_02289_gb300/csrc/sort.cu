@@ -257,25 +257,20 @@ __global__ void k_keys(const double* x, const double* y,
 //
 // Look-back words: digit pass + 1 in the top 4 bits (the words are cleared
 // once per sort, so those of an earlier pass never match), a flag for a
-// running total, and the count; 32 bits below 2^27 keys, else 64.
+// running total, and the count; 32 bits below 2^27 keys, else 64.  A look-back
+// waits for a running block and ends after a bounded number of polls, with an error
+// in the status word; every index it led to is checked against n, and the
+// particles are then left as they were.
+// (Decoupled look-back and one sweep per digit: Merrill and Garland 2016, Adinets and
+// Merrill 2022; the code is this library's own.)
 // Measured against counting, scanning and scattering launches (42 launches,
 // and a host wait for the digit counts): 3,000,001 keys 469 -> 360 us, the
 // evaluation of a 65,537-particle ring 860 -> 675 us.
 // ---------------------------------------------------------------------------
-constexpr int kSortThreads = 384;
 constexpr int kSortWarps = kSortThreads / 32;
-constexpr int kSortItems = 12;                       // keys per lane
 constexpr int kSortTile = kSortThreads * kSortItems; // 4608
-// One small particle set is cut into tiles of 4 keys per lane instead, so that
-// more SMs share it and a tile takes less time (a pass over 65,537 keys 10.5 us
-// -> 6.5 us)
-constexpr int kSortSmallItems = 4;
-constexpr int64_t kSortSmall = 600000;
-constexpr int kRadix = 256;
 constexpr int kSlotShift = 13;                       // kSortTile < 2^13
-constexpr int64_t kSort32 = (int64_t)1 << 27;        // keys that 32-bit look-back words count
 constexpr int kSortHist = 8 * kRadix;                // digit counts per slot
-constexpr int kSortPolls = 1 << 22;                  // look-back polls before a tile gives up
 
 struct TileInfo {
     int64_t start;  // first key of the tile
@@ -379,7 +374,7 @@ template <class W, bool FIRST, int ITEMS>
 __global__ void __launch_bounds__(kSortThreads, 3) k_sweep(
     const uint64_t* kin, const uint32_t* iin, int64_t n, int pass, int ntiles,
     const uint32_t* tmeta, const uint32_t* hist, W* words, uint32_t* ticket,
-    uint64_t* kout, uint32_t* iout, int* status) {
+    uint64_t* kout, uint32_t* iout, int most_polls, int* status) {
     launch_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     SweepSmem<ITEMS>& S = *reinterpret_cast<SweepSmem<ITEMS>*>(smem_raw);
@@ -463,8 +458,8 @@ __global__ void __launch_bounds__(kSortThreads, 3) k_sweep(
             // the tiles that start together all look back over each other
             // (3,000,001 keys: one at a time 358 us, eight 349, 32 400)
             constexpr int LB = 8;
-            int polls = 0;
-            bool done = false;
+            int left = most_polls;
+            bool done = left == 0;  // (0: the wait runs out before it begins)
             for (int t = tile - 1; !done;) {
                 W v[LB];
 #pragma unroll
@@ -479,11 +474,9 @@ __global__ void __launch_bounds__(kSortThreads, 3) k_sweep(
                         got = u + 1;
                     }
                 t -= got;
-                if (got == 0 && ++polls > kSortPolls) {  // (the earlier tile is running: never)
-                    if (status) atomicOr(status, kStatTimeout);
-                    done = true;
-                }
+                if (got == 0 && --left == 0) done = true;  // (the earlier tile is running: never)
             }
+            if (left == 0) atomicOr(status, kStatTimeout);
             Look<W>::store(&mine[tid], tag | Look<W>::kTotal | (excl + (W)total));
         }
         // the patch's first output is its first key's position
@@ -518,30 +511,13 @@ __global__ void __launch_bounds__(kSortThreads, 3) k_sweep(
         if ((int64_t)g[r] < n) iout[g[r]] = S.sidx[r * kSortThreads + tid];
 }
 
-// Scratch of a sort: look-back words, digit counts and tickets, cleared
-// together at its start.
-struct SortScratch {
-    int64_t words, total;  // 32-bit words of the look-back part and in all
-};
-
-SortScratch sort_scratch(int64_t n, int64_t ntiles, int64_t nslots) {
-    SortScratch z;
-    z.words = ntiles * kRadix * (n < kSort32 ? 1 : 2);
-    z.total = z.words + nslots * kSortHist + 8;
-    return z;
-}
-
-int64_t sort_tiles(int64_t n) {  // of one set
-    const int64_t tile = kSortThreads * (n < kSortSmall ? kSortSmallItems : kSortItems);
-    return (n + tile - 1) / tile;
-}
-
 // Sort (key[0]) into (key[0], idx[0]): eight passes, the first one numbering
 // the keys by position.
 template <class W, int ITEMS>
 cudaError_t sort_passes(cudaStream_t s, bool early, uint64_t* const (&kb)[2], uint32_t* const (&ib)[2], int64_t n,
-                        const uint32_t* tmeta, int ntiles, int nslots, int num_sms, uint32_t* scratch, int* status) {
-    const SortScratch z = sort_scratch(n, ntiles, nslots);
+                        const uint32_t* tmeta, int ntiles, int nslots, int num_sms, uint32_t* scratch, SortLimits lim,
+                        int* status) {
+    const SortScratch z = sort_scratch(n, ntiles, nslots, lim.wide_from);
     W* words = reinterpret_cast<W*>(scratch);
     uint32_t* hist = scratch + z.words;
     uint32_t* ticket = hist + (int64_t)nslots * kSortHist;
@@ -557,18 +533,19 @@ cudaError_t sort_passes(cudaStream_t s, bool early, uint64_t* const (&kb)[2], ui
         const int a = pass & 1, b = 1 - a;
         auto kern = pass == 0 ? k_sweep<W, true, ITEMS> : k_sweep<W, false, ITEMS>;
         e = launch_on(s, early, kern, ntiles, kSortThreads, smem, kb[a], ib[a], n, pass, ntiles, tmeta, hist, words,
-                      ticket + pass, kb[b], ib[b], status);
+                      ticket + pass, kb[b], ib[b], lim.polls, status);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
 }
 
 cudaError_t sort_any(cudaStream_t s, bool early, uint64_t* const (&kb)[2], uint32_t* const (&ib)[2], int64_t n,
-                     const uint32_t* tmeta, int ntiles, int nslots, int num_sms, uint32_t* scratch, int* status) {
-    auto run = !tmeta && n < kSortSmall ? sort_passes<uint32_t, kSortSmallItems>
-               : n < kSort32            ? sort_passes<uint32_t, kSortItems>
-                                        : sort_passes<unsigned long long, kSortItems>;
-    return run(s, early, kb, ib, n, tmeta, ntiles, nslots, num_sms, scratch, status);
+                     const uint32_t* tmeta, int ntiles, int nslots, int num_sms, uint32_t* scratch, SortLimits lim,
+                     int* status) {
+    auto run = n >= lim.wide_from               ? sort_passes<unsigned long long, kSortItems>
+               : !tmeta && small_tiles(n, lim.wide_from) ? sort_passes<uint32_t, kSortSmallItems>
+                                                : sort_passes<uint32_t, kSortItems>;
+    return run(s, early, kb, ib, n, tmeta, ntiles, nslots, num_sms, scratch, lim, status);
 }
 constexpr int kSortLaunches = 9;  // kernels of one sort
 
@@ -579,14 +556,15 @@ struct Gather8 {
     const unsigned long long* src[8];
     unsigned long long* dst[8];
     int na;
-    const int* stop;  // status word: with an error in it the particles stay as they are (NULL: not asked)
+    const int* stop;  // status word: with one of stop_bits in it the particles stay as they are
+    int stop_bits;
 };
 
 __global__ void k_gather_all(Gather8 G, unsigned long long* scratch, const uint32_t* perm,
                              int64_t n, int* status) {
     launch_wait();
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n || (G.stop && *G.stop)) return;
+    if (i >= n || (*G.stop & G.stop_bits)) return;
     const uint32_t j = perm[i];
     if (j >= n) {
         atomicOr(status, kStatBounds);
@@ -606,7 +584,7 @@ __global__ void k_gather_all(Gather8 G, unsigned long long* scratch, const uint3
 __global__ void k_copy_back(Gather8 G, const unsigned long long* scratch, int64_t n) {
     launch_wait();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n || (G.stop && *G.stop)) return;
+    if (i >= n || (*G.stop & G.stop_bits)) return;
     unsigned long long v[8];
 #pragma unroll
     for (int a = 0; a < 8; ++a)
@@ -669,16 +647,18 @@ int stage_sort(Ctx* c) {
     const int64_t n = c->n;
     const bool batch = c->n_patches > 1;
     const uint32_t* tmeta = batch ? c->tile_meta.p : nullptr;
-    const int ntiles = batch ? (int)c->n_tiles : (int)sort_tiles(n);
+    const SortLimits lim = c->sort_limits;
+    const int ntiles = batch ? (int)c->n_tiles : (int)sort_tiles(n, lim.wide_from);
     const int nslots = batch ? c->n_sort_slots : ntiles > 1 ? 1 : 0;
-    BH_TRY(grow(c, c->sort_scratch, (size_t)sort_scratch(n, ntiles, nslots).total, "sort scratch"));
+    BH_TRY(grow(c, c->sort_scratch, (size_t)sort_scratch(n, ntiles, nslots, lim.wide_from).total, "sort scratch"));
     if (c->sort_attr_device != c->device) {  // once per device
         BH_CUDA(c, sort_setup_device());
         c->sort_attr_device = c->device;
     }
     uint64_t* const kb[2] = {c->key[0].p, c->key[1].p};
     uint32_t* const ib[2] = {c->idx[0].p, c->idx[1].p};
-    BH_CUDA(c, sort_any(c->stream, !c->capturing, kb, ib, n, tmeta, ntiles, nslots, c->num_sms, c->sort_scratch.p, c->d_status));
+    BH_CUDA(c, sort_any(c->stream, !c->capturing, kb, ib, n, tmeta, ntiles, nslots, c->num_sms, c->sort_scratch.p, lim,
+                        c->d_status));
     c->n_launches += kSortLaunches - (nslots > 0 ? 0 : 1);
     c->key_cur = 0;
     return BH_OK;
@@ -693,7 +673,9 @@ int stage_permute(Ctx* c, bh_particles* p) {
                                    (unsigned long long*)p->m,  (unsigned long long*)p->id};
     const uint32_t* perm = c->idx[c->key_cur].p;
     Gather8 G = {};
-    G.stop = c->dev_build ? nullptr : c->d_status;
+    // (a captured step goes on with any other error in the word: it is one of before the step)
+    G.stop = c->d_status;
+    G.stop_bits = c->dev_build ? kStatTimeout : ~0;
     for (int a = 0; a < 8; ++a)
         if (arrs[a]) {
             G.dst[G.na] = arrs[a];
@@ -726,12 +708,6 @@ int64_t sort_tiles_for(const std::vector<int64_t>& off, std::vector<uint32_t>* m
     return t;
 }
 
-// Context-free form of stage_sort for callers that supply every buffer,
-// ending in (keys, idx) again; nothing here synchronises.
-int64_t sort_scratch_words(int64_t n) {
-    return sort_scratch(n, sort_tiles(n), 1).total;
-}
-
 cudaError_t sort_setup_device() {
     // (the small tiles need less than the default limit)
     const int smem = (int)sizeof(SweepSmem<kSortItems>);
@@ -747,18 +723,19 @@ cudaError_t sort_setup_device() {
     return cudaSuccess;
 }
 
+// Context-free form of stage_sort for callers that supply every buffer,
+// ending in (keys, idx) again; nothing here synchronises.
 cudaError_t sort_pairs_with(cudaStream_t s, uint64_t* keys, uint32_t* idx, uint64_t* ktmp, uint32_t* itmp,
-                            int64_t n, int num_sms, uint32_t* scratch, int* status) {
+                            int64_t n, int num_sms, uint32_t* scratch, int polls, int* status) {
     if (n <= 0) return cudaSuccess;
-    const int ntiles = (int)sort_tiles(n);
+    const int ntiles = (int)sort_tiles(n, kSortWide);
     uint64_t* const kb[2] = {keys, ktmp};
     uint32_t* const ib[2] = {idx, itmp};
     cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;  // (a caller may be capturing its stream)
     const cudaError_t e = cudaStreamIsCapturing(s, &st);
     if (e != cudaSuccess) return e;
     return sort_any(s, st == cudaStreamCaptureStatusNone, kb, ib, n, nullptr, ntiles, ntiles > 1 ? 1 : 0, num_sms,
-                    scratch, status);
+                    scratch, {kSortWide, polls}, status);
 }
-int sort_launches() { return kSortLaunches; }
 
 }  // namespace bh

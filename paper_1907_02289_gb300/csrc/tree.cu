@@ -37,7 +37,10 @@ __device__ __forceinline__ uint32_t compact3(uint64_t x) {
 // two levels: a launch costs 3 to 5 us with its gap, the barrier well under
 // one.  The span_nodes of each pass is where the cluster's 2048 threads, on 8
 // SMs, start to take longer over a level than a launch of its own (the FP64
-// moments early: 8 SMs have 16 FP64 lanes).  A node's particles or children
+// moments early: 8 SMs have 16 FP64 lanes).  A quarter of those values, those and
+// four times those: octree with boxes of a 65,537-particle ring 88, 88 and 106 us,
+// of 262,144 102, 101 and 108; FP32 moments of 65,537 27.5, 27.2 and 33.7, of 2^20
+// 45, 44 and 46; FP64 moments of 4096 131, 139 and 175, of 262,144 239, 242 and 271.  A node's particles or children
 // are loaded several at a time before any of them is used.  Measured with the
 // leaf pass below: force evaluation on kept lists of a 20,000-particle ring 124
 // -> 95 us, evaluation of a 65,537-particle ring 624 -> 540 us, 4 graph steps of
@@ -240,7 +243,7 @@ __global__ void __launch_bounds__(kTreeThreads) k_tree_count(const uint64_t* key
 // counts: sz words kSzLvl.., kSzNg and kSzNl, cut at the node capacity (overflow flagged).
 __global__ void k_tree_sizes(const uint32_t* scan, int64_t ntiles,
                              const unsigned long long* total, unsigned long long cap,
-                             unsigned long long* sz) {
+                             unsigned long long* sz, const int* status) {
     launch_wait();
     const int l = threadIdx.x;
     const unsigned long long nodes = scan[(int64_t)kRowGroups * ntiles], leaf0 = scan[(int64_t)kRowLeaves * ntiles];
@@ -251,7 +254,9 @@ __global__ void k_tree_sizes(const uint32_t* scan, int64_t ntiles,
     if (l == 0) {
         sz[kSzNg] = leaf0 - nodes;
         sz[kSzNl] = *total - leaf0;
-        sz[kSzOvf] = nodes > cap ? kOvfNodes : 0ull;
+        // (keys that a sort which gave up left unsorted make no tree: nothing is built on them)
+        const bool stop = nodes > cap || (*status & kStatTimeout);
+        sz[kSzOvf] = stop ? kOvfNodes : 0ull;
         sz[kSzNeedNodes] = nodes > cap ? nodes : 0ull;
     }
 }
@@ -860,7 +865,7 @@ int stage_octree(Ctx* c) {
     BH_LAUNCH(c);
     BH_TRY(scan_u32(c, cnt, tree_count_words(n), c->d_small));
     BH_CUDA(c, launch(c, k_tree_sizes, 1, 32, 0, cnt, ntiles, c->d_small, dev ? (unsigned long
-                      long)c->cap_nodes : ~0ull, c->d_sz));
+                      long)c->cap_nodes : ~0ull, c->d_sz, c->d_status));
     BH_LAUNCH(c);
     if (dev) {
         c->n_nodes = c->cap_nodes;
