@@ -21,8 +21,9 @@ def _lib():
 
 
 # sort tiles: 1536 keys below 600,000 keys, 4608 from there on; a tile's
-# look-back takes 32 earlier tiles at a time
-@pytest.mark.parametrize("n", [1, 31, 1535, 1536, 1537, 33 * 1536 - 1, 33 * 1536 + 1, 599999, 600000, 600001])
+# look-back takes 8 earlier tiles at a time (all there are, of the ninth tile)
+@pytest.mark.parametrize("n", [1, 31, 1535, 1536, 1537, 8 * 1536, 9 * 1536, 9 * 1536 + 1, 17 * 1536 + 1, 599999,
+                               600000, 600001])
 @pytest.mark.parametrize("kind", ["random", "two digits", "sorted"])
 def test_sort_tiles(n, kind):
     import torch
@@ -109,12 +110,28 @@ def test_walk_of_long_lists():
         assert np.array_equal(L[f], ref.lists[f]), f
 
 
-# a leaf tile holds 128 leaves and 768 particles in shared memory
-@pytest.mark.parametrize("n,n_leaf,n_g", [(5, 8, 64), (1000, 1, 16), (20000, 5, 64), (20000, 6, 64), (20000, 64, 128)])
+# a leaf tile holds 128 leaves and 640 particles in shared memory: "full" leaves of
+# 5 fill it, one of 6 is one particle too many
+@pytest.mark.parametrize("n,n_leaf,n_g", [(5, 8, 64), (1000, 1, 16), (20000, 5, 64), (20000, 6, 64), (20000, 64, 128),
+                                          ("full", 5, 64), ("full + 1", 6, 64)])
 def test_leaf_moments(n, n_leaf, n_g):
-    P = synth.ring(n, n, phi_max=0.2)
-    _, prm = synth.make("ring1m_fp64", 16)
-    prm = dict(prm, n_leaf=n_leaf, n_g=n_g)
+    if isinstance(n, str):
+        rng = np.random.default_rng(4)
+        site = np.repeat(np.arange(256), 5)
+        site = np.append(site, 100) if n_leaf == 6 else site
+        P, n = synth.uniform_cube(len(site), 6), len(site)
+        for f in "xyz":
+            P[f] = rng.random(256)[site]
+        prm = dict(synth.PRESETS["cube4k"]["params"], order=2, n_leaf=n_leaf, n_g=n_g)
+        ref = orc.rebuild(P, orc_params(prm))
+        leaf = ref.tree["nchild"] == 0
+        cnt = (ref.tree["end"].astype(int) - ref.tree["begin"])[leaf][np.argsort(ref.tree["begin"][leaf])]
+        tiles = [cnt[k:k + 128].sum() for k in range(0, len(cnt), 128)]
+        assert sorted(tiles) == ([640, 640] if n_leaf == 5 else [640, 641])
+    else:
+        P = synth.ring(n, n, phi_max=0.2)
+        _, prm = synth.make("ring1m_fp64", 16)
+        prm = dict(prm, n_leaf=n_leaf, n_g=n_g)
     ctx, D, ref = check_build(P, prm, precision=1)
     assert_force_close(accel_of(D), orc.tree_forces(ref, orc_params(prm)), 1e-5)
     mo = ctx.bh_get_moments()
