@@ -755,7 +755,6 @@ int check_tuning(Ctx* c, const bh_tuning* t) {
 }
 
 void apply_tuning(Ctx* c, const bh_tuning* t) {
-    const bool relist = t->n_g != c->prm.n_g || t->chunk != c->tune.chunk || t->order_by_cost != c->tune.order_by_cost;
     if (t->n_g != c->prm.n_g) c->have_lists = false;
     c->prm.n_g = t->n_g;
     c->tune.chunk = t->chunk;
@@ -768,7 +767,6 @@ void apply_tuning(Ctx* c, const bh_tuning* t) {
     c->tune.graph_room = t->graph_room;
     c->graph_ok = false;
     c->rgraph_ok = false;
-    (void)relist;
 }
 
 void read_tuning(const Ctx* c, bh_tuning* t) {
@@ -1070,7 +1068,7 @@ int bh_destroy(bh_ctx* ctx) {
     release(c->M); release(c->cx); release(c->cy);
     release(c->cz); release(c->Q); release(c->cell32); release(c->cell32lo); release(c->refine); release(c->cbnd); release(c->cslot); release(c->cflag); release(c->phi); release(c->plo); release(c->contacts);
     release(c->groups); release(c->leaves); release(c->order); release(c->cnt_p);
-    release(c->cnt_c); release(c->cnt_j); release(c->cnt_jm); release(c->stash_p); release(c->stash_c); release(c->P); release(c->C); release(c->JJ); release(c->ipp);
+    release(c->cnt_c); release(c->cnt_j); release(c->cnt_jm); release(c->stash_p); release(c->stash_c); release(c->P); release(c->C); release(c->JJ);
     release(c->hbuf); release(c->hid);
     for (auto& pr : c->ev_force) {
         cudaEventDestroy(pr.first);

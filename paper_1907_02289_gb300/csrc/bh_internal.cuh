@@ -106,11 +106,11 @@ constexpr uint32_t kWalkCntMax = (1u << 11) - 1;
 
 // Launch tuning of the FP32 force kernel (bh_set_tuning / the autotuner).
 struct Tuning {
-    int chunk = 96;          // largest i-chunk per warp pass: 32, 64 or 96 particles
+    int chunk = 96;          // largest i-chunk of a work item: 32, 64 or 96 particles
     int warps = 4;           // warps per block, 1..8
     int sched = BH_SCHED_DYNAMIC;
     int order_by_cost = 1;   // within a size class, largest estimated cost first
-    int graph = 0;           // capture list-reusing steps of bh_step in a CUDA graph
+    int graph = 0;           // 1: every step of bh_step as a CUDA graph, 2: list-reusing ones only
     int order_window = 0;    // > 0: size-class order within windows of this many groups
     int graph_contact_room = 0;  // > 0: contact candidates a graph step may hold (0: automatic)
     int graph_room = 25;         // percent of room over the last build in a list-constructing graph step
@@ -293,7 +293,6 @@ struct Ctx {
     int64_t n_one_walk_builds = 0;       // list builds whose lists came from one walk
     DBuf<int32_t> P, C;
     DBuf<uint32_t> JJ;
-    DBuf<int64_t> ipp;                   // per group interaction counts (scratch)
 
     // host-buffer stepping
     DBuf<double> hbuf;                   // 10 arrays of n doubles

@@ -13,8 +13,6 @@ struct df {
     float hi, lo;
 };
 
-__device__ __forceinline__ df df_make(float a) { return {a, 0.f}; }
-
 // s + e == a + b exactly, s = fl(a + b) (no condition on the magnitudes)
 __device__ __forceinline__ df two_sum(float a, float b) {
     const float s = __fadd_rn(a, b);

@@ -344,7 +344,10 @@ __device__ __forceinline__ void pp_far_body(const JPair& P, const float2 (&nh)[3
 // discs with Nxx ~ Nyy, so taking Nxx out leaves little of the matrix
 // (rounding error of the term against 64 bits, 4e5 random cells each at
 // theta 0.5: cubic cells 1.532e-7 rms before and after, discs across z
-// 1.523e-7 -> 1.517e-7; taking Nzz out would give 1.540e-7).
+// 1.523e-7 -> 1.517e-7; taking Nzz out would give 1.540e-7; cells of list pairs of
+// rings and sectors across z -0.3% to +0.1%, of cubes -0.3% to +0.1%, of rings
+// across x +0.3% to +0.8%, of which nothing is left in the sums: rms errors
+// of a 131,072-particle ring across x at theta 0.4, 0.5 and 0.8 equal to five digits).
 template <int ORDER, bool EPS>
 __device__ __forceinline__ void pc_body(const CPair& Cp, const float2 (&nh)[3], float2 (&g)[3], float2 eps2) {
     const float2 dx = __fadd2_rn(Cp.x, nh[0]);
@@ -786,7 +789,7 @@ __device__ __forceinline__ unsigned long long global_ns() {
     return t;
 }
 
-// One work item for one warp: an i-chunk of a group (or all of them in turn).
+// One work item for one warp: an i-chunk of a group.
 template <int ORDER, int MODE>
 __device__ __forceinline__ void force_item(const Args& A, Smem32& S, int64_t slot, int lane) {
     const int2 o = A.order[slot];

@@ -47,12 +47,11 @@ __device__ __forceinline__ int64_t count_of(int64_t n, const unsigned long long*
     return v < (unsigned long long)n ? (int64_t)v : n;
 }
 
-// Up to three arrays of one length in one launch: blockIdx.y is the array, its
-// block sums start at blockIdx.y * stride.
+// Up to three arrays of one length in one launch, each scanned in place:
+// blockIdx.y is the array, its block sums start at blockIdx.y * stride.
 template <typename T>
 struct ScanArrays {
-    const T* in[3];
-    T* out[3];
+    T* v[3];
 };
 
 template <typename T>
@@ -61,7 +60,7 @@ __global__ void k_reduce(ScanArrays<T> a, int64_t n, const unsigned long long* d
     launch_wait();
     __shared__ T wt[kThreads / 32];
     __shared__ T tot;
-    const T* in = a.in[blockIdx.y];
+    const T* in = a.v[blockIdx.y];
     sums += blockIdx.y * stride;
     n = count_of(n, dn);
     const int64_t nt = (n + kTile - 1) / kTile;
@@ -79,7 +78,7 @@ __global__ void k_reduce(ScanArrays<T> a, int64_t n, const unsigned long long* d
 }
 
 // One block per array: exclusive scan of the block sums in place; total to
-// d_total[array] and, with close, to element n of the output.
+// d_total[array] and, with close, to the array's element n.
 template <typename T>
 __global__ void k_scan_sums(ScanArrays<T> a, T* sums, int64_t stride, int64_t n, const unsigned long long* dn,
                             unsigned long long* d_total, bool close) {
@@ -98,8 +97,8 @@ __global__ void k_scan_sums(ScanArrays<T> a, T* sums, int64_t stride, int64_t n,
         carry += tot;
         __syncthreads();
     }
-    if (threadIdx.x == 0 && d_total) d_total[blockIdx.y] = (unsigned long long)carry;
-    if (threadIdx.x == 0 && close) a.out[blockIdx.y][n] = carry;
+    if (threadIdx.x == 0) d_total[blockIdx.y] = (unsigned long long)carry;
+    if (threadIdx.x == 0 && close) a.v[blockIdx.y][n] = carry;
 }
 
 // Blocked arrangement: thread t owns items [t*kItems, (t+1)*kItems) of the tile.
@@ -110,8 +109,7 @@ __global__ void k_scan_apply(ScanArrays<T> a, int64_t n, const unsigned long lon
     __shared__ T wt[kThreads / 32];
     __shared__ T tot;
     __shared__ T stage[kTile];
-    const T* in = a.in[blockIdx.y];  // (may be the output)
-    T* out = a.out[blockIdx.y];
+    T* v0 = a.v[blockIdx.y];
     sums += blockIdx.y * stride;
     n = count_of(n, dn);
     const int64_t nt = (n + kTile - 1) / kTile;
@@ -119,7 +117,7 @@ __global__ void k_scan_apply(ScanArrays<T> a, int64_t n, const unsigned long lon
         const int64_t base = tile * kTile;
         for (int k = 0; k < kItems; ++k) {
             int64_t i = base + (int64_t)k * kThreads + threadIdx.x;
-            stage[k * kThreads + threadIdx.x] = (i < n) ? in[i] : T(0);
+            stage[k * kThreads + threadIdx.x] = (i < n) ? v0[i] : T(0);
         }
         __syncthreads();
         T v[kItems], s = 0;
@@ -137,7 +135,7 @@ __global__ void k_scan_apply(ScanArrays<T> a, int64_t n, const unsigned long lon
         __syncthreads();
         for (int k = 0; k < kItems; ++k) {
             int64_t i = base + (int64_t)k * kThreads + threadIdx.x;
-            if (i < n) out[i] = stage[k * kThreads + threadIdx.x];
+            if (i < n) v0[i] = stage[k * kThreads + threadIdx.x];
         }
         __syncthreads();
     }
@@ -164,11 +162,11 @@ int scan_impl(Ctx* c, const ScanArrays<T>& a, int na, int64_t n, unsigned long l
 }  // namespace
 
 int scan_u32(Ctx* c, uint32_t* v, int64_t n, unsigned long long* d_total) {
-    return scan_impl<uint32_t>(c, {{v}, {v}}, 1, n, d_total, nullptr, false);
+    return scan_impl<uint32_t>(c, {{v}}, 1, n, d_total, nullptr, false);
 }
 
 int scan3_i64(Ctx* c, int64_t* const (&v)[3], int64_t n, unsigned long long* d_total, const unsigned long long* dn) {
-    return scan_impl<int64_t>(c, {{v[0], v[1], v[2]}, {v[0], v[1], v[2]}}, 3, n, d_total, dn, true);
+    return scan_impl<int64_t>(c, {{v[0], v[1], v[2]}}, 3, n, d_total, dn, true);
 }
 
 }  // namespace bh

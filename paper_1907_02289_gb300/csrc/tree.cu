@@ -631,14 +631,12 @@ __device__ __forceinline__ void put_moments32(int64_t k, float Mk, df_sum Md, co
 // a block takes kLeafTile consecutive leaves, whose particles are consecutive
 // too; it splits them with coalesced loads, writes the split and keeps it in
 // shared memory, from which a thread per leaf sums the moments (more particles
-// than fit are read back from memory).  Bound by HBM: 32 B read and 32 B
-// written per particle and 52 B per leaf, where a pass of its own re-read the
-// 32 B with a leaf's stride between the lanes.  Split and moments of the 2^24
-// ring, per evaluation: 0.65 -> 0.54 ms.  Room for 640 particles (5 per leaf)
-// lets 10 blocks share an SM, and the masses are summed with the short form of
-// the hi/lo addition (here and in k_moments32), which is a chain per particle:
-// evaluation of a 100,003-particle cube 592 -> 586 us, of a 65,537-particle
-// ring 403 -> 399, four steps of the 2^24 ring 64.1 -> 64.0 ms.
+// than fit are read back from memory).  32 B read and 32 B written per particle and
+// 52 B per leaf, where a pass of its own re-read the 32 B with a leaf's stride
+// between the lanes; it moves about 0.55 of the copy rate, held by the leaves'
+// serial sums between the loads of one tile and the next.  Split and moments of
+// the 2^24 ring, per evaluation: 0.65 -> 0.54 ms.  Room for 640 particles (5 per
+// leaf) lets 10 blocks share an SM (768: four steps of that ring +0.1%).
 constexpr int kLeafTile = 128, kLeafCap = 640;
 
 template <int ORDER>

@@ -413,12 +413,13 @@ struct CoopWalk {
 // The rest of a walk whose tested entries E[0, len) cannot all be opened in the
 // buffer.  E[at, kCoopCap) are the entries whose turn has not come, in order.
 // Those up to the first opened one go to the lists; then a piece from the
-// front of the rest, opened, moves to E[0, ..): as many entries as a quarter of the
-// free room holds (their children's children need room too; a half or a sixth
-// measures the same), at least one.  It is taken level by level until it is settled, or goes back when it does not
-// fit either, by then at least a level further.  Pieces of more than one entry
-// leave kCoopSpare places free, and those of one, a chain down the levels, add
-// at most 7 entries per level, so there is always room for the next one.
+// front of the rest, opened, moves to E[0, ..): as many entries as a quarter of
+// the free room holds (their children's children need room too; a half or a
+// sixth measures the same), at least one.  It is taken level by level until it
+// is settled, or goes back when it does not fit either, by then at least a
+// level further.  Pieces of more than one entry leave kCoopSpare places free,
+// and those of one, a chain down the levels, add at most 7 entries per level,
+// so there is always room for the next one.
 // Measured, the list build of a 1,000,003-particle cube (32,768 groups) with such
 // groups walked by one lane, with k_walk, and with this: 6.4, 1.6 and 1.0 ms at
 // theta 0.5 (2150 entries a group), 13.7, 2.7 and 1.5 ms at theta 0.4 (3500); of a
