@@ -633,10 +633,10 @@ __device__ __forceinline__ void put_moments32(int64_t k, float Mk, df_sum Md, co
 // shared memory, from which a thread per leaf sums the moments (more particles
 // than fit are read back from memory).  32 B read and 32 B written per particle and
 // 52 B per leaf, where a pass of its own re-read the 32 B with a leaf's stride
-// between the lanes; it moves about 0.55 of the copy rate, held by the leaves'
-// serial sums between the loads of one tile and the next.  Split and moments of
-// the 2^24 ring, per evaluation: 0.65 -> 0.54 ms.  Room for 640 particles (5 per
-// leaf) lets 10 blocks share an SM (768: four steps of that ring +0.1%).
+// between the lanes; bound by issue and the loads' latency (2^22 ring: issue slots
+// 68% busy, DRAM at half of its peak).  Split and moments of the 2^24 ring, per
+// evaluation: 0.65 -> 0.54 ms.  Room for 640 particles (5 per leaf) lets 9 blocks
+// share an SM (768: four steps of that ring +0.1%).
 constexpr int kLeafTile = 128, kLeafCap = 640;
 
 template <int ORDER>
