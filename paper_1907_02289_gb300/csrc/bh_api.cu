@@ -546,6 +546,7 @@ int size_dev_build(Ctx* c, const int64_t cap[5]) {
     BH_TRY(grow(c, c->qlo, 3 * (size_t)nodes, "node qlo"));
     BH_TRY(grow(c, c->qhi, 3 * (size_t)nodes, "node qhi"));
     BH_TRY(grow(c, c->wnode, (size_t)nodes, "walk records"));
+    BH_TRY(reserve_sort(c));
     BH_TRY(grow(c, c->tree_cnt, (size_t)tree_count_words(n), "node counts"));
     BH_TRY(grow(c, c->tree_range, (size_t)n, "node ranges"));
     BH_TRY(grow(c, c->tree_top, (size_t)n, "first nodes"));
@@ -933,16 +934,17 @@ int autotune(Ctx* c, bh_particles* p, double* best_ms) {
         BH_TRY(try_force(best));
         const double f_best = best_f;
         const int chunks[3] = {32, 64, 96}, windows[3] = {0, 2048, 8192};
-        std::vector<bh_tuning> tried{best};
+        bh_tuning tried[10] = {best};
+        int ntried = 1;
         for (int q = 0; q < 3; ++q)  // all pairs: the best chunk depends on the window
             for (int w = 0; w < 3; ++w) {
                 bh_tuning t = tried[0];
                 t.chunk = chunks[q];
                 t.order_window = windows[w];
                 bool known = false;
-                for (const bh_tuning& u : tried) known = known || same_items32(c, t, u);
+                for (int u = 0; u < ntried; ++u) known = known || same_items32(c, t, tried[u]);
                 if (known) continue;
-                tried.push_back(t);
+                tried[ntried++] = t;
                 BH_TRY(try_force(t));
             }
         if (best_ms) *best_ms += best_f - f_best;

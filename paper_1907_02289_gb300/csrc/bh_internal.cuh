@@ -377,6 +377,7 @@ int scan3_i64(Ctx* c, int64_t* const (&v)[3], int64_t n, unsigned long long* d_t
 // sort.cu
 int stage_keys(Ctx* c, const bh_particles* p);     // root box + keys (+ status on NaN)
 int stage_sort(Ctx* c);                            // stable LSD radix sort of (key, idx)
+int reserve_sort(Ctx* c);                          // its scratch (before a captured step)
 int stage_permute(Ctx* c, bh_particles* p);        // gather particle arrays into key order
 int setup_patches(Ctx* c, int n_patches, const int64_t* off);  // bh_api.cu
 int64_t sort_tiles_for(const std::vector<int64_t>& off, std::vector<uint32_t>* meta, int* nslots);  // sort.cu

@@ -643,22 +643,34 @@ int stage_keys(Ctx* c, const bh_particles* p) {
     return BH_OK;
 }
 
+// Tiles of the context's sort, and digit-count slots.
+static void sort_shape(const Ctx* c, int* ntiles, int* nslots) {
+    const bool batch = c->n_patches > 1;
+    *ntiles = batch ? (int)c->n_tiles : (int)sort_tiles(c->n, c->sort_limits.wide_from);
+    *nslots = batch ? c->n_sort_slots : *ntiles > 1 ? 1 : 0;
+}
+
+int reserve_sort(Ctx* c) {
+    int ntiles, nslots;
+    sort_shape(c, &ntiles, &nslots);
+    const SortScratch z = sort_scratch(c->n, ntiles, nslots, c->sort_limits.wide_from);
+    return grow(c, c->sort_scratch, (size_t)z.total, "sort scratch");
+}
+
 int stage_sort(Ctx* c) {
     const int64_t n = c->n;
-    const bool batch = c->n_patches > 1;
-    const uint32_t* tmeta = batch ? c->tile_meta.p : nullptr;
-    const SortLimits lim = c->sort_limits;
-    const int ntiles = batch ? (int)c->n_tiles : (int)sort_tiles(n, lim.wide_from);
-    const int nslots = batch ? c->n_sort_slots : ntiles > 1 ? 1 : 0;
-    BH_TRY(grow(c, c->sort_scratch, (size_t)sort_scratch(n, ntiles, nslots, lim.wide_from).total, "sort scratch"));
+    const uint32_t* tmeta = c->n_patches > 1 ? c->tile_meta.p : nullptr;
+    int ntiles, nslots;
+    sort_shape(c, &ntiles, &nslots);
+    BH_TRY(reserve_sort(c));
     if (c->sort_attr_device != c->device) {  // once per device
         BH_CUDA(c, sort_setup_device());
         c->sort_attr_device = c->device;
     }
     uint64_t* const kb[2] = {c->key[0].p, c->key[1].p};
     uint32_t* const ib[2] = {c->idx[0].p, c->idx[1].p};
-    BH_CUDA(c, sort_any(c->stream, !c->capturing, kb, ib, n, tmeta, ntiles, nslots, c->num_sms, c->sort_scratch.p, lim,
-                        c->d_status));
+    BH_CUDA(c, sort_any(c->stream, !c->capturing, kb, ib, n, tmeta, ntiles, nslots, c->num_sms, c->sort_scratch.p,
+                        c->sort_limits, c->d_status));
     c->n_launches += kSortLaunches - (nslots > 0 ? 0 : 1);
     c->key_cur = 0;
     return BH_OK;

@@ -38,6 +38,26 @@ def test_wide_counts_give_the_same_order(sizes):
         assert np.array_equal(a, b)
 
 
+def test_limits_changed_between_graph_steps():
+    """The captured step is made again, with the scratch of the wider counts."""
+    from paper_1907_02289_gb300 import bh
+    P, got = synth.ring(700000, 6), []
+    for wide in (False, True):
+        ctx = bh.Context(**_prm())
+        ctx.bh_set_tuning(graph=1)
+        D = bh.Particles(P)
+        ctx.bh_step(D, 6)
+        if wide:
+            ctx.bh_set_sort_limits(wide_from=1)
+        ctx.bh_step(D, 6)
+        ctx.bh_sync()
+        assert ctx.bh_get_counters()["n_graph_builds"] == 3
+        got.append(D.numpy())
+        ctx.close()
+    for f in got[0]:
+        assert np.array_equal(got[0][f], got[1][f]), f
+
+
 def test_a_wait_that_runs_out_is_reported():
     """No poll allowed: every tile but the first gives up."""
     from paper_1907_02289_gb300 import bh
