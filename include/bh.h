@@ -210,7 +210,7 @@ int bh_create(const bh_params* p, void* stream, bh_ctx** out);
  * the patches one after another, patch q being [offsets[q], offsets[q+1]).
  * Each patch gets its own root box, keys, sort, tree, groups and lists
  * exactly as if it were alone (a patch never interacts with another), but
- * every stage runs once over all patches: one sort, one tree pass per level,
+ * every stage runs once over all patches: one sort, one octree pass,
  * one walk, one force launch.  Trees form a forest whose roots are nodes
  * 0..n_patches-1; node, group and list ids are global.  offsets is a host
  * array of n_patches + 1 entries (copied): offsets[0] = 0, strictly
@@ -293,8 +293,9 @@ int bh_get_tree(bh_ctx* ctx, uint8_t* level, uint32_t* begin, uint32_t* end, int
 int bh_get_moments(bh_ctx* ctx, double* M, double* c3, double* Q6);
 int bh_get_groups(bh_ctx* ctx, int32_t* group_nodes);
 int bh_get_lists(bh_ctx* ctx, int64_t* pp_off, int32_t* pp_ids, int64_t* pc_off, int32_t* pc_ids);
-/* Counters; when timing is on this synchronises the stream to read the
- * stage events. */
+/* Counters, and the times of the stages whose events are complete.  On the FP32
+ * path it waits for the stream after an evaluation, to read its count of refined
+ * particles, and for the list build alone after one. */
 int bh_get_counters(bh_ctx* ctx, bh_counters* out);
 
 /* Change list_capacity (see bh_params) for later list builds; entries >= 0.
@@ -372,7 +373,7 @@ typedef struct {
                           so the warps in flight work on nearby groups whose
                           list data share L2 */
     int graph_contact_room; /* contact candidates a graph step may hold: 0 = twice
-                          the last eager evaluation's count + 65536; n > 0 = n.
+                          the last evaluation's count that was read + 65536; n > 0 = n.
                           More candidates than that in a graph step are
                           dropped and reported as BH_E_LIST_OVERFLOW at the
                           next synchronising call (that step's contact terms
